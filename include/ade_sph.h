@@ -145,7 +145,8 @@ int ade_get_info(const ade_ctx *ctx, ade_info *info_host);
  * caller's particle order), sorted particle copy and the cell start table. */
 int ade_build_cells(ade_ctx *ctx, void *stream);
 
-/* Copy the last cell build out: perm_dev [n] (caller index at each sorted position) and
+/* Copy the last cell build out (after steps: the list of the positions the last step started
+ * from): perm_dev [n] (caller index at each sorted position) and
  * cell_start_dev [ncells + 1] (cell c holds sorted positions cell_start[c] .. cell_start[c+1]-1).
  * Either pointer may be NULL. */
 int ade_get_cells(ade_ctx *ctx, uint32_t *perm_dev, uint32_t *cell_start_dev, void *stream);
@@ -160,12 +161,17 @@ int ade_count_pairs(ade_ctx *ctx, long long *pairs_host, void *stream);
 
 /* nsteps predictor-corrector steps (Eq. 8-9), each: cell build, rate at level l with the fused
  * predictor, rate at level l+1/2 with the fused corrector (which writes one partial of sum C,
- * min C and max C per warp), and the fold of those partials into the step's FP64 statistics. */
+ * min C and max C per warp), and the fold of those partials into the step's FP64 statistics.
+ * In a uniform flow the separations do not change: a call of several steps on a context with
+ * flags = 0 builds the cell list and the pair weights once and evaluates every step from them
+ * (the workspace holds them unless they would exceed 16 GB); results are the same bits as one step
+ * at a time, and as any split of the steps into calls. */
 int ade_step(ade_ctx *ctx, int nsteps, void *stream);
 
 /* As ade_step, replaying captured CUDA graphs: one graph of 32 steps per whole multiple of 32
- * (no launch gap between those steps) and a graph of one step for the rest (each captured on the
- * first call that needs it, outside any capture of the caller's).  With stats_host non-NULL it
+ * (no launch gap between those steps) and one of the remaining steps (a graph of one step, where the
+ * pair weights are not kept), each captured on the first call that needs it, outside any capture of
+ * the caller's.  With stats_host non-NULL it
  * waits for the stream and fills in the last step's statistics (those of the state it wrote; with
  * nsteps = 0, those of the current state as ade_get_stats); with NULL it only enqueues. */
 int ade_run(ade_ctx *ctx, int nsteps, ade_stats *stats_host, void *stream);
@@ -294,7 +300,8 @@ int ade_batch_init(ade_batch **out, int nplumes, const ade_params *p, const int 
 /* nsteps predictor-corrector steps (Eq. 8-9) of every plume, each with its own time step. */
 int ade_batch_step(ade_batch *b, int nsteps, void *stream);
 
-/* As ade_batch_step, replaying one captured CUDA graph per step; only enqueues. */
+/* As ade_batch_step, replaying captured CUDA graphs (of up to 32 steps where several steps share the
+ * pair weights, as in ade_step); only enqueues. */
 int ade_batch_run(ade_batch *b, int nsteps, void *stream);
 
 /* FP64 per-plume mass, min and max (stats_host[nplumes]); waits for the stream. */

@@ -32,11 +32,11 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
                        Args... args)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
@@ -47,6 +47,24 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, 
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
+
+// Origin of the cell grid of a build, in fixed-point words.  Steps of a uniform flow build their
+// cells in a frame that moves with the particles (origin = steps taken x the drift per step), so a
+// particle stays in its cell, and a run gives the same bits wherever it is split into calls and
+// whether the list is rebuilt or kept for a call's next steps.  words[0..2]: the next build's
+// origin; words[4..6]: the last build's.  A build moves words[0..2] to words[4..6] and advances
+// words[0..2] by adv.  words NULL: origin `add` (0: the absolute grid).  A batch holds kFrameWords
+// words per plume, advanced by `steps` times the plume's drift per step (corr[p].inc).
+struct RateParams;
+struct CellFrame {
+    uint32_t *words = nullptr;
+    uint32_t adv[3] = {0u, 0u, 0u};
+    uint32_t add[3] = {0u, 0u, 0u};
+    const RateParams *corr = nullptr;
+    int plumes = 0;
+    uint32_t steps = 0u;
+};
+constexpr int kFrameWords = 8;
 
 // One row of the neighbour-cell stencil: cells (cx - w .. cx + w, cy + dy, cz + dz).
 struct StencilRow {
@@ -86,6 +104,7 @@ struct RateParams {
     int goff;        // batched plumes: first particle (caller and sorted order) of this plume
     int coff;        // batched plumes: first cell of this plume in the global cell table
     int m1;               // -1: the multiplier of the walks' separations (see sep in rate_common.cuh)
+    const uint32_t *frame;   // cell frame of the last build (CellFrame words; NULL: the absolute grid)
     const uint4 *pencil;  // trimmed walks: per pencil (cy, cz) the transverse bounding box
                           // {min y, max y, min z, max z} of its particles at the cell build
 };
@@ -136,6 +155,30 @@ struct SweepOut {
     unsigned long long *pairs;    // pair counter (counting launch)
 };
 
+// Weight table of the evaluations over one cell list (rate_frozen.cu): `cap` lines of 32 words, handed
+// out by an atomic cursor; slots[chunk] = {first line of the chunk's stream, rows, lines, -}.
+constexpr int kFrozenThreads = 128;
+struct FrozenTab {
+    float *words;
+    uint4 *slots;
+    unsigned *cursor;
+    unsigned cap;
+};
+// Concentrations (and Eq. 14's flux) of such a run in sorted order: C at level l, Ch at l + 1/2, each
+// pencil's twice back to back ([2n] words).
+struct FrozenState {
+    float *C, *Ch;
+    float *Q;             // Eq. 14: caller order (read by the build, written by the finish); NULL: Eq. 1
+    float *Qs, *Qh;       // sorted, at l and l + 1/2
+    float tau_inv;
+};
+
+// Batched plumes: chunks y, y + ny, ... of one pencil of one plume; p0: pencils of the plumes before it.
+struct FrozenItem {
+    int plume, pencil, p0;
+    unsigned short y, ny;
+};
+
 // One work item of the batched rate kernel: `count` sorted particles of plume `plume` starting
 // at plume-local sorted index `start`.
 struct BatchTile {
@@ -170,6 +213,7 @@ struct Work {
     uint4 *P0;             // [n] sorted {x, y, z, C} at level l
     uint4 *P1;             // [n] sorted state at level l + 1/2
     uint4 *pencil = nullptr;  // [ncy * ncz] transverse bounding boxes of the pencils (NULL: not built)
+    uint32_t *frame = nullptr;                 // CellFrame words of the steps (NULL: absolute grid)
     uint32_t *tile_sums = nullptr;             // [tiles of 4096 cells, 128 B apart] totals for the one-pass scan
                                                // (k_count adds, k_place clears; null: multi-launch scan)
     double *partials;      // per-block reduction partials (state statistics)
@@ -208,11 +252,14 @@ int cell_build_launches(int n, int ncells, bool onepass);
 // count_zero: w.count[0, ncells) is known to be zero (every build leaves it zero), so the memset
 // that otherwise starts the build is skipped.
 cudaError_t launch_build_cells(int dim, const uint32_t *xq, const float *C, int n, const int *nc,
-                               int ncells, const Work &w, cudaStream_t s, bool count_zero = false);
+                               int ncells, const Work &w, cudaStream_t s, bool count_zero = false,
+                               const CellFrame &frame = CellFrame());
+// Writes a CellFrame's words: the next build's origin, and the last build's.
+cudaError_t launch_set_frame(uint32_t *words, const uint32_t *origin, cudaStream_t s);
 // Batched plumes: keys are coff_p + local key; plume_of[i] gives the plume of caller particle i.
 cudaError_t launch_build_cells_batch(int dim, const uint32_t *xq, const float *C, int n, int ncells,
                                      const RateParams *descs, const uint16_t *plume_of,
-                                     const Work &w, cudaStream_t s);
+                                     const Work &w, cudaStream_t s, const CellFrame &frame);
 // paired: the persistent kernel's threads take two adjacent sorted particles (the paired walk).
 cudaError_t launch_rate_batch(int dim, int kernel, int epi, const uint4 *Pe, const uint32_t *cell_start,
                               const uint32_t *perm, const RateParams *descs, const BatchTile *tiles,
@@ -248,6 +295,23 @@ cudaError_t launch_rate_pair(int dim, int kernel, int epi, bool iso, const uint4
 cudaError_t launch_rate_field(int dim, int kernel, int epi, const uint4 *Pe, const uint32_t *cell_start,
                               const uint32_t *perm, const FieldWork &fw, const RateParams &prm,
                               const FieldParams &fp, const EpiOut &out, cudaStream_t s);
+
+// Evaluations over one cell list with stored weights (rate_frozen.cu): the table, one predictor or
+// corrector (prm.dt), and the final state in the caller's order (prm.inc: the drift of all steps).
+cudaError_t launch_frozen_build(int dim, int kernel, bool iso, const uint4 *P, const uint32_t *cs, const uint32_t *perm,
+                                const RateParams &prm, const FrozenTab &tab, const FrozenState &st, cudaStream_t s);
+cudaError_t launch_frozen_rate(int dim, int kernel, bool iso, int epi, const uint4 *P, const uint32_t *cs,
+                               const RateParams &prm, const FrozenTab &tab, const FrozenState &st, cudaStream_t s);
+cudaError_t launch_frozen_finish(int dim, const uint4 *P, const uint32_t *cs, const uint32_t *perm, const RateParams &prm,
+                                 const FrozenTab &tab, const FrozenState &st, const EpiOut &out, cudaStream_t s);
+
+// The same for a batch: the table and the first predictor (build), or one evaluation.
+cudaError_t launch_frozen_batch(int dim, int kernel, int epi, bool build, const uint4 *P, const uint32_t *cs,
+                                const RateParams *descs, const FrozenItem *items, int nitems, const FrozenTab &tab,
+                                const FrozenState &st, cudaStream_t s);
+cudaError_t launch_frozen_finish_batch(int dim, const uint4 *P, const uint32_t *cs, const uint32_t *perm, int n,
+                                       const RateParams *descs, const uint16_t *plume_of, uint32_t steps,
+                                       const FrozenTab &tab, const FrozenState &st, const EpiOut &out, cudaStream_t s);
 
 // Parameter sweep (sweep.cu).
 cudaError_t launch_sweep_gather(const uint32_t *perm, const float *C, int n, int P, int P4, float *Cs,
@@ -291,14 +355,18 @@ struct ade_ctx {
     double t;
     long long step;
     long long pairs;
-    cudaGraph_t graph;             // one step (ade_run)
-    cudaGraphExec_t graph_exec;
-    cudaGraph_t graph_multi;       // kGraphSteps steps (ade_run)
-    cudaGraphExec_t graph_exec_multi;
+    // captured runs of 1..kGraphSteps steps (ade_run), each on the first call that needs it
+    cudaGraph_t graph[ade::kGraphSteps + 1];
+    cudaGraphExec_t graph_exec[ade::kGraphSteps + 1];
     cudaStream_t cap_stream;
     bool status_cleared;
     cudaEvent_t ev[5];    // per-phase timing events (created on first timed step)
     bool ev_ready;
+    bool frame_set;       // w.frame holds the frame of the current step
+    bool cells_framed;    // the last build was a step's (in the moving frame)
+    bool frozen;          // steps of one call may keep the pair weights (frozen_tab)
+    ade::FrozenTab frozen_tab;
+    float *frozen_C;      // [2][2n] concentrations of such a call (FrozenState)
     // velocity-field mode (p.vmax > 0)
     bool field;
     bool field_set;       // a valid field has been copied in

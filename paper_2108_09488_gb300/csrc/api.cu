@@ -305,7 +305,7 @@ void choose_tiles(int dim, int n, const Grid &g, bool iso, unsigned flags, ade::
 
 struct Layout {
     size_t keys, rank, count, block_sums, perm_tmp, perm, cell_start, P0, P1, partials, wpart, stats,
-        cf_partials, status, pairs, pencil, tile_sums, fVc, fDAc, fDBc, fIncC, fV, fDA, fDB, fInc,
+        cf_partials, status, pairs, pencil, tile_sums, frame, fz_words, fz_slots, fz_C, fz_cursor, fVc, fDAc, fDBc, fIncC, fV, fDA, fDB, fInc,
         fbits, Q, Qh, total;
 };
 
@@ -313,7 +313,7 @@ struct Layout {
 // nw_partials: per-warp corrector partials of the widest rate launch.  npencils: pencil boxes of
 // the trimmed walks (0: none).
 Layout layout(int n, int ncells, int nb_partials, int nw_partials, int field_dim = 0, bool catt = false,
-              int npencils = 0)
+              int npencils = 0, size_t fz_lines = 0, size_t fz_slots = 0)
 {
     Layout L;
     size_t off = 0;
@@ -339,6 +339,11 @@ Layout layout(int n, int ncells, int nb_partials, int nw_partials, int field_dim
     L.pairs = take(64);
     L.pencil = npencils > 0 ? take((size_t)npencils * 16) : 0;
     L.tile_sums = take(ade::tile_sums_bytes(ncells));
+    L.frame = take(ade::kFrameWords * 4);
+    L.fz_words = take(fz_lines * 128);
+    L.fz_slots = take(fz_slots * 16);
+    L.fz_C = take(fz_slots > 0 ? (size_t)n * 16 : 0);
+    L.fz_cursor = take(64);
     L.fVc = L.fDAc = L.fDBc = L.fIncC = L.fV = L.fDA = L.fDB = L.fInc = L.fbits = 0;
     if (field_dim) {
         const size_t rec = (size_t)n * 16, rec3 = field_dim == 3 ? (size_t)n * 16 : 16;
@@ -372,9 +377,33 @@ struct Derived {
     int nw_partials;
     int ncells_cap;
     int pencils_cap;     // pencils (ncy * ncz) of the largest grid the context may use
+    size_t fz_lines;     // weight table of multi-step calls: lines (0: none) and chunk slots
+    size_t fz_slots;
     ade::RateParams tiles;
     Layout L;
 };
+
+// Weight table of multi-step calls (rate_frozen.cu) for grid g: expected lines.  A row of a chunk is as
+// long as its longest lane's range: the particles of the row's pencil within the chord that the
+// smallest transverse distance between the two pencils leaves, plus the spread of 32 lanes' counts
+// on an irregular set.  Chunks that find no room are evaluated from the positions.
+size_t frozen_lines(const ade_params &p, double H, int n, const Grid &g)
+{
+    const double per = (double)n / g.ncells;                  // particles per cell
+    const double sx = p.box[0] / g.nc[0], sy = p.box[1] / g.nc[1], sz = p.dim == 3 ? p.box[2] / g.nc[2] : 0.0;
+    double lines = 8.0;
+    for (int r = 0; r < g.nrows; ++r) {
+        const double ey = fmax(abs(g.rows[r].dy) - 1.0, 0.0) * sy, ez = fmax(abs(g.rows[r].dz) - 1.0, 0.0) * sz;
+        const double mu = 2.0 * sqrt(fmax(H * H - ey * ey - ez * ez, 0.0)) / sx * per;
+        lines += mu + 1.2 * sqrt(mu) + 2.5;                   // and the row's first indices, in use and as scratch
+    }
+    const double np = (double)(g.ncells / g.nc[0]);
+    return (size_t)((n / 32.0 + 0.6 * fmin(np, (double)n)) * lines) + 1024;
+}
+
+// Above this the table is left out and every evaluation computes its weights (a few per cent of the
+// device's memory; a plume of 10^6 particles with 31,000 neighbours would need 125 GB).
+constexpr double kFrozenMaxBytes = 16e9;
 
 int derive(const ade_params *p, int n, Derived *d)
 {
@@ -423,10 +452,25 @@ int derive(const ade_params *p, int n, Derived *d)
         }
     }
     d->ncells_cap = ncells_cap;
+    d->fz_lines = d->fz_slots = 0;
+    if (p->flags == 0u && !(p->vmax > 0.0) && n > 0) {
+        // the library's choice of walk: multi-step calls keep the weights, on any grid it may pick
+        size_t lines = 0, slots = 0;
+        for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
+            Grid g;
+            if ((p->cell_subdiv > 0 && k != p->cell_subdiv) || !make_grid(*p, d->Hgrid, k, &g)) continue;
+            lines = std::max(lines, frozen_lines(*p, d->H, n, g));
+            slots = std::max(slots, (size_t)n / 32 + (size_t)(g.ncells / g.nc[0]) + 2);
+        }
+        if (128.0 * (double)lines <= kFrozenMaxBytes) {
+            d->fz_lines = lines;
+            d->fz_slots = slots;
+        }
+    }
     // pencil boxes serve the trimmed walks of the uniform-velocity kernels
     d->pencils_cap = p->vmax > 0.0 ? 0 : pencils_cap;
     d->L = layout(n, ncells_cap, d->nb_partials, d->nw_partials, p->vmax > 0.0 ? p->dim : 0, p->tau > 0.0,
-                  d->pencils_cap);
+                  d->pencils_cap, d->fz_lines, d->fz_slots);
     return ADE_OK;
 }
 
@@ -470,14 +514,29 @@ int clean_counts(ade_ctx *c, cudaStream_t s)
         ADE_CK(cudaMemsetAsync(c->w.count, 0, (size_t)c->ncells_cap * sizeof(uint32_t), s));
         // the one-pass scan's flags and {ticket, epoch}: from then on each scan leaves them valid
         ADE_CK(cudaMemsetAsync(c->w.tile_sums, 0, ade::tile_sums_bytes(c->ncells_cap), s));
+        if (c->frozen) ADE_CK(cudaMemsetAsync(c->frozen_tab.cursor, 0, sizeof(unsigned), s));
         c->count_clean = true;
     }
     return ADE_OK;
 }
 
+// The frame of the steps' cell grids (CellFrame): the drift of the steps taken so far.  Written
+// once per context and after a restore; from then on every step's build advances it.
+int set_frame_once(ade_ctx *c, cudaStream_t s)
+{
+    if (!c->frame_set && !c->field) {
+        uint32_t w[3];
+        for (int i = 0; i < 3; ++i) w[i] = (uint32_t)c->step * c->inc[i];
+        ADE_CK(ade::launch_set_frame(c->w.frame, w, s));
+        c->frame_set = true;
+    }
+    return ADE_OK;
+}
+
 // Enqueue one cell build; in velocity-field mode followed by the permutation of the v and D
-// records into the sorted order.
-int enqueue_cells(ade_ctx *c, cudaStream_t s)
+// records into the sorted order.  steps > 0: the build of that many steps of a uniform flow, in the
+// moving frame; 0: on the absolute grid.
+int enqueue_cells(ade_ctx *c, cudaStream_t s, int steps = 0)
 {
     int rc = need_field(c);
     if (rc) return rc;
@@ -485,7 +544,13 @@ int enqueue_cells(ade_ctx *c, cudaStream_t s)
     if (rc) return rc;
     rc = clean_counts(c, s);
     if (rc) return rc;
-    cudaError_t e = ade::launch_build_cells(c->dim, c->xq, c->C, c->n, c->nc, c->ncells, c->w, s, true);
+    ade::CellFrame frame;
+    c->cells_framed = steps > 0 && !c->field;
+    if (c->cells_framed) {
+        frame.words = c->w.frame;
+        for (int i = 0; i < 3; ++i) frame.adv[i] = (uint32_t)steps * c->inc[i];
+    }
+    cudaError_t e = ade::launch_build_cells(c->dim, c->xq, c->C, c->n, c->nc, c->ncells, c->w, s, true, frame);
     if (e != cudaSuccess) {
         c->count_clean = false;   // a build that did not run to the end may leave counts behind
         return fail(ADE_ERR_CUDA, "%s", cudaGetErrorString(e));
@@ -516,6 +581,7 @@ int enqueue_eval(ade_ctx *c, Phase ph, ade::EpiOut out, cudaStream_t s)
         rp.inc[i] = ph == PREDICTOR ? c->inc_half[i] : (ph == CORRECTOR ? c->inc[i] : 0u);
         rp.back[i] = ph == CORRECTOR ? c->inc_half[i] : 0u;
     }
+    rp.frame = ph == AT_BUILD || c->field ? nullptr : c->w.frame;
     if (c->catt && ph != AT_BUILD) {
         out.Q = c->Q;
         out.Qh = c->Qh;
@@ -552,10 +618,53 @@ int enqueue_fold(ade_ctx *c, cudaStream_t s)
     return ADE_OK;
 }
 
+// Enqueue `steps` predictor-corrector steps with the pair weights computed once (rate_frozen.cu), and
+// the fold of the last one's diagnostics.
+int enqueue_frozen(ade_ctx *c, int steps, cudaStream_t s)
+{
+    int rc = enqueue_cells(c, s, steps);
+    if (rc) return rc;
+    ade::FrozenState st;
+    memset(&st, 0, sizeof(st));
+    st.C = c->frozen_C;
+    st.Ch = c->frozen_C + 2 * (size_t)c->n;
+    if (c->catt) {
+        st.Q = c->Q;
+        st.Qs = reinterpret_cast<float *>(c->w.perm_tmp);   // free until the next build
+        st.Qh = c->Qh;
+        st.tau_inv = (float)(1.0 / c->p.tau);
+    }
+    ade::RateParams rp = c->rp;
+    rp.frame = c->w.frame;
+    for (int i = 0; i < 3; ++i) {
+        rp.back[i] = 0u;
+        rp.inc[i] = (uint32_t)steps * c->inc[i];
+    }
+    const ade::FrozenTab &tab = c->frozen_tab;
+    rp.dt = (float)(0.5 * c->dt);
+    ADE_CK(ade::launch_frozen_build(c->dim, c->p.kernel, c->iso, c->w.P0, c->w.cell_start, c->w.perm, rp, tab, st, s));
+    for (int k = 0; k < steps; ++k) {
+        rp.dt = (float)(0.5 * c->dt);
+        if (k > 0)
+            ADE_CK(ade::launch_frozen_rate(c->dim, c->p.kernel, c->iso, ade::EPI_PREDICT, c->w.P0, c->w.cell_start, rp, tab, st, s));
+        rp.dt = (float)c->dt;
+        ADE_CK(ade::launch_frozen_rate(c->dim, c->p.kernel, c->iso, ade::EPI_CORRECT, c->w.P0, c->w.cell_start, rp, tab, st, s));
+    }
+    ADE_CK(ade::launch_frozen_finish(c->dim, c->w.P0, c->w.cell_start, c->w.perm, rp, tab, st, epi_corrector(c), s));
+    ADE_CK(ade::launch_fold_warp_partials(c->w.wpart, ade::rate_blocks(c->n) * (ade::kRateThreads / 32), c->w.stats, s));
+    return ADE_OK;
+}
+
+// Whether `steps` steps of one call keep the pair weights.  Filling the table costs about 1.9 evaluations
+// of the tuned walk, one evaluation from it 0.4 to 0.75: from the third step on it always pays, and on
+// sets below about half a million particles from the second (256^2 28 against 38 us per step, 512^2 68
+// against 72, 700^2 irregular 144 against 153; 1024^2 312 against 285).
+bool use_frozen(const ade_ctx *c, int steps) { return c->frozen && (steps >= 3 || (steps == 2 && c->n <= (1 << 19))); }
+
 // Enqueue one predictor-corrector step (Eq. 8-9) and the fold of its diagnostics.
 int enqueue_step(ade_ctx *c, cudaStream_t s)
 {
-    int rc = enqueue_cells(c, s);
+    int rc = enqueue_cells(c, s, 1);
     if (rc) return rc;
     if (c->n == 0) return ADE_OK;
     ade::EpiOut out = epi_none();
@@ -575,7 +684,8 @@ int clear_status_once(ade_ctx *c, cudaStream_t s)
         ADE_CK(cudaMemsetAsync(c->w.status, 0, sizeof(int), s));
         c->status_cleared = true;
     }
-    return clean_counts(c, s);
+    const int rc = set_frame_once(c, s);
+    return rc ? rc : clean_counts(c, s);
 }
 
 // kc of W'(r)/r = kc f(q) for support H: Wendland C2 (support 2h, f = (1-q)^3) kc = -20 B / H^2;
@@ -774,6 +884,13 @@ int ade_init_particles(ade_ctx **out, const ade_params *p, int n, uint32_t *xq_d
     c->w.pairs = at<unsigned long long>(workspace_dev, d.L.pairs);
     c->w.pencil = d.pencils_cap > 0 ? at<uint4>(workspace_dev, d.L.pencil) : nullptr;
     c->w.tile_sums = at<uint32_t>(workspace_dev, d.L.tile_sums);
+    c->w.frame = at<uint32_t>(workspace_dev, d.L.frame);
+    c->frozen = d.fz_lines > 0;
+    c->frozen_tab.words = at<float>(workspace_dev, d.L.fz_words);
+    c->frozen_tab.slots = at<uint4>(workspace_dev, d.L.fz_slots);
+    c->frozen_C = at<float>(workspace_dev, d.L.fz_C);
+    c->frozen_tab.cursor = at<unsigned>(workspace_dev, d.L.fz_cursor);
+    c->frozen_tab.cap = (unsigned)d.fz_lines;
 
     rc = plume_constants(p, n, d, c->D, &c->dt, c->inc, c->inc_half, &c->rp, &c->iso);
     if (rc) {
@@ -815,23 +932,30 @@ namespace {
 // Forget the captured step graphs (the configuration they were captured with has changed).
 void drop_graphs(ade_ctx *c)
 {
-    if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
-    if (c->graph) cudaGraphDestroy(c->graph);
-    if (c->graph_exec_multi) cudaGraphExecDestroy(c->graph_exec_multi);
-    if (c->graph_multi) cudaGraphDestroy(c->graph_multi);
-    c->graph_exec = nullptr;
-    c->graph = nullptr;
-    c->graph_exec_multi = nullptr;
-    c->graph_multi = nullptr;
+    for (int k = 0; k <= ade::kGraphSteps; ++k) {
+        if (c->graph_exec[k]) cudaGraphExecDestroy(c->graph_exec[k]);
+        if (c->graph[k]) cudaGraphDestroy(c->graph[k]);
+        c->graph_exec[k] = nullptr;
+        c->graph[k] = nullptr;
+    }
 }
 
-// Capture `steps` consecutive steps into one graph.
-int capture_steps(ade_ctx *c, int steps, cudaGraph_t *graph, cudaGraphExec_t *exec)
+// Enqueue `steps` steps of one call.
+int enqueue_steps(ade_ctx *c, int steps, cudaStream_t s)
 {
+    if (use_frozen(c, steps)) return enqueue_frozen(c, steps, s);
+    int rc = ADE_OK;
+    for (int k = 0; k < steps && rc == ADE_OK; ++k) rc = enqueue_step(c, s);
+    return rc;
+}
+
+// Capture `steps` consecutive steps into one graph (once).
+int capture_steps(ade_ctx *c, int steps)
+{
+    if (c->graph_exec[steps]) return ADE_OK;
     if (!c->cap_stream) ADE_CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
     ADE_CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-    int rc = ADE_OK;
-    for (int k = 0; k < steps && rc == ADE_OK; ++k) rc = enqueue_step(c, c->cap_stream);
+    const int rc = enqueue_steps(c, steps, c->cap_stream);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
     if (rc) {
@@ -839,13 +963,13 @@ int capture_steps(ade_ctx *c, int steps, cudaGraph_t *graph, cudaGraphExec_t *ex
         return rc;
     }
     ADE_CK(e);
-    cudaError_t ei = cudaGraphInstantiate(exec, g, 0);
+    cudaError_t ei = cudaGraphInstantiate(&c->graph_exec[steps], g, 0);
     if (ei != cudaSuccess) {
         cudaGraphDestroy(g);
-        *exec = nullptr;
+        c->graph_exec[steps] = nullptr;
         return fail(ADE_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(ei));
     }
-    *graph = g;
+    c->graph[steps] = g;
     return ADE_OK;
 }
 
@@ -1079,6 +1203,16 @@ int ade_get_cells(ade_ctx *c, uint32_t *perm_dev, uint32_t *cell_start_dev, void
 {
     if (!c) return fail(ADE_ERR_ARG, "ctx is NULL");
     cudaStream_t s = (cudaStream_t)stream;
+    if (c->cells_framed && c->n > 0) {
+        // a step built its list in the moving frame: the absolute grid's list of the last step's
+        // positions (the current ones minus one drift)
+        int rc = clean_counts(c, s);
+        if (rc) return rc;
+        ade::CellFrame frame;
+        for (int i = 0; i < 3; ++i) frame.add[i] = c->inc[i];
+        ADE_CK(ade::launch_build_cells(c->dim, c->xq, c->C, c->n, c->nc, c->ncells, c->w, s, true, frame));
+        c->cells_framed = false;
+    }
     if (perm_dev && c->n > 0)
         ADE_CK(cudaMemcpyAsync(perm_dev, c->w.perm, (size_t)c->n * 4, cudaMemcpyDeviceToDevice, s));
     if (cell_start_dev)
@@ -1130,10 +1264,8 @@ int ade_step(ade_ctx *c, int nsteps, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     int rc0 = clear_status_once(c, s);
     if (rc0) return rc0;
-    for (int k = 0; k < nsteps; ++k) {
-        int rc = enqueue_step(c, s);
-        if (rc) return rc;
-    }
+    rc0 = enqueue_steps(c, nsteps, s);
+    if (rc0) return rc0;
     c->step += nsteps;
     c->t += nsteps * c->dt;
     return ADE_OK;
@@ -1179,18 +1311,16 @@ int ade_run(ade_ctx *c, int nsteps, ade_stats *st, void *stream)
     rc0 = refresh_field(c, s);
     if (rc0) return rc0;
     // whole multiples of kGraphSteps replay one graph of kGraphSteps steps (no launch gap between
-    // them), the rest a graph of one step
-    const int nmulti = nsteps / ade::kGraphSteps, nsingle = nsteps % ade::kGraphSteps;
-    if (nmulti > 0 && !c->graph_exec_multi) {
-        int rc = capture_steps(c, ade::kGraphSteps, &c->graph_multi, &c->graph_exec_multi);
-        if (rc) return rc;
-    }
-    if (nsingle > 0 && !c->graph_exec) {
-        int rc = capture_steps(c, 1, &c->graph, &c->graph_exec);
-        if (rc) return rc;
-    }
-    for (int k = 0; k < nmulti; ++k) ADE_CK(cudaGraphLaunch(c->graph_exec_multi, s));
-    for (int k = 0; k < nsingle; ++k) ADE_CK(cudaGraphLaunch(c->graph_exec, s));
+    // them), the rest one graph of the remaining steps where they keep the pair weights, else a graph
+    // of one step
+    const int nmulti = nsteps / ade::kGraphSteps, rest = nsteps % ade::kGraphSteps;
+    const int per = use_frozen(c, rest) ? rest : 1;
+    rc0 = nmulti > 0 ? capture_steps(c, ade::kGraphSteps) : ADE_OK;
+    if (rc0 == ADE_OK && rest > 0) rc0 = capture_steps(c, per);
+    if (rc0) return rc0;
+    for (int k = 0; k < nmulti; ++k) ADE_CK(cudaGraphLaunch(c->graph_exec[ade::kGraphSteps], s));
+    for (int k = 0; k < rest; k += per) ADE_CK(cudaGraphLaunch(c->graph_exec[per], s));
+    c->cells_framed = (nsteps > 0 && !c->field) || c->cells_framed;
     c->step += nsteps;
     c->t += nsteps * c->dt;
     if (!st) return ADE_OK;
@@ -1212,7 +1342,7 @@ int ade_step_timed(ade_ctx *c, double *phase_ms, void *stream)
         c->ev_ready = true;
     }
     ADE_CK(cudaEventRecord(c->ev[0], s));
-    rc = enqueue_cells(c, s);
+    rc = enqueue_cells(c, s, 1);
     if (rc) return rc;
     ADE_CK(cudaEventRecord(c->ev[1], s));
     if (c->n > 0) {
@@ -1344,19 +1474,53 @@ struct ade_batch {
     int max_tiles = 0;
     long long step = 0;
     bool status_cleared = false;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t graph_exec = nullptr;
+    // captured runs of 1..kGraphSteps steps, each on the first call that needs it
+    cudaGraph_t graph[ade::kGraphSteps + 1] = {};
+    cudaGraphExec_t graph_exec[ade::kGraphSteps + 1] = {};
     cudaStream_t cap_stream = nullptr;
+    // weight table of multi-step calls (rate_frozen.cu)
+    bool frozen = false;
+    ade::FrozenTab frozen_tab = {};
+    ade::FrozenItem *d_items = nullptr;
+    float *frozen_C = nullptr;
+    std::vector<ade::FrozenItem> items;
 };
 
 namespace {
 
 struct BatchLayout {
-    size_t keys, rank, count, block_sums, tile_sums, perm_tmp, perm, cell_start, P0, P1, pred, corr, tiles,
+    size_t fz_words, fz_slots, fz_C, fz_cursor, fz_items, frames, keys, rank, count, block_sums, tile_sums, perm_tmp, perm, cell_start, P0, P1, pred, corr, tiles,
         queue, plume_of, offsets, stats, status, pairs, total;
 };
 
-BatchLayout batch_layout(int P, int N, int NC_max, int max_tiles)
+// Size of a batch's weight table over every subdivision its plumes may be given (0: none).
+struct BatchFrozen {
+    size_t lines = 0, pencils = 0, items = 0;
+};
+
+BatchFrozen batch_frozen_size(int P, const ade_params *p, const int *n)
+{
+    BatchFrozen f;
+    for (int i = 0; i < P; ++i) {
+        const double H = p[i].kernel == ADE_WENDLAND_C2 ? 2.0 * p[i].h : p[i].h;
+        size_t lines = 0, pencils = 0, items = 0;
+        for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
+            Grid g;
+            if (!make_grid(p[i], H, k, &g)) continue;
+            const size_t np = (size_t)(g.ncells / g.nc[0]);
+            lines = std::max(lines, frozen_lines(p[i], H, n[i], g));
+            pencils = std::max(pencils, np);
+            items = std::max(items, np + (size_t)n[i] / 32);
+        }
+        f.lines += lines;
+        f.pencils += pencils;
+        f.items += items;
+    }
+    if (128.0 * (double)f.lines > kFrozenMaxBytes) f = BatchFrozen();
+    return f;
+}
+
+BatchLayout batch_layout(int P, int N, int NC_max, int max_tiles, const BatchFrozen &fz)
 {
     BatchLayout L;
     size_t off = 0;
@@ -1365,6 +1529,12 @@ BatchLayout batch_layout(int P, int N, int NC_max, int max_tiles)
         off += align256(bytes > 0 ? bytes : 1);
         return o;
     };
+    L.fz_words = take(fz.lines * 128);
+    L.fz_slots = take(fz.lines > 0 ? ((size_t)N / 32 + fz.pencils + 2) * 16 : 0);
+    L.fz_C = take(fz.lines > 0 ? (size_t)N * 16 : 0);
+    L.fz_cursor = take(64);
+    L.fz_items = take(fz.items * sizeof(ade::FrozenItem));
+    L.frames = take((size_t)P * ade::kFrameWords * 4);
     L.keys = take((size_t)N * 4);
     L.rank = take((size_t)N * 4);
     L.count = take((size_t)NC_max * 4);
@@ -1441,6 +1611,8 @@ int batch_max_tiles(int P, const int *n)
 int batch_plan(ade_batch *b)
 {
     b->NC = 0;
+    b->items.clear();
+    int p0 = 0;
     std::vector<std::pair<double, ade::BatchTile>> items;
     for (int i = 0; i < b->P; ++i) {
         ade_params pp = b->params[i];
@@ -1460,6 +1632,7 @@ int batch_plan(ade_batch *b)
         if (rc) return rc;
         rp.goff = b->offsets[i];
         rp.coff = b->NC;
+        rp.frame = b->w.frame + (size_t)i * ade::kFrameWords;
         b->ncells[i] = d.g.ncells;
         b->subdiv_choice[i] = d.g.subdiv;
         b->NC += d.g.ncells;
@@ -1474,6 +1647,15 @@ int batch_plan(ade_batch *b)
         }
         b->pred[i] = pr;
         b->corr[i] = co;
+        // chunks of the weight table: enough items per pencil for its mean population
+        if (b->frozen) {
+            const int np = d.g.ncells / d.g.nc[0];
+            const int ny = std::max(1, std::min(65535, b->n[i] / np / 32));
+            for (int q = 0; q < np; ++q)
+                for (int y = 0; y < ny; ++y)
+                    b->items.push_back(ade::FrozenItem{i, q, p0, (unsigned short)y, (unsigned short)ny});
+            p0 += np;
+        }
         // work items and their estimated cost: candidates per particle x particles
         const double ppc = (double)b->n[i] / d.g.ncells;
         double cand = 0.0;
@@ -1498,6 +1680,16 @@ int batch_plan(ade_batch *b)
     return ADE_OK;
 }
 
+void batch_drop_graphs(ade_batch *b)
+{
+    for (int k = 0; k <= ade::kGraphSteps; ++k) {
+        if (b->graph_exec[k]) cudaGraphExecDestroy(b->graph_exec[k]);
+        if (b->graph[k]) cudaGraphDestroy(b->graph[k]);
+        b->graph_exec[k] = nullptr;
+        b->graph[k] = nullptr;
+    }
+}
+
 int batch_upload(ade_batch *b, cudaStream_t s)
 {
     ADE_CK(cudaMemcpyAsync(b->d_pred, b->pred.data(), b->P * sizeof(ade::RateParams), cudaMemcpyHostToDevice, s));
@@ -1505,27 +1697,29 @@ int batch_upload(ade_batch *b, cudaStream_t s)
     if (!b->tiles.empty())
         ADE_CK(cudaMemcpyAsync(b->d_tiles, b->tiles.data(), b->tiles.size() * sizeof(ade::BatchTile),
                                cudaMemcpyHostToDevice, s));
+    if (!b->items.empty())
+        ADE_CK(cudaMemcpyAsync(b->d_items, b->items.data(), b->items.size() * sizeof(ade::FrozenItem),
+                               cudaMemcpyHostToDevice, s));
     ADE_CK(cudaStreamSynchronize(s));   // the host vectors may change before the next call
-    if (b->graph_exec) {
-        cudaGraphExecDestroy(b->graph_exec);
-        b->graph_exec = nullptr;
-    }
-    if (b->graph) {
-        cudaGraphDestroy(b->graph);
-        b->graph = nullptr;
-    }
+    batch_drop_graphs(b);
     return ADE_OK;
 }
 
-int batch_cells(ade_batch *b, cudaStream_t s)
+// Cell build of the batch in the plumes' moving frames (CellFrame), which `steps` steps advance.
+int batch_cells(ade_batch *b, cudaStream_t s, int steps = 0)
 {
-    ADE_CK(ade::launch_build_cells_batch(b->dim, b->xq, b->C, b->N, b->NC, b->d_pred, b->plume_of, b->w, s));
+    ade::CellFrame frame;
+    frame.words = b->w.frame;
+    frame.corr = b->d_corr;
+    frame.plumes = b->P;
+    frame.steps = (uint32_t)steps;
+    ADE_CK(ade::launch_build_cells_batch(b->dim, b->xq, b->C, b->N, b->NC, b->d_pred, b->plume_of, b->w, s, frame));
     return ADE_OK;
 }
 
 int batch_enqueue_step(ade_batch *b, cudaStream_t s)
 {
-    int rc = batch_cells(b, s);
+    int rc = batch_cells(b, s, 1);
     if (rc) return rc;
     ade::EpiOut out = epi_none();
     out.Pout = b->w.P1;
@@ -1537,6 +1731,69 @@ int batch_enqueue_step(ade_batch *b, cudaStream_t s)
     out.status = b->w.status;
     ADE_CK(ade::launch_rate_batch(b->dim, b->kernel, ade::EPI_CORRECT, b->w.P1, b->w.cell_start, b->w.perm,
                                   b->d_corr, b->d_tiles, (int)b->tiles.size(), b->queue, b->grid, out, s, b->paired));
+    return ADE_OK;
+}
+
+// As enqueue_frozen for every plume of the batch.
+int batch_enqueue_frozen(ade_batch *b, int steps, cudaStream_t s)
+{
+    int rc = batch_cells(b, s, steps);
+    if (rc) return rc;
+    ade::FrozenState st;
+    memset(&st, 0, sizeof(st));
+    st.C = b->frozen_C;
+    st.Ch = b->frozen_C + 2 * (size_t)b->N;
+    const int ni = (int)b->items.size();
+    auto eval = [&](int epi, bool build) {
+        return ade::launch_frozen_batch(b->dim, b->kernel, epi, build, b->w.P0, b->w.cell_start,
+                                        epi == ade::EPI_PREDICT ? b->d_pred : b->d_corr, b->d_items, ni, b->frozen_tab, st, s);
+    };
+    // (the weights need the separations only: the correctors' drift since the build plays no part)
+    for (int k = 0; k < steps; ++k) {
+        ADE_CK(eval(ade::EPI_PREDICT, k == 0));
+        ADE_CK(eval(ade::EPI_CORRECT, false));
+    }
+    ade::EpiOut out = epi_none();
+    out.xq = b->xq;
+    out.C = b->C;
+    out.status = b->w.status;
+    ADE_CK(ade::launch_frozen_finish_batch(b->dim, b->w.P0, b->w.cell_start, b->w.perm, b->N, b->d_corr, b->plume_of,
+                                           (uint32_t)steps, b->frozen_tab, st, out, s));
+    return ADE_OK;
+}
+
+// Whether `steps` steps of one call keep the pair weights.
+bool batch_use_frozen(const ade_batch *b, int steps) { return b->frozen && b->N > 0 && steps >= 2; }
+
+int batch_enqueue_steps(ade_batch *b, int steps, cudaStream_t s)
+{
+    if (batch_use_frozen(b, steps)) return batch_enqueue_frozen(b, steps, s);
+    int rc = ADE_OK;
+    for (int k = 0; k < steps && rc == ADE_OK; ++k) rc = batch_enqueue_step(b, s);
+    return rc;
+}
+
+// Capture `steps` steps into one graph (once).
+int batch_capture(ade_batch *b, int steps)
+{
+    if (b->graph_exec[steps]) return ADE_OK;
+    if (!b->cap_stream) ADE_CK(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking));
+    ADE_CK(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
+    const int rc = batch_enqueue_steps(b, steps, b->cap_stream);
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamEndCapture(b->cap_stream, &g);
+    if (rc) {
+        if (g) cudaGraphDestroy(g);
+        return rc;
+    }
+    ADE_CK(e);
+    cudaError_t ei = cudaGraphInstantiate(&b->graph_exec[steps], g, 0);
+    if (ei != cudaSuccess) {
+        cudaGraphDestroy(g);
+        b->graph_exec[steps] = nullptr;
+        return fail(ADE_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(ei));
+    }
+    b->graph[steps] = g;
     return ADE_OK;
 }
 
@@ -1563,7 +1820,7 @@ int ade_batch_workspace_bytes(int nplumes, const ade_params *p, const int *n, si
     if (rc) return rc;
     long long N = 0;
     for (int i = 0; i < nplumes; ++i) N += n[i];
-    *bytes = batch_layout(nplumes, (int)N, (int)ncm, batch_max_tiles(nplumes, n)).total;
+    *bytes = batch_layout(nplumes, (int)N, (int)ncm, batch_max_tiles(nplumes, n), batch_frozen_size(nplumes, p, n)).total;
     return ADE_OK;
 }
 
@@ -1595,7 +1852,8 @@ int ade_batch_init(ade_batch **out, int nplumes, const ade_params *p, const int 
     b->corr.resize(nplumes);
     b->dt.assign(nplumes, 0.0);
     b->D.assign(9 * (size_t)nplumes, 0.0);
-    const BatchLayout L = batch_layout(nplumes, b->N, b->NC_max, b->max_tiles);
+    const BatchFrozen fz = batch_frozen_size(nplumes, p, n);
+    const BatchLayout L = batch_layout(nplumes, b->N, b->NC_max, b->max_tiles, fz);
     if (b->N > 0 && (!xq_dev || !C_dev)) {
         delete b;
         return fail(ADE_ERR_ARG, "xq_dev and C_dev must be non-NULL");
@@ -1621,6 +1879,14 @@ int ade_batch_init(ade_batch **out, int nplumes, const ade_params *p, const int 
     b->w.perm = at<uint32_t>(workspace_dev, L.perm);
     b->w.cell_start = at<uint32_t>(workspace_dev, L.cell_start);
     b->w.tile_sums = at<uint32_t>(workspace_dev, L.tile_sums);   // cleared with the counts every build
+    b->w.frame = at<uint32_t>(workspace_dev, L.frames);
+    b->frozen = fz.lines > 0;
+    b->frozen_tab.words = at<float>(workspace_dev, L.fz_words);
+    b->frozen_tab.slots = at<uint4>(workspace_dev, L.fz_slots);
+    b->frozen_tab.cursor = at<unsigned>(workspace_dev, L.fz_cursor);
+    b->frozen_tab.cap = (unsigned)fz.lines;
+    b->frozen_C = at<float>(workspace_dev, L.fz_C);
+    b->d_items = at<ade::FrozenItem>(workspace_dev, L.fz_items);
     b->w.P0 = at<uint4>(workspace_dev, L.P0);
     b->w.P1 = at<uint4>(workspace_dev, L.P1);
     b->w.status = at<int>(workspace_dev, L.status);
@@ -1651,6 +1917,8 @@ int ade_batch_init(ade_batch **out, int nplumes, const ade_params *p, const int 
         std::fill(pid.begin() + b->offsets[i], pid.begin() + b->offsets[i + 1], (uint16_t)i);
     e = cudaSuccess;
     if (b->N > 0) e = cudaMemcpyAsync(b->plume_of, pid.data(), pid.size() * 2, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->frozen_tab.cursor, 0, sizeof(unsigned), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->w.frame, 0, (size_t)nplumes * ade::kFrameWords * 4, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->d_offsets, b->offsets.data(), b->offsets.size() * 4, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) {
@@ -1672,7 +1940,7 @@ int ade_batch_step(ade_batch *b, int nsteps, void *stream)
     if (!b || nsteps < 0) return fail(ADE_ERR_ARG, "bad argument");
     cudaStream_t s = (cudaStream_t)stream;
     int rc = batch_clear_status_once(b, s);
-    for (int k = 0; rc == ADE_OK && k < nsteps; ++k) rc = batch_enqueue_step(b, s);
+    if (rc == ADE_OK) rc = batch_enqueue_steps(b, nsteps, s);
     if (rc) return rc;
     b->step += nsteps;
     return ADE_OK;
@@ -1685,26 +1953,15 @@ int ade_batch_run(ade_batch *b, int nsteps, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     int rc = batch_clear_status_once(b, s);
     if (rc) return rc;
-    if (!b->graph_exec && nsteps > 0) {
-        if (!b->cap_stream) ADE_CK(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking));
-        ADE_CK(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
-        rc = batch_enqueue_step(b, b->cap_stream);
-        cudaGraph_t g = nullptr;
-        cudaError_t e = cudaStreamEndCapture(b->cap_stream, &g);
-        if (rc) {
-            if (g) cudaGraphDestroy(g);
-            return rc;
-        }
-        ADE_CK(e);
-        cudaError_t ei = cudaGraphInstantiate(&b->graph_exec, g, 0);
-        if (ei != cudaSuccess) {
-            cudaGraphDestroy(g);
-            b->graph_exec = nullptr;
-            return fail(ADE_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(ei));
-        }
-        b->graph = g;
+    // graphs of kGraphSteps steps and one of the rest where they keep the pair weights, else of one step
+    const int big = batch_use_frozen(b, nsteps) ? ade::kGraphSteps : 1;
+    for (int left = nsteps; left > 0;) {
+        const int k = std::min(left, big);
+        rc = batch_capture(b, k);
+        if (rc) return rc;
+        ADE_CK(cudaGraphLaunch(b->graph_exec[k], s));
+        left -= k;
     }
-    for (int k = 0; k < nsteps; ++k) ADE_CK(cudaGraphLaunch(b->graph_exec, s));
     b->step += nsteps;
     return ADE_OK;
 }
@@ -1905,7 +2162,7 @@ int ade_batch_step_timed(ade_batch *b, double *phase_ms, void *stream)
     cudaEvent_t ev[4];
     for (int k = 0; k < 4; ++k) ADE_CK(cudaEventCreate(&ev[k]));
     ADE_CK(cudaEventRecord(ev[0], s));
-    rc = batch_cells(b, s);
+    rc = batch_cells(b, s, 1);
     if (rc) return rc;
     ADE_CK(cudaEventRecord(ev[1], s));
     ade::EpiOut out = epi_none();
@@ -1942,8 +2199,7 @@ int ade_batch_launches_per_step(const ade_batch *b, int *launches)
 void ade_batch_destroy(ade_batch *b)
 {
     if (!b) return;
-    if (b->graph_exec) cudaGraphExecDestroy(b->graph_exec);
-    if (b->graph) cudaGraphDestroy(b->graph);
+    batch_drop_graphs(b);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
     delete b;
 }

@@ -36,12 +36,13 @@ namespace ade {
 
 namespace {
 
+// org: origin of the cell grid (CellFrame).
 __device__ __forceinline__ uint32_t cell_key(const uint32_t *__restrict__ xq, int n, int i,
-                                             int dim, int ncx, int ncy, int ncz)
+                                             int dim, int ncx, int ncy, int ncz, uint3 org)
 {
-    uint32_t cx = __umulhi(__ldg(xq + i), (uint32_t)ncx);
-    uint32_t cy = __umulhi(__ldg(xq + n + i), (uint32_t)ncy);
-    uint32_t cz = dim == 3 ? __umulhi(__ldg(xq + 2 * (size_t)n + i), (uint32_t)ncz) : 0u;
+    uint32_t cx = __umulhi(__ldg(xq + i) - org.x, (uint32_t)ncx);
+    uint32_t cy = __umulhi(__ldg(xq + n + i) - org.y, (uint32_t)ncy);
+    uint32_t cz = dim == 3 ? __umulhi(__ldg(xq + 2 * (size_t)n + i) - org.z, (uint32_t)ncz) : 0u;
     return (cz * (uint32_t)ncy + cy) * (uint32_t)ncx + cx;
 }
 
@@ -52,6 +53,19 @@ constexpr int kTileCells = kThreads * kTileItems;     // cells per tile (one sca
 constexpr int kTileStride = 32;   // words between two tile totals: one 128-byte line each, so the
                                   // totals' atomics spread over the L2 slices
 constexpr int kTileWindow = 8;    // tiles a block aggregates in shared memory (from its lowest)
+
+// Origin of the grid: the next build's (k_count; at = 0) or the running build's (at = 4, once the
+// scan has moved it).
+__device__ __forceinline__ uint3 frame_origin(const CellFrame &f, int at)
+{
+    uint3 o = make_uint3(f.add[0], f.add[1], f.add[2]);
+    if (f.words) {
+        o.x += f.words[at];
+        o.y += f.words[at + 1];
+        o.z += f.words[at + 2];
+    }
+    return o;
+}
 
 // Adds the block's particles to their tiles' totals (tile = key / kTileCells, 0xffffffff for no
 // particle).  Every thread of the block must call it.
@@ -92,7 +106,7 @@ __global__ __launch_bounds__(kThreads) void k_count(const uint32_t *__restrict__
                                                     uint32_t *__restrict__ rank,
                                                     uint32_t *__restrict__ count,
                                                     uint4 *__restrict__ pencil, int npencils,
-                                                    uint32_t *__restrict__ tile_sums)
+                                                    uint32_t *__restrict__ tile_sums, const CellFrame frame)
 {
     pdl_wait();
     pdl_trigger();
@@ -101,7 +115,7 @@ __global__ __launch_bounds__(kThreads) void k_count(const uint32_t *__restrict__
         for (int q = i; q < npencils; q += gridDim.x * kThreads) pencil[q] = make_uint4(kInfBits, 0u, kInfBits, 0u);
     uint32_t tile = 0xffffffffu;
     if (i < n) {
-        const uint32_t key = cell_key(xq, n, i, dim, ncx, ncy, ncz);
+        const uint32_t key = cell_key(xq, n, i, dim, ncx, ncy, ncz, frame_origin(frame, 0));
         keys[i] = key;
         rank[i] = atomicAdd(count + key, 1u);
         tile = key / (uint32_t)kTileCells;
@@ -241,7 +255,8 @@ __global__ __launch_bounds__(kThreads) void k_scan_apply(uint32_t *__restrict__ 
 // k_scan_apply; k_place clears the tile totals once every block has read them.
 __global__ __launch_bounds__(kThreads) void k_scan_tiles(uint32_t *__restrict__ count, int m,
                                                          uint32_t *__restrict__ start,
-                                                         const uint32_t *__restrict__ tile_sums)
+                                                         const uint32_t *__restrict__ tile_sums,
+                                                         const CellFrame frame)
 {
     pdl_wait();
     pdl_trigger();
@@ -306,6 +321,16 @@ __global__ __launch_bounds__(kThreads) void k_scan_tiles(uint32_t *__restrict__ 
         }
     }
     if (base <= m - 1 && m - 1 < base + kTileItems) start[m] = run;  // holder of the last element
+    if (frame.words && blockIdx.x == 0) {   // k_count has read it: this build's origin moves over, the
+        const int nf = frame.corr ? frame.plumes : 1;                          // next build's advances
+        for (int q = threadIdx.x; q < 3 * nf; q += kThreads) {
+            const int p = q / 3, d = q - 3 * p;
+            uint32_t *w = frame.words + (size_t)p * kFrameWords;
+            const uint32_t o = w[d];
+            w[4 + d] = o;
+            w[d] = o + (frame.corr ? frame.corr[p].inc[d] * frame.steps : frame.adv[d]);
+        }
+    }
 }
 
 __global__ __launch_bounds__(kThreads) void k_place(const uint32_t *__restrict__ keys,
@@ -370,9 +395,11 @@ struct Box {
 struct BoxAcc {
     Box *box;
     uint32_t ncy, ncz;
-    __device__ __forceinline__ void operator()(const uint4 &r) const
+    uint32_t oy, oz;      // origin of the cell grid
+    __device__ __forceinline__ void operator()(const uint4 &r) const { into(box, r); }
+    __device__ __forceinline__ void into(Box *b, const uint4 &r) const
     {
-        if (box) box->add(cell_frac_bits(r.y, ncy), cell_frac_bits(r.z, ncz));
+        if (b) b->add(cell_frac_bits(r.y - oy, ncy), cell_frac_bits(r.z - oz, ncz));
     }
 };
 
@@ -415,7 +442,7 @@ __device__ __forceinline__ void merge_pencils(int c, int ncells, int ncx, Box b,
 template <class Rec>
 __device__ __forceinline__ void order_small_cell(uint32_t s, uint32_t e, const uint32_t *__restrict__ perm_tmp,
                                                  uint32_t *__restrict__ perm, uint4 *__restrict__ P, Rec rec,
-                                                 BoxAcc acc = BoxAcc{nullptr, 0u, 0u})
+                                                 BoxAcc acc = BoxAcc{nullptr, 0u, 0u, 0u, 0u})
 {
     const uint32_t m = e - s;
     if (m <= 4) {
@@ -483,7 +510,7 @@ template <class Rec>
 __device__ __forceinline__ void order_big_cells(bool big, uint32_t s, uint32_t e,
                                                 const uint32_t *__restrict__ perm_tmp,
                                                 uint32_t *__restrict__ perm, uint4 *__restrict__ P, Rec rec,
-                                                BoxAcc acc = BoxAcc{nullptr, 0u, 0u})
+                                                BoxAcc acc = BoxAcc{nullptr, 0u, 0u, 0u, 0u})
 {
     const int lane = threadIdx.x & 31;
     unsigned todo = __ballot_sync(0xffffffffu, big);
@@ -505,7 +532,7 @@ __device__ __forceinline__ void order_big_cells(bool big, uint32_t s, uint32_t e
             if (has && bs + rank < be) {
                 perm[bs + rank] = v;
                 const uint4 r = rec(v);
-                if (acc.box) cb.add(cell_frac_bits(r.y, acc.ncy), cell_frac_bits(r.z, acc.ncz));
+                if (acc.box) acc.into(&cb, r);
                 P[bs + rank] = r;
             }
         }
@@ -541,7 +568,7 @@ __global__ __launch_bounds__(kThreads) void k_order(const uint32_t *__restrict__
                                                     const float *__restrict__ C, int n, int dim,
                                                     uint32_t *__restrict__ perm,
                                                     uint4 *__restrict__ P, int ncx, int ncy, int ncz,
-                                                    uint4 *__restrict__ pencil)
+                                                    uint4 *__restrict__ pencil, const CellFrame frame)
 {
     pdl_wait();
     pdl_trigger();
@@ -554,7 +581,8 @@ __global__ __launch_bounds__(kThreads) void k_order(const uint32_t *__restrict__
     const bool valid = e > s && e <= (uint32_t)n;
     const PlainRec rec{xq, C, n, dim};
     Box box;
-    const BoxAcc bacc{pencil ? &box : nullptr, (uint32_t)ncy, (uint32_t)ncz};
+    const uint3 org = frame_origin(frame, 4);
+    const BoxAcc bacc{pencil ? &box : nullptr, (uint32_t)ncy, (uint32_t)ncz, org.y, org.z};
     if (valid && e - s <= kSmallCell) order_small_cell(s, e, perm_tmp, perm, P, rec, bacc);
     order_big_cells(valid && e - s > kSmallCell, s, e, perm_tmp, perm, P, rec, bacc);
     if (pencil) merge_pencils(c, ncells, ncx, box, pencil);
@@ -571,7 +599,8 @@ __global__ __launch_bounds__(kThreads) void k_order_block(const uint32_t *__rest
                                                           const uint32_t *__restrict__ xq,
                                                           const float *__restrict__ C, int n, int dim,
                                                           uint32_t *__restrict__ perm, uint4 *__restrict__ P,
-                                                          int ncx, int ncy, int ncz, uint4 *__restrict__ pencil)
+                                                          int ncx, int ncy, int ncz, uint4 *__restrict__ pencil,
+                                                          const CellFrame frame)
 {
     pdl_wait();
     pdl_trigger();
@@ -582,7 +611,9 @@ __global__ __launch_bounds__(kThreads) void k_order_block(const uint32_t *__rest
     const uint32_t s = __ldg(start + c), e = __ldg(start + c + 1);
     if (e <= s || e > (uint32_t)n) return;                       // uniform over the block
     const PlainRec rec{xq, C, n, dim};
+    const uint3 org = frame_origin(frame, 4);
     Box box;
+    const BoxAcc bacc{pencil ? &box : nullptr, (uint32_t)ncy, (uint32_t)ncz, org.y, org.z};
     for (uint32_t k0 = s; k0 < e; k0 += kThreads * kRankItems) {
         uint32_t v[kRankItems], rank[kRankItems];
 #pragma unroll
@@ -608,7 +639,7 @@ __global__ __launch_bounds__(kThreads) void k_order_block(const uint32_t *__rest
             if (k < e && s + rank[r] < e) {
                 perm[s + rank[r]] = v[r];
                 const uint4 q = rec(v[r]);
-                if (pencil) box.add(cell_frac_bits(q.y, (uint32_t)ncy), cell_frac_bits(q.z, (uint32_t)ncz));
+                bacc(q);
                 P[s + rank[r]] = q;
             }
         }
@@ -642,20 +673,30 @@ __global__ __launch_bounds__(kThreads) void k_count_batch(const uint32_t *__rest
                                                           uint32_t *__restrict__ keys,
                                                           uint32_t *__restrict__ rank,
                                                           uint32_t *__restrict__ count,
-                                                          uint32_t *__restrict__ tile_sums)
+                                                          uint32_t *__restrict__ tile_sums,
+                                                          const uint32_t *__restrict__ frames)
 {
     const int i = blockIdx.x * kThreads + threadIdx.x;
     uint32_t tile = 0xffffffffu;
     if (i < n) {
-        const RateParams &d = descs[__ldg(plume_of + i)];
+        const int plume = __ldg(plume_of + i);
+        const RateParams &d = descs[plume];
         const int np = d.n, goff = d.goff;
+        const uint32_t *f = frames ? frames + (size_t)plume * kFrameWords : nullptr;
         const uint32_t key =
-            (uint32_t)d.coff + cell_key(xq + (size_t)dim * goff, np, i - goff, dim, d.ncx, d.ncy, d.ncz);
+            (uint32_t)d.coff + cell_key(xq + (size_t)dim * goff, np, i - goff, dim, d.ncx, d.ncy, d.ncz,
+                                        f ? make_uint3(f[0], f[1], f[2]) : make_uint3(0u, 0u, 0u));
         keys[i] = key;
         rank[i] = atomicAdd(count + key, 1u);
         tile = key / (uint32_t)kTileCells;
     }
     if (tile_sums) add_tile_totals(tile, tile_sums);
+}
+
+__global__ void k_set_frame(uint32_t *words, uint32_t x, uint32_t y, uint32_t z)
+{
+    const int t = threadIdx.x & 3;
+    if (threadIdx.x < kFrameWords) words[threadIdx.x] = t == 0 ? x : (t == 1 ? y : (t == 2 ? z : 0u));
 }
 
 struct BatchRec {
@@ -701,6 +742,12 @@ __global__ __launch_bounds__(kThreads) void k_order_batch(const uint32_t *__rest
 
 }  // namespace
 
+cudaError_t launch_set_frame(uint32_t *words, const uint32_t *origin, cudaStream_t s)
+{
+    k_set_frame<<<1, 32, 0, s>>>(words, origin[0], origin[1], origin[2]);
+    return cudaGetLastError();
+}
+
 int scan_blocks(int m) { return (m + kScanTile - 1) / kScanTile; }
 
 int tile_blocks(int m) { return (m + kTileCells - 1) / kTileCells; }
@@ -714,7 +761,7 @@ int cell_build_launches(int n, int ncells, bool onepass)
 
 cudaError_t launch_build_cells_batch(int dim, const uint32_t *xq, const float *C, int n, int ncells,
                                      const RateParams *descs, const uint16_t *plume_of,
-                                     const Work &w, cudaStream_t s)
+                                     const Work &w, cudaStream_t s, const CellFrame &frame)
 {
     const int nt = tile_blocks(ncells);
     cudaError_t e = cudaMemsetAsync(w.count, 0, (size_t)ncells * sizeof(uint32_t), s);
@@ -722,9 +769,10 @@ cudaError_t launch_build_cells_batch(int dim, const uint32_t *xq, const float *C
     if (e != cudaSuccess) return e;
     const int nb = (n + kThreads - 1) / kThreads;
     if (nb > 0)
-        k_count_batch<<<nb, kThreads, 0, s>>>(xq, n, dim, descs, plume_of, w.keys, w.rank, w.count, w.tile_sums);
+        k_count_batch<<<nb, kThreads, 0, s>>>(xq, n, dim, descs, plume_of, w.keys, w.rank, w.count, w.tile_sums,
+                                              frame.words);
     if (w.tile_sums) {
-        k_scan_tiles<<<nt, kThreads, 0, s>>>(w.count, ncells, w.cell_start, (const uint32_t *)w.tile_sums);
+        k_scan_tiles<<<nt, kThreads, 0, s>>>(w.count, ncells, w.cell_start, (const uint32_t *)w.tile_sums, frame);
     } else {
         const int sb = scan_blocks(ncells);
         k_scan_blocks<<<sb, kThreads, 0, s>>>(w.count, ncells, w.block_sums);
@@ -740,7 +788,7 @@ cudaError_t launch_build_cells_batch(int dim, const uint32_t *xq, const float *C
 }
 
 cudaError_t launch_build_cells(int dim, const uint32_t *xq, const float *C, int n, const int *nc,
-                               int ncells, const Work &w, cudaStream_t s, bool count_zero)
+                               int ncells, const Work &w, cudaStream_t s, bool count_zero, const CellFrame &frame)
 {
     const int nt = tile_blocks(ncells);
     cudaError_t e = count_zero ? cudaSuccess : cudaMemsetAsync(w.count, 0, (size_t)ncells * sizeof(uint32_t), s);
@@ -750,12 +798,12 @@ cudaError_t launch_build_cells(int dim, const uint32_t *xq, const float *C, int 
     const int nb = (n + kThreads - 1) / kThreads;
     if (nb > 0 && e == cudaSuccess)
         e = launch_pdl(k_count, nb, kThreads, 0, s, xq, n, dim, nc[0], nc[1], nc[2], w.keys, w.rank, w.count,
-                       w.pencil, ncells / nc[0], w.tile_sums);
+                       w.pencil, ncells / nc[0], w.tile_sums, frame);
     const int sb = scan_blocks(ncells);
     if (w.tile_sums) {
         if (e == cudaSuccess)
             e = launch_pdl(k_scan_tiles, nt, kThreads, 0, s, w.count, ncells, w.cell_start,
-                           (const uint32_t *)w.tile_sums);
+                           (const uint32_t *)w.tile_sums, frame);
     } else if (sb <= kScanFoldBlocks) {
         if (e == cudaSuccess) e = launch_pdl(k_scan_blocks, sb, kThreads, 0, s, w.count, ncells, w.block_sums);
         if (e == cudaSuccess)
@@ -771,10 +819,10 @@ cudaError_t launch_build_cells(int dim, const uint32_t *xq, const float *C, int 
         if (e != cudaSuccess) return e;
         if ((long long)n >= 16ll * ncells)   // many particles per cell: one block per cell
             e = launch_pdl(k_order_block, ncells, kThreads, 0, s, w.cell_start, ncells, w.perm_tmp, xq, C, n,
-                           dim, w.perm, w.P0, nc[0], nc[1], nc[2], w.pencil);
+                           dim, w.perm, w.P0, nc[0], nc[1], nc[2], w.pencil, frame);
         else
             e = launch_pdl(k_order, (ncells + kThreads - 1) / kThreads, kThreads, 0, s, w.cell_start, ncells,
-                           w.perm_tmp, xq, C, n, dim, w.perm, w.P0, nc[0], nc[1], nc[2], w.pencil);
+                           w.perm_tmp, xq, C, n, dim, w.perm, w.P0, nc[0], nc[1], nc[2], w.pencil, frame);
     }
     return e;
 }

@@ -188,6 +188,7 @@ int ade_checkpoint_load(ade_ctx *c, const void *host_buf, size_t bytes, void *st
         c->field_dirty = false;
     }
     if (c->catt) c->flux_set = true;
+    c->frame_set = false;        // the cell frame follows the restored step
     c->status_cleared = false;   // the status word is cleared again before the next step
     return ADE_OK;
 }

@@ -61,10 +61,11 @@ __global__ __launch_bounds__(kRateThreads) void k_rate(const uint4 *__restrict__
     const bool valid = i < prm.n;
     const int ii = valid ? i : prm.n - 1;
     const uint4 pa = __ldg(Pe + ii);
-    // cell of the cell build: evaluation position minus the drift since the build
-    const int cx = (int)__umulhi(pa.x - prm.back[0], (uint32_t)prm.ncx);
-    const int cy = (int)__umulhi(pa.y - prm.back[1], (uint32_t)prm.ncy);
-    const int cz = DIM == 3 ? (int)__umulhi(pa.z - prm.back[2], (uint32_t)prm.ncz) : 0;
+    // cell of the cell build: evaluation position minus the drift since the build, in its frame
+    const uint3 org = cell_origin(prm);
+    const int cx = (int)__umulhi(pa.x - org.x, (uint32_t)prm.ncx);
+    const int cy = (int)__umulhi(pa.y - org.y, (uint32_t)prm.ncy);
+    const int cz = DIM == 3 ? (int)__umulhi(pa.z - org.z, (uint32_t)prm.ncz) : 0;
     Acc acc{0.f, 0.f, __int_as_float(0x7f800000), __int_as_float(0xff800000), 0u};
     unsigned cnt = 0u;
     // Corrector: the caller index and C^l are loaded ahead of the pair loop (not in the trimmed
@@ -200,11 +201,12 @@ __global__ __launch_bounds__(kTileThreads, 2) void k_rate_tiled(const uint4 *__r
     const bool staged = carry <= prm.cap;
 
     // 3. stage the halo: one thread per halo cell copies that cell's particles
+    const uint3 org = cell_origin(prm);
     if (staged) {
-        const uint32_t ox = (uint32_t)(((unsigned long long)(2 * tx0 + TX) << 31) / (unsigned)ncx);
-        const uint32_t oy = (uint32_t)(((unsigned long long)(2 * ty0 + TY) << 31) / (unsigned)ncy);
+        const uint32_t ox = (uint32_t)(((unsigned long long)(2 * tx0 + TX) << 31) / (unsigned)ncx) + org.x;
+        const uint32_t oy = (uint32_t)(((unsigned long long)(2 * ty0 + TY) << 31) / (unsigned)ncy) + org.y;
         const uint32_t oz =
-            DIM == 3 ? (uint32_t)(((unsigned long long)(2 * tz0 + TZ) << 31) / (unsigned)ncz) : 0u;
+            DIM == 3 ? (uint32_t)(((unsigned long long)(2 * tz0 + TZ) << 31) / (unsigned)ncz) + org.z : 0u;
         for (int h = threadIdx.x; h < NH; h += kTileThreads) {
             const int hx = h % HX, row = h / HX;
             const int hy = row % HY, hz = row / HY;
@@ -231,9 +233,9 @@ __global__ __launch_bounds__(kTileThreads, 2) void k_rate_tiled(const uint4 *__r
         const int off = t - tpre[r];
         const int gi = tglb[r] + off;
         const uint4 pe = __ldg(Pe + gi);
-        const int cx = (int)__umulhi(pe.x - prm.back[0], (uint32_t)ncx);
-        const int cy = (int)__umulhi(pe.y - prm.back[1], (uint32_t)ncy);
-        const int cz = DIM == 3 ? (int)__umulhi(pe.z - prm.back[2], (uint32_t)ncz) : 0;
+        const int cx = (int)__umulhi(pe.x - org.x, (uint32_t)ncx);
+        const int cy = (int)__umulhi(pe.y - org.y, (uint32_t)ncy);
+        const int cz = DIM == 3 ? (int)__umulhi(pe.z - org.z, (uint32_t)ncz) : 0;
         float rate;
         unsigned cnt = 0u;
         if (staged) {
@@ -300,6 +302,7 @@ __global__ __launch_bounds__(kRateThreads) void k_rate_batch(const uint4 *__rest
     const int lane = threadIdx.x & 31;
     RateParams &mine = sp[threadIdx.x >> 5];
     int cur = -1;
+    uint3 org = make_uint3(0u, 0u, 0u);
     unsigned cnt = 0u;
     for (;;) {
         int item = 0;
@@ -313,6 +316,7 @@ __global__ __launch_bounds__(kRateThreads) void k_rate_batch(const uint4 *__rest
             for (int w = lane; w < kWords; w += 32) dst[w] = __ldg(src + w);
             cur = t.plume;
             __syncwarp();
+            org = cell_origin(mine);
         }
         const RateParams &prm = mine;
         EpiOut o = out;
@@ -323,12 +327,12 @@ __global__ __launch_bounds__(kRateThreads) void k_rate_batch(const uint4 *__rest
                 const bool v1 = k + 1 < t.count;
                 const uint4 pa0 = __ldg(Pe + g0);
                 const uint4 pa1 = __ldg(Pe + (v1 ? g0 + 1 : g0));
-                const int cx0 = (int)__umulhi(pa0.x - prm.back[0], (uint32_t)prm.ncx);
-                const int cy0 = (int)__umulhi(pa0.y - prm.back[1], (uint32_t)prm.ncy);
-                const int cz0 = DIM == 3 ? (int)__umulhi(pa0.z - prm.back[2], (uint32_t)prm.ncz) : 0;
-                const int cx1 = (int)__umulhi(pa1.x - prm.back[0], (uint32_t)prm.ncx);
-                const int cy1 = (int)__umulhi(pa1.y - prm.back[1], (uint32_t)prm.ncy);
-                const int cz1 = DIM == 3 ? (int)__umulhi(pa1.z - prm.back[2], (uint32_t)prm.ncz) : 0;
+                const int cx0 = (int)__umulhi(pa0.x - org.x, (uint32_t)prm.ncx);
+                const int cy0 = (int)__umulhi(pa0.y - org.y, (uint32_t)prm.ncy);
+                const int cz0 = DIM == 3 ? (int)__umulhi(pa0.z - org.z, (uint32_t)prm.ncz) : 0;
+                const int cx1 = (int)__umulhi(pa1.x - org.x, (uint32_t)prm.ncx);
+                const int cy1 = (int)__umulhi(pa1.y - org.y, (uint32_t)prm.ncy);
+                const int cz1 = DIM == 3 ? (int)__umulhi(pa1.z - org.z, (uint32_t)prm.ncz) : 0;
                 float r0, r1 = 0.f;
                 unsigned c = 0u;
                 if (v1 && can_pair(cx0, cy0, cz0, cx1, cy1, cz1, prm.ncx)) {
@@ -346,9 +350,9 @@ __global__ __launch_bounds__(kRateThreads) void k_rate_batch(const uint4 *__rest
             for (int k = lane; k < t.count; k += 32) {
                 const int gi = prm.goff + t.start + k;
                 const uint4 pa = __ldg(Pe + gi);
-                const int cx = (int)__umulhi(pa.x - prm.back[0], (uint32_t)prm.ncx);
-                const int cy = (int)__umulhi(pa.y - prm.back[1], (uint32_t)prm.ncy);
-                const int cz = DIM == 3 ? (int)__umulhi(pa.z - prm.back[2], (uint32_t)prm.ncz) : 0;
+                const int cx = (int)__umulhi(pa.x - org.x, (uint32_t)prm.ncx);
+                const int cy = (int)__umulhi(pa.y - org.y, (uint32_t)prm.ncy);
+                const int cz = DIM == 3 ? (int)__umulhi(pa.z - org.z, (uint32_t)prm.ncz) : 0;
                 unsigned c = 0u;
                 const float rate = rate_direct<DIM, KERNEL, true, COUNT>(Pe, cs + prm.coff, pa, cx, cy, cz, prm, c);
                 cnt += c;

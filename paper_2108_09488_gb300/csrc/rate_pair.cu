@@ -31,12 +31,13 @@ __global__ __launch_bounds__(kRateThreads, (BF && !TRIM) ? 10 : 0) void k_rate_p
     const int ii0 = v0 ? i0 : prm.n - 1, ii1 = v1 ? i1 : ii0;
     const uint4 pa0 = __ldg(Pe + ii0);
     const uint4 pa1 = __ldg(Pe + ii1);
-    const int cx0 = (int)__umulhi(pa0.x - prm.back[0], (uint32_t)prm.ncx);
-    const int cy0 = (int)__umulhi(pa0.y - prm.back[1], (uint32_t)prm.ncy);
-    const int cz0 = DIM == 3 ? (int)__umulhi(pa0.z - prm.back[2], (uint32_t)prm.ncz) : 0;
-    const int cx1 = (int)__umulhi(pa1.x - prm.back[0], (uint32_t)prm.ncx);
-    const int cy1 = (int)__umulhi(pa1.y - prm.back[1], (uint32_t)prm.ncy);
-    const int cz1 = DIM == 3 ? (int)__umulhi(pa1.z - prm.back[2], (uint32_t)prm.ncz) : 0;
+    const uint3 org = cell_origin(prm);
+    const int cx0 = (int)__umulhi(pa0.x - org.x, (uint32_t)prm.ncx);
+    const int cy0 = (int)__umulhi(pa0.y - org.y, (uint32_t)prm.ncy);
+    const int cz0 = DIM == 3 ? (int)__umulhi(pa0.z - org.z, (uint32_t)prm.ncz) : 0;
+    const int cx1 = (int)__umulhi(pa1.x - org.x, (uint32_t)prm.ncx);
+    const int cy1 = (int)__umulhi(pa1.y - org.y, (uint32_t)prm.ncy);
+    const int cz1 = DIM == 3 ? (int)__umulhi(pa1.z - org.z, (uint32_t)prm.ncz) : 0;
     Acc acc{0.f, 0.f, __int_as_float(0x7f800000), __int_as_float(0xff800000), 0u};
     unsigned cnt = 0u;
     float r0, r1;

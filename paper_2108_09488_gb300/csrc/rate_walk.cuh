@@ -19,6 +19,20 @@ __device__ __forceinline__ unsigned in_support_fp64(int ix, int iy, int iz, cons
     return (r2 > 0.0 && r2 < prm.H2d) ? 1u : 0u;
 }
 
+// Evaluation position minus this word gives the position in the frame of the cell build: the drift
+// since the build plus the origin of the build's grid (0 on the absolute grid).
+template <class P>
+__device__ __forceinline__ uint3 cell_origin(const P &prm)
+{
+    uint3 o = make_uint3(prm.back[0], prm.back[1], prm.back[2]);
+    if (prm.frame) {
+        o.x += __ldg(prm.frame + 4);
+        o.y += __ldg(prm.frame + 5);
+        o.z += __ldg(prm.frame + 6);
+    }
+    return o;
+}
+
 // Per-pair constants, copied into registers once per particle (the parameter block may live in
 // shared or constant memory).
 struct PairConst {
@@ -92,11 +106,12 @@ struct TrimSelf {
 template <int DIM>
 __device__ __forceinline__ TrimSelf trim_self(const uint4 &pa, int cy, int cz, const RateParams &prm)
 {
+    const uint3 org = cell_origin(prm);
     const float inv32 = 2.3283064365386963e-10f;   // 2^-32
     TrimSelf t;
-    t.fx = (float)((pa.x - prm.back[0]) * (uint32_t)prm.ncx) * inv32;
-    t.fy = (float)((pa.y - prm.back[1]) * (uint32_t)prm.ncy) * inv32;
-    t.fz = DIM == 3 ? (float)((pa.z - prm.back[2]) * (uint32_t)prm.ncz) * inv32 : 0.f;
+    t.fx = (float)((pa.x - org.x) * (uint32_t)prm.ncx) * inv32;
+    t.fy = (float)((pa.y - org.y) * (uint32_t)prm.ncy) * inv32;
+    t.fz = DIM == 3 ? (float)((pa.z - org.z) * (uint32_t)prm.ncz) * inv32 : 0.f;
     t.p0 = cz * prm.ncy + cy;
     t.interior = cy >= prm.k && cy < prm.ncy - prm.k && (DIM == 2 || (cz >= prm.k && cz < prm.ncz - prm.k));
     return t;

@@ -68,9 +68,16 @@ __global__ __launch_bounds__(kT) void k_rate_sweep(const uint4 *__restrict__ Pe,
     float Ca[NT];
     load_group<NT>(Ce + (size_t)ii * P4 + g0, Ca);
     const int ncx = prm.ncx, ncy = prm.ncy, ncz = prm.ncz;
-    const int cx = (int)__umulhi(pa.x - prm.back[0], (uint32_t)ncx);
-    const int cy = (int)__umulhi(pa.y - prm.back[1], (uint32_t)ncy);
-    const int cz = DIM == 3 ? (int)__umulhi(pa.z - prm.back[2], (uint32_t)ncz) : 0;
+    // cell of the build: position minus the drift since it, in the build's frame
+    uint3 org = make_uint3(prm.back[0], prm.back[1], prm.back[2]);
+    if (prm.frame) {
+        org.x += __ldg(prm.frame + 4);
+        org.y += __ldg(prm.frame + 5);
+        org.z += __ldg(prm.frame + 6);
+    }
+    const int cx = (int)__umulhi(pa.x - org.x, (uint32_t)ncx);
+    const int cy = (int)__umulhi(pa.y - org.y, (uint32_t)ncy);
+    const int cz = DIM == 3 ? (int)__umulhi(pa.z - org.z, (uint32_t)ncz) : 0;
     const float H2 = prm.H2, invH = prm.invH, sy = prm.sy, sz = prm.sz;
     const float vx = sp.vh[0], vy = sp.vh[1], vz = sp.vh[2];
     float acc[NT], comp[NT];
