@@ -7,6 +7,8 @@
 
 #include "../../include/ade_sph.h"
 
+struct ade_ctx;
+
 namespace ade {
 
 constexpr int kMaxSubdiv = 6;                                   // cells per support radius
@@ -235,9 +237,7 @@ struct NvtxRange {
 // Records msg as the calling thread's last error (read by ade_last_error) and returns code.
 int report_error(int code, const char *msg);
 
-// Pair-factor constants Kc[6], c0 of a uniform dispersion tensor D (dim x dim, Eq. 5, K = 2D).
-void pair_coeffs(int dim, double gamma, const double *D, float *Kc, float *c0);
-// The interaction walks' form of the same factor for the tensor of Eq. 3 (RateParams uw, ub, upf;
+// The interaction walks' form of Eq. 5's pair factor for the tensor of Eq. 3 (RateParams uw, ub, upf;
 // pf must be set first).
 void rate_pair_consts(int dim, double gamma, const double *v, double alpha_L, double alpha_T, double D_m,
                       RateParams *rp);
@@ -296,6 +296,11 @@ cudaError_t launch_rate_field(int dim, int kernel, int epi, const uint4 *Pe, con
                               const uint32_t *perm, const FieldWork &fw, const RateParams &prm,
                               const FieldParams &fp, const EpiOut &out, cudaStream_t s);
 
+// Launch grid of the table's kernels (kFrozenThreads threads a block).
+dim3 frozen_grid(const RateParams &prm);
+// Lines and slots of a table with `val` words per pair (lines bounded by the table's size limit), and blocks
+// of frozen_grid, enough for every grid the context may switch to.
+void frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots, int *blocks);
 // Evaluations over one cell list with stored weights (rate_frozen.cu): the table, one predictor or
 // corrector (prm.dt), and the final state in the caller's order (prm.inc: the drift of all steps).
 cudaError_t launch_frozen_build(int dim, int kernel, bool iso, const uint4 *P, const uint32_t *cs, const uint32_t *perm,

@@ -17,256 +17,388 @@
 // Forward states are kept as checkpoints every `ckpt_every` steps and recomputed segment by segment
 // on the way back.  All operators use one cell list built at the initial positions (the geometry
 // is frozen, which is exact for a uniform drift), so forward and adjoint apply the same L.
+// With a uniform v every one of these operators is a combination of two sums over the pairs,
+//   S_L = pf sum_b g_L (x_a - x_b),  S_T = pf sum_b g_T (x_a - x_b),
+// g_L and g_T the weights for D = vhat vhat^T and I - vhat vhat^T (frozen_table.cuh):
+//   L_L = |v| S_L,  L_T = |v| S_T,  L_m = S_L + S_T,  L = d_L S_L + d_T S_T, d_i = alpha_i |v| + D_m
+// (sums with D's other split, a (vhat . e)^2 + b, cancel: dJ/dalpha lost up to a factor of 8 in
+// accuracy).  g_L and g_T never change during a call, so
+// they are computed once (frozen_table.cuh) and an evaluation streams them; the state and the adjoint
+// state of a backward step share one pass, and the dot products are taken in that pass from S_L and S_T,
+// so a backward step is two launches and a forward step two.
+// Bound: L2 / HBM, 8 bytes a pair.  512^2 lattice, 20 neighbours, 40 steps: 13.5 -> 4.3 ms (the dot
+// products' kernel alone took 97 us a step: nine threads folded 1024 FP64 partials one by one).
 // Pair arithmetic is FP32 with compensated row sums (as in rate.cu); dot products and J are FP64.
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "ade_internal.h"
 
+namespace ade {
+
 namespace {
 
-constexpr int kT = 256;
+#include "rate_common.cuh"
 
-// Up to three pair-factor sets (operators) and the weights of their combination.
-struct ApplyCoef {
-    float Kc[3][6];
-    float c0[3];
-    float theta[3];
+#include "rate_walk.cuh"
+
+#include "frozen_table.cuh"
+
+constexpr int kT = kFrozenThreads;
+constexpr double kTwo32 = 4294967296.0;
+constexpr int kDots = 6;   // per backward step: p.S_L u, p.S_T u, b.S_L u, b.S_T u (b = L p), p.S_L a, p.S_T a (a = L u)
+
+// S_L (0) and S_T (1) of NR fields.
+template <int NR>
+struct ShapeSums {
+    const float *x[NR];
+    float xa[NR], r0[NR], r1[NR], a0[NR], c0[NR], a1[NR], c1[NR];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int q = 0; q < NR; ++q) r0[q] = r1[q] = a0[q] = c0[q] = a1[q] = c1[q] = 0.f;
+    }
+    __device__ __forceinline__ void add(int q, float2 w, float xb)
+    {
+        const float d = xa[q] - xb;
+        r0[q] = fmaf(w.x, d, r0[q]);
+        r1[q] = fmaf(w.y, d, r1[q]);
+    }
+    template <int M>
+    __device__ __forceinline__ void lines(const float *w, int s)
+    {
+        float2 wv[M];
+        float xv[NR][M];
+#pragma unroll
+        for (int u = 0; u < M; ++u) {
+            wv[u] = __ldg(reinterpret_cast<const float2 *>(w) + u * 32);
+#pragma unroll
+            for (int q = 0; q < NR; ++q) xv[q][u] = x[q][s + u];
+        }
+#pragma unroll
+        for (int u = 0; u < M; ++u)
+#pragma unroll
+            for (int q = 0; q < NR; ++q) add(q, wv[u], xv[q][u]);
+    }
+    __device__ __forceinline__ void end_row()
+    {
+#pragma unroll
+        for (int q = 0; q < NR; ++q) {
+            neumaier_add(a0[q], c0[q], r0[q]);
+            neumaier_add(a1[q], c1[q], r1[q]);
+            r0[q] = r1[q] = 0.f;
+        }
+    }
+    __device__ __forceinline__ float s0(int q) const { return a0[q] + c0[q]; }
+    __device__ __forceinline__ float s1(int q) const { return a1[q] + c1[q]; }
 };
 
-__device__ __forceinline__ void nadd(float &sum, float &comp, float x)
+// The same sums over the positions, for a chunk without room in the table.
+template <int DIM, int KERNEL, bool ISO, int NR>
+__device__ __noinline__ void walk_sums(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs, const RateParams &prm,
+                                       const Chunk &c, const ShapeConst sc, ShapeSums<NR> &op)
 {
-    float t = sum + x;
-    if (fabsf(sum) >= fabsf(x))
-        comp += (sum - t) + x;
-    else
-        comp += (x - t) + sum;
-    sum = t;
-}
-
-template <int KERNEL>
-__device__ __forceinline__ float shape_f(float omq)
-{
-    if (KERNEL == ADE_WENDLAND_C2) return omq * omq * omq;
-    float o2 = omq * omq;
-    return o2 * o2 * omq * fmaf(-5.f, omq, 6.f);
-}
-
-template <int DIM>
-__device__ __forceinline__ float dcal_k(float dx, float dy, float dz, float rinv2, const float *Kc, float c0)
-{
-    float Q;
-    if (DIM == 2) {
-        Q = dx * fmaf(Kc[0], dx, Kc[3] * dy);
-    } else {
-        float qx = fmaf(Kc[0], dx, fmaf(Kc[3], dy, Kc[4] * dz));
-        float qy = fmaf(Kc[1], dy, Kc[5] * dz);
-        Q = fmaf(dx, qx, dy * qy);
-    }
-    return fmaf(Q, rinv2, c0);
-}
-
-// out_k[i] = (L_k v)_i for sorted particle i, k < NOUT; with NOUT == 3 and comb != NULL also
-// comb[i] = sum_k theta_k out_k[i]; with NOUT == 1 and axpy != NULL also axpy[i] = base[i] + alpha
-// (L v)_i.  Same candidate walk and summation order as the rate kernel's direct variant.
-template <int DIM, int KERNEL, int NOUT>
-__global__ __launch_bounds__(kT) void k_apply(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
-                                              const float *__restrict__ v, const ade::RateParams prm,
-                                              const ApplyCoef co, float *__restrict__ out0,
-                                              float *__restrict__ out1, float *__restrict__ out2,
-                                              float *__restrict__ comb, const float *__restrict__ base,
-                                              float alpha, float *__restrict__ axpy)
-{
-    const int i = blockIdx.x * kT + threadIdx.x;
-    if (i >= prm.n) return;
-    const uint4 pa = __ldg(P + i);
-    const float va = __ldg(v + i);
-    const int ncx = prm.ncx, ncy = prm.ncy, ncz = prm.ncz;
-    const int cx = (int)__umulhi(pa.x, (uint32_t)ncx);
-    const int cy = (int)__umulhi(pa.y, (uint32_t)ncy);
-    const int cz = DIM == 3 ? (int)__umulhi(pa.z, (uint32_t)ncz) : 0;
-    float acc[NOUT], cmp[NOUT];
+    const uint4 pa = __ldg(P + min(c.i0 + (int)(threadIdx.x & 31), c.pe - 1));
+    const int ncx = prm.ncx;
+    const int cx = (int)__umulhi(pa.x - frame_x(prm), (uint32_t)ncx);
+    const PairConst k(prm);
+    for (int r = 0; r < prm.nrows; ++r) {
+        const StencilRow row = prm.rows[r];
+        const int q = row_pencil_of<DIM>(row, c.cy, c.cz, prm);
+        const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
+        int s, cnt;
+        cyclic_range(cs, q * ncx, cx - (int)row.w, cx + row.w + 1, ncx, qs, qe, s, cnt);
+        for (int t = 0; t < cnt; ++t) {
+            int j = s + t;
+            j = j >= qe ? j - len : j;
+            const float2 w = pair_shape<DIM, KERNEL, ISO>(pa, __ldg(P + j), k, sc);
 #pragma unroll
-    for (int k = 0; k < NOUT; ++k) acc[k] = cmp[k] = 0.f;
-    for (int ri = 0; ri < prm.nrows; ++ri) {
-        const ade::StencilRow row = prm.rows[ri];
-        int yy = cy + row.dy;
-        yy += (yy < 0) ? ncy : 0;
-        yy -= (yy >= ncy) ? ncy : 0;
-        int zz = 0;
-        if (DIM == 3) {
-            zz = cz + row.dz;
-            zz += (zz < 0) ? ncz : 0;
-            zz -= (zz >= ncz) ? ncz : 0;
+            for (int f = 0; f < NR; ++f) op.add(f, w, op.x[f][qs + j]);
         }
-        const int basec = (zz * ncy + yy) * ncx;
-        const int lo = cx - row.w, hi = cx + row.w + 1;
-        int r0[2], r1[2];
-        if (lo < 0) {
-            r0[0] = __ldg(cs + basec + lo + ncx);
-            r1[0] = __ldg(cs + basec + ncx);
-            r0[1] = __ldg(cs + basec);
-            r1[1] = __ldg(cs + basec + hi);
-        } else if (hi > ncx) {
-            r0[0] = __ldg(cs + basec + lo);
-            r1[0] = __ldg(cs + basec + ncx);
-            r0[1] = __ldg(cs + basec);
-            r1[1] = __ldg(cs + basec + hi - ncx);
-        } else {
-            r0[0] = __ldg(cs + basec + lo);
-            r1[0] = __ldg(cs + basec + hi);
-            r0[1] = r1[1] = 0;
-        }
-        float rs[NOUT];
-#pragma unroll
-        for (int k = 0; k < NOUT; ++k) rs[k] = 0.f;
-        for (int piece = 0; piece < 2; ++piece)
-            for (int j = r0[piece]; j < r1[piece]; ++j) {
-                const uint4 pb = __ldg(P + j);
-                float dx = (float)(int)(pa.x - pb.x);
-                float dy = (float)(int)(pa.y - pb.y) * prm.sy;
-                float dz = DIM == 3 ? (float)(int)(pa.z - pb.z) * prm.sz : 0.f;
-                float r2 = fmaf(dx, dx, dy * dy);
-                if (DIM == 3) r2 = fmaf(dz, dz, r2);
-                if (r2 < prm.H2 && r2 > 0.f) {
-                    const float rinv = rsqrtf(r2);
-                    const float f = shape_f<KERNEL>(fmaf(-(r2 * rinv), prm.invH, 1.f));
-                    const float dv = va - __ldg(v + j);
-                    const float ri2 = rinv * rinv;
-#pragma unroll
-                    for (int k = 0; k < NOUT; ++k)
-                        rs[k] = fmaf(f * dcal_k<DIM>(dx, dy, dz, ri2, co.Kc[k], co.c0[k]), dv, rs[k]);
-                }
-            }
-#pragma unroll
-        for (int k = 0; k < NOUT; ++k) nadd(acc[k], cmp[k], rs[k]);
-    }
-    float r[NOUT];
-#pragma unroll
-    for (int k = 0; k < NOUT; ++k) r[k] = prm.pf * (acc[k] + cmp[k]);
-    out0[i] = r[0];
-    if (NOUT == 3) {
-        out1[i] = r[1 % NOUT];
-        out2[i] = r[2 % NOUT];
-        if (comb) comb[i] = fmaf(co.theta[0], r[0], fmaf(co.theta[1], r[1 % NOUT], co.theta[2] * r[2 % NOUT]));
-    } else if (axpy) {
-        axpy[i] = fmaf(alpha, r[0], __ldg(base + i));
+        op.end_row();
     }
 }
 
-__global__ void k_axpy(float *out, const float *x, float alpha, const float *y, int n)
+// The table (prm.uw = vhat, prm.ub = 0) and the initial concentrations, doubled per pencil.
+template <int DIM, int KERNEL, bool ISO>
+__global__ __launch_bounds__(kT) void k_adj_table(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
+                                                  const RateParams prm, const FrozenTab tab, const ShapeConst sc, float *__restrict__ C0)
 {
-    const int i = blockIdx.x * kT + threadIdx.x;
-    if (i < n) out[i] = fmaf(alpha, y[i], x[i]);
+    pdl_wait();
+    __shared__ TrimRow srow[ISO ? kMaxRows : 1];
+    if (ISO) stage_trim_rows(srow, prm);
+    for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), gridDim.y * (kT / 32), [&](const Chunk &c) {
+        const int i = c.i0 + (threadIdx.x & 31);
+        const uint4 pa = __ldg(P + min(i, c.pe - 1));
+        build_chunk<DIM, KERNEL, ISO, ISO, 2>(P, cs, prm, c, pa, srow, tab, sc);
+        if (i < c.pe) C0[c.ps + i] = C0[c.pe + i] = __uint_as_float(pa.w);
+    });
 }
 
-__global__ void k_gather(float *out, const float *in, const uint32_t *perm, int n)
-{
-    const int i = blockIdx.x * kT + threadIdx.x;
-    if (i < n) out[i] = in[perm[i]];
-}
-
-__global__ void k_scatter(float *out, const float *in, const uint32_t *perm, int n)
-{
-    const int i = blockIdx.x * kT + threadIdx.x;
-    if (i < n) out[perm[i]] = in[i];
-}
-
-__global__ void k_sorted_C(float *out, const uint4 *P, int n)
-{
-    const int i = blockIdx.x * kT + threadIdx.x;
-    if (i < n) out[i] = __uint_as_float(P[i].w);
-}
-
-// ND FP64 dot products x_d . y_d, d < ND; per-block partials, the last block folds them in a fixed
-// order into out[0..ND) and resets the counter.
-constexpr int kMaxDots = 9;
-struct DotArgs {
-    const float *x[kMaxDots];
-    const float *y[kMaxDots];
+// One pass over the table; fields doubled per pencil.
+//   HALF, FULL  out1 = base + step L x1 (HALF: base = x1)
+//   BACK1       out0 = a = L x0 (x0 = u), out1 = x1 + step L x1 (x1 = p); dots of p and b = L p with S_L u, S_T u
+//   BACK2       out1 = base + step L x1 (x1 = hp, base = p; out1 may be base); dots of p with S_L a, S_T a (x0 = a)
+enum AdjMode { HALF = 0, FULL = 1, BACK1 = 2, BACK2 = 3 };
+struct AdjPass {
+    const float *x0, *x1, *base;
+    float *out0, *out1;
+    float ca, cb, cal, cbl;   // L x = ca S_L + cb S_T (hi + lo), pf folded in
+    float step;
+    ShapeConst sc;
+    double *partials;      // [blocks][kDots] of the step (BACK1: the first four, BACK2: the last two)
 };
 
+__device__ __forceinline__ float combine(const AdjPass &ps, float s0, float s1)
+{
+    return fmaf(ps.ca, s0, fmaf(ps.cb, s1, fmaf(ps.cal, s0, ps.cbl * s1)));
+}
+
+// Sum of v[0..4) over the warp's lanes: every exchange halves the values a lane holds, so four sums take
+// 6 FP64 additions a lane instead of 20 (FP64 runs at a sixtieth of the FP32 rate here).  Lanes
+// 0, 8, 16, 24 hold sums 0, 1, 2, 3.
+__device__ __forceinline__ double warp_sums4(double v0, double v1, double v2, double v3)
+{
+    const int lane = threadIdx.x & 31;
+    const bool hi = (lane & 16) != 0, h8 = (lane & 8) != 0;
+    const double t0 = (hi ? v2 : v0) + __shfl_xor_sync(kFull, hi ? v0 : v2, 16);
+    const double t1 = (hi ? v3 : v1) + __shfl_xor_sync(kFull, hi ? v1 : v3, 16);
+    double r = (h8 ? t1 : t0) + __shfl_xor_sync(kFull, h8 ? t0 : t1, 8);
+    for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
+    return r;
+}
+
+// Block sums of d[0..ND) into out[0..ND) (a fixed order).  Every thread must call it.
 template <int ND>
-__global__ __launch_bounds__(kT) void k_dots(DotArgs a, int n, double *partials, unsigned *done,
-                                             double *out)
+__device__ __forceinline__ void block_sums(const double (&d)[ND], double *out)
 {
-    __shared__ double sh[ND][kT / 32];
-    __shared__ bool last;
-    const int i = blockIdx.x * kT + threadIdx.x;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr int G = (ND + 3) / 4;
+    __shared__ double sh[kT / 32][4 * G];
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int d = 0; d < ND; ++d) {
-        double v = i < n ? (double)a.x[d][i] * (double)a.y[d][i] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) sh[d][wid] = v;
+    for (int g = 0; g < G; ++g) {
+        const double r = warp_sums4(d[4 * g], 4 * g + 1 < ND ? d[(4 * g + 1) % ND] : 0.0, 4 * g + 2 < ND ? d[(4 * g + 2) % ND] : 0.0,
+                                    4 * g + 3 < ND ? d[(4 * g + 3) % ND] : 0.0);
+        if ((lane & 7) == 0) sh[threadIdx.x >> 5][4 * g + (lane >> 3)] = r;
     }
     __syncthreads();
     if (threadIdx.x < ND) {
-        double s = 0.0;
-        for (int w = 0; w < kT / 32; ++w) s += sh[threadIdx.x][w];
-        partials[(size_t)blockIdx.x * ND + threadIdx.x] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last) {
-        __threadfence();
-        if (threadIdx.x < ND) {
-            double s = 0.0;
-            for (int b = 0; b < (int)gridDim.x; ++b) s += __ldcg(partials + (size_t)b * ND + threadIdx.x);
-            out[threadIdx.x] = s;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) *done = 0u;
+        double t = 0.0;
+        for (int w = 0; w < kT / 32; ++w) t += sh[w][threadIdx.x];
+        out[threadIdx.x] = t;
     }
 }
 
-int blocks(int n) { return (n + kT - 1) / kT; }
+template <int DIM, int KERNEL, bool ISO, int MODE>
+__global__ __launch_bounds__(kT) void k_adj_pass(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
+                                                 const RateParams prm, const FrozenTab tab, const AdjPass ps)
+{
+    pdl_wait();
+    constexpr bool BACK = MODE >= BACK1;
+    constexpr int NR = BACK ? 2 : 1, ND = MODE == BACK1 ? 4 : 2;   // fields: x1, then x0
+    double dot[ND];
+#pragma unroll
+    for (int q = 0; q < ND; ++q) dot[q] = 0.0;
+    for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), gridDim.y * (kT / 32), [&](const Chunk &c) {
+        const int i = c.i0 + (threadIdx.x & 31);
+        const int at = c.ps + min(i, c.pe - 1);
+        ShapeSums<NR> op;
+        op.zero();
+        op.x[0] = ps.x1;
+        op.xa[0] = ps.x1[at];
+        if (BACK) {
+            op.x[NR - 1] = ps.x0;
+            op.xa[NR - 1] = ps.x0[at];
+        }
+        const uint4 sl = __ldg(tab.slots + c.slot);
+        if (sl.x != kNoRoom) stream_rows<2>(sl, tab, op);
+        else walk_sums<DIM, KERNEL, ISO, NR>(P, cs, prm, c, ps.sc, op);
+        if (i >= c.pe) return;
+        const int again = c.pe + i;
+        const float L1 = combine(ps, op.s0(0), op.s1(0));
+        const float p = MODE == HALF || MODE == BACK1 ? op.xa[0] : ps.base[at];
+        ps.out1[at] = ps.out1[again] = fmaf(ps.step, L1, p);
+        if (BACK) {
+            const float s0 = op.s0(NR - 1), s1 = op.s1(NR - 1);
+            dot[0] = fma((double)p, (double)s0, dot[0]);
+            dot[1] = fma((double)p, (double)s1, dot[1]);
+            if (MODE == BACK1) {
+                dot[2 % ND] = fma((double)L1, (double)s0, dot[2 % ND]);
+                dot[3 % ND] = fma((double)L1, (double)s1, dot[3 % ND]);
+                ps.out0[at] = ps.out0[again] = combine(ps, s0, s1);
+            }
+        }
+    });
+    if (BACK)
+        block_sums<ND>(dot, ps.partials + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kDots + (MODE == BACK2 ? 4 : 0));
+}
 
-// Adjoint workspace layout (floats in units of n, then doubles).
-struct AdjLayout {
-    size_t ckpt, seg, a, h, p, b, hp, lam, r3, la3, tgt, tmp, dots, partials, J, done, total;
-    int nck;
+// lambda^N = C^N - C* (doubled per pencil) and its squares' block sums.
+template <int DIM>
+__global__ __launch_bounds__(kT) void k_adj_misfit(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
+                                                   const uint32_t *__restrict__ perm, const RateParams prm,
+                                                   const float *__restrict__ CN, const float *__restrict__ target,
+                                                   float *__restrict__ p, double *__restrict__ partials)
+{
+    pdl_wait();
+    double d[kDots] = {0.0};
+    for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), gridDim.y * (kT / 32), [&](const Chunk &c) {
+        const int i = c.i0 + (threadIdx.x & 31);
+        if (i >= c.pe) return;
+        const uint32_t a = __ldg(perm + i);
+        const float t = a < (uint32_t)prm.n ? __ldg(target + a) : 0.f;
+        const float v = fmaf(-1.f, t, CN[c.ps + i]);
+        p[c.ps + i] = p[c.pe + i] = v;
+        d[0] = fma((double)v, (double)v, d[0]);
+    });
+    block_sums<kDots>(d, partials + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kDots);
+}
+
+// out[step][q] = sum over the blocks' partials, one CTA per step, in a fixed order.
+constexpr int kFoldT = 256;
+__global__ __launch_bounds__(kFoldT) void k_adj_fold(const double *__restrict__ partials, int blocks, double *__restrict__ out)
+{
+    pdl_wait();
+    __shared__ double sh[kFoldT / 32][kDots];
+    const double *p = partials + (size_t)blockIdx.x * blocks * kDots;
+    double s[kDots];
+#pragma unroll
+    for (int q = 0; q < kDots; ++q) s[q] = 0.0;
+    for (int b = threadIdx.x; b < blocks; b += kFoldT)
+#pragma unroll
+        for (int q = 0; q < kDots; ++q) s[q] += p[(size_t)b * kDots + q];
+#pragma unroll
+    for (int q = 0; q < kDots; ++q)
+        for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_down_sync(kFull, s[q], o);
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int q = 0; q < kDots; ++q) sh[threadIdx.x >> 5][q] = s[q];
+    __syncthreads();
+    if (threadIdx.x < kDots) {
+        double t = 0.0;
+        for (int w = 0; w < kFoldT / 32; ++w) t += sh[w][threadIdx.x];
+        out[(size_t)blockIdx.x * kDots + threadIdx.x] = t;
+    }
+}
+
+// out[perm[i]] = the doubled field's value of sorted particle i.
+__global__ __launch_bounds__(kT) void k_adj_scatter(const uint32_t *__restrict__ cs, const uint32_t *__restrict__ perm,
+                                                    const RateParams prm, const float *__restrict__ x, float *__restrict__ out)
+{
+    pdl_wait();
+    for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), gridDim.y * (kT / 32), [&](const Chunk &c) {
+        const int i = c.i0 + (threadIdx.x & 31);
+        if (i >= c.pe) return;
+        const uint32_t a = __ldg(perm + i);
+        if (a < (uint32_t)prm.n) out[a] = x[c.ps + i];
+    });
+}
+
+// Everything one call needs.
+struct Adj {
+    const ade_ctx *c;
+    cudaStream_t s;
+    RateParams rp;         // uw = vhat, ub = 0
+    FrozenTab tab;
+    float ca, cb, cal, cbl;   // L(theta) x = ca S_L + cb S_T (hi + lo)
+    ShapeConst sc;
+    dim3 grid;
 };
 
-size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
+template <int DIM, int KERNEL, bool ISO>
+cudaError_t pass_t(const Adj &A, int mode, const AdjPass &ps)
+{
+    const uint4 *P = A.c->w.P0;
+    const uint32_t *cs = A.c->w.cell_start;
+    switch (mode) {
+    case HALF: return launch_pdl(k_adj_pass<DIM, KERNEL, ISO, HALF>, A.grid, kT, 0, A.s, P, cs, A.rp, A.tab, ps);
+    case FULL: return launch_pdl(k_adj_pass<DIM, KERNEL, ISO, FULL>, A.grid, kT, 0, A.s, P, cs, A.rp, A.tab, ps);
+    case BACK1: return launch_pdl(k_adj_pass<DIM, KERNEL, ISO, BACK1>, A.grid, kT, 0, A.s, P, cs, A.rp, A.tab, ps);
+    default: return launch_pdl(k_adj_pass<DIM, KERNEL, ISO, BACK2>, A.grid, kT, 0, A.s, P, cs, A.rp, A.tab, ps);
+    }
+}
 
-AdjLayout adj_layout(int n, int nsteps, int ck)
+template <int DIM, int KERNEL, bool ISO>
+cudaError_t table_t(const Adj &A, float *C0)
+{
+    return launch_pdl(k_adj_table<DIM, KERNEL, ISO>, A.grid, kT, 0, A.s, A.c->w.P0, A.c->w.cell_start, A.rp, A.tab, A.sc, C0);
+}
+
+#define ADE_ADJ_CALL(F, ...)                                                                                          \
+    (A.c->dim == 2 ? (A.c->p.kernel == ADE_WENDLAND_C2                                                                \
+                          ? (A.c->iso ? F<2, ADE_WENDLAND_C2, true>(__VA_ARGS__) : F<2, ADE_WENDLAND_C2, false>(__VA_ARGS__))   \
+                          : (A.c->iso ? F<2, ADE_WENDLAND_C4, true>(__VA_ARGS__) : F<2, ADE_WENDLAND_C4, false>(__VA_ARGS__)))  \
+                   : (A.c->p.kernel == ADE_WENDLAND_C2                                                                \
+                          ? (A.c->iso ? F<3, ADE_WENDLAND_C2, true>(__VA_ARGS__) : F<3, ADE_WENDLAND_C2, false>(__VA_ARGS__))   \
+                          : (A.c->iso ? F<3, ADE_WENDLAND_C4, true>(__VA_ARGS__) : F<3, ADE_WENDLAND_C4, false>(__VA_ARGS__))))
+
+cudaError_t pass(const Adj &A, int mode, const AdjPass &ps) { return ADE_ADJ_CALL(pass_t, A, mode, ps); }
+cudaError_t table(const Adj &A, float *C0) { return ADE_ADJ_CALL(table_t, A, C0); }
+
+// One forward step C_out = S C_in: h = u + dt/2 L u, C_out = u + dt L h.
+cudaError_t fwd_step(const Adj &A, const float *u, float *h, float *out, float dt)
+{
+    AdjPass ps;
+    memset(&ps, 0, sizeof(ps));
+    ps.ca = A.ca;
+    ps.cb = A.cb;
+    ps.cal = A.cal;
+    ps.cbl = A.cbl;
+    ps.sc = A.sc;
+    ps.x1 = u;
+    ps.out1 = h;
+    ps.step = 0.5f * dt;
+    cudaError_t e = pass(A, HALF, ps);
+    if (e != cudaSuccess) return e;
+    ps.x1 = h;
+    ps.base = u;
+    ps.out1 = out;
+    ps.step = dt;
+    return pass(A, FULL, ps);
+}
+
+// Adjoint workspace: fields (doubled per pencil), the weight table, FP64 partials of one segment.
+struct AdjLayout {
+    size_t ckpt, seg, h, p, hp, a, dots, partials, words, slots, cursor, total;
+    size_t lines;
+    int nck, blocks;
+};
+
+AdjLayout adj_layout(const ade_ctx *c, int nsteps, int ck)
 {
     AdjLayout L;
     size_t off = 0;
     auto take = [&](size_t bytes) {
         size_t o = off;
-        off += al256(bytes > 0 ? bytes : 1);
+        off += ((bytes > 0 ? bytes : 1) + 255) & ~(size_t)255;
         return o;
     };
-    const size_t fv = (size_t)n * 4;
+    const size_t f2 = (size_t)c->n * 8;
+    size_t slots = 0;
+    frozen_extent(c, 2, &L.lines, &slots, &L.blocks);
     L.nck = (nsteps + ck - 1) / ck;
-    L.ckpt = take(fv * (L.nck + 1));
-    L.seg = take(fv * ck);
-    L.a = take(fv);
-    L.h = take(fv);
-    L.p = take(fv);
-    L.b = take(fv);
-    L.hp = take(fv);
-    L.lam = take(fv);
-    L.r3 = take(fv * 3);
-    L.la3 = take(fv * 3);
-    L.tgt = take(fv);
-    L.tmp = take(fv);
-    L.dots = take((size_t)nsteps * kMaxDots * 8);
-    L.partials = take((size_t)blocks(n) * kMaxDots * 8);
-    L.J = take(64);
-    L.done = take(64);
+    L.ckpt = take(f2 * (L.nck + 1));
+    L.seg = take(f2 * std::min(ck, nsteps));
+    L.h = take(f2);
+    L.p = take(f2);
+    L.hp = take(f2);
+    L.a = take(f2);
+    L.dots = take(((size_t)nsteps + 1) * kDots * 8);
+    L.partials = take((size_t)L.blocks * std::min(ck, nsteps) * kDots * 8);
+    L.words = take(L.lines * 128);
+    L.slots = take(slots * 16);
+    L.cursor = take(64);
     L.total = off;
     return L;
 }
+
+}  // namespace
+
+}  // namespace ade
 
 #define ADJ_CK(call)                                                                               \
     do {                                                                                           \
@@ -278,54 +410,12 @@ AdjLayout adj_layout(int n, int nsteps, int ck)
         }                                                                                          \
     } while (0)
 
-struct Adj {
-    ade_ctx *c;
-    cudaStream_t s;
-    ApplyCoef op;     // the operator L(theta) in slot 0
-    ApplyCoef basis;  // L_L, L_T, L_m in slots 0..2, theta as combination weights
-    int n;
-};
-
-template <int DIM, int KERNEL>
-cudaError_t apply_t(const Adj &A, const float *v, int multi, float *o0, float *o1, float *o2, float *comb,
-                    const float *base, float alpha, float *axpy)
-{
-    const int nb = blocks(A.n);
-    const ade::Work &w = A.c->w;
-    if (multi)
-        k_apply<DIM, KERNEL, 3><<<nb, kT, 0, A.s>>>(w.P0, w.cell_start, v, A.c->rp, A.basis, o0, o1, o2, comb,
-                                                    nullptr, 0.f, nullptr);
-    else
-        k_apply<DIM, KERNEL, 1><<<nb, kT, 0, A.s>>>(w.P0, w.cell_start, v, A.c->rp, A.op, o0, nullptr, nullptr,
-                                                    nullptr, base, alpha, axpy);
-    return cudaGetLastError();
-}
-
-cudaError_t apply(const Adj &A, const float *v, int multi, float *o0, float *o1, float *o2, float *comb,
-                  const float *base, float alpha, float *axpy)
-{
-    const int dim = A.c->dim, kern = A.c->p.kernel;
-    if (dim == 2)
-        return kern == ADE_WENDLAND_C2 ? apply_t<2, ADE_WENDLAND_C2>(A, v, multi, o0, o1, o2, comb, base, alpha, axpy)
-                                       : apply_t<2, ADE_WENDLAND_C4>(A, v, multi, o0, o1, o2, comb, base, alpha, axpy);
-    return kern == ADE_WENDLAND_C2 ? apply_t<3, ADE_WENDLAND_C2>(A, v, multi, o0, o1, o2, comb, base, alpha, axpy)
-                                   : apply_t<3, ADE_WENDLAND_C4>(A, v, multi, o0, o1, o2, comb, base, alpha, axpy);
-}
-
-// One forward step C_out = S C_in: a = L u, h = u + dt/2 a, C_out = u + dt L h.
-cudaError_t fwd_step(const Adj &A, const float *u, float *a, float *h, float *out, float dt)
-{
-    cudaError_t e = apply(A, u, 0, a, nullptr, nullptr, nullptr, u, 0.5f * dt, h);
-    if (e != cudaSuccess) return e;
-    return apply(A, h, 0, a, nullptr, nullptr, nullptr, u, dt, out);
-}
-
-}  // namespace
+using namespace ade;
 
 extern "C" int ade_adjoint_workspace_bytes(const ade_ctx *c, int nsteps, int ckpt_every, size_t *bytes)
 {
     if (!c || !bytes || nsteps < 1 || ckpt_every < 1) return ade::report_error(ADE_ERR_ARG, "bad argument");
-    *bytes = adj_layout(c->n, nsteps, ckpt_every).total;
+    *bytes = adj_layout(c, nsteps, ckpt_every).total;
     return ADE_OK;
 }
 
@@ -338,7 +428,7 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
         return ade::report_error(ADE_ERR_ARG, "bad argument");
     if (c->field) return ade::report_error(ADE_ERR_STATE, "the adjoint is for a uniform velocity (vmax = 0)");
     if (c->catt) return ade::report_error(ADE_ERR_STATE, "the adjoint is for Eq. 1 (tau = 0)");
-    const AdjLayout L = adj_layout(c->n, nsteps, ckpt_every);
+    const AdjLayout L = adj_layout(c, nsteps, ckpt_every);
     if (aws_bytes < L.total || ((uintptr_t)aws & 255u)) return ade::report_error(ADE_ERR_CAPACITY, "adjoint workspace too small or misaligned");
     const int n = c->n;
     if (n == 0) {
@@ -346,131 +436,125 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
         if (J_host) *J_host = 0.0;
         return ADE_OK;
     }
+    const double gamma = c->p.gamma > 0.0 ? c->p.gamma : c->dim + 2.0;
+    double vabs = 0.0;
+    for (int i = 0; i < c->dim; ++i) vabs += c->p.v[i] * c->p.v[i];
+    vabs = sqrt(vabs);
+    // the table's shapes are those of 2 (1 - q): 2^3 f (C2) or 2^5 f (C4), undone in the prefactor
+    const double pf = (double)c->rp.pf * (c->p.kernel == ADE_WENDLAND_C2 ? 0.125 : 0.03125);
     Adj A;
     A.c = c;
     A.s = (cudaStream_t)stream;
-    A.n = n;
-    memset(&A.op, 0, sizeof(A.op));
-    memset(&A.basis, 0, sizeof(A.basis));
-    const double gamma = c->p.gamma > 0.0 ? c->p.gamma : c->dim + 2.0;
-    ade::pair_coeffs(c->dim, gamma, c->D, A.op.Kc[0], &A.op.c0[0]);
-    const double theta[3] = {c->p.alpha_L, c->p.alpha_T, c->p.D_m};
-    double vabs2 = 0.0;
-    for (int i = 0; i < c->dim; ++i) vabs2 += c->p.v[i] * c->p.v[i];
-    const double vabs = sqrt(vabs2);
-    for (int k = 0; k < 3; ++k) {
-        // B_L = v v^T / |v|, B_T = |v| I - v v^T / |v|, B_m = I (the theta-derivatives of Eq. 3)
-        double B[9] = {0};
-        for (int i = 0; i < c->dim; ++i)
-            for (int j = 0; j < c->dim; ++j) {
-                const double vv = vabs > 0.0 ? c->p.v[i] * c->p.v[j] / vabs : 0.0;
-                const double I = i == j ? 1.0 : 0.0;
-                B[i * c->dim + j] = k == 0 ? vv : (k == 1 ? vabs * I - vv : I);
-            }
-        ade::pair_coeffs(c->dim, gamma, B, A.basis.Kc[k], &A.basis.c0[k]);
-        A.basis.theta[k] = (float)theta[k];
+    A.rp = c->rp;
+    A.rp.frame = nullptr;
+    A.rp.ub = 0.f;
+    float lo[3];
+    for (int i = 0; i < 3; ++i) {
+        const double vh = vabs > 0.0 ? (i < c->dim ? c->p.v[i] / vabs : 0.0) : (i == 0 ? 1.0 : 0.0);
+        A.rp.uw[i] = (float)vh;
+        lo[i] = (float)(vh - (double)A.rp.uw[i]);
     }
+    // 1/H in x-axis words, and the part of it that FP32 leaves
+    A.sc.lo = make_float4(lo[0], lo[1], lo[2], (float)(c->p.box[0] / kTwo32 / c->H - (double)c->rp.invH));
+    A.sc.g2 = (float)(2.0 * gamma);
+    A.sc.bT = (float)(2.0 * (gamma - c->dim) + 2.0);
+    const double sa = c->p.alpha_L * vabs + c->p.D_m, sb = c->p.alpha_T * vabs + c->p.D_m;
+    A.ca = (float)(pf * sa);
+    A.cb = (float)(pf * sb);
+    A.cal = (float)(pf * sa - (double)A.ca);
+    A.cbl = (float)(pf * sb - (double)A.cb);
+    A.grid = frozen_grid(A.rp);
     char *base = static_cast<char *>(aws);
-    float *ckpt = reinterpret_cast<float *>(base + L.ckpt);
-    float *seg = reinterpret_cast<float *>(base + L.seg);
-    float *a = reinterpret_cast<float *>(base + L.a);
-    float *h = reinterpret_cast<float *>(base + L.h);
-    float *p = reinterpret_cast<float *>(base + L.p);
-    float *bb = reinterpret_cast<float *>(base + L.b);
-    float *hp = reinterpret_cast<float *>(base + L.hp);
-    float *lam = reinterpret_cast<float *>(base + L.lam);
-    float *r3 = reinterpret_cast<float *>(base + L.r3);
-    float *la3 = reinterpret_cast<float *>(base + L.la3);
-    float *tgt = reinterpret_cast<float *>(base + L.tgt);
-    float *tmp = reinterpret_cast<float *>(base + L.tmp);
+    auto field = [&](size_t o) { return reinterpret_cast<float *>(base + o); };
+    const size_t n2 = 2 * (size_t)n;
+    float *ckpt = field(L.ckpt), *seg = field(L.seg), *h = field(L.h), *p = field(L.p), *hp = field(L.hp), *a = field(L.a);
     double *dots = reinterpret_cast<double *>(base + L.dots);
     double *partials = reinterpret_cast<double *>(base + L.partials);
-    double *Jd = reinterpret_cast<double *>(base + L.J);
-    unsigned *done = reinterpret_cast<unsigned *>(base + L.done);
+    A.tab.words = field(L.words);
+    A.tab.slots = reinterpret_cast<uint4 *>(base + L.slots);
+    A.tab.cursor = reinterpret_cast<unsigned *>(base + L.cursor);
+    A.tab.cap = (unsigned)L.lines;
+    const int nb = (int)(A.grid.x * A.grid.y);
+    if (nb > L.blocks) return ade::report_error(ADE_ERR_CAPACITY, "adjoint partials exceed the workspace");
     const float dt = (float)c->dt;
-    const int nb = blocks(n);
     cudaStream_t s = A.s;
+    const uint32_t *cs = c->w.cell_start, *perm = c->w.perm;
 
     // frozen geometry: one cell list at the current positions (counts and tile totals cleared first)
-    cudaError_t e = ade::launch_build_cells(c->dim, c->xq, c->C, n, c->nc, c->ncells, c->w, s);
-    if (e != cudaSuccess) return ade::report_error(ADE_ERR_CUDA, cudaGetErrorString(e));
-    ADJ_CK(cudaMemsetAsync(done, 0, sizeof(unsigned), s));
-    k_sorted_C<<<nb, kT, 0, s>>>(ckpt, c->w.P0, n);
-    k_gather<<<nb, kT, 0, s>>>(tgt, C_target_dev, c->w.perm, n);
-    // forward with checkpoints every ckpt_every steps
+    ADJ_CK(cudaMemsetAsync(A.tab.cursor, 0, sizeof(unsigned), s));
+    ADJ_CK(ade::launch_build_cells(c->dim, c->xq, c->C, n, c->nc, c->ncells, c->w, s));
+    c->cells_framed = false;
+    ADJ_CK(table(A, ckpt));
+    // forward: checkpoints every ckpt_every steps, the last segment's states straight into seg
+    const int l0_last = (L.nck - 1) * ckpt_every;
+    float *tmp[2] = {hp, a};   // free until the backward pass
+    const float *u = ckpt;
     for (int l = 0; l < nsteps; ++l) {
-        const float *u = (l % ckpt_every == 0) ? ckpt + (size_t)(l / ckpt_every) * n : tmp;
-        float *out = ((l + 1) % ckpt_every == 0 || l + 1 == nsteps) ? ckpt + (size_t)((l + ckpt_every) / ckpt_every) * n : tmp;
-        if (u == tmp && out == tmp) {
-            ADJ_CK(fwd_step(A, tmp, a, h, lam, dt));
-            ADJ_CK(cudaMemcpyAsync(tmp, lam, (size_t)n * 4, cudaMemcpyDeviceToDevice, s));
-        } else {
-            ADJ_CK(fwd_step(A, u, a, h, out, dt));
-        }
+        float *out;
+        if (l + 1 == nsteps) out = ckpt + (size_t)L.nck * n2;
+        else if (l + 1 > l0_last) out = seg + (size_t)(l + 1 - l0_last) * n2;
+        else if ((l + 1) % ckpt_every == 0) out = ckpt + (size_t)((l + 1) / ckpt_every) * n2;
+        else out = tmp[l & 1];
+        ADJ_CK(fwd_step(A, u, h, out, dt));
+        u = out;
     }
     // C^N sits in checkpoint slot nck (the last step always writes a slot)
-    const float *CN = ckpt + (size_t)L.nck * n;
-    if (C_final_dev) k_scatter<<<nb, kT, 0, s>>>(C_final_dev, CN, c->w.perm, n);
+    const float *CN = ckpt + (size_t)L.nck * n2;
+    if (C_final_dev) ADJ_CK(launch_pdl(k_adj_scatter, A.grid, kT, 0, s, cs, perm, A.rp, CN, C_final_dev));
     // lambda^N = C^N - C*, J = 1/2 |lambda^N|^2
-    k_axpy<<<nb, kT, 0, s>>>(p, CN, -1.0f, tgt, n);
-    {
-        DotArgs da;
-        memset(&da, 0, sizeof(da));
-        da.x[0] = p;
-        da.y[0] = p;
-        k_dots<1><<<nb, kT, 0, s>>>(da, n, partials, done, Jd);
-        ADJ_CK(cudaGetLastError());
-    }
+    if (c->dim == 2) ADJ_CK(launch_pdl(k_adj_misfit<2>, A.grid, kT, 0, s, c->w.P0, cs, perm, A.rp, CN, C_target_dev, p, partials));
+    else ADJ_CK(launch_pdl(k_adj_misfit<3>, A.grid, kT, 0, s, c->w.P0, cs, perm, A.rp, CN, C_target_dev, p, partials));
+    ADJ_CK(launch_pdl(k_adj_fold, 1, kFoldT, 0, s, partials, nb, dots + (size_t)nsteps * kDots));
     // backward, segment by segment
-    float *r[3] = {r3, r3 + n, r3 + 2 * (size_t)n};
-    float *la[3] = {la3, la3 + n, la3 + 2 * (size_t)n};
+    AdjPass ps;
+    memset(&ps, 0, sizeof(ps));
+    ps.ca = A.ca;
+    ps.cb = A.cb;
+    ps.cal = A.cal;
+    ps.cbl = A.cbl;
+    ps.sc = A.sc;
     for (int sgi = L.nck - 1; sgi >= 0; --sgi) {
         const int l0 = sgi * ckpt_every;
         const int l1 = l0 + ckpt_every < nsteps ? l0 + ckpt_every : nsteps;
-        ADJ_CK(cudaMemcpyAsync(seg, ckpt + (size_t)sgi * n, (size_t)n * 4, cudaMemcpyDeviceToDevice, s));
-        for (int l = l0; l + 1 < l1; ++l)
-            ADJ_CK(fwd_step(A, seg + (size_t)(l - l0) * n, a, h, seg + (size_t)(l + 1 - l0) * n, dt));
+        auto state = [&](int l) { return l == l0 ? ckpt + (size_t)sgi * n2 : seg + (size_t)(l - l0) * n2; };
+        if (sgi < L.nck - 1)
+            for (int l = l0; l + 1 < l1; ++l) ADJ_CK(fwd_step(A, state(l), h, state(l + 1), dt));
         for (int l = l1 - 1; l >= l0; --l) {
-            const float *u = seg + (size_t)(l - l0) * n;
-            // r_k = L_k u and a = L u;  la_k = L_k a
-            ADJ_CK(apply(A, u, 1, r[0], r[1], r[2], a, nullptr, 0.f, nullptr));
-            ADJ_CK(apply(A, a, 1, la[0], la[1], la[2], nullptr, nullptr, 0.f, nullptr));
-            // b = L p, hp = p + dt/2 b
-            ADJ_CK(apply(A, p, 0, bb, nullptr, nullptr, nullptr, p, 0.5f * dt, hp));
-            DotArgs da;
-            for (int k = 0; k < 3; ++k) {
-                da.x[k] = p;
-                da.y[k] = r[k];
-                da.x[3 + k] = p;
-                da.y[3 + k] = la[k];
-                da.x[6 + k] = bb;
-                da.y[6 + k] = r[k];
-            }
-            k_dots<9><<<nb, kT, 0, s>>>(da, n, partials, done, dots + (size_t)l * kMaxDots);
-            ADJ_CK(cudaGetLastError());
-            // lambda^l = p + dt L hp
-            ADJ_CK(apply(A, hp, 0, bb, nullptr, nullptr, nullptr, p, dt, lam));
-            ADJ_CK(cudaMemcpyAsync(p, lam, (size_t)n * 4, cudaMemcpyDeviceToDevice, s));
+            // a = L u, b = L p, hp = p + dt/2 b, then lambda^l = p + dt L hp (into p)
+            ps.partials = partials + (size_t)(l - l0) * nb * kDots;
+            ps.x0 = state(l);
+            ps.x1 = p;
+            ps.base = nullptr;
+            ps.out0 = a;
+            ps.out1 = hp;
+            ps.step = 0.5f * dt;
+            ADJ_CK(pass(A, BACK1, ps));
+            ps.x0 = a;
+            ps.x1 = hp;
+            ps.base = p;
+            ps.out0 = nullptr;
+            ps.out1 = p;
+            ps.step = dt;
+            ADJ_CK(pass(A, BACK2, ps));
         }
+        ADJ_CK(launch_pdl(k_adj_fold, (unsigned)(l1 - l0), kFoldT, 0, s, partials, nb, dots + (size_t)l0 * kDots));
     }
-    if (dJdC0_dev) k_scatter<<<nb, kT, 0, s>>>(dJdC0_dev, p, c->w.perm, n);
-    ADJ_CK(cudaGetLastError());
-    std::vector<double> hd((size_t)nsteps * kMaxDots);
-    double Jh = 0.0;
+    if (dJdC0_dev) ADJ_CK(launch_pdl(k_adj_scatter, A.grid, kT, 0, s, cs, perm, A.rp, (const float *)p, dJdC0_dev));
+    std::vector<double> hd(((size_t)nsteps + 1) * kDots);
     ADJ_CK(cudaMemcpyAsync(hd.data(), dots, hd.size() * 8, cudaMemcpyDeviceToHost, s));
-    ADJ_CK(cudaMemcpyAsync(&Jh, Jd, 8, cudaMemcpyDeviceToHost, s));
     ADJ_CK(cudaStreamSynchronize(s));
-    if (J_host) *J_host = 0.5 * Jh;
+    if (J_host) *J_host = 0.5 * hd[(size_t)nsteps * kDots];
     if (dJdtheta_host) {
+        // sum_l dt p.(L_k u) + dt^2/2 (p.(L_k a) + b.(L_k u)) of S_L and S_T
         const double dtd = (double)dt;
-        for (int k = 0; k < 3; ++k) {
-            double g = 0.0;
-            for (int l = 0; l < nsteps; ++l) {
-                const double *d = hd.data() + (size_t)l * kMaxDots;
-                g += dtd * d[k] + 0.5 * dtd * dtd * (d[3 + k] + d[6 + k]);
-            }
-            dJdtheta_host[k] = g;
+        double g[2] = {0.0, 0.0};
+        for (int l = 0; l < nsteps; ++l) {
+            const double *d = hd.data() + (size_t)l * kDots;
+            for (int q = 0; q < 2; ++q) g[q] += dtd * d[q] + 0.5 * dtd * dtd * (d[4 + q] + d[2 + q]);
         }
+        dJdtheta_host[0] = pf * vabs * g[0];
+        dJdtheta_host[1] = pf * vabs * g[1];
+        dJdtheta_host[2] = pf * (g[0] + g[1]);
     }
     return ADE_OK;
 }

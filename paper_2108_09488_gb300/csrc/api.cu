@@ -387,7 +387,7 @@ struct Derived {
 // long as its longest lane's range: the particles of the row's pencil within the chord that the
 // smallest transverse distance between the two pencils leaves, plus the spread of 32 lanes' counts
 // on an irregular set.  Chunks that find no room are evaluated from the positions.
-size_t frozen_lines(const ade_params &p, double H, int n, const Grid &g)
+size_t frozen_lines(const ade_params &p, double H, int n, const Grid &g, int val = 1)
 {
     const double per = (double)n / g.ncells;                  // particles per cell
     const double sx = p.box[0] / g.nc[0], sy = p.box[1] / g.nc[1], sz = p.dim == 3 ? p.box[2] / g.nc[2] : 0.0;
@@ -395,7 +395,7 @@ size_t frozen_lines(const ade_params &p, double H, int n, const Grid &g)
     for (int r = 0; r < g.nrows; ++r) {
         const double ey = fmax(abs(g.rows[r].dy) - 1.0, 0.0) * sy, ez = fmax(abs(g.rows[r].dz) - 1.0, 0.0) * sz;
         const double mu = 2.0 * sqrt(fmax(H * H - ey * ey - ez * ez, 0.0)) / sx * per;
-        lines += mu + 1.2 * sqrt(mu) + 2.5;                   // and the row's first indices, in use and as scratch
+        lines += val * (mu + 1.2 * sqrt(mu) + 0.5) + 2.0;     // and the row's first indices, in use and as scratch
     }
     const double np = (double)(g.ncells / g.nc[0]);
     return (size_t)((n / 32.0 + 0.6 * fmin(np, (double)n)) * lines) + 1024;
@@ -780,21 +780,25 @@ T *at(void *base, size_t off)
 
 }  // namespace
 
-// Pair-factor constants for a uniform tensor D (Eq. 5 with K = 2D):
-// Gamma x^T K x / r^2 - tr K = x^T Gamma (K - K_last I) x / r^2 + (Gamma K_last - tr K).
-void ade::pair_coeffs(int dm, double gamma, const double *D, float *Kc, float *c0)
+void ade::frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots, int *blocks)
 {
-    auto K = [&](int i, int j) { return 2.0 * D[i * dm + j]; };  // harmonic mean of equal D
-    const double Klast = K(dm - 1, dm - 1);
-    double trK = 0.0;
-    for (int i = 0; i < dm; ++i) trK += K(i, i);
-    Kc[0] = (float)(gamma * (K(0, 0) - Klast));
-    Kc[1] = dm == 3 ? (float)(gamma * (K(1, 1) - Klast)) : 0.0f;
-    Kc[2] = 0.0f;
-    Kc[3] = (float)(2.0 * gamma * K(0, 1));
-    Kc[4] = dm == 3 ? (float)(2.0 * gamma * K(0, 2)) : 0.0f;
-    Kc[5] = dm == 3 ? (float)(2.0 * gamma * K(1, 2)) : 0.0f;
-    *c0 = (float)(gamma * Klast - trK);
+    *lines = *slots = 0;
+    *blocks = 1;
+    const bool fixed = c->p.cell_subdiv > 0 || c->p.flags != 0u;   // no autotuning: the grid in use
+    for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
+        Grid g;
+        if ((fixed && k != c->subdiv) || !make_grid(c->p, c->Hgrid, k, &g)) continue;
+        *lines = std::max(*lines, frozen_lines(c->p, c->H, c->n, g, val));
+        *slots = std::max(*slots, (size_t)c->n / 32 + (size_t)(g.ncells / g.nc[0]) + 2);
+        ade::RateParams rp;
+        memset(&rp, 0, sizeof(rp));
+        rp.n = c->n;
+        rp.ncy = g.nc[1];
+        rp.ncz = g.nc[2];
+        const dim3 d = ade::frozen_grid(rp);
+        *blocks = std::max(*blocks, (int)(d.x * d.y));
+    }
+    *lines = std::min(*lines, (size_t)(kFrozenMaxBytes / 128.0));
 }
 
 // Eq. 3 gives D = d_T I + (d_L - d_T) vhat vhat^T with d_T = alpha_T |v| + D_m, d_L = alpha_L |v| + D_m;

@@ -8,16 +8,7 @@
 // instead of about 39 instructions.  The table belongs to one call: it is rebuilt from the
 // positions by every call that uses it.
 //
-// Layout.  A warp owns up to 32 consecutive sorted particles (lane = particle) of one pencil (the
-// cells of one (cy, cz) row along x), so its lanes share the stencil rows.  Per row the lanes' in-
-// support candidates are contiguous index ranges, trimmed at both ends to the first and last
-// candidate that can lie inside H; m = the longest lane's length.  All storage is in 32-word lines
-// (128 B, lane = word): per chunk the rows' m (one word each), then per row, in stencil order, one
-// line of first indices and m lines of weights: one linear stream per chunk.  The concentrations are
-// kept twice per pencil, back to back (particle j of pencil [ps, pe) at ps + j and again at pe + j),
-// so that a range that runs over the periodic x seam stays contiguous.  A chunk that finds no room in
-// the table is marked and evaluated from the positions instead (the same sums), so a table that is
-// too small costs time, never a result.
+// The table's layout is described in frozen_table.cuh.
 //
 // The arithmetic of each weight, the order of the sum inside a row (FP32) and over the rows
 // (Neumaier) are those of the branch-free walks of rate.cu, and every candidate left out has
@@ -32,386 +23,9 @@ namespace {
 
 #include "rate_walk.cuh"
 
+#include "frozen_table.cuh"
+
 constexpr int kT = kFrozenThreads;
-constexpr unsigned kFull = 0xffffffffu;
-constexpr unsigned kNoRoom = 0xffffffffu;
-
-// Where one warp's chunk lies: particles [i0, min(i0 + 32, pe)) of pencil p (cy, cz).
-struct Chunk {
-    int cy, cz, i0, ps, pe, slot;
-};
-
-// Origin of the build's cell grid along x (the records hold the positions of the build: no drift).
-__device__ __forceinline__ uint32_t frame_x(const RateParams &prm) { return prm.frame ? __ldg(prm.frame + 4) : 0u; }
-
-// Weight of the pair (a, b): the branch-free walks' product of shape and pair factor; 0 outside the
-// support and at zero separation.
-template <int DIM, int KERNEL, bool ISO>
-__device__ __forceinline__ float pair_weight(const uint4 &pa, const uint4 &pb, const PairConst &k)
-{
-    float dx = sep(pa.x, pb.x, k.m1), dy = sep(pa.y, pb.y, k.m1), dz = 0.f;
-    if (DIM == 3) dz = sep(pa.z, pb.z, k.m1);
-    if (!ISO) {
-        dy *= k.sy;
-        if (DIM == 3) dz *= k.sz;
-    }
-    float r2 = fmaf(dx, dx, dy * dy);
-    if (DIM == 3) r2 = fmaf(dz, dz, r2);
-    const float rinv = rsqrt_ftz(r2);
-    const float om = fmaf(-(r2 * rinv), k.invH, 1.f);
-    const float omq2 = fmaxf(om + om, 0.f);
-    const float s = fmaxf(dcal<DIM>(dx, dy, dz, rinv, k), -3.402823466e38f);
-    return shape2x<KERNEL>(omq2) * s;
-}
-
-// Squared separation in x units^2.
-template <int DIM, bool ISO>
-__device__ __forceinline__ float sep2(const uint4 &pa, const uint4 &pb, const PairConst &k)
-{
-    float dx = sep(pa.x, pb.x, k.m1), dy = sep(pa.y, pb.y, k.m1), dz = 0.f;
-    if (DIM == 3) dz = sep(pa.z, pb.z, k.m1);
-    if (!ISO) {
-        dy *= k.sy;
-        if (DIM == 3) dz *= k.sz;
-    }
-    float r2 = fmaf(dx, dx, dy * dy);
-    if (DIM == 3) r2 = fmaf(dz, dz, r2);
-    return r2;
-}
-
-// The weights of two candidates, the FP32 part in packed FP32x2 instructions (each half with the
-// operations of pair_weight, so the same bits).
-template <int DIM, int KERNEL, bool ISO>
-__device__ __forceinline__ float2 pair_weight2(const uint4 &pa, const uint4 &p0, const uint4 &p1, const PairConst2 &k)
-{
-    float2 dx = f2(sep(pa.x, p0.x, k.m1), sep(pa.x, p1.x, k.m1));
-    float2 dy = f2(sep(pa.y, p0.y, k.m1), sep(pa.y, p1.y, k.m1));
-    float2 dz = f2(0.f, 0.f);
-    if (DIM == 3) dz = f2(sep(pa.z, p0.z, k.m1), sep(pa.z, p1.z, k.m1));
-    if (!ISO) {
-        dy = __fmul2_rn(dy, k.sy);
-        if (DIM == 3) dz = __fmul2_rn(dz, k.sz);
-    }
-    float2 r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
-    if (DIM == 3) r2 = __ffma2_rn(dz, dz, r2);
-    const float2 rinv = f2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-    const float2 om = __ffma2_rn(__fmul2_rn(r2, rinv), k.ninvH, f2(1.f, 1.f));
-    const float2 omq2 = f2(fmaxf(om.x + om.x, 0.f), fmaxf(om.y + om.y, 0.f));
-    const float2 sr = dcal2<DIM>(dx, dy, dz, rinv, k);
-    const float2 sc = f2(fmaxf(sr.x, -3.402823466e38f), fmaxf(sr.y, -3.402823466e38f));
-    return __fmul2_rn(shape2x2<KERNEL>(omq2), sc);
-}
-
-// Cyclic candidate range of cells [lo, hi) of the pencil row whose cells start at `base` and whose
-// particles are [qs, qe): first index and count (a range over the seam continues at qs).
-__device__ __forceinline__ void cyclic_range(const uint32_t *__restrict__ cs, int base, int lo, int hi, int ncx,
-                                             int qs, int qe, int &s, int &cnt)
-{
-    const bool wl = lo < 0, wh = hi > ncx;
-    s = (int)__ldg(cs + base + (wl ? lo + ncx : lo));
-    const int e = (int)__ldg(cs + base + (wh ? hi - ncx : hi));
-    cnt = (wl || wh) ? (qe - s) + (e - qs) : e - s;
-}
-
-// Stencil row r seen from pencil (cy, cz): its pencil index.
-template <int DIM>
-__device__ __forceinline__ int row_pencil_of(const StencilRow &r, int cy, int cz, const RateParams &prm)
-{
-    int yy = cy + r.dy;
-    yy += yy < 0 ? prm.ncy : 0;
-    yy -= yy >= prm.ncy ? prm.ncy : 0;
-    int zz = 0;
-    if (DIM == 3) {
-        zz = cz + r.dz;
-        zz += zz < 0 ? prm.ncz : 0;
-        zz -= zz >= prm.ncz ? prm.ncz : 0;
-    }
-    return zz * prm.ncy + yy;
-}
-
-// Row sums over the positions for a chunk without room in the table: the full stencil, concentrations
-// from C (doubled per pencil), or from the records where C is NULL.
-template <int DIM, int KERNEL, bool ISO>
-__device__ __noinline__ float walk_chunk(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
-                                         const RateParams &prm, const Chunk &c, const float *__restrict__ C)
-{
-    const int lane = threadIdx.x & 31;
-    const int i = min(c.i0 + lane, c.pe - 1);
-    const uint4 pa = __ldg(P + i);
-    const float Ca = C ? C[c.ps + i] : __uint_as_float(pa.w);
-    const int ncx = prm.ncx;
-    const int cx = (int)__umulhi(pa.x - frame_x(prm), (uint32_t)ncx);
-    const PairConst k(prm);
-    float acc = 0.f, comp = 0.f;
-    for (int r = 0; r < prm.nrows; ++r) {
-        const StencilRow row = prm.rows[r];
-        const int q = row_pencil_of<DIM>(row, c.cy, c.cz, prm);
-        const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
-        int s, cnt;
-        cyclic_range(cs, q * ncx, cx - (int)row.w, cx + row.w + 1, ncx, qs, qe, s, cnt);
-        float rs = 0.f;
-        for (int t = 0; t < cnt; ++t) {
-            int j = s + t;
-            j = j >= qe ? j - len : j;
-            const uint4 pb = __ldg(P + j);
-            rs = fmaf(pair_weight<DIM, KERNEL, ISO>(pa, pb, k), Ca - (C ? C[qs + j] : __uint_as_float(pb.w)), rs);
-        }
-        neumaier_add(acc, comp, rs);
-    }
-    return acc + comp;
-}
-
-// Weights of one chunk into the table, and the row sums of the first evaluation (the concentrations
-// of the records).  BOX: the pencils' transverse boxes and the staged rows are at hand (square or
-// cubic single plumes): rows out of the warp's reach are skipped, as in the trimmed walks, and a
-// lane's range is cut at the x half-extent its own distance to the row leaves.  Otherwise every row is
-// looked at and a range is cut by the separations themselves.
-template <int DIM, int KERNEL, bool ISO, bool BOX>
-__device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs, const RateParams &prm,
-                             const Chunk &c, const uint4 &pa, const TrimRow *srow, const FrozenTab &tab)
-{
-    const int lane = threadIdx.x & 31;
-    const int ncx = prm.ncx, nrows = prm.nrows;
-    const int cx = (int)__umulhi(pa.x - frame_x(prm), (uint32_t)ncx);
-    const bool valid = c.i0 + lane < c.pe;
-    TrimSelf me = {};
-    float ylo = 0.f, yhi = 0.f, zlo = 0.f, zhi = 0.f;
-    const TrimGeom g(prm);
-    const float wpc = 4294967296.f / (float)ncx;     // x words per cell
-    const PairConst k(prm);
-    const float far2 = prm.H2 * (1.f + 1.f / 4096.f);   // beyond this the weight is exactly 0
-    int nr = nrows;
-    if (BOX) {
-        me = trim_self<DIM>(pa, c.cy, c.cz, prm);
-        ylo = yhi = me.fy;
-        zlo = zhi = me.fz;
-        warp_interval<DIM>(ylo, yhi, zlo, zhi);
-        nr = 0;
-        for (int rb = 0; rb < nrows; rb += 32) {
-            float xe;
-            int pidx, wx;
-            nr += __popc(__ballot_sync(kFull, warp_row_test<DIM>(rb, srow, nrows, me, c.cy, c.cz, prm, g, ylo, yhi, zlo, zhi,
-                                                                 xe, pidx, wx)));
-        }
-    }
-    // scratch lines for the rows in reach of the chunk: {m, pencil} of each row, then its first indices
-    const int hl = (nr + 15) >> 4;
-    unsigned meta = 0u;
-    if (lane == 0) meta = atomicAdd(tab.cursor, (unsigned)(hl + nr));
-    meta = __shfl_sync(kFull, meta, 0);
-    bool room = meta <= tab.cap && tab.cap - meta >= (unsigned)(hl + nr);
-    if (!room) {
-        if (lane == 0) tab.slots[c.slot] = make_uint4(kNoRoom, 0u, 0u, 0u);
-        return walk_chunk<DIM, KERNEL, ISO>(P, cs, prm, c, nullptr);
-    }
-    int2 *row = reinterpret_cast<int2 *>(tab.words + (size_t)meta * 32);
-    int *first = reinterpret_cast<int *>(tab.words) + (size_t)(meta + hl) * 32;
-    unsigned R = 0u, lines = 0u;
-    for (int rb = 0; rb < nrows; rb += 32) {
-        float xe = 0.f;
-        int pidx = 0, wx = 0;
-        bool reach;
-        if (BOX) {
-            reach = warp_row_test<DIM>(rb, srow, nrows, me, c.cy, c.cz, prm, g, ylo, yhi, zlo, zhi, xe, pidx, wx);
-        } else {
-            reach = rb + lane < nrows;
-            if (reach) {
-                const StencilRow r = prm.rows[rb + lane];
-                pidx = row_pencil_of<DIM>(r, c.cy, c.cz, prm);
-                wx = r.w;
-            }
-        }
-        for (unsigned mask = __ballot_sync(kFull, reach); mask != 0u; mask &= mask - 1u) {
-            const int b = __ffs(mask) - 1;
-            const int q = __shfl_sync(kFull, pidx, b), w = __shfl_sync(kFull, wx, b) & 0xff;
-            int dlo = -w, dhi = w;
-            int xw = 0x7fffffff;                      // the lane's x half-extent in words
-            if (BOX) {
-                const TrimRow r = srow[rb + b];
-                const float e2 = row_gap2<DIM>(load_box(prm, q), r, me.fy, me.fy, 0.f, me.fz, me.fz, 0.f, g);
-                const float t = g.Hm2 - e2;
-                const float xl = t > 0.f ? fmaf(t * rsqrt_ftz(t), g.inv_wx, 1.f / 4096.f) : 0.f;
-                dlo = max(__float2int_rd(me.fx - xl), -w);
-                dhi = min(__float2int_rd(me.fx + xl), w);
-                xw = t > 0.f ? __float2int_ru(fminf(xl * wpc, 2.0e9f)) : -1;
-            }
-            const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
-            int s, cnt;
-            cyclic_range(cs, q * ncx, cx + dlo, cx + dhi + 1, ncx, qs, qe, s, cnt);
-            if (!valid || xw < 0) cnt = 0;
-            if (s >= qe) s = qs;                     // (the range's first cells are empty)
-            if (BOX) {
-                // candidates farther than xw along x lie beyond H (1 + 2^-12): weight exactly 0
-                while (cnt > 0) {
-                    const int d = (int)(__ldg(&P[s].x) - pa.x);
-                    if (d >= -xw && d <= xw) break;
-                    --cnt;
-                    s = s + 1 < qe ? s + 1 : qs;
-                }
-                while (cnt > 0) {
-                    const int j = s + cnt - 1;
-                    const int d = (int)(__ldg(&P[j >= qe ? j - len : j].x) - pa.x);
-                    if (d >= -xw && d <= xw) break;
-                    --cnt;
-                }
-            } else {
-                while (cnt > 0 && !(sep2<DIM, ISO>(pa, __ldg(P + s), k) < far2)) {
-                    --cnt;
-                    s = s + 1 < qe ? s + 1 : qs;
-                }
-                while (cnt > 0) {
-                    const int j = s + cnt - 1;
-                    if (sep2<DIM, ISO>(pa, __ldg(P + (j >= qe ? j - len : j)), k) < far2) break;
-                    --cnt;
-                }
-            }
-            const int m = (int)__reduce_max_sync(kFull, (unsigned)cnt);
-            if (m == 0) continue;
-            // idle tail iterations of a shorter lane stay inside the doubled pencil (m <= len)
-            if (lane == 0) row[R] = make_int2(m, q);
-            first[R * 32 + lane] = s;
-            ++R;
-            lines += (unsigned)m;
-        }
-    }
-    const unsigned hs = (R + 31u) >> 5;
-    unsigned off = 0u;
-    if (lane == 0) off = atomicAdd(tab.cursor, hs + R + lines);
-    off = __shfl_sync(kFull, off, 0);
-    room = off <= tab.cap && tab.cap - off >= hs + R + lines;
-    if (lane == 0) tab.slots[c.slot] = make_uint4(room ? off : kNoRoom, R, hs + R + lines, 0u);
-    if (!room) return walk_chunk<DIM, KERNEL, ISO>(P, cs, prm, c, nullptr);
-    __syncwarp();
-    const PairConst2 k2(k, k.m1);
-    const float Ca = __uint_as_float(pa.w);
-    float acc = 0.f, comp = 0.f;
-    float *out = tab.words + (size_t)off * 32 + lane;
-    for (unsigned r = lane; r < hs * 32; r += 32) out[r - lane] = __int_as_float(r < R ? row[r].x : 0);
-    out += (size_t)hs * 32;
-    for (unsigned r = 0; r < R; ++r) {
-        const int2 h = row[r];
-        const int m = h.x, qs = (int)__ldg(cs + h.y * ncx), qe = (int)__ldg(cs + h.y * ncx + ncx), len = qe - qs;
-        const int s = first[r * 32 + lane];
-        out[0] = __int_as_float(s + qs);            // index into the doubled concentrations
-        out += 32;
-        float rs = 0.f;
-        int t = 0;
-#pragma unroll 2
-        for (; t + 1 < m; t += 2, out += 64) {
-            const int j0 = s + t, j1 = j0 + 1;
-            const uint4 p0 = __ldg(P + (j0 >= qe ? j0 - len : j0)), p1 = __ldg(P + (j1 >= qe ? j1 - len : j1));
-            const float2 w = pair_weight2<DIM, KERNEL, ISO>(pa, p0, p1, k2);
-            out[0] = w.x;
-            out[32] = w.y;
-            rs = fmaf(w.x, Ca - __uint_as_float(p0.w), rs);
-            rs = fmaf(w.y, Ca - __uint_as_float(p1.w), rs);
-        }
-        if (t < m) {
-            const int j = s + t;
-            const uint4 pb = __ldg(P + (j >= qe ? j - len : j));
-            const float w = pair_weight<DIM, KERNEL, ISO>(pa, pb, k);
-            out[0] = w;
-            rs = fmaf(w, Ca - __uint_as_float(pb.w), rs);
-            out += 32;
-        }
-        neumaier_add(acc, comp, rs);
-    }
-    return acc + comp;
-}
-
-// Weights are read once per evaluation: keep them out of L1, where the concentrations live.
-__device__ __forceinline__ float ld_weight(const float *p)
-{
-    float v;
-    asm("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
-
-// M lines of one row (M a compile-time count: every load of the row in flight at once).
-template <int M>
-__device__ __forceinline__ float row_lines(const float *__restrict__ w, const float *__restrict__ Cr, float Ca, float rs)
-{
-    float wv[M], cv[M];
-#pragma unroll
-    for (int u = 0; u < M; ++u) {
-        wv[u] = ld_weight(w + u * 32);
-        cv[u] = Cr[u];
-    }
-#pragma unroll
-    for (int u = 0; u < M; ++u) rs = fmaf(wv[u], Ca - cv[u], rs);
-    return rs;
-}
-
-__device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes)
-{
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-// sum_b w_ab (C_a - C_b) of the chunk's particles from the table (`C` doubled per pencil).  Lane 0
-// keeps the stream kAhead lines ahead in L2 with bulk prefetches; the next row's first indices are
-// loaded before the current row's lines.
-constexpr int kAhead = 32, kPiece = 16;   // lines
-
-__device__ __forceinline__ float stream_chunk(const uint4 sl, const FrozenTab &tab, const float *__restrict__ C, float Ca)
-{
-    const int lane = threadIdx.x & 31;
-    const int R = (int)sl.y;
-    const float *base = tab.words + (size_t)sl.x * 32;
-    const float *w = base + lane;
-    const int total = (int)sl.z;
-    int ahead = min(total, kAhead);
-    if (lane == 0) prefetch_l2(base, (unsigned)ahead * 128u);
-    const float *hdr = w;
-    w += (size_t)((R + 31) >> 5) * 32;
-    float acc = 0.f, comp = 0.f;
-    int hm = 0;
-    float s = ld_weight(w);
-    for (int r = 0; r < R; ++r) {
-        if ((r & 31) == 0) hm = __float_as_int(ld_weight(hdr + r));
-        const int m = __shfl_sync(kFull, hm, r & 31);
-        const float *Cr = C + __float_as_int(s);
-        const float *wl = w + 32;
-        w = wl + m * 32;
-        if (r + 1 < R) s = ld_weight(w);
-        const int pos = (int)((w - base) >> 5);
-        if (ahead < total && pos + kAhead > ahead + kPiece) {
-            const int n = min(total - ahead, pos + kAhead - ahead);
-            if (lane == 0) prefetch_l2(base + (size_t)ahead * 32, (unsigned)n * 128u);
-            ahead += n;
-        }
-        float rs = 0.f;
-        int k = m;
-        for (; k > 8; k -= 8, wl += 256, Cr += 8) rs = row_lines<8>(wl, Cr, Ca, rs);
-        switch (k) {
-        case 1: rs = row_lines<1>(wl, Cr, Ca, rs); break;
-        case 2: rs = row_lines<2>(wl, Cr, Ca, rs); break;
-        case 3: rs = row_lines<3>(wl, Cr, Ca, rs); break;
-        case 4: rs = row_lines<4>(wl, Cr, Ca, rs); break;
-        case 5: rs = row_lines<5>(wl, Cr, Ca, rs); break;
-        case 6: rs = row_lines<6>(wl, Cr, Ca, rs); break;
-        case 7: rs = row_lines<7>(wl, Cr, Ca, rs); break;
-        default: rs = row_lines<8>(wl, Cr, Ca, rs); break;
-        }
-        neumaier_add(acc, comp, rs);
-    }
-    return acc + comp;
-}
-
-// The warp's chunks: warp v of pencil p takes chunks v, v + nv, ...
-template <class F>
-__device__ __forceinline__ void for_chunks(const uint32_t *__restrict__ cs, const RateParams &prm, int p, int p0, int v, int nv,
-                                           F f)
-{
-    Chunk c;
-    c.cy = p % prm.ncy;
-    c.cz = p / prm.ncy;
-    c.ps = (int)__ldg(cs + p * prm.ncx);
-    c.pe = (int)__ldg(cs + p * prm.ncx + prm.ncx);
-    for (c.i0 = c.ps + 32 * v; c.i0 < c.pe; c.i0 += 32 * nv) {
-        c.slot = (c.i0 >> 5) + p0 + p;   // increases strictly from chunk to chunk
-        f(c);
-    }
-}
 
 // Predictor (C -> Ch) or corrector (C updated from the rate at Ch) of one particle, Eq. 8-9, or the
 // same for Cattaneo's (C, Q), Eq. 14 (see epilogue in rate_walk.cuh); Cl, ql: C and Q at level l.
@@ -449,7 +63,7 @@ __global__ __launch_bounds__(kT) void k_frozen_build(const uint4 *__restrict__ P
     for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), nv, [&](const Chunk &c) {
         const int i = c.i0 + (threadIdx.x & 31);
         const uint4 pa = __ldg(P + min(i, c.pe - 1));
-        const float sum = build_chunk<DIM, KERNEL, ISO, ISO>(P, cs, prm, c, pa, srow, tab);
+        const float sum = build_chunk<DIM, KERNEL, ISO, ISO, 1>(P, cs, prm, c, pa, srow, tab);
         if (i >= c.pe) return;
         const float Cl = __uint_as_float(pa.w);
         st.C[c.ps + i] = st.C[c.pe + i] = Cl;
@@ -497,7 +111,7 @@ __global__ __launch_bounds__(kT) void k_frozen_build_batch(const uint4 *__restri
     for_chunks(cs + prm.coff, prm, it.pencil, it.p0, it.y, it.ny, [&](const Chunk &c) {
         const int i = c.i0 + (threadIdx.x & 31);
         const uint4 pa = __ldg(P + min(i, c.pe - 1));
-        const float sum = build_chunk<DIM, KERNEL, true, false>(P, cs + prm.coff, prm, c, pa, nullptr, tab);
+        const float sum = build_chunk<DIM, KERNEL, true, false, 1>(P, cs + prm.coff, prm, c, pa, nullptr, tab);
         if (i >= c.pe) return;
         const float Cl = __uint_as_float(pa.w);
         st.C[c.ps + i] = st.C[c.pe + i] = Cl;
@@ -593,24 +207,11 @@ __global__ __launch_bounds__(kT) void k_frozen_finish(const uint4 *__restrict__ 
     warp_finish<EPI_CORRECT, false, kT>(acc, out);
 }
 
-// Grid: one block column per pencil, enough blocks along y for the mean pencil's chunks (a fuller
-// pencil's warps take several).  A grid of less than about four waves gets twice that, so that on a
-// small set one full pencil (two lattice lines where the others hold one) does not make a tail:
-// 256^2 at 3 cells per H 11.6 -> 8.3 us per evaluation.
-dim3 chunk_grid(const RateParams &prm)
-{
-    const int np = prm.ncy * prm.ncz;
-    const int mean = (prm.n + np - 1) / np;
-    int y = (mean + kT - 1) / kT;
-    if ((long long)np * y < 8192) y *= 2;
-    return dim3((unsigned)np, (unsigned)y, 1);
-}
-
 template <int DIM, int KERNEL, bool ISO>
 cudaError_t build_t(const uint4 *P, const uint32_t *cs, const uint32_t *perm, const RateParams &prm,
                     const FrozenTab &tab, const FrozenState &st, cudaStream_t s)
 {
-    return launch_pdl(k_frozen_build<DIM, KERNEL, ISO>, chunk_grid(prm), kT, 0, s, P, cs, perm, prm, tab, st);
+    return launch_pdl(k_frozen_build<DIM, KERNEL, ISO>, frozen_grid(prm), kT, 0, s, P, cs, perm, prm, tab, st);
 }
 
 template <int DIM, int KERNEL, bool ISO>
@@ -618,11 +219,24 @@ cudaError_t rate_t(int epi, const uint4 *P, const uint32_t *cs, const RateParams
                    const FrozenState &st, cudaStream_t s)
 {
     return epi == EPI_PREDICT
-               ? launch_pdl(k_frozen_rate<DIM, KERNEL, ISO, EPI_PREDICT>, chunk_grid(prm), kT, 0, s, P, cs, prm, tab, st)
-               : launch_pdl(k_frozen_rate<DIM, KERNEL, ISO, EPI_CORRECT>, chunk_grid(prm), kT, 0, s, P, cs, prm, tab, st);
+               ? launch_pdl(k_frozen_rate<DIM, KERNEL, ISO, EPI_PREDICT>, frozen_grid(prm), kT, 0, s, P, cs, prm, tab, st)
+               : launch_pdl(k_frozen_rate<DIM, KERNEL, ISO, EPI_CORRECT>, frozen_grid(prm), kT, 0, s, P, cs, prm, tab, st);
 }
 
 }  // namespace
+
+// Grid: one block column per pencil, enough blocks along y for the mean pencil's chunks (a fuller
+// pencil's warps take several).  A grid of less than about four waves gets twice that, so that on a
+// small set one full pencil (two lattice lines where the others hold one) does not make a tail:
+// 256^2 at 3 cells per H 11.6 -> 8.3 us per evaluation.
+dim3 frozen_grid(const RateParams &prm)
+{
+    const int np = prm.ncy * prm.ncz;
+    const int mean = (prm.n + np - 1) / np;
+    int y = (mean + kT - 1) / kT;
+    if ((long long)np * y < 8192) y *= 2;
+    return dim3((unsigned)np, (unsigned)(y > 0 ? y : 1), 1);
+}
 
 cudaError_t launch_frozen_build(int dim, int kernel, bool iso, const uint4 *P, const uint32_t *cs, const uint32_t *perm,
                                 const RateParams &prm, const FrozenTab &tab, const FrozenState &st, cudaStream_t s)
