@@ -144,16 +144,16 @@ struct SweepParams {
     float b[kSweepGroup];
     int g0;                       // first set of the group
     int nt;                       // sets in the group: 1, 2, 4 or 8
-    int P4;                       // stride of the interleaved sorted concentrations
+    float dL[kSweepGroup];        // alpha_L |v| + D_m and alpha_T |v| + D_m per set (0 beyond nt)
+    float dT[kSweepGroup];
 };
 
 struct SweepOut {
-    float *rate;                  // EPI_RATE: [P][n] caller order (may be NULL)
-    float *Cout;                  // EPI_PREDICT: sorted half-step concentrations [n][P4]
-    uint4 *Pout;                  // EPI_PREDICT: sorted half-step positions (group 0 writes)
-    float *C;                     // EPI_CORRECT: caller concentrations [P][n], updated in place
-    uint32_t *xq;                 // EPI_CORRECT: caller positions (group 0 writes)
-    int *status;                  // EPI_CORRECT: set to 1 on a non-finite C
+    float *rate;                  // single evaluation: [P][n] caller order (may be NULL)
+    float *Cout;                  // on-the-fly predictor: sorted half-step concentrations
+    float *C;                     // final state: caller concentrations [P][n]
+    uint32_t *xq;                 // final state: caller positions
+    int *status;                  // set to 1 on a non-finite C
     unsigned long long *pairs;    // pair counter (counting launch)
 };
 
@@ -179,6 +179,17 @@ struct FrozenState {
 struct FrozenItem {
     int plume, pencil, p0;
     unsigned short y, ny;
+};
+
+// Steps of one sweep call: sorted positions, cell table, weight table, concentrations (planes of
+// four sets, doubled per pencil) at levels l and l + 1/2, and the constants of the table's weights.
+struct SweepRun {
+    const uint4 *P;
+    const uint32_t *cs, *perm;
+    FrozenTab tab;
+    float *C, *Ch;
+    float4 lo;                    // low parts of vhat and 1/H
+    float g2, bT;                 // 2 Gamma, 2 (Gamma - d) + 2
 };
 
 // One work item of the batched rate kernel: `count` sorted particles of plume `plume` starting
@@ -318,9 +329,14 @@ cudaError_t launch_frozen_finish_batch(int dim, const uint4 *P, const uint32_t *
                                        const RateParams *descs, const uint16_t *plume_of, uint32_t steps,
                                        const FrozenTab &tab, const FrozenState &st, const EpiOut &out, cudaStream_t s);
 
-// Parameter sweep (sweep.cu).
-cudaError_t launch_sweep_gather(const uint32_t *perm, const float *C, int n, int P, int P4, float *Cs,
-                                cudaStream_t s);
+// Parameter sweep (sweep.cu): the table and the sorted concentrations (doubled pencils), one predictor or
+// corrector of a group (prm.dt; out.C set: the call's last corrector, prm.inc the drift of all steps); and
+// for short calls the gather and one evaluation with the geometry on the fly.
+cudaError_t launch_sweep_table(int dim, int kernel, bool iso, const SweepRun &r, const RateParams &prm, const float *C,
+                               int sets, int P4, cudaStream_t s);
+cudaError_t launch_sweep_pass(int dim, int kernel, bool iso, int epi, const SweepRun &r, const SweepParams &sp,
+                              const RateParams &prm, const SweepOut &out, cudaStream_t s);
+cudaError_t launch_sweep_gather(const uint32_t *perm, const float *C, int n, int P, int P4, float *Cs, cudaStream_t s);
 cudaError_t launch_rate_sweep(int dim, int kernel, int epi, bool count, const uint4 *Pe, const float *Ce,
                               const uint32_t *cell_start, const uint32_t *perm, const RateParams &prm,
                               const SweepParams &sp, const SweepOut &out, cudaStream_t s);

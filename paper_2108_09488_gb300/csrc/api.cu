@@ -2222,7 +2222,7 @@ struct ade_sweep {
     uint32_t *xq = nullptr;
     float *C = nullptr;                // caller concentrations [P][n]
     ade::Work w;
-    float *Cs0 = nullptr, *Cs1 = nullptr;   // sorted, interleaved [n][P4] at l and l + 1/2
+    float *Cs0 = nullptr, *Cs1 = nullptr;   // sorted, planes of four sets, at l and l + 1/2
     double *pstats = nullptr;               // {sum, min, max} per set
     ade::RateParams rp;
     std::vector<ade::SweepParams> groups;
@@ -2230,9 +2230,11 @@ struct ade_sweep {
     double dt = 0.0, t = 0.0;
     long long step = 0, pairs = 0;
     uint32_t inc[3], inc_half[3];
-    bool status_cleared = false;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t graph_exec = nullptr;
+    bool status_cleared = false, count_clean = false, iso = false;
+    ade::SweepRun run = {};
+    // captured runs of 1..kGraphSteps steps, each on the first call that needs it
+    cudaGraph_t graph[ade::kGraphSteps + 1] = {};
+    cudaGraphExec_t graph_exec[ade::kGraphSteps + 1] = {};
     cudaStream_t cap_stream = nullptr;
     cudaEvent_t ev[4];
     bool ev_ready = false;
@@ -2242,7 +2244,7 @@ namespace {
 
 struct SweepLayout {
     Derived d;
-    size_t Cs0, Cs1, pstats, total;
+    size_t Cs0, Cs1, pstats, words, slots, cursor, lines, total;
 };
 
 // Common parameters and workspace of a sweep.  theta may be NULL (workspace size only: the layout
@@ -2298,64 +2300,133 @@ int sweep_layout(const ade_params *p, int n, int P, const double *theta, ade_par
         off += align256(bytes > 0 ? bytes : 1);
         return o;
     };
-    L->Cs0 = take((size_t)n * P4 * 4);
-    L->Cs1 = take((size_t)n * P4 * 4);
+    L->Cs0 = take((size_t)n * P4 * 8);   // each pencil twice
+    L->Cs1 = take((size_t)n * P4 * 8);
     L->pstats = take((size_t)3 * P * 8);
+    L->lines = n > 0 ? std::min(frozen_lines(pp, L->d.H, n, L->d.g, 2), (size_t)(kFrozenMaxBytes / 128.0)) : 0;
+    L->words = take(L->lines * 128);
+    L->slots = take(((size_t)n / 32 + (size_t)(L->d.g.ncells / L->d.g.nc[0]) + 2) * 16);
+    L->cursor = take(64);
     L->total = off;
     if (pp_out) *pp_out = pp;
     return ADE_OK;
 }
 
-int sweep_cells(ade_sweep *sw, cudaStream_t s)
+// Counts, tile totals and the table's cursor arrive uninitialised: cleared once (before any capture);
+// the frame starts at the absolute grid.
+int sweep_clear_once(ade_sweep *sw, cudaStream_t s)
 {
-    ADE_CK(ade::launch_build_cells(sw->dim, sw->xq, sw->C, sw->n, sw->nc, sw->ncells, sw->w, s));
+    if (!sw->count_clean) {
+        ADE_CK(cudaMemsetAsync(sw->w.count, 0, (size_t)sw->ncells * sizeof(uint32_t), s));
+        ADE_CK(cudaMemsetAsync(sw->w.tile_sums, 0, ade::tile_sums_bytes(sw->ncells), s));
+        ADE_CK(cudaMemsetAsync(sw->run.tab.cursor, 0, sizeof(unsigned), s));
+        ADE_CK(cudaMemsetAsync(sw->w.frame, 0, ade::kFrameWords * 4, s));
+        sw->count_clean = true;
+    }
+    return ADE_OK;
+}
+
+// Cell build (in the moving frame of `steps` steps; 0: where the steps' frame stands).
+int sweep_cells(ade_sweep *sw, int steps, cudaStream_t s)
+{
+    int rc = sweep_clear_once(sw, s);
+    if (rc) return rc;
+    ade::CellFrame frame;
+    frame.words = sw->w.frame;
+    for (int i = 0; i < 3; ++i) frame.adv[i] = (uint32_t)steps * sw->inc[i];
+    cudaError_t e = ade::launch_build_cells(sw->dim, sw->xq, sw->C, sw->n, sw->nc, sw->ncells, sw->w, s, true, frame);
+    if (e != cudaSuccess) {
+        sw->count_clean = false;
+        return fail(ADE_ERR_CUDA, "%s", cudaGetErrorString(e));
+    }
+    return ADE_OK;
+}
+
+// The predictors or correctors of every group; steps > 0: the last correctors of a call of that many.
+int sweep_evals(ade_sweep *sw, int epi, int steps, cudaStream_t s)
+{
+    ade::RateParams rp = sw->rp;
+    rp.dt = (float)(epi == ade::EPI_PREDICT ? 0.5 * sw->dt : sw->dt);
+    ade::SweepOut out;
+    memset(&out, 0, sizeof(out));
+    if (steps > 0) {
+        out.C = sw->C;
+        out.xq = sw->xq;
+        out.status = sw->w.status;
+        for (int i = 0; i < 3; ++i) rp.inc[i] = (uint32_t)steps * sw->inc[i];
+    }
+    for (const ade::SweepParams &g : sw->groups)
+        ADE_CK(ade::launch_sweep_pass(sw->dim, sw->p.kernel, sw->iso, epi, sw->run, g, rp, out, s));
+    return ADE_OK;
+}
+
+// Cells, concentrations and weights of a call of `steps` steps.
+int sweep_begin(ade_sweep *sw, int steps, cudaStream_t s)
+{
+    int rc = sweep_cells(sw, steps, s);
+    if (rc || sw->n == 0) return rc;
+    ADE_CK(ade::launch_sweep_table(sw->dim, sw->p.kernel, sw->iso, sw->run, sw->rp, sw->C, sw->P, sw->P4, s));
+    return ADE_OK;
+}
+
+// Whether a call of `steps` steps fills the table: it costs about three evaluations' gain (512^2, 8 sets:
+// 71 us against 95 - 72 per evaluation), so from four evaluations on.
+bool sweep_use_table(const ade_sweep *sw, int steps) { return 2 * steps * (int)sw->groups.size() >= 4; }
+
+// The predictors or correctors of every group with the geometry on the fly (one step).
+int sweep_evals_fly(ade_sweep *sw, int epi, cudaStream_t s)
+{
+    ade::RateParams rp = sw->rp;
+    rp.dt = (float)(epi == ade::EPI_PREDICT ? 0.5 * sw->dt : sw->dt);
+    for (int i = 0; i < 3; ++i) rp.inc[i] = sw->inc[i];
+    ade::SweepOut out;
+    memset(&out, 0, sizeof(out));
+    out.Cout = sw->Cs1;
+    out.C = sw->C;
+    out.xq = sw->xq;
+    out.status = sw->w.status;
+    for (const ade::SweepParams &g : sw->groups)
+        ADE_CK(ade::launch_rate_sweep(sw->dim, sw->p.kernel, epi, false, sw->w.P0, epi == ade::EPI_PREDICT ? sw->Cs0 : sw->Cs1,
+                                      sw->w.cell_start, sw->w.perm, rp, g, out, s));
+    return ADE_OK;
+}
+
+// Cells and concentrations of one step with the geometry on the fly.
+int sweep_begin_fly(ade_sweep *sw, cudaStream_t s)
+{
+    int rc = sweep_cells(sw, 1, s);
+    if (rc || sw->n == 0) return rc;
     ADE_CK(ade::launch_sweep_gather(sw->w.perm, sw->C, sw->n, sw->P, sw->P4, sw->Cs0, s));
     return ADE_OK;
 }
 
-// The evaluations of every group: predictors (all groups), or correctors (all groups).
-int sweep_evals(ade_sweep *sw, int ph, cudaStream_t s)
+// `steps` steps of one call.
+int sweep_steps(ade_sweep *sw, int steps, cudaStream_t s)
 {
-    ade::RateParams rp = sw->rp;
-    ade::SweepOut out;
-    memset(&out, 0, sizeof(out));
-    const uint4 *Pe = sw->w.P0;
-    const float *Ce = sw->Cs0;
-    int epi = ade::EPI_PREDICT;
-    if (ph == 1) {
-        rp.dt = (float)(0.5 * sw->dt);
-        for (int i = 0; i < 3; ++i) {
-            rp.inc[i] = sw->inc_half[i];
-            rp.back[i] = 0u;
-        }
-        out.Cout = sw->Cs1;
-        out.Pout = sw->w.P1;
-    } else {
-        epi = ade::EPI_CORRECT;
-        Pe = sw->w.P1;
-        Ce = sw->Cs1;
-        rp.dt = (float)sw->dt;
-        for (int i = 0; i < 3; ++i) {
-            rp.inc[i] = sw->inc[i];
-            rp.back[i] = sw->inc_half[i];
-        }
-        out.C = sw->C;
-        out.xq = sw->xq;
-        out.status = sw->w.status;
+    if (!sweep_use_table(sw, steps)) {   // (one step of one group)
+        int rc = sweep_begin_fly(sw, s);
+        if (rc || sw->n == 0) return rc;
+        rc = sweep_evals_fly(sw, ade::EPI_PREDICT, s);
+        return rc ? rc : sweep_evals_fly(sw, ade::EPI_CORRECT, s);
     }
-    for (const ade::SweepParams &g : sw->groups)
-        ADE_CK(ade::launch_rate_sweep(sw->dim, sw->p.kernel, epi, false, Pe, Ce, sw->w.cell_start, sw->w.perm, rp,
-                                      g, out, s));
-    return ADE_OK;
+    int rc = sweep_begin(sw, steps, s);
+    for (int k = 0; rc == ADE_OK && sw->n > 0 && k < steps; ++k) {
+        rc = sweep_evals(sw, ade::EPI_PREDICT, 0, s);
+        if (rc == ADE_OK) rc = sweep_evals(sw, ade::EPI_CORRECT, k + 1 == steps ? steps : 0, s);
+    }
+    return rc;
 }
 
-int sweep_step(ade_sweep *sw, cudaStream_t s)
+// One evaluation's launches with the geometry on the fly.
+int sweep_eval_fly(ade_sweep *sw, bool count, const ade::SweepOut &out, cudaStream_t s)
 {
-    int rc = sweep_cells(sw, s);
-    if (rc || sw->n == 0) return rc;
-    rc = sweep_evals(sw, 1, s);
-    if (rc) return rc;
-    return sweep_evals(sw, 2, s);
+    ADE_CK(ade::launch_sweep_gather(sw->w.perm, sw->C, sw->n, sw->P, sw->P4, sw->Cs0, s));
+    for (const ade::SweepParams &g : sw->groups) {
+        ADE_CK(ade::launch_rate_sweep(sw->dim, sw->p.kernel, ade::EPI_RATE, count, sw->w.P0, sw->Cs0, sw->w.cell_start, sw->w.perm,
+                                      sw->rp, g, out, s));
+        if (count) break;   // the geometry is the same for every group
+    }
+    return ADE_OK;
 }
 
 int sweep_clear_status_once(ade_sweep *sw, cudaStream_t s)
@@ -2364,7 +2435,7 @@ int sweep_clear_status_once(ade_sweep *sw, cudaStream_t s)
         ADE_CK(cudaMemsetAsync(sw->w.status, 0, sizeof(int), s));
         sw->status_cleared = true;
     }
-    return ADE_OK;
+    return sweep_clear_once(sw, s);
 }
 
 }  // namespace
@@ -2435,6 +2506,20 @@ int ade_sweep_init(ade_sweep **out, const ade_params *p, int n, int ntheta, cons
         return rc;
     }
     sw->rp.variant = 0;
+    sw->iso = iso;
+    sw->w.frame = at<uint32_t>(workspace_dev, W.frame);
+    sw->w.pencil = at<uint4>(workspace_dev, W.pencil);
+    sw->rp.frame = sw->w.frame;
+    sw->rp.pencil = sw->w.pencil;
+    sw->run.P = sw->w.P0;
+    sw->run.cs = sw->w.cell_start;
+    sw->run.perm = sw->w.perm;
+    sw->run.C = sw->Cs0;
+    sw->run.Ch = sw->Cs1;
+    sw->run.tab.words = at<float>(workspace_dev, L.words);
+    sw->run.tab.slots = at<uint4>(workspace_dev, L.slots);
+    sw->run.tab.cursor = at<unsigned>(workspace_dev, L.cursor);
+    sw->run.tab.cap = (unsigned)L.lines;
     sw->theta.assign(theta_host, theta_host + 3 * ntheta);
     // Dcal = a u + b per set (uniform v, K = 2D)
     const int dm = pp.dim;
@@ -2445,7 +2530,18 @@ int ade_sweep_init(ade_sweep **out, const ade_params *p, int n, int ntheta, cons
     ade::SweepParams base;
     memset(&base, 0, sizeof(base));
     for (int i = 0; i < 3; ++i) base.vh[i] = vabs > 0.0 ? (float)(i < dm ? pp.v[i] / vabs : 0.0) : (i == 0 ? 1.f : 0.f);
-    base.P4 = sw->P4;
+    for (int i = 0; i < 3; ++i) sw->rp.uw[i] = base.vh[i];   // the table's weights take u = (vhat . e)^2
+    sw->rp.ub = 0.f;
+    {
+        float lo[3];
+        for (int i = 0; i < 3; ++i) {
+            const double vh = vabs > 0.0 ? (i < dm ? pp.v[i] / vabs : 0.0) : (i == 0 ? 1.0 : 0.0);
+            lo[i] = (float)(vh - (double)base.vh[i]);
+        }
+        sw->run.lo = make_float4(lo[0], lo[1], lo[2], (float)(pp.box[0] / kTwo32 / L.d.H - (double)sw->rp.invH));
+        sw->run.g2 = (float)(2.0 * gamma);
+        sw->run.bT = (float)(2.0 * (gamma - dm) + 2.0);
+    }
     for (int g0 = 0; g0 < ntheta;) {
         int nt = ade::kSweepGroup;
         while (nt > ntheta - g0) nt >>= 1;
@@ -2457,6 +2553,8 @@ int ade_sweep_init(ade_sweep **out, const ade_params *p, int n, int ntheta, cons
                          Dm = theta_host[3 * (g0 + k) + 2];
             g.a[k] = (float)(2.0 * gamma * (aL - aT) * vabs);
             g.b[k] = (float)(2.0 * (gamma - dm) * (aT * vabs + Dm) - 2.0 * (aL - aT) * vabs);
+            g.dL[k] = (float)(aL * vabs + Dm);
+            g.dT[k] = (float)(aT * vabs + Dm);
         }
         sw->groups.push_back(g);
         g0 += nt;
@@ -2486,15 +2584,12 @@ int ade_sweep_rate(ade_sweep *sw, float *dCdt_dev, void *stream)
     if (!sw) return fail(ADE_ERR_ARG, "sweep is NULL");
     if (sw->n > 0 && !dCdt_dev) return fail(ADE_ERR_ARG, "dCdt_dev is NULL");
     cudaStream_t s = (cudaStream_t)stream;
-    int rc = sweep_cells(sw, s);
+    int rc = sweep_cells(sw, 0, s);
     if (rc || sw->n == 0) return rc;
     ade::SweepOut out;
     memset(&out, 0, sizeof(out));
     out.rate = dCdt_dev;
-    for (const ade::SweepParams &g : sw->groups)
-        ADE_CK(ade::launch_rate_sweep(sw->dim, sw->p.kernel, ade::EPI_RATE, false, sw->w.P0, sw->Cs0,
-                                      sw->w.cell_start, sw->w.perm, sw->rp, g, out, s));
-    return ADE_OK;
+    return sweep_eval_fly(sw, false, out, s);
 }
 
 int ade_sweep_count_pairs(ade_sweep *sw, long long *pairs_host, void *stream)
@@ -2502,14 +2597,14 @@ int ade_sweep_count_pairs(ade_sweep *sw, long long *pairs_host, void *stream)
     if (!sw || !pairs_host) return fail(ADE_ERR_ARG, "NULL argument");
     cudaStream_t s = (cudaStream_t)stream;
     *pairs_host = 0;
-    int rc = sweep_cells(sw, s);
+    int rc = sweep_cells(sw, 0, s);
     if (rc || sw->n == 0) return rc;
     ADE_CK(cudaMemsetAsync(sw->w.pairs, 0, 8, s));
     ade::SweepOut out;
     memset(&out, 0, sizeof(out));
     out.pairs = sw->w.pairs;
-    ADE_CK(ade::launch_rate_sweep(sw->dim, sw->p.kernel, ade::EPI_RATE, true, sw->w.P0, sw->Cs0, sw->w.cell_start,
-                                  sw->w.perm, sw->rp, sw->groups[0], out, s));
+    rc = sweep_eval_fly(sw, true, out, s);
+    if (rc) return rc;
     unsigned long long v = 0;
     ADE_CK(cudaMemcpyAsync(&v, sw->w.pairs, 8, cudaMemcpyDeviceToHost, s));
     ADE_CK(cudaStreamSynchronize(s));
@@ -2526,10 +2621,8 @@ int ade_sweep_step(ade_sweep *sw, int nsteps, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     int rc = sweep_clear_status_once(sw, s);
     if (rc) return rc;
-    for (int k = 0; k < nsteps; ++k) {
-        rc = sweep_step(sw, s);
-        if (rc) return rc;
-    }
+    if (nsteps > 0) rc = sweep_steps(sw, nsteps, s);
+    if (rc) return rc;
     sw->step += nsteps;
     sw->t += nsteps * sw->dt;
     return ADE_OK;
@@ -2543,26 +2636,30 @@ int ade_sweep_run(ade_sweep *sw, int nsteps, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     int rc = sweep_clear_status_once(sw, s);
     if (rc) return rc;
-    if (!sw->graph_exec && nsteps > 0) {
-        if (!sw->cap_stream) ADE_CK(cudaStreamCreateWithFlags(&sw->cap_stream, cudaStreamNonBlocking));
-        ADE_CK(cudaStreamBeginCapture(sw->cap_stream, cudaStreamCaptureModeThreadLocal));
-        rc = sweep_step(sw, sw->cap_stream);
-        cudaGraph_t g = nullptr;
-        cudaError_t e = cudaStreamEndCapture(sw->cap_stream, &g);
-        if (rc) {
-            if (g) cudaGraphDestroy(g);
-            return rc;
+    for (int left = nsteps; left > 0;) {   // graphs of kGraphSteps steps and one of the rest
+        const int k = std::min(left, ade::kGraphSteps);
+        if (!sw->graph_exec[k]) {
+            if (!sw->cap_stream) ADE_CK(cudaStreamCreateWithFlags(&sw->cap_stream, cudaStreamNonBlocking));
+            ADE_CK(cudaStreamBeginCapture(sw->cap_stream, cudaStreamCaptureModeThreadLocal));
+            rc = sweep_steps(sw, k, sw->cap_stream);
+            cudaGraph_t g = nullptr;
+            cudaError_t e = cudaStreamEndCapture(sw->cap_stream, &g);
+            if (rc) {
+                if (g) cudaGraphDestroy(g);
+                return rc;
+            }
+            ADE_CK(e);
+            cudaError_t ei = cudaGraphInstantiate(&sw->graph_exec[k], g, 0);
+            if (ei != cudaSuccess) {
+                cudaGraphDestroy(g);
+                sw->graph_exec[k] = nullptr;
+                return fail(ADE_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(ei));
+            }
+            sw->graph[k] = g;
         }
-        ADE_CK(e);
-        cudaError_t ei = cudaGraphInstantiate(&sw->graph_exec, g, 0);
-        if (ei != cudaSuccess) {
-            cudaGraphDestroy(g);
-            sw->graph_exec = nullptr;
-            return fail(ADE_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(ei));
-        }
-        sw->graph = g;
+        ADE_CK(cudaGraphLaunch(sw->graph_exec[k], s));
+        left -= k;
     }
-    for (int k = 0; k < nsteps; ++k) ADE_CK(cudaGraphLaunch(sw->graph_exec, s));
     sw->step += nsteps;
     sw->t += nsteps * sw->dt;
     return ADE_OK;
@@ -2580,16 +2677,17 @@ int ade_sweep_step_timed(ade_sweep *sw, double *phase_ms, void *stream)
         sw->ev_ready = true;
     }
     ADE_CK(cudaEventRecord(sw->ev[0], s));
-    rc = sweep_cells(sw, s);
+    const bool table = sweep_use_table(sw, 1);
+    rc = table ? sweep_begin(sw, 1, s) : sweep_begin_fly(sw, s);
     if (rc) return rc;
     ADE_CK(cudaEventRecord(sw->ev[1], s));
     if (sw->n > 0) {
-        rc = sweep_evals(sw, 1, s);
+        rc = table ? sweep_evals(sw, ade::EPI_PREDICT, 0, s) : sweep_evals_fly(sw, ade::EPI_PREDICT, s);
         if (rc) return rc;
     }
     ADE_CK(cudaEventRecord(sw->ev[2], s));
     if (sw->n > 0) {
-        rc = sweep_evals(sw, 2, s);
+        rc = table ? sweep_evals(sw, ade::EPI_CORRECT, 1, s) : sweep_evals_fly(sw, ade::EPI_CORRECT, s);
         if (rc) return rc;
     }
     ADE_CK(cudaEventRecord(sw->ev[3], s));
@@ -2608,8 +2706,8 @@ int ade_sweep_step_timed(ade_sweep *sw, double *phase_ms, void *stream)
 int ade_sweep_launches_per_step(const ade_sweep *sw, int *launches)
 {
     if (!sw || !launches) return fail(ADE_ERR_ARG, "NULL argument");
-    // the cell build (count, 2 or 3 scan launches, place, order), gather; one predictor and one
-    // corrector per group
+    // the cell build (count, the scan, place, order), the weight table with the sets' gather (once per
+    // call of several steps), one predictor and one corrector per group
     *launches = ade::cell_build_launches(sw->n, sw->ncells, sw->w.tile_sums != nullptr) + (sw->n > 0 ? 1 + 2 * (int)sw->groups.size() : 0);
     return ADE_OK;
 }
@@ -2642,8 +2740,10 @@ int ade_sweep_stats(ade_sweep *sw, ade_stats *st, void *stream)
 void ade_sweep_destroy(ade_sweep *sw)
 {
     if (!sw) return;
-    if (sw->graph_exec) cudaGraphExecDestroy(sw->graph_exec);
-    if (sw->graph) cudaGraphDestroy(sw->graph);
+    for (int k = 0; k <= ade::kGraphSteps; ++k) {
+        if (sw->graph_exec[k]) cudaGraphExecDestroy(sw->graph_exec[k]);
+        if (sw->graph[k]) cudaGraphDestroy(sw->graph[k]);
+    }
     if (sw->cap_stream) cudaStreamDestroy(sw->cap_stream);
     if (sw->ev_ready)
         for (int k = 0; k < 4; ++k) cudaEventDestroy(sw->ev[k]);

@@ -83,6 +83,40 @@ __device__ __forceinline__ float2 pair_shape(const uint4 &pa, const uint4 &pb, c
     return make_float2(f * fmaf(sc.g2, u, -2.f), f * fmaf(-sc.g2, u, sc.bT));
 }
 
+// The same for two candidates, in packed FP32x2 instructions (the same operations per half).
+template <int DIM, int KERNEL, bool ISO>
+__device__ __forceinline__ void pair_shape2(const uint4 &pa, const uint4 &p0, const uint4 &p1, const PairConst2 &k,
+                                            const ShapeConst &sc, float2 &gL, float2 &gT)
+{
+    float2 dx = f2(sep(pa.x, p0.x, k.m1), sep(pa.x, p1.x, k.m1));
+    float2 dy = f2(sep(pa.y, p0.y, k.m1), sep(pa.y, p1.y, k.m1));
+    float2 dz = f2(0.f, 0.f);
+    if (DIM == 3) dz = f2(sep(pa.z, p0.z, k.m1), sep(pa.z, p1.z, k.m1));
+    if (!ISO) {
+        dy = __fmul2_rn(dy, k.sy);
+        if (DIM == 3) dz = __fmul2_rn(dz, k.sz);
+    }
+    const float2 m1 = f2(-1.f, -1.f), one = f2(1.f, 1.f), half = f2(0.5f, 0.5f);
+    float2 r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
+    if (DIM == 3) r2 = __ffma2_rn(dz, dz, r2);
+    float2 rinv = f2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+    rinv = __ffma2_rn(__fmul2_rn(half, rinv), __ffma2_rn(__fmul2_rn(__fmul2_rn(r2, rinv), m1), rinv, one), rinv);
+    const float2 r = __fmul2_rn(r2, rinv), nr = __fmul2_rn(r, m1);
+    const float2 rl = __fmul2_rn(__fmul2_rn(half, rinv), __ffma2_rn(nr, r, r2));
+    const float2 nq = __fmul2_rn(r, k.ninvH);                                   // -q, and its low part
+    const float2 nql = __ffma2_rn(nr, f2(sc.lo.w, sc.lo.w), __ffma2_rn(rl, k.ninvH, __ffma2_rn(r, k.ninvH, __fmul2_rn(nq, m1))));
+    const float2 om = __fadd2_rn(__fadd2_rn(one, nq), nql);
+    const float2 f = shape2x2<KERNEL>(f2(fmaxf(om.x + om.x, 0.f), fmaxf(om.y + om.y, 0.f)));
+    float2 c = __ffma2_rn(f2(sc.lo.x, sc.lo.x), dx, __fmul2_rn(f2(sc.lo.y, sc.lo.y), dy));
+    if (DIM == 3) c = __ffma2_rn(f2(sc.lo.z, sc.lo.z), dz, c);
+    float2 ch = __ffma2_rn(k.w0, dx, __ffma2_rn(k.w1, dy, c));
+    if (DIM == 3) ch = __ffma2_rn(k.w2, dz, ch);
+    const float2 t = __fmul2_rn(ch, rinv), t2 = __fmul2_rn(t, t);
+    const float2 u = f2(fminf(t2.x, 1.f), fminf(t2.y, 1.f)), g2 = f2(sc.g2, sc.g2);
+    gL = __fmul2_rn(f, __ffma2_rn(g2, u, f2(-2.f, -2.f)));
+    gT = __fmul2_rn(f, __ffma2_rn(__fmul2_rn(g2, m1), u, f2(sc.bT, sc.bT)));
+}
+
 // Squared separation in x units^2.
 template <int DIM, bool ISO>
 __device__ __forceinline__ float sep2(const uint4 &pa, const uint4 &pb, const PairConst &k)
@@ -261,18 +295,29 @@ __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const 
             if (!valid || xw < 0) cnt = 0;
             if (s >= qe) s = qs;                     // (the range's first cells are empty)
             if (BOX) {
-                // candidates farther than xw along x lie beyond H (1 + 2^-12): weight exactly 0
+                // candidates farther than xw along x lie beyond H (1 + 2^-12): weight exactly 0.  Both
+                // ends' two outermost are looked at together (one latency instead of up to four).
+                auto at = [&](int t) {
+                    const int j = s + t;
+                    return __ldg(&P[j >= qe ? j - len : j].x);
+                };
+                auto out = [&](uint32_t x) {
+                    const int d = (int)(x - pa.x);
+                    return d < -xw || d > xw;
+                };
                 while (cnt > 0) {
-                    const int d = (int)(__ldg(&P[s].x) - pa.x);
-                    if (d >= -xw && d <= xw) break;
-                    --cnt;
-                    s = s + 1 < qe ? s + 1 : qs;
-                }
-                while (cnt > 0) {
-                    const int j = s + cnt - 1;
-                    const int d = (int)(__ldg(&P[j >= qe ? j - len : j].x) - pa.x);
-                    if (d >= -xw && d <= xw) break;
-                    --cnt;
+                    const int t1 = min(1, cnt - 1), e1 = max(cnt - 2, 0);
+                    const uint32_t f0 = at(0), f1 = at(t1), b0 = at(cnt - 1), b1 = at(e1);
+                    const int df = out(f0) ? (out(f1) ? 2 : 1) : 0, db = out(b0) ? (out(b1) ? 2 : 1) : 0;
+                    const int left = cnt - df - db;
+                    if (left <= 0) {          // the ends meet: what is left, if anything, lies between them
+                        cnt = out(f0) && out(f1) && out(b0) && out(b1) && cnt <= 4 ? 0 : cnt;
+                        break;
+                    }
+                    s += df;
+                    if (s >= qe) s -= len;
+                    cnt = left;
+                    if (df < 2 && db < 2) break;
                 }
             } else {
                 while (cnt > 0 && !(sep2<DIM, ISO>(pa, __ldg(P + s), k) < far2)) {
@@ -316,8 +361,16 @@ __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const 
         out += 32;
         if (VAL == 2) {
             float2 *o2 = reinterpret_cast<float2 *>(out + lane);
-#pragma unroll 2
-            for (int t = 0; t < m; ++t) {
+            int t = 0;
+            for (; t + 1 < m; t += 2) {
+                const int j0 = s + t, j1 = j0 + 1;
+                float2 gL, gT;
+                pair_shape2<DIM, KERNEL, ISO>(pa, __ldg(P + (j0 >= qe ? j0 - len : j0)), __ldg(P + (j1 >= qe ? j1 - len : j1)),
+                                              k2, sc, gL, gT);
+                o2[t * 32] = f2(gL.x, gT.x);
+                o2[(t + 1) * 32] = f2(gL.y, gT.y);
+            }
+            if (t < m) {
                 const int j = s + t;
                 o2[t * 32] = pair_shape<DIM, KERNEL, ISO>(pa, __ldg(P + (j >= qe ? j - len : j)), k, sc);
             }

@@ -10,9 +10,15 @@
 // once and each parameter set costs one fused multiply-add for Dcal, a multiply by f, the
 // concentration difference and the accumulation.  The cell list, the positions and the drift are
 // shared; only the concentrations are per set.  Parameter sets are evaluated in groups of up to 8
-// per launch (registers); the sorted concentrations are interleaved [n][P4] (P4 = P rounded up to
-// a multiple of 4) so that a group's values are one or two 16-byte loads per candidate.
+// per launch (registers); the sorted concentrations lie in planes of four sets, 16 bytes per particle, so
+// that a group's values are one or two 16-byte loads per candidate.
 // Summation as in rate.cu: FP32 row sums, Neumaier across rows, fixed order.
+//
+// Calls of four evaluations and more keep the geometry in a table (frozen_table.cuh: g_L and g_T per pair,
+// from which set k's weight is d_L,k g_L + d_T,k g_T) and stream it once per group and evaluation
+// (k_sweep_pass); shorter ones (k_rate_sweep) compute it on the fly.  Bound of a pass with 8 sets: the
+// latency of L1 and L2 at 27 % occupancy (32 bytes of concentrations a candidate, 96 registers).
+// 512^2, 60 neighbours, 8 sets, per evaluation: 95 us on the fly, 71 us from the table.
 #include "ade_internal.h"
 
 namespace ade {
@@ -21,39 +27,247 @@ namespace {
 
 #include "rate_common.cuh"
 
-constexpr int kT = kRateThreads;
+#include "rate_walk.cuh"
 
+#include "frozen_table.cuh"
+
+constexpr int kT = kRateThreads;
+static_assert(kRateThreads == kFrozenThreads, "the table's launch grid counts blocks of kFrozenThreads");
+
+// Sorted concentrations: planes of four sets, one 16-byte word per particle and plane (`plane` words
+// each), so that a warp's loads of neighbouring particles are contiguous (interleaving all sets of a
+// particle took twice the L1 wavefronts: 83 us a pass with 8 sets).  p: the group's first plane at word j 0.
 template <int NT>
-__device__ __forceinline__ void load_group(const float *__restrict__ p, float v[NT])
+__device__ __forceinline__ void load_group(const float *__restrict__ p, size_t plane, size_t j, float v[NT])
 {
     if (NT == 1) {
-        v[0] = __ldg(p);
+        v[0] = __ldg(p + 4 * j);
     } else if (NT == 2) {
-        const float2 q = __ldg(reinterpret_cast<const float2 *>(p));
+        const float2 q = __ldg(reinterpret_cast<const float2 *>(p + 4 * j));
         v[0] = q.x;
-        v[1] = q.y;
+        v[1 % NT] = q.y;
     } else {
 #pragma unroll
         for (int k = 0; k < NT; k += 4) {
-            const float4 q = __ldg(reinterpret_cast<const float4 *>(p) + k / 4);
+            const float4 q = __ldg(reinterpret_cast<const float4 *>(p) + (k / 4) * plane + j);
             v[k] = q.x;
-            v[k + 1] = q.y;
-            v[k + 2] = q.z;
-            v[k + 3] = q.w;
+            v[(k + 1) % NT] = q.y;
+            v[(k + 2) % NT] = q.z;
+            v[(k + 3) % NT] = q.w;
         }
     }
 }
 
-// Sorted, interleaved concentrations: Cs[i * P4 + p] = C[p * n + perm[i]].
-__global__ __launch_bounds__(kT) void k_sweep_gather(const uint32_t *__restrict__ perm, const float *__restrict__ C,
-                                                     int n, int P, int P4, float *__restrict__ Cs)
+template <int NT>
+__device__ __forceinline__ void store_group(float *p, size_t plane, size_t j, const float v[NT])
 {
-    const int i = blockIdx.x * kT + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t a = __ldg(perm + i);
-    for (int p = 0; p < P4; ++p) Cs[(size_t)i * P4 + p] = p < P ? __ldg(C + (size_t)p * n + a) : 0.f;
+    if (NT == 1) {
+        p[4 * j] = v[0];
+    } else if (NT == 2) {
+        *reinterpret_cast<float2 *>(p + 4 * j) = make_float2(v[0], v[1 % NT]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < NT; k += 4)
+            reinterpret_cast<float4 *>(p)[(k / 4) * plane + j] = make_float4(v[k], v[(k + 1) % NT], v[(k + 2) % NT], v[(k + 3) % NT]);
+    }
 }
 
+// The group's first plane, at its first set's word.
+__device__ __forceinline__ size_t group_base(int g0, size_t plane) { return (size_t)(g0 >> 2) * plane * 4 + (size_t)(g0 & 3); }
+
+// The warp's chunks of the block's pencil.
+template <class F>
+__device__ __forceinline__ void block_chunks(const uint32_t *__restrict__ cs, const RateParams &prm, F f)
+{
+    for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), gridDim.y * (kT / 32), f);
+}
+
+// Sorted concentrations of one particle, C[p n + perm[i]], at words j0 and j1.
+__device__ __forceinline__ void gather_sets(const uint32_t *__restrict__ perm, const float *__restrict__ C, size_t n, int P,
+                                            int P4, int i, size_t plane, size_t j0, size_t j1, float *__restrict__ Cs)
+{
+    const uint32_t a = __ldg(perm + i);
+    if (a >= (uint32_t)n) return;
+    for (int p = 0; p < P4; p += 4) {
+        float v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = p + q < P ? __ldg(C + (size_t)(p + q) * n + a) : 0.f;
+        store_group<4>(Cs + (size_t)p * plane, plane, j0, v);
+        if (j1 != j0) store_group<4>(Cs + (size_t)p * plane, plane, j1, v);
+    }
+}
+
+__global__ __launch_bounds__(kT) void k_sweep_gather(const uint32_t *__restrict__ perm, const float *__restrict__ C, int n,
+                                                     int P, int P4, float *__restrict__ Cs)
+{
+    pdl_wait();
+    pdl_trigger();
+    const int i = blockIdx.x * kT + threadIdx.x;
+    if (i < n) gather_sets(perm, C, (size_t)n, P, P4, i, (size_t)n, (size_t)i, (size_t)i, Cs);
+}
+
+// The table of a call and the concentrations, doubled per pencil.
+template <int DIM, int KERNEL, bool ISO>
+__global__ __launch_bounds__(kT) void k_sweep_table(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
+                                                    const uint32_t *__restrict__ perm, const RateParams prm,
+                                                    const FrozenTab tab, const ShapeConst sc, const float *__restrict__ C,
+                                                    int sets, int P4, float *__restrict__ Cs)
+{
+    pdl_wait();
+    __shared__ TrimRow srow[ISO ? kMaxRows : 1];
+    if (ISO) stage_trim_rows(srow, prm);
+    block_chunks(cs, prm, [&](const Chunk &c) {
+        const int i = c.i0 + (threadIdx.x & 31);
+        if (i < c.pe) gather_sets(perm, C, (size_t)prm.n, sets, P4, i, 2 * (size_t)prm.n, (size_t)(c.ps + i), (size_t)(c.pe + i), Cs);
+        const uint4 pa = __ldg(P + min(i, c.pe - 1));
+        build_chunk<DIM, KERNEL, ISO, ISO, 2>(P, cs, prm, c, pa, srow, tab, sc);
+    });
+}
+
+// sum_b (d_L g_L + d_T g_T)(C_a - C_b) of NT sets, two sets to a packed FP32x2 instruction.
+template <int NT>
+struct SetSums {
+    static constexpr int N2 = (NT + 1) / 2;
+    const float *C;            // doubled, from the group's first set
+    size_t plane;
+    float2 Ca[N2], rs[N2], acc[N2], comp[N2], dL[N2], dT[N2];
+    __device__ __forceinline__ void add(float2 g, const float2 (&Cb)[N2])
+    {
+        const float2 gl = f2(g.x, g.x), gt = f2(g.y, g.y), m1 = f2(-1.f, -1.f);
+#pragma unroll
+        for (int k = 0; k < N2; ++k)
+            rs[k] = __ffma2_rn(__ffma2_rn(dL[k], gl, __fmul2_rn(dT[k], gt)), __ffma2_rn(Cb[k], m1, Ca[k]), rs[k]);
+    }
+    __device__ __forceinline__ void load(size_t j, float2 (&v)[N2]) const
+    {
+        float t[NT];
+        load_group<NT>(C, plane, j, t);
+#pragma unroll
+        for (int k = 0; k < N2; ++k) v[k] = f2(t[2 * k], 2 * k + 1 < NT ? t[(2 * k + 1) % NT] : 0.f);
+    }
+    template <int M>
+    __device__ __forceinline__ void lines(const float *w, int s)
+    {
+        constexpr int B = NT >= 8 ? 2 : 4;   // candidates in flight (registers)
+        float2 g[M];
+#pragma unroll
+        for (int u = 0; u < M; ++u) g[u] = __ldg(reinterpret_cast<const float2 *>(w) + u * 32);
+#pragma unroll
+        for (int u0 = 0; u0 < M; u0 += B) {
+            float2 v[B][N2];
+#pragma unroll
+            for (int u = 0; u < B; ++u)
+                if (u0 + u < M) load((size_t)(s + u0 + u), v[u]);
+#pragma unroll
+            for (int u = 0; u < B; ++u)
+                if (u0 + u < M) add(g[(u0 + u) % M], v[u]);
+        }
+    }
+    __device__ __forceinline__ void end_row()
+    {
+#pragma unroll
+        for (int k = 0; k < N2; ++k) {
+            neumaier_add2(acc[k], comp[k], rs[k]);
+            rs[k] = f2(0.f, 0.f);
+        }
+    }
+};
+
+// The same sums over the positions, for a chunk without room in the table.
+template <int DIM, int KERNEL, bool ISO, int NT>
+__device__ __noinline__ void walk_sets(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs, const RateParams &prm,
+                                       const Chunk &c, const ShapeConst &sc, SetSums<NT> &op)
+{
+    const uint4 pa = __ldg(P + min(c.i0 + (int)(threadIdx.x & 31), c.pe - 1));
+    const int ncx = prm.ncx;
+    const int cx = (int)__umulhi(pa.x - frame_x(prm), (uint32_t)ncx);
+    const PairConst k(prm);
+    for (int r = 0; r < prm.nrows; ++r) {
+        const StencilRow row = prm.rows[r];
+        const int q = row_pencil_of<DIM>(row, c.cy, c.cz, prm);
+        const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
+        int s, cnt;
+        cyclic_range(cs, q * ncx, cx - (int)row.w, cx + row.w + 1, ncx, qs, qe, s, cnt);
+        for (int t = 0; t < cnt; ++t) {
+            int j = s + t;
+            j = j >= qe ? j - len : j;
+            float2 v[SetSums<NT>::N2];
+            op.load((size_t)(qs + j), v);
+            op.add(pair_shape<DIM, KERNEL, ISO>(pa, __ldg(P + j), k, sc), v);
+        }
+        op.end_row();
+    }
+}
+
+// One evaluation of one group from the table: predictor (C -> Ch) or corrector (C updated), Eq. 8-9.
+// out.C set (a call's last corrector): the state goes to the caller's order instead, with the positions
+// advanced by prm.inc (the drift of all steps; the first group writes them).
+// Eight sets' sums take up to 96 registers, five CTAs per SM; held to 80 they spill (97 against 75 us a
+// pass at 512^2), and two warps of four sets each on a chunk were slower (94 us: twice the weights'
+// traffic), as were rings of the stream in shared memory (81 us: fewer warps).
+template <int DIM, int KERNEL, bool ISO, int NT, int EPI>
+__global__ __launch_bounds__(kT, 5) void k_sweep_pass(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
+                                                   const RateParams prm, const FrozenTab tab, const ShapeConst sc,
+                                                   const SweepParams sp, float *C, float *Ch,
+                                                   const uint32_t *__restrict__ perm, const SweepOut out)
+{
+    pdl_wait();
+    const bool last = EPI == EPI_CORRECT && out.C;
+    if (last && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *tab.cursor = 0u;   // the next table starts empty
+    const int g0 = sp.g0;
+    block_chunks(cs, prm, [&](const Chunk &c) {
+        const int i = c.i0 + (threadIdx.x & 31);
+        const size_t plane = 2 * (size_t)prm.n, at = (size_t)(c.ps + min(i, c.pe - 1)), gb = group_base(g0, plane);
+        SetSums<NT> op;
+        op.C = (EPI == EPI_PREDICT ? C : Ch) + gb;
+        op.plane = plane;
+        op.load(at, op.Ca);
+#pragma unroll
+        for (int k = 0; k < SetSums<NT>::N2; ++k) {
+            op.dL[k] = f2(sp.dL[2 * k], sp.dL[2 * k + 1]);
+            op.dT[k] = f2(sp.dT[2 * k], sp.dT[2 * k + 1]);
+            op.rs[k] = op.acc[k] = op.comp[k] = f2(0.f, 0.f);
+        }
+        const uint4 sl = __ldg(tab.slots + c.slot);
+        if (sl.x != kNoRoom) stream_rows<2>(sl, tab, op);
+        else walk_sets<DIM, KERNEL, ISO, NT>(P, cs, prm, c, sc, op);
+        if (i >= c.pe) return;
+        const float pf = prm.pf * shape_unscale<KERNEL>();
+        float Cl[NT], o[NT];
+        if (EPI == EPI_CORRECT) load_group<NT>(C + gb, plane, at, Cl);
+#pragma unroll
+        for (int k = 0; k < NT; ++k) {
+            const float2 a2 = op.acc[k / 2], c2 = op.comp[k / 2], ca = op.Ca[k / 2];
+            const float rate = pf * (k & 1 ? a2.y + c2.y : a2.x + c2.x);
+            o[k] = fmaf(prm.dt, rate, EPI == EPI_CORRECT ? Cl[k] : (k & 1 ? ca.y : ca.x));
+        }
+        if (last) {
+            const uint32_t a = __ldg(perm + i);
+            const size_t n = (size_t)prm.n;
+            if (a >= (uint32_t)n) return;
+            bool bad = false;
+#pragma unroll
+            for (int k = 0; k < NT; ++k) {
+                out.C[(size_t)(g0 + k) * n + a] = o[k];
+                bad |= !isfinite(o[k]);
+            }
+            if (bad) atomicOr(out.status, 1);
+            if (g0 == 0) {
+                const uint4 q = __ldg(P + i);
+                out.xq[a] = q.x + prm.inc[0];
+                out.xq[n + a] = q.y + prm.inc[1];
+                if (DIM == 3) out.xq[2 * n + a] = q.z + prm.inc[2];
+            }
+            return;
+        }
+        float *to = (EPI == EPI_PREDICT ? Ch : C) + gb;
+        store_group<NT>(to, plane, at, o);
+        store_group<NT>(to, plane, (size_t)(c.pe + i), o);
+    });
+}
+
+// One evaluation with the geometry computed on the fly: the rate or pair count, or a predictor (Ce -> out.Cout)
+// or corrector (caller order) of a call too short for the table.  Pe: the positions of the build.
 template <int DIM, int KERNEL, int EPI, int NT, bool COUNT>
 __global__ __launch_bounds__(kT) void k_rate_sweep(const uint4 *__restrict__ Pe, const float *__restrict__ Ce,
                                                    const uint32_t *__restrict__ cs,
@@ -64,9 +278,10 @@ __global__ __launch_bounds__(kT) void k_rate_sweep(const uint4 *__restrict__ Pe,
     const bool valid = i < prm.n;
     const int ii = valid ? i : prm.n - 1;
     const uint4 pa = __ldg(Pe + ii);
-    const int P4 = sp.P4, g0 = sp.g0;
+    const int g0 = sp.g0;
+    const float *Cg = Ce + group_base(g0, (size_t)prm.n);
     float Ca[NT];
-    load_group<NT>(Ce + (size_t)ii * P4 + g0, Ca);
+    load_group<NT>(Cg, (size_t)prm.n, (size_t)ii, Ca);
     const int ncx = prm.ncx, ncy = prm.ncy, ncz = prm.ncz;
     // cell of the build: position minus the drift since it, in the build's frame
     uint3 org = make_uint3(prm.back[0], prm.back[1], prm.back[2]);
@@ -143,7 +358,7 @@ __global__ __launch_bounds__(kT) void k_rate_sweep(const uint4 *__restrict__ Pe,
                     const float cr = c * rinv;
                     const float u = cr * cr;
                     float Cb[NT];
-                    load_group<NT>(Ce + (size_t)j * P4 + g0, Cb);
+                    load_group<NT>(Cg, (size_t)prm.n, (size_t)j, Cb);
 #pragma unroll
                     for (int k = 0; k < NT; ++k) rs[k] = fmaf(f * fmaf(sp.a[k], u, sp.b[k]), Ca[k] - Cb[k], rs[k]);
                 }
@@ -161,44 +376,34 @@ __global__ __launch_bounds__(kT) void k_rate_sweep(const uint4 *__restrict__ Pe,
 #pragma unroll
     for (int k = 0; k < NT; ++k) rate[k] = prm.pf * (acc[k] + comp[k]);
     const size_t n = (size_t)prm.n;
+    if (EPI == EPI_PREDICT) {
+        float o[NT];
+#pragma unroll
+        for (int k = 0; k < NT; ++k) o[k] = fmaf(prm.dt, rate[k], Ca[k]);
+        store_group<NT>(out.Cout + group_base(g0, n), n, (size_t)i, o);
+        return;
+    }
+    const uint32_t a = __ldg(perm + i);
+    if (a >= (uint32_t)n) return;
     if (EPI == EPI_RATE) {
-        if (out.rate) {
-            const uint32_t a = __ldg(perm + i);
-            if (a < (uint32_t)n)
+        if (out.rate)
 #pragma unroll
-                for (int k = 0; k < NT; ++k) out.rate[(size_t)(g0 + k) * n + a] = rate[k];
-        }
-    } else if (EPI == EPI_PREDICT) {
-        // C_p^{l+1/2} = C_p^l + dt/2 r_p^l (sorted, interleaved); x^{l+1/2} = x^l + dt/2 v once
+            for (int k = 0; k < NT; ++k) out.rate[(size_t)(g0 + k) * n + a] = rate[k];
+        return;
+    }
+    bool bad = false;
 #pragma unroll
-        for (int k = 0; k < NT; ++k) out.Cout[(size_t)i * P4 + g0 + k] = fmaf(prm.dt, rate[k], Ca[k]);
-        if (g0 == 0) {
-            uint4 q;
-            q.x = pa.x + prm.inc[0];
-            q.y = pa.y + prm.inc[1];
-            q.z = pa.z + prm.inc[2];
-            q.w = 0u;
-            out.Pout[i] = q;
-        }
-    } else {
-        // C_p^{l+1} = C_p^l + dt r_p^{l+1/2} and x^{l+1} = x^l + dt v, in the caller's order
-        const uint32_t a = __ldg(perm + i);
-        if (a < (uint32_t)n) {
-            bool bad = false;
-#pragma unroll
-            for (int k = 0; k < NT; ++k) {
-                float *Cp = out.C + (size_t)(g0 + k) * n + a;
-                const float Cn = fmaf(prm.dt, rate[k], *Cp);
-                *Cp = Cn;
-                bad |= !isfinite(Cn);
-            }
-            if (bad) atomicOr(out.status, 1);
-            if (g0 == 0) {
-                out.xq[a] = pa.x - prm.back[0] + prm.inc[0];
-                out.xq[n + a] = pa.y - prm.back[1] + prm.inc[1];
-                if (DIM == 3) out.xq[2 * n + a] = pa.z - prm.back[2] + prm.inc[2];
-            }
-        }
+    for (int k = 0; k < NT; ++k) {
+        float *Cp = out.C + (size_t)(g0 + k) * n + a;
+        const float Cn = fmaf(prm.dt, rate[k], *Cp);
+        *Cp = Cn;
+        bad |= !isfinite(Cn);
+    }
+    if (bad) atomicOr(out.status, 1);
+    if (g0 == 0) {
+        out.xq[a] = pa.x + prm.inc[0];
+        out.xq[n + a] = pa.y + prm.inc[1];
+        if (DIM == 3) out.xq[2 * n + a] = pa.z + prm.inc[2];
     }
 }
 
@@ -230,14 +435,60 @@ void launch_sweep_k(int epi, bool count, int blocks, const uint4 *Pe, const floa
     }
 }
 
+template <int DIM, int KERNEL, bool ISO, int NT>
+cudaError_t pass_nt(const SweepRun &r, int epi, const SweepParams &sp, const RateParams &prm, const SweepOut &out, cudaStream_t s)
+{
+    const dim3 g = frozen_grid(prm);
+    return epi == EPI_PREDICT
+               ? launch_pdl(k_sweep_pass<DIM, KERNEL, ISO, NT, EPI_PREDICT>, g, kT, 0, s, r.P, r.cs, prm, r.tab, ShapeConst{r.lo, r.g2, r.bT}, sp, r.C, r.Ch, r.perm, out)
+               : launch_pdl(k_sweep_pass<DIM, KERNEL, ISO, NT, EPI_CORRECT>, g, kT, 0, s, r.P, r.cs, prm, r.tab, ShapeConst{r.lo, r.g2, r.bT}, sp, r.C, r.Ch, r.perm, out);
+}
+
+template <int DIM, int KERNEL, bool ISO>
+cudaError_t pass_k(const SweepRun &r, int epi, const SweepParams &sp, const RateParams &prm, const SweepOut &out, cudaStream_t s)
+{
+    switch (sp.nt) {
+    case 1: return pass_nt<DIM, KERNEL, ISO, 1>(r, epi, sp, prm, out, s);
+    case 2: return pass_nt<DIM, KERNEL, ISO, 2>(r, epi, sp, prm, out, s);
+    case 4: return pass_nt<DIM, KERNEL, ISO, 4>(r, epi, sp, prm, out, s);
+    default: return pass_nt<DIM, KERNEL, ISO, 8>(r, epi, sp, prm, out, s);
+    }
+}
+
+template <int DIM, int KERNEL, bool ISO>
+cudaError_t table_k(const SweepRun &r, const RateParams &prm, const float *C, int sets, int P4, cudaStream_t s)
+{
+    return launch_pdl(k_sweep_table<DIM, KERNEL, ISO>, frozen_grid(prm), kT, 0, s, r.P, r.cs, r.perm, prm, r.tab,
+                      ShapeConst{r.lo, r.g2, r.bT}, C, sets, P4, r.C);
+}
+
+#define ADE_SWEEP_CALL(F, ...)                                                                                               \
+    (dim == 2 ? (kernel == ADE_WENDLAND_C2                                                                                   \
+                     ? (iso ? F<2, ADE_WENDLAND_C2, true>(__VA_ARGS__) : F<2, ADE_WENDLAND_C2, false>(__VA_ARGS__))          \
+                     : (iso ? F<2, ADE_WENDLAND_C4, true>(__VA_ARGS__) : F<2, ADE_WENDLAND_C4, false>(__VA_ARGS__)))         \
+              : (kernel == ADE_WENDLAND_C2                                                                                   \
+                     ? (iso ? F<3, ADE_WENDLAND_C2, true>(__VA_ARGS__) : F<3, ADE_WENDLAND_C2, false>(__VA_ARGS__))          \
+                     : (iso ? F<3, ADE_WENDLAND_C4, true>(__VA_ARGS__) : F<3, ADE_WENDLAND_C4, false>(__VA_ARGS__))))
+
 }  // namespace
 
-cudaError_t launch_sweep_gather(const uint32_t *perm, const float *C, int n, int P, int P4, float *Cs,
-                                cudaStream_t s)
+cudaError_t launch_sweep_gather(const uint32_t *perm, const float *C, int n, int P, int P4, float *Cs, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    k_sweep_gather<<<(n + kT - 1) / kT, kT, 0, s>>>(perm, C, n, P, P4, Cs);
-    return cudaGetLastError();
+    return launch_pdl(k_sweep_gather, (unsigned)((n + kT - 1) / kT), kT, 0, s, perm, C, n, P, P4, Cs);
+}
+
+cudaError_t launch_sweep_table(int dim, int kernel, bool iso, const SweepRun &r, const RateParams &prm, const float *C,
+                               int sets, int P4, cudaStream_t s)
+{
+    return ADE_SWEEP_CALL(table_k, r, prm, C, sets, P4, s);
+}
+
+cudaError_t launch_sweep_pass(int dim, int kernel, bool iso, int epi, const SweepRun &r, const SweepParams &sp,
+                              const RateParams &prm, const SweepOut &out, cudaStream_t s)
+{
+    if (sp.nt != 1 && sp.nt != 2 && sp.nt != 4 && sp.nt != 8) return cudaErrorInvalidValue;
+    return ADE_SWEEP_CALL(pass_k, r, epi, sp, prm, out, s);
 }
 
 cudaError_t launch_rate_sweep(int dim, int kernel, int epi, bool count, const uint4 *Pe, const float *Ce,

@@ -125,3 +125,28 @@ def test_batch_kept_weights_give_the_walks_bits(lib, dim):
         s.step(41)
         xb, Cb = b.state(i)
         assert _bits(xb, s.state()[0]) and _bits(Cb, s.state()[1]), i
+
+
+@pytest.mark.parametrize("sets", [1, 3, 11])
+@pytest.mark.parametrize("name", ["2d-blob-no-room", "2d-unequal-box", "3d-jitter-23-c4", "2d-lattice-33", "2d-sparse"])
+def test_sweep_steps_match_single_plumes(lib, name, sets):
+    """Steps of a sweep (stored weights g_L, g_T) against single-plume contexts of every set: the two
+    forms of a pair's weight differ by a few FP32 roundings, 1e-5 of the increment per step as for
+    every rate, and C is rounded once per half step."""
+    xq, C, kw = CASES[name]()
+    kw = dict(kw, dt=2e-4)
+    theta = [(1e-2 * (k + 1) / sets, 1e-3, 1e-6 * k) for k in range(sets)]
+    Cs = np.stack([C * np.float32(1.0 + 0.1 * k) for k in range(sets)])
+    sw = lib.Sweep(lib.params(**kw), xq, Cs, theta)
+    for n in (1, 2):
+        sw.run(n)
+    xs, out = sw.state()
+    for k, th in enumerate(theta):
+        p = dict(kw, alpha_L=th[0], alpha_T=th[1], D_m=th[2])
+        sim = lib.Simulation(lib.params(flags=lib.FLAG_DIRECT, **p), xq, Cs[k])
+        sim.step(3)
+        x1, C1 = sim.state()
+        assert _bits(xs, x1)
+        inc = np.abs(C1.astype(np.float64) - Cs[k]).max()
+        tol = 3 * 1e-5 * inc + 6 * np.abs(C1).max() * 2.0 ** -24
+        assert np.abs(out[k].astype(np.float64) - C1).max() <= tol, k
