@@ -103,6 +103,7 @@ struct RateParams {
     int cap;         // staged-particle capacity of a tile
     double u[3];     // FP64 length of one fixed-point unit per axis (L_i / 2^32)
     double H2d;      // FP64 support radius squared (pair counting decides support in FP64)
+    unsigned fz_base, fz_stride;   // weight table: first line and lines per chunk (FrozenTab)
     int goff;        // batched plumes: first particle (caller and sorted order) of this plume
     int coff;        // batched plumes: first cell of this plume in the global cell table
     int m1;               // -1: the multiplier of the walks' separations (see sep in rate_common.cuh)
@@ -157,14 +158,16 @@ struct SweepOut {
     unsigned long long *pairs;    // pair counter (counting launch)
 };
 
-// Weight table of the evaluations over one cell list (rate_frozen.cu): `cap` lines of 32 words, handed
-// out by an atomic cursor; slots[chunk] = {first line of the chunk's stream, rows, lines, -}.
+// Weight table of the evaluations over one cell list (rate_frozen.cu), in lines of 32 words: a region of
+// RateParams::fz_stride lines per chunk from RateParams::fz_base on, and from line `pool` on `cap` lines
+// that an atomic cursor hands out to chunks that outgrow theirs; slots[chunk] = {first line of the
+// chunk's stream, rows, lines, header lines}.
 constexpr int kFrozenThreads = 128;
 struct FrozenTab {
     float *words;
     uint4 *slots;
     unsigned *cursor;
-    unsigned cap;
+    unsigned pool, cap;
 };
 // Concentrations (and Eq. 14's flux) of such a run in sorted order: C at level l, Ch at l + 1/2, each
 // pencil's twice back to back ([2n] words).
@@ -310,8 +313,10 @@ cudaError_t launch_rate_field(int dim, int kernel, int epi, const uint4 *Pe, con
 // Launch grid of the table's kernels (kFrozenThreads threads a block).
 dim3 frozen_grid(const RateParams &prm);
 // Lines and slots of a table with `val` words per pair (lines bounded by the table's size limit), and blocks
-// of frozen_grid, enough for every grid the context may switch to.
+// of frozen_grid, enough for every grid the context may switch to; and the table's division among the
+// chunks of the grid in use (fz_base, fz_stride, pool, cap).
 void frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots, int *blocks);
+void frozen_divide(const ade_ctx *c, int val, size_t lines, RateParams *rp, FrozenTab *tab);
 // Evaluations over one cell list with stored weights (rate_frozen.cu): the table, one predictor or
 // corrector (prm.dt), and the final state in the caller's order (prm.inc: the drift of all steps).
 cudaError_t launch_frozen_build(int dim, int kernel, bool iso, const uint4 *P, const uint32_t *cs, const uint32_t *perm,
@@ -387,6 +392,7 @@ struct ade_ctx {
     bool cells_framed;    // the last build was a step's (in the moving frame)
     bool frozen;          // steps of one call may keep the pair weights (frozen_tab)
     ade::FrozenTab frozen_tab;
+    size_t frozen_lines;  // lines of the table
     float *frozen_C;      // [2][2n] concentrations of such a call (FrozenState)
     // velocity-field mode (p.vmax > 0)
     bool field;

@@ -134,7 +134,7 @@ __global__ __launch_bounds__(kT) void k_adj_table(const uint4 *__restrict__ P, c
     for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), gridDim.y * (kT / 32), [&](const Chunk &c) {
         const int i = c.i0 + (threadIdx.x & 31);
         const uint4 pa = __ldg(P + min(i, c.pe - 1));
-        build_chunk<DIM, KERNEL, ISO, ISO, 2>(P, cs, prm, c, pa, srow, tab, sc);
+        build_chunk<DIM, KERNEL, ISO, ISO ? kCutBox : kCutFull, 2>(P, cs, prm, c, pa, srow, tab, sc);
         if (i < c.pe) C0[c.ps + i] = C0[c.pe + i] = __uint_as_float(pa.w);
     });
 }
@@ -473,7 +473,7 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     A.tab.words = field(L.words);
     A.tab.slots = reinterpret_cast<uint4 *>(base + L.slots);
     A.tab.cursor = reinterpret_cast<unsigned *>(base + L.cursor);
-    A.tab.cap = (unsigned)L.lines;
+    frozen_divide(c, 2, L.lines, &A.rp, &A.tab);
     const int nb = (int)(A.grid.x * A.grid.y);
     if (nb > L.blocks) return ade::report_error(ADE_ERR_CAPACITY, "adjoint partials exceed the workspace");
     const float dt = (float)c->dt;

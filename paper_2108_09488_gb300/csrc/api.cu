@@ -383,22 +383,36 @@ struct Derived {
     Layout L;
 };
 
-// Weight table of multi-step calls (rate_frozen.cu) for grid g: expected lines.  A row of a chunk is as
-// long as its longest lane's range: the particles of the row's pencil within the chord that the
-// smallest transverse distance between the two pencils leaves, plus the spread of 32 lanes' counts
-// on an irregular set.  Chunks that find no room are evaluated from the positions.
-size_t frozen_lines(const ade_params &p, double H, int n, const Grid &g, int val = 1)
+// Weight table of multi-step calls (rate_frozen.cu) for grid g.  chunk_lines: lines one chunk may need.  A
+// row is as long as its longest lane's range: the particles of the row's pencil within the chord that
+// the smallest transverse distance between the two pencils leaves, plus what the cells at its ends hold
+// outside of it and the spread of 32 lanes' counts on an irregular set.
+unsigned chunk_lines(const ade_params &p, double H, int n, const Grid &g, int val)
 {
     const double per = (double)n / g.ncells;                  // particles per cell
     const double sx = p.box[0] / g.nc[0], sy = p.box[1] / g.nc[1], sz = p.dim == 3 ? p.box[2] / g.nc[2] : 0.0;
-    double lines = 8.0;
+    double lines = (g.nrows + 31) / 32 + 4.0;
     for (int r = 0; r < g.nrows; ++r) {
         const double ey = fmax(abs(g.rows[r].dy) - 1.0, 0.0) * sy, ez = fmax(abs(g.rows[r].dz) - 1.0, 0.0) * sz;
         const double mu = 2.0 * sqrt(fmax(H * H - ey * ey - ez * ez, 0.0)) / sx * per;
-        lines += val * (mu + 1.2 * sqrt(mu) + 0.5) + 2.0;     // and the row's first indices, in use and as scratch
+        lines += val * (mu + 1.2 * sqrt(mu) + 0.8 * per + 0.5) + 1.0;   // whole cells at the ends; the first indices
     }
-    const double np = (double)(g.ncells / g.nc[0]);
-    return (size_t)((n / 32.0 + 0.6 * fmin(np, (double)n)) * lines) + 1024;
+    return (unsigned)fmin(ceil(lines), 1e9);
+}
+
+size_t frozen_slots(int n, const Grid &g) { return (size_t)n / 32 + (size_t)(g.ncells / g.nc[0]) + 2; }
+
+// A region per chunk, and an eighth more for chunks that outgrow theirs.
+size_t frozen_lines(const ade_params &p, double H, int n, const Grid &g, int val = 1)
+{
+    const size_t l = frozen_slots(n, g) * chunk_lines(p, H, n, g, val);
+    return l + l / 8 + 64;
+}
+
+// Lines of a chunk's region when `lines` are at hand.
+unsigned frozen_stride(const ade_params &p, double H, int n, const Grid &g, int val, size_t lines)
+{
+    return (unsigned)std::min<size_t>(chunk_lines(p, H, n, g, val), lines / frozen_slots(n, g));
 }
 
 // Above this the table is left out and every evaluation computes its weights (a few per cent of the
@@ -460,7 +474,7 @@ int derive(const ade_params *p, int n, Derived *d)
             Grid g;
             if ((p->cell_subdiv > 0 && k != p->cell_subdiv) || !make_grid(*p, d->Hgrid, k, &g)) continue;
             lines = std::max(lines, frozen_lines(*p, d->H, n, g));
-            slots = std::max(slots, (size_t)n / 32 + (size_t)(g.ncells / g.nc[0]) + 2);
+            slots = std::max(slots, frozen_slots(n, g));
         }
         if (128.0 * (double)lines <= kFrozenMaxBytes) {
             d->fz_lines = lines;
@@ -640,7 +654,8 @@ int enqueue_frozen(ade_ctx *c, int steps, cudaStream_t s)
         rp.back[i] = 0u;
         rp.inc[i] = (uint32_t)steps * c->inc[i];
     }
-    const ade::FrozenTab &tab = c->frozen_tab;
+    ade::FrozenTab tab = c->frozen_tab;
+    ade::frozen_divide(c, 1, c->frozen_lines, &rp, &tab);
     rp.dt = (float)(0.5 * c->dt);
     ADE_CK(ade::launch_frozen_build(c->dim, c->p.kernel, c->iso, c->w.P0, c->w.cell_start, c->w.perm, rp, tab, st, s));
     for (int k = 0; k < steps; ++k) {
@@ -655,11 +670,12 @@ int enqueue_frozen(ade_ctx *c, int steps, cudaStream_t s)
     return ADE_OK;
 }
 
-// Whether `steps` steps of one call keep the pair weights.  Filling the table costs about 1.9 evaluations
-// of the tuned walk, one evaluation from it 0.4 to 0.75: from the third step on it always pays, and on
-// sets below about half a million particles from the second (256^2 28 against 38 us per step, 512^2 68
-// against 72, 700^2 irregular 144 against 153; 1024^2 312 against 285).
-bool use_frozen(const ade_ctx *c, int steps) { return c->frozen && (steps >= 3 || (steps == 2 && c->n <= (1 << 19))); }
+// Whether `steps` steps of one call keep the pair weights: filling the table takes 1.5 to 1.9 evaluations of
+// the tuned walk and gives the first predictor, a later evaluation from it takes 0.4 to 0.8, so it pays
+// from the second step on (two steps, us per step: 128^3 1241 against 1465, 1024^2 276 against 285,
+// 512^2 59 against 72, 256^2 23 against 38).  A single step stays with the walks (the cube's would
+// take 1.5 ms).
+bool use_frozen(const ade_ctx *c, int steps) { return c->frozen && steps >= 2; }
 
 // Enqueue one predictor-corrector step (Eq. 8-9) and the fold of its diagnostics.
 int enqueue_step(ade_ctx *c, cudaStream_t s)
@@ -789,7 +805,7 @@ void ade::frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots,
         Grid g;
         if ((fixed && k != c->subdiv) || !make_grid(c->p, c->Hgrid, k, &g)) continue;
         *lines = std::max(*lines, frozen_lines(c->p, c->H, c->n, g, val));
-        *slots = std::max(*slots, (size_t)c->n / 32 + (size_t)(g.ncells / g.nc[0]) + 2);
+        *slots = std::max(*slots, frozen_slots(c->n, g));
         ade::RateParams rp;
         memset(&rp, 0, sizeof(rp));
         rp.n = c->n;
@@ -799,6 +815,16 @@ void ade::frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots,
         *blocks = std::max(*blocks, (int)(d.x * d.y));
     }
     *lines = std::min(*lines, (size_t)(kFrozenMaxBytes / 128.0));
+}
+
+void ade::frozen_divide(const ade_ctx *c, int val, size_t lines, RateParams *rp, FrozenTab *tab)
+{
+    Grid g;
+    if (!make_grid(c->p, c->Hgrid, c->subdiv, &g)) return;   // (the grid in use fits)
+    rp->fz_base = 0u;
+    rp->fz_stride = frozen_stride(c->p, c->H, c->n, g, val, lines);
+    tab->pool = (unsigned)(frozen_slots(c->n, g) * rp->fz_stride);
+    tab->cap = (unsigned)(lines - tab->pool);
 }
 
 // Eq. 3 gives D = d_T I + (d_L - d_T) vhat vhat^T with d_T = alpha_T |v| + D_m, d_L = alpha_L |v| + D_m;
@@ -894,7 +920,7 @@ int ade_init_particles(ade_ctx **out, const ade_params *p, int n, uint32_t *xq_d
     c->frozen_tab.slots = at<uint4>(workspace_dev, d.L.fz_slots);
     c->frozen_C = at<float>(workspace_dev, d.L.fz_C);
     c->frozen_tab.cursor = at<unsigned>(workspace_dev, d.L.fz_cursor);
-    c->frozen_tab.cap = (unsigned)d.fz_lines;
+    c->frozen_lines = d.fz_lines;
 
     rc = plume_constants(p, n, d, c->D, &c->dt, c->inc, c->inc_half, &c->rp, &c->iso);
     if (rc) {
@@ -1488,6 +1514,7 @@ struct ade_batch {
     ade::FrozenItem *d_items = nullptr;
     float *frozen_C = nullptr;
     std::vector<ade::FrozenItem> items;
+    std::vector<size_t> frozen_plume;   // table lines of each plume
 };
 
 namespace {
@@ -1500,6 +1527,7 @@ struct BatchLayout {
 // Size of a batch's weight table over every subdivision its plumes may be given (0: none).
 struct BatchFrozen {
     size_t lines = 0, pencils = 0, items = 0;
+    std::vector<size_t> plume;          // lines of each plume
 };
 
 BatchFrozen batch_frozen_size(int P, const ade_params *p, const int *n)
@@ -1517,6 +1545,7 @@ BatchFrozen batch_frozen_size(int P, const ade_params *p, const int *n)
             items = std::max(items, np + (size_t)n[i] / 32);
         }
         f.lines += lines;
+        f.plume.push_back(lines);
         f.pencils += pencils;
         f.items += items;
     }
@@ -1617,6 +1646,7 @@ int batch_plan(ade_batch *b)
     b->NC = 0;
     b->items.clear();
     int p0 = 0;
+    unsigned fz_line = 0u;
     std::vector<std::pair<double, ade::BatchTile>> items;
     for (int i = 0; i < b->P; ++i) {
         ade_params pp = b->params[i];
@@ -1637,6 +1667,11 @@ int batch_plan(ade_batch *b)
         rp.goff = b->offsets[i];
         rp.coff = b->NC;
         rp.frame = b->w.frame + (size_t)i * ade::kFrameWords;
+        if (b->frozen) {   // the plume's chunks' regions, one plume behind the other; what is left is the pool
+            rp.fz_base = fz_line;
+            rp.fz_stride = frozen_stride(pp, d.H, b->n[i], d.g, 1, b->frozen_plume[i]);
+            fz_line += (unsigned)(frozen_slots(b->n[i], d.g) * rp.fz_stride);
+        }
         b->ncells[i] = d.g.ncells;
         b->subdiv_choice[i] = d.g.subdiv;
         b->NC += d.g.ncells;
@@ -1674,6 +1709,10 @@ int batch_plan(ade_batch *b)
         }
     }
     if (b->NC > b->NC_max) return fail(ADE_ERR_CAPACITY, "batch cell table exceeds the workspace");
+    size_t fz_total = 0;
+    for (size_t l : b->frozen_plume) fz_total += l;
+    b->frozen_tab.pool = fz_line;
+    b->frozen_tab.cap = (unsigned)(fz_total - fz_line);
     std::stable_sort(items.begin(), items.end(),
                      [](const std::pair<double, ade::BatchTile> &x, const std::pair<double, ade::BatchTile> &y) {
                          return x.first > y.first;
@@ -1888,7 +1927,7 @@ int ade_batch_init(ade_batch **out, int nplumes, const ade_params *p, const int 
     b->frozen_tab.words = at<float>(workspace_dev, L.fz_words);
     b->frozen_tab.slots = at<uint4>(workspace_dev, L.fz_slots);
     b->frozen_tab.cursor = at<unsigned>(workspace_dev, L.fz_cursor);
-    b->frozen_tab.cap = (unsigned)fz.lines;
+    b->frozen_plume = fz.plume;
     b->frozen_C = at<float>(workspace_dev, L.fz_C);
     b->d_items = at<ade::FrozenItem>(workspace_dev, L.fz_items);
     b->w.P0 = at<uint4>(workspace_dev, L.P0);
@@ -2305,7 +2344,7 @@ int sweep_layout(const ade_params *p, int n, int P, const double *theta, ade_par
     L->pstats = take((size_t)3 * P * 8);
     L->lines = n > 0 ? std::min(frozen_lines(pp, L->d.H, n, L->d.g, 2), (size_t)(kFrozenMaxBytes / 128.0)) : 0;
     L->words = take(L->lines * 128);
-    L->slots = take(((size_t)n / 32 + (size_t)(L->d.g.ncells / L->d.g.nc[0]) + 2) * 16);
+    L->slots = take(frozen_slots(n, L->d.g) * 16);
     L->cursor = take(64);
     L->total = off;
     if (pp_out) *pp_out = pp;
@@ -2519,7 +2558,9 @@ int ade_sweep_init(ade_sweep **out, const ade_params *p, int n, int ntheta, cons
     sw->run.tab.words = at<float>(workspace_dev, L.words);
     sw->run.tab.slots = at<uint4>(workspace_dev, L.slots);
     sw->run.tab.cursor = at<unsigned>(workspace_dev, L.cursor);
-    sw->run.tab.cap = (unsigned)L.lines;
+    sw->rp.fz_stride = n > 0 ? frozen_stride(pp, L.d.H, n, L.d.g, 2, L.lines) : 0u;
+    sw->run.tab.pool = (unsigned)(frozen_slots(n, L.d.g) * sw->rp.fz_stride);
+    sw->run.tab.cap = (unsigned)L.lines - sw->run.tab.pool;
     sw->theta.assign(theta_host, theta_host + 3 * ntheta);
     // Dcal = a u + b per set (uniform v, K = 2D)
     const int dm = pp.dim;

@@ -21,7 +21,8 @@ constexpr unsigned kNoRoom = 0xffffffffu;
 
 // Where one warp's chunk lies: particles [i0, min(i0 + 32, pe)) of pencil p (cy, cz).
 struct Chunk {
-    int cy, cz, i0, ps, pe, slot;
+    int cy, cz, i0, ps, pe;
+    int local, slot;       // the chunk's number within its plume, and in the slot table
 };
 
 // Origin of the build's cell grid along x (the records hold the positions of the build: no drift).
@@ -133,8 +134,9 @@ __device__ __forceinline__ float sep2(const uint4 &pa, const uint4 &pb, const Pa
 }
 
 // The weights of two candidates, the FP32 part in packed FP32x2 instructions (each half with the
-// operations of pair_weight, so the same bits).
-template <int DIM, int KERNEL, bool ISO>
+// operations of pair_weight, so the same bits).  ZS = false: zero separation does not occur (rows other
+// than the particles' own), as in pair_range_direct.
+template <int DIM, int KERNEL, bool ISO, bool ZS>
 __device__ __forceinline__ float2 pair_weight2(const uint4 &pa, const uint4 &p0, const uint4 &p1, const PairConst2 &k)
 {
     float2 dx = f2(sep(pa.x, p0.x, k.m1), sep(pa.x, p1.x, k.m1));
@@ -149,10 +151,38 @@ __device__ __forceinline__ float2 pair_weight2(const uint4 &pa, const uint4 &p0,
     if (DIM == 3) r2 = __ffma2_rn(dz, dz, r2);
     const float2 rinv = f2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
     const float2 om = __ffma2_rn(__fmul2_rn(r2, rinv), k.ninvH, f2(1.f, 1.f));
-    const float2 omq2 = f2(fmaxf(om.x + om.x, 0.f), fmaxf(om.y + om.y, 0.f));
+    const float2 omq2 = ZS ? f2(fmaxf(om.x + om.x, 0.f), fmaxf(om.y + om.y, 0.f)) : f2(om.x + fabsf(om.x), om.y + fabsf(om.y));
     const float2 sr = dcal2<DIM>(dx, dy, dz, rinv, k);
-    const float2 sc = f2(fmaxf(sr.x, -3.402823466e38f), fmaxf(sr.y, -3.402823466e38f));
+    const float2 sc = ZS ? f2(fmaxf(sr.x, -3.402823466e38f), fmaxf(sr.y, -3.402823466e38f)) : sr;
     return __fmul2_rn(shape2x2<KERNEL>(omq2), sc);
+}
+
+// Weights of one row's m candidates s, s + 1, ... (WRAP: beyond qe on from qe - len) into out, a line each,
+// and the row sum of the records' concentrations.
+template <int DIM, int KERNEL, bool ISO, bool ZS, bool WRAP>
+__device__ __forceinline__ float row_weights(const uint4 *__restrict__ P, const uint4 &pa, float Ca, const PairConst &k,
+                                             const PairConst2 &k2, int s, int m, int qe, int len, float *__restrict__ out)
+{
+    float rs = 0.f;
+    const uint4 *Ps = P + s;
+    int t = 0;
+#pragma unroll 2
+    for (; t + 1 < m; t += 2) {
+        const uint4 p0 = __ldg(WRAP && s + t >= qe ? Ps + t - len : Ps + t);
+        const uint4 p1 = __ldg(WRAP && s + t + 1 >= qe ? Ps + t + 1 - len : Ps + t + 1);
+        const float2 w = pair_weight2<DIM, KERNEL, ISO, ZS>(pa, p0, p1, k2);
+        out[t * 32] = w.x;
+        out[(t + 1) * 32] = w.y;
+        rs = fmaf(w.x, Ca - __uint_as_float(p0.w), rs);
+        rs = fmaf(w.y, Ca - __uint_as_float(p1.w), rs);
+    }
+    if (t < m) {
+        const uint4 pb = __ldg(WRAP && s + t >= qe ? Ps + t - len : Ps + t);
+        const float w = pair_weight<DIM, KERNEL, ISO>(pa, pb, k);
+        out[t * 32] = w;
+        rs = fmaf(w, Ca - __uint_as_float(pb.w), rs);
+    }
+    return rs;
 }
 
 // Cyclic candidate range of cells [lo, hi) of the pencil row whose cells start at `base` and whose
@@ -214,12 +244,19 @@ __device__ __noinline__ float walk_chunk(const uint4 *__restrict__ P, const uint
     return acc + comp;
 }
 
-// Weights (VAL 1) or g_L, g_T (VAL 2) of one chunk into the table; VAL 1 returns the row sums of the first evaluation (the concentrations
-// of the records).  BOX: the pencils' transverse boxes and the staged rows are at hand (square or
-// cubic single plumes): rows out of the warp's reach are skipped, as in the trimmed walks, and a
-// lane's range is cut at the x half-extent its own distance to the row leaves.  Otherwise every row is
-// looked at and a range is cut by the separations themselves.
-template <int DIM, int KERNEL, bool ISO, bool BOX, int VAL>
+// How a chunk's rows and ranges are cut before the separations are evaluated: every row and range
+// (kCutFull: unequal boxes), by the cell bands (kCutBand: no pencil boxes at hand), or by the pencils'
+// transverse boxes (kCutBox), as in the trimmed walks.
+enum ChunkCut { kCutFull = 0, kCutBand = 1, kCutBox = 2 };
+
+// Weights (VAL 1) or g_L, g_T (VAL 2) of one chunk into the table; VAL 1 returns the row sums of the
+// first evaluation (the concentrations of the records).  One pass over the rows: the chunk's lines go
+// to a region of fixed size (prm.fz_stride lines, the host's estimate for the grid) and only a chunk that
+// outgrows it is done again into room taken from the pool behind.  Rows are tested once per warp, each
+// lane's range is cut by its own distance to the row and then to its first and last candidate that may
+// lie inside H.  Bound: instruction issue.  128^3 cube 1.55 -> 1.15 ms, 1024^2 258 -> 200 us against a
+// form that counted every chunk's lines in a pass of its own.
+template <int DIM, int KERNEL, bool ISO, int CUT, int VAL>
 __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs, const RateParams &prm,
                              const Chunk &c, const uint4 &pa, const TrimRow *srow, const FrozenTab &tab,
                              const ShapeConst &sc = ShapeConst())
@@ -233,85 +270,80 @@ __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const 
     const TrimGeom g(prm);
     const float wpc = 4294967296.f / (float)ncx;     // x words per cell
     const PairConst k(prm);
+    const PairConst2 k2(k, k.m1);
     const float far2 = prm.H2 * (1.f + 1.f / 4096.f);   // beyond this the weight is exactly 0
-    int nr = nrows;
-    if (BOX) {
+    const float Ca = __uint_as_float(pa.w);
+    if (CUT != kCutFull) {
         me = trim_self<DIM>(pa, c.cy, c.cz, prm);
         ylo = yhi = me.fy;
         zlo = zhi = me.fz;
         warp_interval<DIM>(ylo, yhi, zlo, zhi);
-        nr = 0;
+    }
+    const unsigned hs = (unsigned)(nrows + 31) >> 5;    // header lines: a word per row
+    unsigned base = prm.fz_base + (unsigned)c.local * prm.fz_stride, room = prm.fz_stride;
+    float acc = 0.f, comp = 0.f;
+    unsigned R = 0u, used = 0u;
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        acc = comp = 0.f;
+        R = 0u;
+        used = hs;
+        float *hdr = tab.words + (size_t)base * 32;
+        float *out = hdr + hs * 32 + lane;
         for (int rb = 0; rb < nrows; rb += 32) {
-            float xe;
-            int pidx, wx;
-            nr += __popc(__ballot_sync(kFull, warp_row_test<DIM>(rb, srow, nrows, me, c.cy, c.cz, prm, g, ylo, yhi, zlo, zhi,
-                                                                 xe, pidx, wx)));
-        }
-    }
-    // scratch lines for the rows in reach of the chunk: {m, pencil} of each row, then its first indices
-    const int hl = (nr + 15) >> 4;
-    unsigned meta = 0u;
-    if (lane == 0) meta = atomicAdd(tab.cursor, (unsigned)(hl + nr));
-    meta = __shfl_sync(kFull, meta, 0);
-    bool room = meta <= tab.cap && tab.cap - meta >= (unsigned)(hl + nr);
-    if (!room) {
-        if (lane == 0) tab.slots[c.slot] = make_uint4(kNoRoom, 0u, 0u, 0u);
-        return VAL == 1 ? walk_chunk<DIM, KERNEL, ISO>(P, cs, prm, c, nullptr) : 0.f;
-    }
-    int2 *row = reinterpret_cast<int2 *>(tab.words + (size_t)meta * 32);
-    int *first = reinterpret_cast<int *>(tab.words) + (size_t)(meta + hl) * 32;
-    unsigned R = 0u, lines = 0u;
-    for (int rb = 0; rb < nrows; rb += 32) {
-        float xe = 0.f;
-        int pidx = 0, wx = 0;
-        bool reach;
-        if (BOX) {
-            reach = warp_row_test<DIM>(rb, srow, nrows, me, c.cy, c.cz, prm, g, ylo, yhi, zlo, zhi, xe, pidx, wx);
-        } else {
-            reach = rb + lane < nrows;
-            if (reach) {
+            float xe = 0.f;
+            int pidx = 0, wx = 0;
+            bool reach = rb + lane < nrows;
+            if (CUT == kCutBox) {
+                reach = warp_row_test<DIM>(rb, srow, nrows, me, c.cy, c.cz, prm, g, ylo, yhi, zlo, zhi, xe, pidx, wx);
+            } else if (reach) {
                 const StencilRow r = prm.rows[rb + lane];
                 pidx = row_pencil_of<DIM>(r, c.cy, c.cz, prm);
-                wx = r.w;
+                wx = (r.w & 0xff) | (r.dy == 0 && (DIM == 2 || r.dz == 0) ? 1 << 24 : 0);
+                if (CUT == kCutBand) {
+                    const TrimRow tr{(float)r.dy, (float)r.dz, 0, 0};
+                    const float e2 = row_gap2<DIM>(make_float4(0.f, 1.f, 0.f, DIM == 3 ? 1.f : 0.f), tr, ylo, yhi, yhi - ylo, zlo, zhi,
+                                                   zhi - zlo, g);
+                    const float t = fmaxf(g.Hm2 - e2, 0.f);
+                    xe = fmaf(t * rsqrt_ftz(fmaxf(t, 1.f)), g.inv_wx, 1.f / 4096.f);
+                    reach = e2 < g.Hm2;
+                }
             }
-        }
-        for (unsigned mask = __ballot_sync(kFull, reach); mask != 0u; mask &= mask - 1u) {
-            const int b = __ffs(mask) - 1;
-            const int q = __shfl_sync(kFull, pidx, b), w = __shfl_sync(kFull, wx, b) & 0xff;
-            int dlo = -w, dhi = w;
-            int xw = 0x7fffffff;                      // the lane's x half-extent in words
-            if (BOX) {
-                const TrimRow r = srow[rb + b];
-                const float e2 = row_gap2<DIM>(load_box(prm, q), r, me.fy, me.fy, 0.f, me.fz, me.fz, 0.f, g);
-                const float t = g.Hm2 - e2;
-                const float xl = t > 0.f ? fmaf(t * rsqrt_ftz(t), g.inv_wx, 1.f / 4096.f) : 0.f;
-                dlo = max(__float2int_rd(me.fx - xl), -w);
-                dhi = min(__float2int_rd(me.fx + xl), w);
-                xw = t > 0.f ? __float2int_ru(fminf(xl * wpc, 2.0e9f)) : -1;
-            }
-            const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
-            int s, cnt;
-            cyclic_range(cs, q * ncx, cx + dlo, cx + dhi + 1, ncx, qs, qe, s, cnt);
-            if (!valid || xw < 0) cnt = 0;
-            if (s >= qe) s = qs;                     // (the range's first cells are empty)
-            if (BOX) {
-                // candidates farther than xw along x lie beyond H (1 + 2^-12): weight exactly 0.  Both
-                // ends' two outermost are looked at together (one latency instead of up to four).
-                auto at = [&](int t) {
-                    const int j = s + t;
-                    return __ldg(&P[j >= qe ? j - len : j].x);
-                };
-                auto out = [&](uint32_t x) {
-                    const int d = (int)(x - pa.x);
-                    return d < -xw || d > xw;
+            for (unsigned mask = __ballot_sync(kFull, reach); mask != 0u; mask &= mask - 1u) {
+                const int b = __ffs(mask) - 1;
+                const int q = __shfl_sync(kFull, pidx, b), wb = __shfl_sync(kFull, wx, b), w = wb & 0xff;
+                int dlo = -w, dhi = w, xw = 0x7fffffff;          // xw: the lane's x half-extent in words
+                if (CUT == kCutBox) {
+                    const TrimRow tr = srow[rb + b];
+                    const float e2 = row_gap2<DIM>(load_box(prm, q), tr, me.fy, me.fy, 0.f, me.fz, me.fz, 0.f, g);
+                    const float t = g.Hm2 - e2, xl = t > 0.f ? fmaf(t * rsqrt_ftz(t), g.inv_wx, 1.f / 4096.f) : 0.f;
+                    dlo = max(__float2int_rd(me.fx - xl), -w);
+                    dhi = min(__float2int_rd(me.fx + xl), w);
+                    xw = t > 0.f ? __float2int_ru(fminf(xl * wpc, 2.0e9f)) : -1;
+                } else if (CUT == kCutBand) {
+                    const float xeb = __shfl_sync(kFull, xe, b);
+                    dlo = max(__float2int_rd(me.fx - xeb), -w);
+                    dhi = min(__float2int_rd(me.fx + xeb), w);
+                }
+                const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
+                int s, cnt;
+                cyclic_range(cs, q * ncx, cx + dlo, cx + dhi + 1, ncx, qs, qe, s, cnt);
+                if (!valid || xw < 0) cnt = 0;
+                if (s >= qe) s = qs;                     // (the range's first cells are empty)
+                // Both ends' two outermost candidates are looked at together (one latency): farther than xw
+                // along x, or than H, their weight is exactly 0.
+                auto out_of = [&](int t) {
+                    const int j = s + t, jj = j >= qe ? j - len : j;
+                    if (CUT == kCutBox) {
+                        const int d = (int)(__ldg(&P[jj].x) - pa.x);
+                        return d < -xw || d > xw;
+                    }
+                    return !(sep2<DIM, ISO>(pa, __ldg(P + jj), k) < far2);
                 };
                 while (cnt > 0) {
-                    const int t1 = min(1, cnt - 1), e1 = max(cnt - 2, 0);
-                    const uint32_t f0 = at(0), f1 = at(t1), b0 = at(cnt - 1), b1 = at(e1);
-                    const int df = out(f0) ? (out(f1) ? 2 : 1) : 0, db = out(b0) ? (out(b1) ? 2 : 1) : 0;
-                    const int left = cnt - df - db;
-                    if (left <= 0) {          // the ends meet: what is left, if anything, lies between them
-                        cnt = out(f0) && out(f1) && out(b0) && out(b1) && cnt <= 4 ? 0 : cnt;
+                    const bool f0 = out_of(0), f1 = out_of(min(1, cnt - 1)), b0 = out_of(cnt - 1), b1 = out_of(max(cnt - 2, 0));
+                    const int df = f0 ? (f1 ? 2 : 1) : 0, db = b0 ? (b1 ? 2 : 1) : 0, left = cnt - df - db;
+                    if (left <= 0) {                     // the ends meet: what is left, if anything, lies between
+                        if (f0 && f1 && b0 && b1 && cnt <= 4) cnt = 0;
                         break;
                     }
                     s += df;
@@ -319,86 +351,56 @@ __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const 
                     cnt = left;
                     if (df < 2 && db < 2) break;
                 }
-            } else {
-                while (cnt > 0 && !(sep2<DIM, ISO>(pa, __ldg(P + s), k) < far2)) {
-                    --cnt;
-                    s = s + 1 < qe ? s + 1 : qs;
+                const int m = (int)__reduce_max_sync(kFull, (unsigned)cnt);
+                if (m == 0) continue;
+                // idle tail iterations of a shorter lane stay inside the doubled pencil (m <= len)
+                used += 1u + (unsigned)(m * VAL);
+                const bool keep = used <= room;
+                if (keep) {
+                    if (lane == 0) hdr[R] = __int_as_float(m);
+                    out[0] = __int_as_float(s + qs);     // index into the doubled concentrations
                 }
-                while (cnt > 0) {
-                    const int j = s + cnt - 1;
-                    if (sep2<DIM, ISO>(pa, __ldg(P + (j >= qe ? j - len : j)), k) < far2) break;
-                    --cnt;
+                ++R;
+                if (!keep) continue;                     // to be done again
+                out += 32;
+                float rs = 0.f;
+                if (VAL == 2) {
+                    float2 *o2 = reinterpret_cast<float2 *>(out + lane);
+                    int t = 0;
+                    for (; t + 1 < m; t += 2) {
+                        const int j0 = s + t, j1 = j0 + 1;
+                        float2 gL, gT;
+                        pair_shape2<DIM, KERNEL, ISO>(pa, __ldg(P + (j0 >= qe ? j0 - len : j0)), __ldg(P + (j1 >= qe ? j1 - len : j1)),
+                                                      k2, sc, gL, gT);
+                        o2[t * 32] = f2(gL.x, gT.x);
+                        o2[(t + 1) * 32] = f2(gL.y, gT.y);
+                    }
+                    if (t < m) {
+                        const int j = s + t;
+                        o2[t * 32] = pair_shape<DIM, KERNEL, ISO>(pa, __ldg(P + (j >= qe ? j - len : j)), k, sc);
+                    }
+                } else if (__any_sync(kFull, s + m > qe)) {
+                    rs = row_weights<DIM, KERNEL, ISO, true, true>(P, pa, Ca, k, k2, s, m, qe, len, out);
+                } else if ((wb >> 24) != 0) {
+                    rs = row_weights<DIM, KERNEL, ISO, true, false>(P, pa, Ca, k, k2, s, m, qe, len, out);
+                } else {
+                    rs = row_weights<DIM, KERNEL, ISO, false, false>(P, pa, Ca, k, k2, s, m, qe, len, out);
                 }
+                out += m * 32 * VAL;
+                neumaier_add(acc, comp, rs);
             }
-            const int m = (int)__reduce_max_sync(kFull, (unsigned)cnt);
-            if (m == 0) continue;
-            // idle tail iterations of a shorter lane stay inside the doubled pencil (m <= len)
-            if (lane == 0) row[R] = make_int2(m, q);
-            first[R * 32 + lane] = s;
-            ++R;
-            lines += (unsigned)(m * VAL);
         }
+        if (used <= room || attempt == 1) break;
+        // outgrown: once more into the pool
+        unsigned at = 0u;
+        if (lane == 0) at = atomicAdd(tab.cursor, used);
+        at = __shfl_sync(kFull, at, 0);
+        base = tab.pool + at;
+        room = at <= tab.cap && tab.cap - at >= used ? used : 0u;
+        if (room == 0u) break;
     }
-    const unsigned hs = (R + 31u) >> 5;
-    unsigned off = 0u;
-    if (lane == 0) off = atomicAdd(tab.cursor, hs + R + lines);
-    off = __shfl_sync(kFull, off, 0);
-    room = off <= tab.cap && tab.cap - off >= hs + R + lines;
-    if (lane == 0) tab.slots[c.slot] = make_uint4(room ? off : kNoRoom, R, hs + R + lines, 0u);
-    if (!room) return VAL == 1 ? walk_chunk<DIM, KERNEL, ISO>(P, cs, prm, c, nullptr) : 0.f;
-    __syncwarp();
-    const PairConst2 k2(k, k.m1);
-    const float Ca = __uint_as_float(pa.w);
-    float acc = 0.f, comp = 0.f;
-    float *out = tab.words + (size_t)off * 32 + lane;
-    for (unsigned r = lane; r < hs * 32; r += 32) out[r - lane] = __int_as_float(r < R ? row[r].x : 0);
-    out += (size_t)hs * 32;
-    for (unsigned r = 0; r < R; ++r) {
-        const int2 h = row[r];
-        const int m = h.x, qs = (int)__ldg(cs + h.y * ncx), qe = (int)__ldg(cs + h.y * ncx + ncx), len = qe - qs;
-        const int s = first[r * 32 + lane];
-        out[0] = __int_as_float(s + qs);            // index into the doubled concentrations
-        out += 32;
-        if (VAL == 2) {
-            float2 *o2 = reinterpret_cast<float2 *>(out + lane);
-            int t = 0;
-            for (; t + 1 < m; t += 2) {
-                const int j0 = s + t, j1 = j0 + 1;
-                float2 gL, gT;
-                pair_shape2<DIM, KERNEL, ISO>(pa, __ldg(P + (j0 >= qe ? j0 - len : j0)), __ldg(P + (j1 >= qe ? j1 - len : j1)),
-                                              k2, sc, gL, gT);
-                o2[t * 32] = f2(gL.x, gT.x);
-                o2[(t + 1) * 32] = f2(gL.y, gT.y);
-            }
-            if (t < m) {
-                const int j = s + t;
-                o2[t * 32] = pair_shape<DIM, KERNEL, ISO>(pa, __ldg(P + (j >= qe ? j - len : j)), k, sc);
-            }
-            out += 64 * m;
-            continue;
-        }
-        float rs = 0.f;
-        int t = 0;
-#pragma unroll 2
-        for (; t + 1 < m; t += 2, out += 64) {
-            const int j0 = s + t, j1 = j0 + 1;
-            const uint4 p0 = __ldg(P + (j0 >= qe ? j0 - len : j0)), p1 = __ldg(P + (j1 >= qe ? j1 - len : j1));
-            const float2 w = pair_weight2<DIM, KERNEL, ISO>(pa, p0, p1, k2);
-            out[0] = w.x;
-            out[32] = w.y;
-            rs = fmaf(w.x, Ca - __uint_as_float(p0.w), rs);
-            rs = fmaf(w.y, Ca - __uint_as_float(p1.w), rs);
-        }
-        if (t < m) {
-            const int j = s + t;
-            const uint4 pb = __ldg(P + (j >= qe ? j - len : j));
-            const float w = pair_weight<DIM, KERNEL, ISO>(pa, pb, k);
-            out[0] = w;
-            rs = fmaf(w, Ca - __uint_as_float(pb.w), rs);
-            out += 32;
-        }
-        neumaier_add(acc, comp, rs);
-    }
+    if (lane == 0) tab.slots[c.slot] = make_uint4(used <= room ? base : kNoRoom, R, used, hs);
+    if (VAL == 1 && used > room) return walk_chunk<DIM, KERNEL, ISO>(P, cs, prm, c, nullptr);
     return acc + comp;
 }
 
@@ -433,7 +435,7 @@ __device__ __forceinline__ void stream_rows(const uint4 sl, const FrozenTab &tab
     int ahead = min(total, kAhead);
     if (lane == 0) prefetch_l2(base, (unsigned)ahead * 128u);
     const float *hdr = w;
-    w += (size_t)((R + 31) >> 5) * 32;
+    w += (size_t)sl.w * 32;
     int hm = 0;
     float s = ld_weight(w);
     for (int r = 0; r < R; ++r) {
@@ -507,7 +509,8 @@ __device__ __forceinline__ void for_chunks(const uint32_t *__restrict__ cs, cons
     c.ps = (int)__ldg(cs + p * prm.ncx);
     c.pe = (int)__ldg(cs + p * prm.ncx + prm.ncx);
     for (c.i0 = c.ps + 32 * v; c.i0 < c.pe; c.i0 += 32 * nv) {
-        c.slot = (c.i0 >> 5) + p0 + p;   // increases strictly from chunk to chunk
+        c.local = ((c.i0 - prm.goff) >> 5) + p;   // increases strictly from chunk to chunk
+        c.slot = (c.i0 >> 5) + p0 + p;
         f(c);
     }
 }

@@ -63,7 +63,7 @@ __global__ __launch_bounds__(kT) void k_frozen_build(const uint4 *__restrict__ P
     for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), nv, [&](const Chunk &c) {
         const int i = c.i0 + (threadIdx.x & 31);
         const uint4 pa = __ldg(P + min(i, c.pe - 1));
-        const float sum = build_chunk<DIM, KERNEL, ISO, ISO, 1>(P, cs, prm, c, pa, srow, tab);
+        const float sum = build_chunk<DIM, KERNEL, ISO, ISO ? kCutBox : kCutFull, 1>(P, cs, prm, c, pa, srow, tab);
         if (i >= c.pe) return;
         const float Cl = __uint_as_float(pa.w);
         st.C[c.ps + i] = st.C[c.pe + i] = Cl;
@@ -111,7 +111,7 @@ __global__ __launch_bounds__(kT) void k_frozen_build_batch(const uint4 *__restri
     for_chunks(cs + prm.coff, prm, it.pencil, it.p0, it.y, it.ny, [&](const Chunk &c) {
         const int i = c.i0 + (threadIdx.x & 31);
         const uint4 pa = __ldg(P + min(i, c.pe - 1));
-        const float sum = build_chunk<DIM, KERNEL, true, false, 1>(P, cs + prm.coff, prm, c, pa, nullptr, tab);
+        const float sum = build_chunk<DIM, KERNEL, true, kCutBand, 1>(P, cs + prm.coff, prm, c, pa, nullptr, tab);
         if (i >= c.pe) return;
         const float Cl = __uint_as_float(pa.w);
         st.C[c.ps + i] = st.C[c.pe + i] = Cl;

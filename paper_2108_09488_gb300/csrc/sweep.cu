@@ -120,7 +120,7 @@ __global__ __launch_bounds__(kT) void k_sweep_table(const uint4 *__restrict__ P,
         const int i = c.i0 + (threadIdx.x & 31);
         if (i < c.pe) gather_sets(perm, C, (size_t)prm.n, sets, P4, i, 2 * (size_t)prm.n, (size_t)(c.ps + i), (size_t)(c.pe + i), Cs);
         const uint4 pa = __ldg(P + min(i, c.pe - 1));
-        build_chunk<DIM, KERNEL, ISO, ISO, 2>(P, cs, prm, c, pa, srow, tab, sc);
+        build_chunk<DIM, KERNEL, ISO, ISO ? kCutBox : kCutFull, 2>(P, cs, prm, c, pa, srow, tab, sc);
     });
 }
 
