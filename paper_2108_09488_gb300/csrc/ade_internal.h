@@ -81,6 +81,7 @@ struct RateParams {
     int nrows;
     StencilRow rows[kMaxRows];
     float H2;        // support radius squared
+    float Hg2;       // squared radius the cell grid is built for (velocity-field mode: H + skin)
     float invH;      // 1 / support radius
     float sy, sz;    // L_y / L_x, L_z / L_x (1 for a cubic box)
     // Pair factor of Eq. 5 for the uniform tensor of Eq. 3 (K = 2D): Dcal = a (vhat . e)^2 + b with
@@ -306,6 +307,8 @@ cudaError_t launch_field_permute(int dim, const uint32_t *perm, int n, const Fie
 cudaError_t launch_rate_pair(int dim, int kernel, int epi, bool iso, const uint4 *Pe, const uint4 *Pc,
                              const uint32_t *cs, const uint32_t *perm, const RateParams &prm, const EpiOut &out,
                              cudaStream_t s);
+// Partials the velocity-field corrector writes.
+int field_partials(int dim, const RateParams &prm);
 cudaError_t launch_rate_field(int dim, int kernel, int epi, const uint4 *Pe, const uint32_t *cell_start,
                               const uint32_t *perm, const FieldWork &fw, const RateParams &prm,
                               const FieldParams &fp, const EpiOut &out, cudaStream_t s);
@@ -393,6 +396,7 @@ struct ade_ctx {
     bool frozen;          // steps of one call may keep the pair weights (frozen_tab)
     ade::FrozenTab frozen_tab;
     size_t frozen_lines;  // lines of the table
+    bool frozen_fits;     // the table has room for the grid in use
     float *frozen_C;      // [2][2n] concentrations of such a call (FrozenState)
     // velocity-field mode (p.vmax > 0)
     bool field;

@@ -204,6 +204,16 @@ int choose_grid(const ade_params &p, double H, int n, Grid *g)
     for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
         Grid t;
         if (!make_grid(p, H, k, &t)) continue;
+        // 3D: the finest grid of at least one particle per cell on average (else the coarsest).  Finer
+        // ones leave rows of few candidates and pencils of few particles (us per step at this rule's
+        // choice and one finer: 45^3 jittered, velocity field 504 / 536, weights kept 121 / 205; 64^3 at one
+        // per cell, field 1882 / 2304, weights kept 165 / 179), coarser ones longer ranges.
+        if (p.dim == 3) {
+            if (found && (double)n < 0.999 * t.ncells) break;
+            *g = t;
+            found = true;
+            continue;
+        }
         double c = grid_cost(t, n);
         if (!found || c < best) {
             *g = t;
@@ -309,6 +319,8 @@ struct Layout {
         fbits, Q, Qh, total;
 };
 
+constexpr size_t kStatusAt = 64, kStatsBytes = 128;
+
 // field_dim: 0 for a uniform velocity, else dim (velocity-field buffers are added at the end).
 // nw_partials: per-warp corrector partials of the widest rate launch.  npencils: pencil boxes of
 // the trimmed walks (0: none).
@@ -333,9 +345,9 @@ Layout layout(int n, int ncells, int nb_partials, int nw_partials, int field_dim
     L.P1 = take((size_t)n * 16);
     L.partials = take((size_t)3 * (nb_partials > 0 ? nb_partials : 1) * 8);
     L.wpart = take((size_t)(nw_partials > 0 ? nw_partials : 1) * 16);
-    L.stats = take(8 * 8);
+    L.stats = take(kStatsBytes);
     L.cf_partials = take((size_t)3 * (nb_partials > 0 ? nb_partials : 1) * 8);
-    L.status = take(64);
+    L.status = L.stats + kStatusAt;   // behind the statistics, so that one copy brings both to the host
     L.pairs = take(64);
     L.pencil = npencils > 0 ? take((size_t)npencils * 16) : 0;
     L.tile_sums = take(ade::tile_sums_bytes(ncells));
@@ -383,6 +395,14 @@ struct Derived {
     Layout L;
 };
 
+// Particles within H of one at the mean density.
+double expected_neighbours(const ade_params &p, double H, int n)
+{
+    double nb = (double)n * (p.dim == 2 ? kPi * H * H : 4.0 / 3.0 * kPi * H * H * H);
+    for (int i = 0; i < p.dim; ++i) nb /= p.box[i];
+    return nb;
+}
+
 // Weight table of multi-step calls (rate_frozen.cu) for grid g.  chunk_lines: lines one chunk may need.  A
 // row is as long as its longest lane's range: the particles of the row's pencil within the chord that
 // the smallest transverse distance between the two pencils leaves, plus what the cells at its ends hold
@@ -413,6 +433,20 @@ size_t frozen_lines(const ade_params &p, double H, int n, const Grid &g, int val
 unsigned frozen_stride(const ade_params &p, double H, int n, const Grid &g, int val, size_t lines)
 {
     return (unsigned)std::min<size_t>(chunk_lines(p, H, n, g, val), lines / frozen_slots(n, g));
+}
+
+// Lines a table may take on the grids the autotuner may switch to: a fifth more than the smallest, and what
+// the grid in use needs.  (Coarse grids hold several lattice lines per pencil and need much more; a
+// context tuned to one evaluates every step anew.)
+size_t frozen_room(const ade_params &p, double Hgrid, double H, int n, const Grid &in_use, bool fixed, int val)
+{
+    size_t least = frozen_lines(p, H, n, in_use, val);
+    const size_t own = least;
+    for (int k = 1; !fixed && k <= ade::kMaxSubdiv; ++k) {
+        Grid g;
+        if (make_grid(p, Hgrid, k, &g)) least = std::min(least, frozen_lines(p, H, n, g, val));
+    }
+    return std::max(own, least + least / 5);
 }
 
 // Above this the table is left out and every evaluation computes its weights (a few per cent of the
@@ -448,6 +482,17 @@ int derive(const ade_params *p, int n, Derived *d)
     d->nb_partials = nbr > nbc ? nbr : nbc;
     if (nbt > d->nb_partials) d->nb_partials = nbt;
     d->nw_partials = std::max(nbr * (ade::kRateThreads / 32), ade::rate_launch_warps(p->dim, d->tiles, iso));
+    if (p->vmax > 0.0)   // the velocity-field kernel's blocks go by pencils, on any grid the context may be given
+        for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
+            Grid g;
+            if ((p->cell_subdiv > 0 && k != p->cell_subdiv) || !make_grid(*p, d->Hgrid, k, &g)) continue;
+            ade::RateParams t;
+            memset(&t, 0, sizeof(t));
+            t.n = n;
+            t.ncy = g.nc[1];
+            t.ncz = g.nc[2];
+            d->nw_partials = std::max(d->nw_partials, ade::field_partials(p->dim, t));
+        }
     int ncells_cap = d->g.ncells;
     int pencils_cap = d->g.ncells / d->g.nc[0];
     if (p->cell_subdiv == 0 && p->flags == 0u) {
@@ -467,12 +512,18 @@ int derive(const ade_params *p, int n, Derived *d)
     }
     d->ncells_cap = ncells_cap;
     d->fz_lines = d->fz_slots = 0;
-    if (p->flags == 0u && !(p->vmax > 0.0) && n > 0) {
+    // Wide kernels on sets that fill the chip stay with the walks: a table of 12 GB streams no faster than
+    // they evaluate (405^2 irregular, 9,400 neighbours: 2.2 ms either way; 248^2, 4,900, whose 1,900 warps do
+    // not fill it: 0.58 against 0.93 ms).
+    const bool wide = expected_neighbours(*p, d->H, n) > 500.0 && n > 80000;
+    if (p->flags == 0u && !(p->vmax > 0.0) && n > 0 && !wide) {
         // the library's choice of walk: multi-step calls keep the weights, on any grid it may pick
         size_t lines = 0, slots = 0;
+        const size_t room = frozen_room(*p, d->Hgrid, d->H, n, d->g, p->cell_subdiv > 0, 1);
         for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
             Grid g;
             if ((p->cell_subdiv > 0 && k != p->cell_subdiv) || !make_grid(*p, d->Hgrid, k, &g)) continue;
+            if (frozen_lines(*p, d->H, n, g) > room) continue;
             lines = std::max(lines, frozen_lines(*p, d->H, n, g));
             slots = std::max(slots, frozen_slots(n, g));
         }
@@ -625,7 +676,7 @@ ade::EpiOut epi_corrector(ade_ctx *c)
 // partials into w.stats (the step's diagnostics of Eq. 9).
 int enqueue_fold(ade_ctx *c, cudaStream_t s)
 {
-    const int m = c->field ? ade::rate_blocks(c->n) * (ade::kRateThreads / 32)
+    const int m = c->field ? ade::field_partials(c->dim, c->rp)
                            : ade::rate_launch_warps(c->dim, c->rp, c->iso);
     if (m > c->wpart_cap) return fail(ADE_ERR_CAPACITY, "corrector partials exceed the workspace");
     ADE_CK(ade::launch_fold_warp_partials(c->w.wpart, m, c->w.stats, s));
@@ -675,7 +726,7 @@ int enqueue_frozen(ade_ctx *c, int steps, cudaStream_t s)
 // from the second step on (two steps, us per step: 128^3 1241 against 1465, 1024^2 276 against 285,
 // 512^2 59 against 72, 256^2 23 against 38).  A single step stays with the walks (the cube's would
 // take 1.5 ms).
-bool use_frozen(const ade_ctx *c, int steps) { return c->frozen && steps >= 2; }
+bool use_frozen(const ade_ctx *c, int steps) { return c->frozen && c->frozen_fits && steps >= 2; }
 
 // Enqueue one predictor-corrector step (Eq. 8-9) and the fold of its diagnostics.
 int enqueue_step(ade_ctx *c, cudaStream_t s)
@@ -761,6 +812,7 @@ int plume_constants(const ade_params *p, int n, const Derived &d, double *D, dou
     const double u = p->box[0] / kTwo32;
     const double Hu = d.H / u;
     rp.H2 = (float)(Hu * Hu);
+    rp.Hg2 = (float)((d.Hgrid / u) * (d.Hgrid / u));
     for (int i = 0; i < 3; ++i) rp.u[i] = (i < p->dim ? p->box[i] : 1.0) / kTwo32;
     rp.H2d = d.H * d.H;
     rp.invH = (float)(1.0 / Hu);
@@ -774,6 +826,12 @@ int plume_constants(const ade_params *p, int n, const Derived &d, double *D, dou
     rp.m1 = -1;
     rp.variant = d.tiles.variant == 1 ? 1 : ((p->flags & ADE_FLAG_BRANCHED) ? 2 : 0);
     if (rp.variant != 1 && (p->flags & ADE_FLAG_TRIMMED)) rp.variant = rp.variant == 2 ? 4 : 3;  // trimmed rows
+    // The library's choice without autotuning: trimmed rows in 3D, and in 2D from about 100 neighbours on
+    // (us per step, full / trimmed: 128^3 4424 / 2298, 57^3 jittered 505 / 439, 2D 160^2 with 2,700
+    // neighbours 828 / 693, 1024^2 with 120 385 / 375; 300^2 jittered with 45 68 / 82).  The paired walks
+    // are left to the autotuner: on an irregular set they lose (57^3 980).
+    if (p->flags == 0u && !(p->vmax > 0.0) && *iso && (p->dim == 3 || expected_neighbours(*p, d.H, n) >= 100.0))
+        rp.variant = 3;
     if (p->flags & ADE_FLAG_PAIRED)                                                           // paired walks
         rp.variant = (p->flags & ADE_FLAG_BRANCHED) ? ((p->flags & ADE_FLAG_TRIMMED) ? 8 : 7)
                                                     : ((p->flags & ADE_FLAG_TRIMMED) ? 6 : 5);
@@ -801,10 +859,23 @@ void ade::frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots,
     *lines = *slots = 0;
     *blocks = 1;
     const bool fixed = c->p.cell_subdiv > 0 || c->p.flags != 0u;   // no autotuning: the grid in use
+    // (the same before and after autotuning: callers size a workspace with it; a grid that needs more has
+    // chunks evaluated from the positions)
+    Grid first;
+    size_t room = 0;
+    for (int k = 1; k <= ade::kMaxSubdiv && room == 0; ++k)
+        if ((!fixed || k == c->subdiv) && make_grid(c->p, c->Hgrid, k, &first)) {
+            Grid best = first;
+            for (int q = k; !fixed && q <= ade::kMaxSubdiv; ++q) {
+                Grid g;
+                if (make_grid(c->p, c->Hgrid, q, &g) && frozen_lines(c->p, c->H, c->n, g, val) < frozen_lines(c->p, c->H, c->n, best, val)) best = g;
+            }
+            room = frozen_room(c->p, c->Hgrid, c->H, c->n, best, fixed, val);
+        }
     for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
         Grid g;
         if ((fixed && k != c->subdiv) || !make_grid(c->p, c->Hgrid, k, &g)) continue;
-        *lines = std::max(*lines, frozen_lines(c->p, c->H, c->n, g, val));
+        *lines = std::max(*lines, std::min(room, frozen_lines(c->p, c->H, c->n, g, val)));
         *slots = std::max(*slots, frozen_slots(c->n, g));
         ade::RateParams rp;
         memset(&rp, 0, sizeof(rp));
@@ -921,6 +992,7 @@ int ade_init_particles(ade_ctx **out, const ade_params *p, int n, uint32_t *xq_d
     c->frozen_C = at<float>(workspace_dev, d.L.fz_C);
     c->frozen_tab.cursor = at<unsigned>(workspace_dev, d.L.fz_cursor);
     c->frozen_lines = d.fz_lines;
+    c->frozen_fits = true;
 
     rc = plume_constants(p, n, d, c->D, &c->dt, c->inc, c->inc_half, &c->rp, &c->iso);
     if (rc) {
@@ -1022,6 +1094,7 @@ int apply_config(ade_ctx *c, int k, int variant)
     for (int i = 0; i < 3; ++i) c->nc[i] = g.nc[i];
     c->ncells = g.ncells;
     c->subdiv = g.subdiv;
+    c->frozen_fits = frozen_lines(c->p, c->H, c->n, g) <= c->frozen_lines;
     ade::RateParams &rp = c->rp;
     rp.ncx = g.nc[0];
     rp.ncy = g.nc[1];
@@ -1304,11 +1377,11 @@ int ade_step(ade_ctx *c, int nsteps, void *stream)
 // Copies {sum C, min C, max C} from w.stats and the status word out (waits for the stream).
 static int read_stats(ade_ctx *c, ade_stats *st, cudaStream_t s)
 {
-    double h[3];
+    double h[kStatusAt / sizeof(double) + 1];
     int status = 0;
-    ADE_CK(cudaMemcpyAsync(h, c->w.stats, sizeof(h), cudaMemcpyDeviceToHost, s));
-    ADE_CK(cudaMemcpyAsync(&status, c->w.status, sizeof(int), cudaMemcpyDeviceToHost, s));
+    ADE_CK(cudaMemcpyAsync(h, c->w.stats, sizeof(h), cudaMemcpyDeviceToHost, s));   // the status word follows
     ADE_CK(cudaStreamSynchronize(s));
+    memcpy(&status, reinterpret_cast<const char *>(h) + kStatusAt, sizeof(status));
     st->mass = h[0] * c->p.mass;
     st->c_min = h[1];
     st->c_max = h[2];
@@ -1509,7 +1582,7 @@ struct ade_batch {
     cudaGraphExec_t graph_exec[ade::kGraphSteps + 1] = {};
     cudaStream_t cap_stream = nullptr;
     // weight table of multi-step calls (rate_frozen.cu)
-    bool frozen = false;
+    bool frozen = false, frozen_fits = false;   // frozen_fits: room for the grids in use
     ade::FrozenTab frozen_tab = {};
     ade::FrozenItem *d_items = nullptr;
     float *frozen_C = nullptr;
@@ -1535,12 +1608,18 @@ BatchFrozen batch_frozen_size(int P, const ade_params *p, const int *n)
     BatchFrozen f;
     for (int i = 0; i < P; ++i) {
         const double H = p[i].kernel == ADE_WENDLAND_C2 ? 2.0 * p[i].h : p[i].h;
-        size_t lines = 0, pencils = 0, items = 0;
+        size_t lines = 0, pencils = 0, items = 0, least = 0;
         for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
             Grid g;
             if (!make_grid(p[i], H, k, &g)) continue;
-            const size_t np = (size_t)(g.ncells / g.nc[0]);
-            lines = std::max(lines, frozen_lines(p[i], H, n[i], g));
+            const size_t l = frozen_lines(p[i], H, n[i], g);
+            least = least ? std::min(least, l) : l;
+        }
+        for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
+            Grid g;
+            if (!make_grid(p[i], H, k, &g)) continue;
+            const size_t np = (size_t)(g.ncells / g.nc[0]), l = frozen_lines(p[i], H, n[i], g);
+            if (l <= least + least / 5) lines = std::max(lines, l);   // (see frozen_room)
             pencils = std::max(pencils, np);
             items = std::max(items, np + (size_t)n[i] / 32);
         }
@@ -1647,6 +1726,7 @@ int batch_plan(ade_batch *b)
     b->items.clear();
     int p0 = 0;
     unsigned fz_line = 0u;
+    b->frozen_fits = true;
     std::vector<std::pair<double, ade::BatchTile>> items;
     for (int i = 0; i < b->P; ++i) {
         ade_params pp = b->params[i];
@@ -1668,6 +1748,7 @@ int batch_plan(ade_batch *b)
         rp.coff = b->NC;
         rp.frame = b->w.frame + (size_t)i * ade::kFrameWords;
         if (b->frozen) {   // the plume's chunks' regions, one plume behind the other; what is left is the pool
+            b->frozen_fits = b->frozen_fits && frozen_lines(pp, d.H, b->n[i], d.g) <= b->frozen_plume[i];
             rp.fz_base = fz_line;
             rp.fz_stride = frozen_stride(pp, d.H, b->n[i], d.g, 1, b->frozen_plume[i]);
             fz_line += (unsigned)(frozen_slots(b->n[i], d.g) * rp.fz_stride);
@@ -1806,7 +1887,7 @@ int batch_enqueue_frozen(ade_batch *b, int steps, cudaStream_t s)
 }
 
 // Whether `steps` steps of one call keep the pair weights.
-bool batch_use_frozen(const ade_batch *b, int steps) { return b->frozen && b->N > 0 && steps >= 2; }
+bool batch_use_frozen(const ade_batch *b, int steps) { return b->frozen && b->frozen_fits && b->N > 0 && steps >= 2; }
 
 int batch_enqueue_steps(ade_batch *b, int steps, cudaStream_t s)
 {

@@ -78,6 +78,20 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x, float
     lo = lo + (err + xlo);
 }
 
+// {hi, lo, min, max} of the warp's particles' new C (lane 0 holds it), by a fixed shuffle tree.
+__device__ __forceinline__ float4 warp_partial(const Acc &acc)
+{
+    float mn = acc.mn, mx = acc.mx, hi = acc.hi, lo = acc.lo;
+    for (int o = 16; o > 0; o >>= 1) {
+        mn = fminf(mn, __shfl_down_sync(0xffffffffu, mn, o));
+        mx = fmaxf(mx, __shfl_down_sync(0xffffffffu, mx, o));
+        const float h2 = __shfl_down_sync(0xffffffffu, hi, o);
+        const float l2 = __shfl_down_sync(0xffffffffu, lo, o);
+        two_sum_add(hi, lo, h2, l2);
+    }
+    return make_float4(hi, lo, mn, mx);
+}
+
 // Warp-wide part of the epilogue: pair count, and for the corrector one partial per warp
 // {hi, lo, min, max} of its particles' new C, folded by a fixed shuffle tree (error-free two-sum
 // for the sum, exact FP32 min and max).  No block barrier, fence or atomic: the grid-wide fold
@@ -92,14 +106,6 @@ __device__ __forceinline__ void warp_finish(Acc acc, const EpiOut &out)
         if ((threadIdx.x & 31) == 0 && c) atomicAdd(out.pairs, (unsigned long long)c);
     }
     if (EPI != EPI_CORRECT) return;
-    float mn = acc.mn, mx = acc.mx, hi = acc.hi, lo = acc.lo;
-    for (int o = 16; o > 0; o >>= 1) {
-        mn = fminf(mn, __shfl_down_sync(0xffffffffu, mn, o));
-        mx = fmaxf(mx, __shfl_down_sync(0xffffffffu, mx, o));
-        const float h2 = __shfl_down_sync(0xffffffffu, hi, o);
-        const float l2 = __shfl_down_sync(0xffffffffu, lo, o);
-        two_sum_add(hi, lo, h2, l2);
-    }
-    if ((threadIdx.x & 31) == 0)
-        out.wpart[(size_t)blockIdx.x * (NT / 32) + (threadIdx.x >> 5)] = make_float4(hi, lo, mn, mx);
+    const float4 r = warp_partial(acc);
+    if ((threadIdx.x & 31) == 0) out.wpart[(size_t)blockIdx.x * (NT / 32) + (threadIdx.x >> 5)] = r;
 }

@@ -25,6 +25,8 @@
 // minus hi); the pair's denominator is (hi_a + hi_b) + (lo_a + lo_b), whose first sum is exact when
 // the two cancel (Sterbenz), so K_ij keeps FP32 relative accuracy.  The lo words ride in the
 // otherwise unused fourth lanes of the float4 records, so the pair loop loads nothing extra.
+#include <algorithm>
+
 #include "ade_internal.h"
 
 namespace ade {
@@ -32,6 +34,10 @@ namespace ade {
 namespace {
 
 #include "rate_common.cuh"
+
+#include "rate_walk.cuh"
+
+#include "frozen_table.cuh"
 
 constexpr int kT = kRateThreads;
 
@@ -149,14 +155,110 @@ __global__ __launch_bounds__(kT) void k_field_permute(const uint32_t *__restrict
     Inc[i] = __ldg(IncC + a);
 }
 
-template <int DIM, int KERNEL, int EPI, bool COUNT>
-__global__ __launch_bounds__(kT) void k_rate_field(const uint4 *__restrict__ Pe, const uint32_t *__restrict__ cs,
+// Ordered in-support pairs (FP64 test), one thread per sorted particle over the full stencil.
+template <int DIM>
+__global__ __launch_bounds__(kT) void k_count_field(const uint4 *__restrict__ Pe, const uint32_t *__restrict__ cs,
+                                                    const RateParams prm, const EpiOut out)
+{
+    pdl_wait();
+    const int i = blockIdx.x * kT + threadIdx.x;
+    const bool valid = i < prm.n;
+    const uint4 pa = __ldg(Pe + (valid ? i : prm.n - 1));
+    const int ncx = prm.ncx, ncy = prm.ncy, ncz = prm.ncz;
+    const int cx = (int)__umulhi(pa.x, (uint32_t)ncx);
+    const int cy = (int)__umulhi(pa.y, (uint32_t)ncy);
+    const int cz = DIM == 3 ? (int)__umulhi(pa.z, (uint32_t)ncz) : 0;
+    unsigned cnt = 0u;
+    for (int ri = 0; ri < prm.nrows; ++ri) {
+        const StencilRow row = prm.rows[ri];
+        const int q = row_pencil_of<DIM>(row, cy, cz, prm);
+        int s0, e0, s1, e1;
+        row_ranges(cs, q * ncx, cx - (int)row.w, cx + row.w + 1, ncx, s0, e0, s1, e1);
+        for (int piece = 0; piece < 2; ++piece)
+            for (int j = piece ? s1 : s0; j < (piece ? e1 : e0); ++j) {
+                const uint4 pb = __ldg(Pe + j);
+                cnt += in_support_fp64<DIM>((int)(pa.x - pb.x), (int)(pa.y - pb.y), (int)(pa.z - pb.z), prm);
+            }
+    }
+    Acc acc{0.f, 0.f, 0.f, 0.f, valid ? cnt : 0u};
+    warp_finish<EPI_RATE, true, kT>(acc, out);
+}
+
+// One target's own records for the pair terms.
+template <int DIM>
+struct FieldTarget {
+    uint4 p;
+    float4 v, da, db, da4, db4;
+    float Ca;
+    __device__ __forceinline__ FieldTarget(const uint4 &p_, float Ca_, const float4 &v_, const float4 &da_, const float4 &db_)
+        : p(p_), v(v_), da(da_), db(db_), Ca(Ca_)
+    {
+        // 4 D (diagonal) and 8 D (off-diagonal) for the harmonic means (da.z is Dyy in 2D, Dxz in 3D)
+        da4 = make_float4(4.f * da.x, 8.f * da.y, (DIM == 2 ? 4.f : 8.f) * da.z, 0.f);
+        db4 = make_float4(4.f * db.x, 8.f * db.y, 4.f * db.z, 0.f);
+    }
+};
+
+template <int DIM>
+__device__ __forceinline__ float field_sep(const FieldTarget<DIM> &t, const uint4 &pb, const PairConst &k, float &dx, float &dy,
+                                           float &dz)
+{
+    dx = sep(t.p.x, pb.x, k.m1);
+    dy = sep(t.p.y, pb.y, k.m1) * k.sy;
+    dz = DIM == 3 ? sep(t.p.z, pb.z, k.m1) * k.sz : 0.f;
+    float r2 = fmaf(dx, dx, dy * dy);
+    if (DIM == 3) r2 = fmaf(dz, dz, r2);
+    return r2;
+}
+
+// Both terms of Eq. 4 for an in-support candidate j.
+template <int DIM, int KERNEL>
+__device__ __forceinline__ void field_pair(const FieldTarget<DIM> &t, const uint4 *__restrict__ Pe, const float4 *__restrict__ V,
+                                           const float4 *__restrict__ DA, const float4 *__restrict__ DB, unsigned j,
+                                           const PairConst &k, float gam, float &rd, float &rc)
+{
+    const uint4 pb = __ldg(Pe + j);
+    const float4 vb = __ldg(V + j), d1 = __ldg(DA + j);
+    float dx, dy, dz;
+    const float r2 = field_sep<DIM>(t, pb, k, dx, dy, dz);
+    const float rinv = rsqrt_ftz(r2);
+    const float f = shape<KERNEL>(fmaf(-(r2 * rinv), k.invH, 1.f));
+    const float kxx = hmean_diag(t.da.x, t.da4.x, d1.x), kxy2 = hmean_off2(t.da.y, t.da4.y, t.da.w, d1.y, d1.w);
+    float Q, tr;
+    if (DIM == 2) {
+        const float kyy = hmean_diag(t.da.z, t.da4.z, d1.z);
+        Q = fmaf(dx, fmaf(kxx, dx, kxy2 * dy), kyy * dy * dy);
+        tr = kxx + kyy;
+    } else {
+        const float4 d2 = __ldg(DB + j);
+        const float kxz2 = hmean_off2(t.da.z, t.da4.z, t.v.w, d1.z, vb.w);
+        const float kyy = hmean_diag(t.db.x, t.db4.x, d2.x);
+        const float kyz2 = hmean_off2(t.db.y, t.db4.y, t.db.w, d2.y, d2.w);
+        const float kzz = hmean_diag(t.db.z, t.db4.z, d2.z);
+        const float qx = fmaf(kxx, dx, fmaf(kxy2, dy, kxz2 * dz));
+        const float qy = fmaf(kyy, dy, kyz2 * dz);
+        Q = fmaf(dx, qx, fmaf(dy, qy, kzz * dz * dz));
+        tr = kxx + kyy + kzz;
+    }
+    const float s = fmaf(gam * Q, rinv * rinv, -tr);
+    rd = fmaf(f * s, t.Ca - __uint_as_float(pb.w), rd);
+    float dvx = fmaf(t.v.x - vb.x, dx, (t.v.y - vb.y) * dy);
+    if (DIM == 3) dvx = fmaf(t.v.z - vb.z, dz, dvx);
+    rc = fmaf(f, dvx, rc);
+}
+
+// 2D: one thread per sorted particle evaluates the in-support candidates of the full stencil as it meets
+// them (rows of ten and more candidates: the lists of the 3D kernel cost more than the lanes they keep busy,
+// 459 against 430 us on the 1024^2 rung).
+template <int KERNEL, int EPI>
+__global__ __launch_bounds__(kT) void k_rate_field2(const uint4 *__restrict__ Pe, const uint32_t *__restrict__ cs,
                                                    const uint32_t *__restrict__ perm,
                                                    const float4 *__restrict__ V, const float4 *__restrict__ DA,
                                                    const float4 *__restrict__ DB, const uint4 *__restrict__ Inc,
                                                    const RateParams prm, const FieldParams fp, const EpiOut out)
 {
     pdl_wait();   // no early trigger: see pdl_trigger
+    constexpr int DIM = 2;
     const int i = blockIdx.x * kT + threadIdx.x;
     const bool valid = i < prm.n;
     const int ii = valid ? i : prm.n - 1;
@@ -180,7 +282,6 @@ __global__ __launch_bounds__(kT) void k_rate_field(const uint4 *__restrict__ Pe,
     const float4 da4 = make_float4(4.f * da.x, 8.f * da.y, (DIM == 2 ? 4.f : 8.f) * da.z, 0.f);
     const float4 db4 = make_float4(4.f * db.x, 8.f * db.y, 4.f * db.z, 0.f);
     float sd = 0.f, cd = 0.f, sc = 0.f, cc = 0.f;
-    unsigned cnt = 0u;
     for (int ri = 0; ri < prm.nrows; ++ri) {
         const StencilRow row = prm.rows[ri];
         int yy = cy + row.dy;
@@ -216,15 +317,6 @@ __global__ __launch_bounds__(kT) void k_rate_field(const uint4 *__restrict__ Pe,
             for (int j = r0[piece]; j < r1[piece]; ++j) {
                 const uint4 pb = __ldg(Pe + j);
                 const int ix = (int)(pa.x - pb.x), iy = (int)(pa.y - pb.y), iz = (int)(pa.z - pb.z);
-                if (COUNT) {
-                    const double dxd = (double)ix * prm.u[0], dyd = (double)iy * prm.u[1];
-                    double r2d = __dadd_rn(__dmul_rn(dxd, dxd), __dmul_rn(dyd, dyd));
-                    if (DIM == 3) {
-                        const double dzd = (double)iz * prm.u[2];
-                        r2d = __dadd_rn(r2d, __dmul_rn(dzd, dzd));
-                    }
-                    cnt += (r2d > 0.0 && r2d < prm.H2d) ? 1u : 0u;
-                }
                 const float dx = (float)ix;
                 const float dy = (float)iy * sy;
                 const float dz = DIM == 3 ? (float)iz * sz : 0.f;
@@ -267,7 +359,7 @@ __global__ __launch_bounds__(kT) void k_rate_field(const uint4 *__restrict__ Pe,
     }
     const float rate = fmaf(prm.pf, sd + cd, fp.pconv * Ca * (sc + cc));
 
-    Acc acc{0.f, 0.f, __int_as_float(0x7f800000), __int_as_float(0xff800000), valid ? cnt : 0u};
+    Acc acc{0.f, 0.f, __int_as_float(0x7f800000), __int_as_float(0xff800000), 0u};
     if (valid) {
         if (EPI == EPI_RATE) {
             if (out.rate) {
@@ -304,39 +396,213 @@ __global__ __launch_bounds__(kT) void k_rate_field(const uint4 *__restrict__ Pe,
             acc.mx = fmaxf(acc.mx, Cn);
         }
     }
-    warp_finish<EPI, COUNT, kT>(acc, out);
+    warp_finish<EPI, false, kT>(acc, out);
 }
 
-template <int DIM, int KERNEL, bool COUNT>
-void launch_field_epi(int epi, int blocks, const uint4 *Pe, const uint32_t *cs, const uint32_t *perm,
-                      const FieldWork &fw, const RateParams &prm, const FieldParams &fp, const EpiOut &out,
-                      cudaStream_t s)
+// 3D: a warp takes chunks of up to 32 consecutive particles of one pencil (for_chunks), so its lanes share the
+// stencil rows; each lane's range of a row is cut by the distance its own cell position leaves to the
+// row's cell band, for the grid's radius H + dt vmax (positions of the build: the drift since cannot
+// bring a pair within H that was beyond it).  The candidates are only tested first, and those in support
+// noted in the lane's list in shared memory; full lists are evaluated together.  On an irregular set the
+// lanes' ranges of a row differ, and a warp that evaluated where it tested would spend the pair's 110
+// instructions on the longest lane's candidates, in support or not: 6.7 a pair on 45^3
+// jittered particles.  SPLIT 4 (sets that leave the chip idle): the block's four warps share a chunk, each
+// takes every fourth row, and warp 0 adds their sums in order.
+// Per evaluation: 45^3 jittered, 195 neighbours, 425 -> 235 us (at the grid of about two
+// particles per cell; 24^3 345 -> 105).
+constexpr int kList = 40;   // entries per lane (one flush is one FP32 partial sum)
+
+template <int KERNEL, int EPI, int SPLIT>
+__global__ __launch_bounds__(kT) void k_rate_field3(const uint4 *__restrict__ Pe, const uint32_t *__restrict__ cs,
+                                                   const uint32_t *__restrict__ perm,
+                                                   const float4 *__restrict__ V, const float4 *__restrict__ DA,
+                                                   const float4 *__restrict__ DB, const uint4 *__restrict__ Inc,
+                                                   const RateParams prm, const FieldParams fp, const EpiOut out)
 {
-    switch (epi) {
-    case EPI_RATE:
-        launch_pdl(k_rate_field<DIM, KERNEL, EPI_RATE, COUNT>, blocks, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.DB, fw.Inc, prm, fp, out);
-        break;
-    case EPI_PREDICT:
-        launch_pdl(k_rate_field<DIM, KERNEL, EPI_PREDICT, COUNT>, blocks, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.DB, fw.Inc, prm, fp, out);
-        break;
-    default:
-        launch_pdl(k_rate_field<DIM, KERNEL, EPI_CORRECT, COUNT>, blocks, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.DB, fw.Inc, prm, fp, out);
-        break;
+    constexpr int DIM = 3;
+    pdl_wait();   // no early trigger: see pdl_trigger
+    __shared__ float4 part[SPLIT > 1 ? kT : 1];
+    __shared__ unsigned lists[kT / 32][kList * 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int ncx = prm.ncx;
+    Acc acc{0.f, 0.f, __int_as_float(0x7f800000), __int_as_float(0xff800000), 0u};
+    const PairConst kc(prm);
+    unsigned *list = lists[wid] + lane;
+    TrimGeom g(prm);
+    g.Hm2 = prm.Hg2 * (1.f + 1.f / 2048.f);
+    const int v = SPLIT > 1 ? blockIdx.y : blockIdx.y * (kT / 32) + wid;
+    const int nv = SPLIT > 1 ? gridDim.y : gridDim.y * (kT / 32);
+    for_chunks(cs, prm, blockIdx.x, 0, v, nv, [&](const Chunk &c) {
+        const int i = c.i0 + lane;
+        const bool valid = i < c.pe;
+        const int ii = valid ? i : c.pe - 1;
+        const uint4 pa = __ldg(Pe + ii);
+        // fixed-point drift of this particle; the cell of the cell build is the evaluation position
+        // minus the drift since the build (the half step, in the corrector)
+        const uint4 ic = EPI == EPI_RATE ? make_uint4(0u, 0u, 0u, 0u) : __ldg(Inc + ii);
+        uint32_t back[3] = {0u, 0u, 0u};
+        if (EPI == EPI_CORRECT) half_drift(ic, back);
+        const FieldTarget<DIM> t(pa, __uint_as_float(pa.w), __ldg(V + ii), __ldg(DA + ii), DIM == 3 ? __ldg(DB + ii) : make_float4(0.f, 0.f, 0.f, 0.f));
+        const int cx = (int)__umulhi(pa.x - back[0], (uint32_t)ncx);
+        const float inv32 = 2.3283064365386963e-10f;   // 2^-32
+        const float fx = (float)((pa.x - back[0]) * (uint32_t)ncx) * inv32;
+        const float fy = (float)((pa.y - back[1]) * (uint32_t)prm.ncy) * inv32;
+        const float fz = DIM == 3 ? (float)((pa.z - back[2]) * (uint32_t)prm.ncz) * inv32 : 0.f;
+        float sd = 0.f, cd = 0.f, sc = 0.f, cc = 0.f;
+        int have = 0;
+        auto flush = [&]() {
+            float rd = 0.f, rc = 0.f;
+#pragma unroll 2
+            for (int e = 0; e < have; ++e) field_pair<DIM, KERNEL>(t, Pe, V, DA, DB, list[32 * e], kc, fp.gamma, rd, rc);
+            neumaier_add(sd, cd, rd);
+            neumaier_add(sc, cc, rc);
+            have = 0;
+        };
+        for (int ri = SPLIT > 1 ? wid : 0; ri < prm.nrows; ri += SPLIT) {
+            const StencilRow row = prm.rows[ri];
+            const TrimRow tr{(float)row.dy, (float)row.dz, 0, 0};
+            const float e2 = row_gap2<DIM>(make_float4(0.f, 1.f, 0.f, DIM == 3 ? 1.f : 0.f), tr, fy, fy, 0.f, fz, fz, 0.f, g);
+            const float d2 = fmaxf(g.Hm2 - e2, 0.f);
+            if (!__any_sync(kFull, e2 < g.Hm2)) continue;
+            const float xe = fmaf(d2 * rsqrt_ftz(fmaxf(d2, 1.f)), g.inv_wx, 1.f / 4096.f);
+            const int w = row.w;
+            const int q = row_pencil_of<DIM>(row, c.cy, c.cz, prm);
+            const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
+            int s, cnt;
+            cyclic_range(cs, q * ncx, cx + max(__float2int_rd(fx - xe), -w), cx + min(__float2int_rd(fx + xe), w) + 1, ncx, qs, qe,
+                         s, cnt);
+            if (!(e2 < g.Hm2)) cnt = 0;
+            for (int u = 0; __any_sync(kFull, u < cnt);) {
+                // up to the room every lane's list has
+                const int room = kList - (int)__reduce_max_sync(kFull, (unsigned)have);
+                const int end = min(cnt, u + room);
+                for (; u < end; ++u) {
+                    const int j = s + u, jj = j >= qe ? j - len : j;
+                    float dx, dy, dz;
+                    const float r2 = field_sep<DIM>(t, __ldg(Pe + jj), kc, dx, dy, dz);
+                    if (r2 < prm.H2 && r2 > 0.f) list[32 * have++] = (unsigned)jj;
+                }
+                if (room < kList / 4) flush();
+            }
+        }
+        flush();
+        if (SPLIT > 1) {
+            part[threadIdx.x] = make_float4(sd, cd, sc, cc);
+            __syncthreads();
+            if (wid == 0)
+                for (int q = 1; q < SPLIT; ++q) {
+                    const float4 o = part[32 * q + lane];
+                    neumaier_add(sd, cd, o.x);
+                    neumaier_add(sc, cc, o.z);
+                    cd += o.y;
+                    cc += o.w;
+                }
+            __syncthreads();
+            if (wid != 0) return;
+        }
+        if (!valid) return;
+        const float rate = fmaf(prm.pf, sd + cd, fp.pconv * t.Ca * (sc + cc));
+        if (EPI == EPI_RATE) {
+            if (out.rate) {
+                const uint32_t a = __ldg(perm + i);
+                if (a < (uint32_t)prm.n) out.rate[a] = rate;
+            }
+        } else if (EPI == EPI_PREDICT) {
+            // C^{l+1/2} = C^l + dt/2 r^l, x_a^{l+1/2} = x_a^l + dt/2 v_a
+            uint32_t inc[3];
+            half_drift(ic, inc);
+            uint4 o;
+            o.x = pa.x + inc[0];
+            o.y = pa.y + inc[1];
+            o.z = pa.z + inc[2];
+            o.w = __float_as_uint(fmaf(prm.dt, rate, t.Ca));
+            out.Pout[i] = o;
+        } else {
+            // C^{l+1} = C^l + dt r^{l+1/2}, x_a^{l+1} = x_a^l + dt v_a (caller order); x^l is the
+            // evaluation position minus this particle's half-step drift (exact in fixed point)
+            const uint32_t a = __ldg(perm + i);
+            uint32_t inc[3];
+            full_drift(ic, inc);
+            float Cn = 0.f;
+            if (a < (uint32_t)prm.n) {
+                Cn = fmaf(prm.dt, rate, out.C[a]);
+                out.C[a] = Cn;
+                out.xq[a] = pa.x - back[0] + inc[0];
+                out.xq[(size_t)prm.n + a] = pa.y - back[1] + inc[1];
+                if (DIM == 3) out.xq[2 * (size_t)prm.n + a] = pa.z - back[2] + inc[2];
+            }
+            if (!isfinite(Cn)) atomicOr(out.status, 1);
+            two_sum_add(acc.hi, acc.lo, Cn, 0.f);
+            acc.mn = fminf(acc.mn, Cn);
+            acc.mx = fmaxf(acc.mx, Cn);
+        }
+    });
+    if (EPI == EPI_CORRECT) {   // one partial per warp that took chunks (SPLIT: the block's first)
+        const float4 r = warp_partial(acc);
+        if (lane == 0 && (SPLIT == 1 || wid == 0)) {
+            const size_t blk = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
+            out.wpart[SPLIT == 1 ? blk * (kT / 32) + wid : blk] = r;
+        }
     }
 }
 
-template <int DIM, int KERNEL>
-void launch_field_count(bool count, int epi, int blocks, const uint4 *Pe, const uint32_t *cs,
-                        const uint32_t *perm, const FieldWork &fw, const RateParams &prm,
-                        const FieldParams &fp, const EpiOut &out, cudaStream_t s)
+template <int KERNEL, int SPLIT>
+cudaError_t launch_field3(int epi, dim3 grid, const uint4 *Pe, const uint32_t *cs, const uint32_t *perm,
+                          const FieldWork &fw, const RateParams &prm, const FieldParams &fp, const EpiOut &out,
+                          cudaStream_t s)
 {
-    if (count)
-        launch_field_epi<DIM, KERNEL, true>(epi, blocks, Pe, cs, perm, fw, prm, fp, out, s);
-    else
-        launch_field_epi<DIM, KERNEL, false>(epi, blocks, Pe, cs, perm, fw, prm, fp, out, s);
+    switch (epi) {
+    case EPI_RATE:
+        return launch_pdl(k_rate_field3<KERNEL, EPI_RATE, SPLIT>, grid, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.DB, fw.Inc, prm, fp, out);
+    case EPI_PREDICT:
+        return launch_pdl(k_rate_field3<KERNEL, EPI_PREDICT, SPLIT>, grid, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.DB, fw.Inc, prm, fp, out);
+    default:
+        return launch_pdl(k_rate_field3<KERNEL, EPI_CORRECT, SPLIT>, grid, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.DB, fw.Inc, prm, fp, out);
+    }
+}
+
+template <int KERNEL>
+cudaError_t launch_field2(int epi, const uint4 *Pe, const uint32_t *cs, const uint32_t *perm, const FieldWork &fw,
+                          const RateParams &prm, const FieldParams &fp, const EpiOut &out, cudaStream_t s)
+{
+    const unsigned g = (unsigned)((prm.n + kT - 1) / kT);
+    switch (epi) {
+    case EPI_RATE:
+        return launch_pdl(k_rate_field2<KERNEL, EPI_RATE>, g, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.DB, fw.Inc, prm, fp, out);
+    case EPI_PREDICT:
+        return launch_pdl(k_rate_field2<KERNEL, EPI_PREDICT>, g, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.DB, fw.Inc, prm, fp, out);
+    default:
+        return launch_pdl(k_rate_field2<KERNEL, EPI_CORRECT>, g, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.DB, fw.Inc, prm, fp, out);
+    }
+}
+
+// Chunks of a set that fills the chip less than about twice (152 SMs of 24 warps) are shared by the four
+// warps of a block.
+bool field_split(const RateParams &prm) { return prm.n / 32 < 2 * 152 * 24; }
+unsigned field_split_y(const RateParams &prm)   // a block per chunk of the mean pencil
+{
+    return (unsigned)std::max(1, (prm.n / (prm.ncy * prm.ncz) + 31) / 32);
+}
+
+template <int KERNEL>
+cudaError_t launch_field_k(int dim, int epi, const uint4 *Pe, const uint32_t *cs, const uint32_t *perm, const FieldWork &fw,
+                    const RateParams &prm, const FieldParams &fp, const EpiOut &out, cudaStream_t s)
+{
+    if (dim == 2) return launch_field2<KERNEL>(epi, Pe, cs, perm, fw, prm, fp, out, s);
+    dim3 g = frozen_grid(prm);
+    if (!field_split(prm)) return launch_field3<KERNEL, 1>(epi, g, Pe, cs, perm, fw, prm, fp, out, s);
+    g.y = field_split_y(prm);
+    return launch_field3<KERNEL, 4>(epi, g, Pe, cs, perm, fw, prm, fp, out, s);
 }
 
 }  // namespace
+
+int field_partials(int dim, const RateParams &prm)
+{
+    if (dim == 2) return (prm.n + kT - 1) / kT * (kT / 32);
+    const dim3 g = frozen_grid(prm);
+    return field_split(prm) ? (int)(g.x * field_split_y(prm)) : (int)(g.x * g.y) * (kT / 32);
+}
 
 cudaError_t launch_field_records(int dim, const float *v_dev, int n, const FieldParams &fp, const FieldWork &fw,
                                  cudaStream_t s)
@@ -373,20 +639,13 @@ cudaError_t launch_rate_field(int dim, int kernel, int epi, const uint4 *Pe, con
                               const FieldParams &fp, const EpiOut &out, cudaStream_t s)
 {
     if (prm.n == 0) return cudaSuccess;
-    const int blocks = (prm.n + kT - 1) / kT;
-    const bool count = out.pairs != nullptr;
-    if (dim == 2) {
-        if (kernel == ADE_WENDLAND_C2)
-            launch_field_count<2, ADE_WENDLAND_C2>(count, epi, blocks, Pe, cell_start, perm, fw, prm, fp, out, s);
-        else
-            launch_field_count<2, ADE_WENDLAND_C4>(count, epi, blocks, Pe, cell_start, perm, fw, prm, fp, out, s);
-    } else {
-        if (kernel == ADE_WENDLAND_C2)
-            launch_field_count<3, ADE_WENDLAND_C2>(count, epi, blocks, Pe, cell_start, perm, fw, prm, fp, out, s);
-        else
-            launch_field_count<3, ADE_WENDLAND_C4>(count, epi, blocks, Pe, cell_start, perm, fw, prm, fp, out, s);
+    if (out.pairs) {
+        const unsigned blocks = (unsigned)((prm.n + kT - 1) / kT);
+        return dim == 2 ? launch_pdl(k_count_field<2>, blocks, kT, 0, s, Pe, cell_start, prm, out)
+                        : launch_pdl(k_count_field<3>, blocks, kT, 0, s, Pe, cell_start, prm, out);
     }
-    return cudaGetLastError();
+    return kernel == ADE_WENDLAND_C2 ? launch_field_k<ADE_WENDLAND_C2>(dim, epi, Pe, cell_start, perm, fw, prm, fp, out, s)
+                                     : launch_field_k<ADE_WENDLAND_C4>(dim, epi, Pe, cell_start, perm, fw, prm, fp, out, s);
 }
 
 }  // namespace ade
