@@ -184,8 +184,7 @@ __global__ __launch_bounds__(kT) void k_count_field(const uint4 *__restrict__ Pe
     warp_finish<EPI_RATE, true, kT>(acc, out);
 }
 
-// One target's own records for the pair terms.
-template <int DIM>
+// 3D: one target's own records for the pair terms.
 struct FieldTarget {
     uint4 p;
     float4 v, da, db, da4, db4;
@@ -193,57 +192,46 @@ struct FieldTarget {
     __device__ __forceinline__ FieldTarget(const uint4 &p_, float Ca_, const float4 &v_, const float4 &da_, const float4 &db_)
         : p(p_), v(v_), da(da_), db(db_), Ca(Ca_)
     {
-        // 4 D (diagonal) and 8 D (off-diagonal) for the harmonic means (da.z is Dyy in 2D, Dxz in 3D)
-        da4 = make_float4(4.f * da.x, 8.f * da.y, (DIM == 2 ? 4.f : 8.f) * da.z, 0.f);
+        // 4 D (diagonal) and 8 D (off-diagonal) for the harmonic means
+        da4 = make_float4(4.f * da.x, 8.f * da.y, 8.f * da.z, 0.f);
         db4 = make_float4(4.f * db.x, 8.f * db.y, 4.f * db.z, 0.f);
     }
 };
 
-template <int DIM>
-__device__ __forceinline__ float field_sep(const FieldTarget<DIM> &t, const uint4 &pb, const PairConst &k, float &dx, float &dy,
+__device__ __forceinline__ float field_sep(const FieldTarget &t, const uint4 &pb, const PairConst &k, float &dx, float &dy,
                                            float &dz)
 {
     dx = sep(t.p.x, pb.x, k.m1);
     dy = sep(t.p.y, pb.y, k.m1) * k.sy;
-    dz = DIM == 3 ? sep(t.p.z, pb.z, k.m1) * k.sz : 0.f;
-    float r2 = fmaf(dx, dx, dy * dy);
-    if (DIM == 3) r2 = fmaf(dz, dz, r2);
-    return r2;
+    dz = sep(t.p.z, pb.z, k.m1) * k.sz;
+    return fmaf(dz, dz, fmaf(dx, dx, dy * dy));
 }
 
 // Both terms of Eq. 4 for an in-support candidate j.
-template <int DIM, int KERNEL>
-__device__ __forceinline__ void field_pair(const FieldTarget<DIM> &t, const uint4 *__restrict__ Pe, const float4 *__restrict__ V,
+template <int KERNEL>
+__device__ __forceinline__ void field_pair(const FieldTarget &t, const uint4 *__restrict__ Pe, const float4 *__restrict__ V,
                                            const float4 *__restrict__ DA, const float4 *__restrict__ DB, unsigned j,
                                            const PairConst &k, float gam, float &rd, float &rc)
 {
     const uint4 pb = __ldg(Pe + j);
     const float4 vb = __ldg(V + j), d1 = __ldg(DA + j);
     float dx, dy, dz;
-    const float r2 = field_sep<DIM>(t, pb, k, dx, dy, dz);
+    const float r2 = field_sep(t, pb, k, dx, dy, dz);
     const float rinv = rsqrt_ftz(r2);
     const float f = shape<KERNEL>(fmaf(-(r2 * rinv), k.invH, 1.f));
     const float kxx = hmean_diag(t.da.x, t.da4.x, d1.x), kxy2 = hmean_off2(t.da.y, t.da4.y, t.da.w, d1.y, d1.w);
-    float Q, tr;
-    if (DIM == 2) {
-        const float kyy = hmean_diag(t.da.z, t.da4.z, d1.z);
-        Q = fmaf(dx, fmaf(kxx, dx, kxy2 * dy), kyy * dy * dy);
-        tr = kxx + kyy;
-    } else {
-        const float4 d2 = __ldg(DB + j);
-        const float kxz2 = hmean_off2(t.da.z, t.da4.z, t.v.w, d1.z, vb.w);
-        const float kyy = hmean_diag(t.db.x, t.db4.x, d2.x);
-        const float kyz2 = hmean_off2(t.db.y, t.db4.y, t.db.w, d2.y, d2.w);
-        const float kzz = hmean_diag(t.db.z, t.db4.z, d2.z);
-        const float qx = fmaf(kxx, dx, fmaf(kxy2, dy, kxz2 * dz));
-        const float qy = fmaf(kyy, dy, kyz2 * dz);
-        Q = fmaf(dx, qx, fmaf(dy, qy, kzz * dz * dz));
-        tr = kxx + kyy + kzz;
-    }
+    const float4 d2 = __ldg(DB + j);
+    const float kxz2 = hmean_off2(t.da.z, t.da4.z, t.v.w, d1.z, vb.w);
+    const float kyy = hmean_diag(t.db.x, t.db4.x, d2.x);
+    const float kyz2 = hmean_off2(t.db.y, t.db4.y, t.db.w, d2.y, d2.w);
+    const float kzz = hmean_diag(t.db.z, t.db4.z, d2.z);
+    const float qx = fmaf(kxx, dx, fmaf(kxy2, dy, kxz2 * dz));
+    const float qy = fmaf(kyy, dy, kyz2 * dz);
+    const float Q = fmaf(dx, qx, fmaf(dy, qy, kzz * dz * dz));
+    const float tr = kxx + kyy + kzz;
     const float s = fmaf(gam * Q, rinv * rinv, -tr);
     rd = fmaf(f * s, t.Ca - __uint_as_float(pb.w), rd);
-    float dvx = fmaf(t.v.x - vb.x, dx, (t.v.y - vb.y) * dy);
-    if (DIM == 3) dvx = fmaf(t.v.z - vb.z, dz, dvx);
+    const float dvx = fmaf(t.v.z - vb.z, dz, fmaf(t.v.x - vb.x, dx, (t.v.y - vb.y) * dy));
     rc = fmaf(f, dvx, rc);
 }
 
@@ -254,46 +242,34 @@ template <int KERNEL, int EPI>
 __global__ __launch_bounds__(kT) void k_rate_field2(const uint4 *__restrict__ Pe, const uint32_t *__restrict__ cs,
                                                    const uint32_t *__restrict__ perm,
                                                    const float4 *__restrict__ V, const float4 *__restrict__ DA,
-                                                   const float4 *__restrict__ DB, const uint4 *__restrict__ Inc,
-                                                   const RateParams prm, const FieldParams fp, const EpiOut out)
+                                                   const uint4 *__restrict__ Inc, const RateParams prm, const FieldParams fp, const EpiOut out)
 {
     pdl_wait();   // no early trigger: see pdl_trigger
-    constexpr int DIM = 2;
     const int i = blockIdx.x * kT + threadIdx.x;
     const bool valid = i < prm.n;
     const int ii = valid ? i : prm.n - 1;
     const uint4 pa = __ldg(Pe + ii);
     const float4 va = __ldg(V + ii);
     const float4 da = __ldg(DA + ii);
-    const float4 db = DIM == 3 ? __ldg(DB + ii) : make_float4(0.f, 0.f, 0.f, 0.f);
     // fixed-point drift of this particle; the cell of the cell build is the evaluation position
     // minus the drift since the build (the half step, in the corrector)
     const uint4 ic = EPI == EPI_RATE ? make_uint4(0u, 0u, 0u, 0u) : __ldg(Inc + ii);
     uint32_t back[3] = {0u, 0u, 0u};
     if (EPI == EPI_CORRECT) half_drift(ic, back);
-    const int ncx = prm.ncx, ncy = prm.ncy, ncz = prm.ncz;
+    const int ncx = prm.ncx, ncy = prm.ncy;
     const int cx = (int)__umulhi(pa.x - back[0], (uint32_t)ncx);
     const int cy = (int)__umulhi(pa.y - back[1], (uint32_t)ncy);
-    const int cz = DIM == 3 ? (int)__umulhi(pa.z - back[2], (uint32_t)ncz) : 0;
     const float Ca = __uint_as_float(pa.w);
-    const float H2 = prm.H2, invH = prm.invH, sy = prm.sy, sz = prm.sz, gam = fp.gamma;
+    const float H2 = prm.H2, invH = prm.invH, sy = prm.sy, gam = fp.gamma;
     // 4 D (diagonal) and 8 D (off-diagonal) of this particle for the harmonic means
-    // (da.z is Dyy in 2D, Dxz in 3D)
-    const float4 da4 = make_float4(4.f * da.x, 8.f * da.y, (DIM == 2 ? 4.f : 8.f) * da.z, 0.f);
-    const float4 db4 = make_float4(4.f * db.x, 8.f * db.y, 4.f * db.z, 0.f);
+    const float4 da4 = make_float4(4.f * da.x, 8.f * da.y, 4.f * da.z, 0.f);
     float sd = 0.f, cd = 0.f, sc = 0.f, cc = 0.f;
     for (int ri = 0; ri < prm.nrows; ++ri) {
         const StencilRow row = prm.rows[ri];
         int yy = cy + row.dy;
         yy += (yy < 0) ? ncy : 0;
         yy -= (yy >= ncy) ? ncy : 0;
-        int zz = 0;
-        if (DIM == 3) {
-            zz = cz + row.dz;
-            zz += (zz < 0) ? ncz : 0;
-            zz -= (zz >= ncz) ? ncz : 0;
-        }
-        const int base = (zz * ncy + yy) * ncx;
+        const int base = yy * ncx;
         const int lo = cx - row.w, hi = cx + row.w + 1;
         int r0[2], r1[2];
         if (lo < 0) {
@@ -316,42 +292,22 @@ __global__ __launch_bounds__(kT) void k_rate_field2(const uint4 *__restrict__ Pe
 #pragma unroll 4
             for (int j = r0[piece]; j < r1[piece]; ++j) {
                 const uint4 pb = __ldg(Pe + j);
-                const int ix = (int)(pa.x - pb.x), iy = (int)(pa.y - pb.y), iz = (int)(pa.z - pb.z);
+                const int ix = (int)(pa.x - pb.x), iy = (int)(pa.y - pb.y);
                 const float dx = (float)ix;
                 const float dy = (float)iy * sy;
-                const float dz = DIM == 3 ? (float)iz * sz : 0.f;
-                float r2 = fmaf(dx, dx, dy * dy);
-                if (DIM == 3) r2 = fmaf(dz, dz, r2);
+                const float r2 = fmaf(dx, dx, dy * dy);
                 if (r2 < H2 && r2 > 0.f) {
                     const float rinv = rsqrtf(r2);
                     const float f = shape<KERNEL>(fmaf(-(r2 * rinv), invH, 1.f));
                     const float4 vb = __ldg(V + j);
                     const float4 d1 = __ldg(DA + j);
-                    float Q, tr;
-                    if (DIM == 2) {
-                        const float kxx = hmean_diag(da.x, da4.x, d1.x);
-                        const float kxy2 = hmean_off2(da.y, da4.y, da.w, d1.y, d1.w);
-                        const float kyy = hmean_diag(da.z, da4.z, d1.z);
-                        Q = fmaf(dx, fmaf(kxx, dx, kxy2 * dy), kyy * dy * dy);
-                        tr = kxx + kyy;
-                    } else {
-                        const float4 d2 = __ldg(DB + j);
-                        const float kxx = hmean_diag(da.x, da4.x, d1.x);
-                        const float kxy2 = hmean_off2(da.y, da4.y, da.w, d1.y, d1.w);
-                        const float kxz2 = hmean_off2(da.z, da4.z, va.w, d1.z, vb.w);
-                        const float kyy = hmean_diag(db.x, db4.x, d2.x);
-                        const float kyz2 = hmean_off2(db.y, db4.y, db.w, d2.y, d2.w);
-                        const float kzz = hmean_diag(db.z, db4.z, d2.z);
-                        const float qx = fmaf(kxx, dx, fmaf(kxy2, dy, kxz2 * dz));
-                        const float qy = fmaf(kyy, dy, kyz2 * dz);
-                        Q = fmaf(dx, qx, fmaf(dy, qy, kzz * dz * dz));
-                        tr = kxx + kyy + kzz;
-                    }
-                    const float s = fmaf(gam * Q, rinv * rinv, -tr);
+                    const float kxx = hmean_diag(da.x, da4.x, d1.x);
+                    const float kxy2 = hmean_off2(da.y, da4.y, da.w, d1.y, d1.w);
+                    const float kyy = hmean_diag(da.z, da4.z, d1.z);
+                    const float Q = fmaf(dx, fmaf(kxx, dx, kxy2 * dy), kyy * dy * dy);
+                    const float s = fmaf(gam * Q, rinv * rinv, -(kxx + kyy));
                     rd = fmaf(f * s, Ca - __uint_as_float(pb.w), rd);
-                    float dvx = fmaf(va.x - vb.x, dx, (va.y - vb.y) * dy);
-                    if (DIM == 3) dvx = fmaf(va.z - vb.z, dz, dvx);
-                    rc = fmaf(f, dvx, rc);
+                    rc = fmaf(f, fmaf(va.x - vb.x, dx, (va.y - vb.y) * dy), rc);
                 }
             }
         neumaier_add(sd, cd, rd);
@@ -388,7 +344,6 @@ __global__ __launch_bounds__(kT) void k_rate_field2(const uint4 *__restrict__ Pe
                 out.C[a] = Cn;
                 out.xq[a] = pa.x - back[0] + inc[0];
                 out.xq[(size_t)prm.n + a] = pa.y - back[1] + inc[1];
-                if (DIM == 3) out.xq[2 * (size_t)prm.n + a] = pa.z - back[2] + inc[2];
             }
             if (!isfinite(Cn)) atomicOr(out.status, 1);
             two_sum_add(acc.hi, acc.lo, Cn, 0.f);
@@ -442,18 +397,18 @@ __global__ __launch_bounds__(kT) void k_rate_field3(const uint4 *__restrict__ Pe
         const uint4 ic = EPI == EPI_RATE ? make_uint4(0u, 0u, 0u, 0u) : __ldg(Inc + ii);
         uint32_t back[3] = {0u, 0u, 0u};
         if (EPI == EPI_CORRECT) half_drift(ic, back);
-        const FieldTarget<DIM> t(pa, __uint_as_float(pa.w), __ldg(V + ii), __ldg(DA + ii), DIM == 3 ? __ldg(DB + ii) : make_float4(0.f, 0.f, 0.f, 0.f));
+        const FieldTarget t(pa, __uint_as_float(pa.w), __ldg(V + ii), __ldg(DA + ii), __ldg(DB + ii));
         const int cx = (int)__umulhi(pa.x - back[0], (uint32_t)ncx);
         const float inv32 = 2.3283064365386963e-10f;   // 2^-32
         const float fx = (float)((pa.x - back[0]) * (uint32_t)ncx) * inv32;
         const float fy = (float)((pa.y - back[1]) * (uint32_t)prm.ncy) * inv32;
-        const float fz = DIM == 3 ? (float)((pa.z - back[2]) * (uint32_t)prm.ncz) * inv32 : 0.f;
+        const float fz = (float)((pa.z - back[2]) * (uint32_t)prm.ncz) * inv32;
         float sd = 0.f, cd = 0.f, sc = 0.f, cc = 0.f;
         int have = 0;
         auto flush = [&]() {
             float rd = 0.f, rc = 0.f;
 #pragma unroll 2
-            for (int e = 0; e < have; ++e) field_pair<DIM, KERNEL>(t, Pe, V, DA, DB, list[32 * e], kc, fp.gamma, rd, rc);
+            for (int e = 0; e < have; ++e) field_pair<KERNEL>(t, Pe, V, DA, DB, list[32 * e], kc, fp.gamma, rd, rc);
             neumaier_add(sd, cd, rd);
             neumaier_add(sc, cc, rc);
             have = 0;
@@ -461,7 +416,7 @@ __global__ __launch_bounds__(kT) void k_rate_field3(const uint4 *__restrict__ Pe
         for (int ri = SPLIT > 1 ? wid : 0; ri < prm.nrows; ri += SPLIT) {
             const StencilRow row = prm.rows[ri];
             const TrimRow tr{(float)row.dy, (float)row.dz, 0, 0};
-            const float e2 = row_gap2<DIM>(make_float4(0.f, 1.f, 0.f, DIM == 3 ? 1.f : 0.f), tr, fy, fy, 0.f, fz, fz, 0.f, g);
+            const float e2 = row_gap2<DIM>(make_float4(0.f, 1.f, 0.f, 1.f), tr, fy, fy, 0.f, fz, fz, 0.f, g);
             const float d2 = fmaxf(g.Hm2 - e2, 0.f);
             if (!__any_sync(kFull, e2 < g.Hm2)) continue;
             const float xe = fmaf(d2 * rsqrt_ftz(fmaxf(d2, 1.f)), g.inv_wx, 1.f / 4096.f);
@@ -479,7 +434,7 @@ __global__ __launch_bounds__(kT) void k_rate_field3(const uint4 *__restrict__ Pe
                 for (; u < end; ++u) {
                     const int j = s + u, jj = j >= qe ? j - len : j;
                     float dx, dy, dz;
-                    const float r2 = field_sep<DIM>(t, __ldg(Pe + jj), kc, dx, dy, dz);
+                    const float r2 = field_sep(t, __ldg(Pe + jj), kc, dx, dy, dz);
                     if (r2 < prm.H2 && r2 > 0.f) list[32 * have++] = (unsigned)jj;
                 }
                 if (room < kList / 4) flush();
@@ -529,7 +484,7 @@ __global__ __launch_bounds__(kT) void k_rate_field3(const uint4 *__restrict__ Pe
                 out.C[a] = Cn;
                 out.xq[a] = pa.x - back[0] + inc[0];
                 out.xq[(size_t)prm.n + a] = pa.y - back[1] + inc[1];
-                if (DIM == 3) out.xq[2 * (size_t)prm.n + a] = pa.z - back[2] + inc[2];
+                out.xq[2 * (size_t)prm.n + a] = pa.z - back[2] + inc[2];
             }
             if (!isfinite(Cn)) atomicOr(out.status, 1);
             two_sum_add(acc.hi, acc.lo, Cn, 0.f);
@@ -568,11 +523,11 @@ cudaError_t launch_field2(int epi, const uint4 *Pe, const uint32_t *cs, const ui
     const unsigned g = (unsigned)((prm.n + kT - 1) / kT);
     switch (epi) {
     case EPI_RATE:
-        return launch_pdl(k_rate_field2<KERNEL, EPI_RATE>, g, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.DB, fw.Inc, prm, fp, out);
+        return launch_pdl(k_rate_field2<KERNEL, EPI_RATE>, g, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.Inc, prm, fp, out);
     case EPI_PREDICT:
-        return launch_pdl(k_rate_field2<KERNEL, EPI_PREDICT>, g, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.DB, fw.Inc, prm, fp, out);
+        return launch_pdl(k_rate_field2<KERNEL, EPI_PREDICT>, g, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.Inc, prm, fp, out);
     default:
-        return launch_pdl(k_rate_field2<KERNEL, EPI_CORRECT>, g, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.DB, fw.Inc, prm, fp, out);
+        return launch_pdl(k_rate_field2<KERNEL, EPI_CORRECT>, g, kT, 0, s, Pe, cs, perm, fw.V, fw.DA, fw.Inc, prm, fp, out);
     }
 }
 
