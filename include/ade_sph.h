@@ -86,7 +86,9 @@ typedef struct ade_params {
     int dt_rule;       /* ADE_DT_LAMBDA_MAX or ADE_DT_TRACE */
     double dt_coef;    /* coefficient of the rule; <= 0 selects 0.1 (Eq. 10) */
     int cell_subdiv;   /* cells per support radius along each axis, 1..6; 0 = automatic */
-    unsigned flags;    /* 0 (library's choice), ADE_FLAG_DIRECT, ADE_FLAG_TILED, ADE_FLAG_BRANCHED,
+    unsigned flags;    /* 0 (library's choice: without ade_autotune the branch-free walk over trimmed rows
+                          in 3D and from 100 expected neighbours on, over full rows otherwise; kept pair
+                          weights in calls of several steps), ADE_FLAG_DIRECT, ADE_FLAG_TILED, ADE_FLAG_BRANCHED,
                           or ADE_FLAG_TRIMMED alone or with DIRECT or BRANCHED */
     double vmax;       /* 0: uniform velocity v.  > 0: velocity-field mode -- each particle carries
                           its own constant velocity (ade_set_velocity_field), |v_a| <= vmax; v is
@@ -121,7 +123,7 @@ typedef struct ade_info {
     int sort_passes;  /* radix-sort passes per cell build */
     int variant;      /* interaction kernel: 0 direct walk (branch-free), 1 shared-memory tiles,
                          2 direct walk branching on the support test, 3 and 4 the two direct
-                         walks with per-particle trimmed rows */
+                         walks with per-particle trimmed rows, 5 to 8 their paired forms */
     int tile[3];      /* target cells per tile (tiled variant) */
     int tile_capacity;/* staged particles per tile (tiled variant) */
     size_t workspace_bytes;

@@ -192,7 +192,6 @@ struct SweepRun {
     const uint32_t *cs, *perm;
     FrozenTab tab;
     float *C, *Ch;
-    float4 lo;                    // low parts of vhat and 1/H
     float g2, bT;                 // 2 Gamma, 2 (Gamma - d) + 2
 };
 

@@ -105,7 +105,8 @@ __device__ __noinline__ void walk_sums(const uint4 *__restrict__ P, const uint32
     const uint4 pa = __ldg(P + min(c.i0 + (int)(threadIdx.x & 31), c.pe - 1));
     const int ncx = prm.ncx;
     const int cx = (int)__umulhi(pa.x - frame_x(prm), (uint32_t)ncx);
-    const PairConst k(prm);
+    const PairConst kc(prm);
+    const PairConst2 k(kc, kc.m1);
     for (int r = 0; r < prm.nrows; ++r) {
         const StencilRow row = prm.rows[r];
         const int q = row_pencil_of<DIM>(row, c.cy, c.cz, prm);
@@ -115,7 +116,7 @@ __device__ __noinline__ void walk_sums(const uint4 *__restrict__ P, const uint32
         for (int t = 0; t < cnt; ++t) {
             int j = s + t;
             j = j >= qe ? j - len : j;
-            const float2 w = pair_shape<DIM, KERNEL, ISO>(pa, __ldg(P + j), k, sc);
+            const float2 w = pair_shape<DIM, KERNEL, ISO, true>(pa, __ldg(P + j), k, sc);
 #pragma unroll
             for (int f = 0; f < NR; ++f) op.add(f, w, op.x[f][qs + j]);
         }
@@ -134,7 +135,7 @@ __global__ __launch_bounds__(kT) void k_adj_table(const uint4 *__restrict__ P, c
     for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), gridDim.y * (kT / 32), [&](const Chunk &c) {
         const int i = c.i0 + (threadIdx.x & 31);
         const uint4 pa = __ldg(P + min(i, c.pe - 1));
-        build_chunk<DIM, KERNEL, ISO, ISO ? kCutBox : kCutFull, 2>(P, cs, prm, c, pa, srow, tab, sc);
+        build_chunk<DIM, KERNEL, ISO, ISO ? kCutBox : kCutFull, 2, true>(P, cs, prm, c, pa, srow, tab, sc);
         if (i < c.pe) C0[c.ps + i] = C0[c.pe + i] = __uint_as_float(pa.w);
     });
 }

@@ -2654,16 +2654,8 @@ int ade_sweep_init(ade_sweep **out, const ade_params *p, int n, int ntheta, cons
     for (int i = 0; i < 3; ++i) base.vh[i] = vabs > 0.0 ? (float)(i < dm ? pp.v[i] / vabs : 0.0) : (i == 0 ? 1.f : 0.f);
     for (int i = 0; i < 3; ++i) sw->rp.uw[i] = base.vh[i];   // the table's weights take u = (vhat . e)^2
     sw->rp.ub = 0.f;
-    {
-        float lo[3];
-        for (int i = 0; i < 3; ++i) {
-            const double vh = vabs > 0.0 ? (i < dm ? pp.v[i] / vabs : 0.0) : (i == 0 ? 1.0 : 0.0);
-            lo[i] = (float)(vh - (double)base.vh[i]);
-        }
-        sw->run.lo = make_float4(lo[0], lo[1], lo[2], (float)(pp.box[0] / kTwo32 / L.d.H - (double)sw->rp.invH));
-        sw->run.g2 = (float)(2.0 * gamma);
-        sw->run.bT = (float)(2.0 * (gamma - dm) + 2.0);
-    }
+    sw->run.g2 = (float)(2.0 * gamma);
+    sw->run.bT = (float)(2.0 * (gamma - dm) + 2.0);
     for (int g0 = 0; g0 < ntheta;) {
         int nt = ade::kSweepGroup;
         while (nt > ntheta - g0) nt >>= 1;

@@ -51,41 +51,46 @@ __device__ __forceinline__ float pair_weight(const uint4 &pa, const uint4 &pb, c
 // The pair's weights for D = vhat vhat^T and D = I - vhat vhat^T (Eq. 3-5 with K = 2D),
 //   g_L = f (2 Gamma u - 2),  g_T = f (-2 Gamma u + 2 (Gamma - d) + 2),  u = (vhat . e)^2,
 // from which every uniform tensor's weight is (alpha_L |v| + D_m) g_L + (alpha_T |v| + D_m) g_T (sums of
-// f and f u would cancel in that).  Both 0 outside the support and at zero separation.  Computed once per
-// call, so 1/r takes a Newton step, and r, 1/H and vhat (sc.lo: low parts {vhat, 1/H}) are taken to twice
-// FP32: on a lattice the same few separations recur, and their rounding would bias every pair alike.
+// f and f u would cancel in that).  Both 0 outside the support and at zero separation.  FINE (the adjoint):
+// 1/r takes a Newton step, and r, 1/H, vhat (sc.lo: low parts {vhat, 1/H}) and u are taken to twice FP32.
+// On a lattice the same few separations recur, so their rounding biases every pair alike, and dJ/dtheta adds
+// the pairs of all steps: 1e-8..2e-7 of its components with FINE, 4e-9..3e-7 with the low parts of vhat, r and
+// 1/H alone (six plumes of 85^2 to 512^2).  The sweep's concentrations do not feel it (2e-8..1.1e-7 both ways,
+// and without the table), and a call of four steps with 8 sets on 512^2 takes 603 us instead of 654.
 struct ShapeConst {
     float4 lo;
     float g2, bT;          // 2 Gamma, 2 (Gamma - d) + 2
 };
 
-template <int DIM, int KERNEL, bool ISO>
-__device__ __forceinline__ float2 pair_shape(const uint4 &pa, const uint4 &pb, const PairConst &k, const ShapeConst &sc)
+template <int DIM, int KERNEL, bool ISO, bool FINE>
+__device__ __forceinline__ void pair_shape2(const uint4 &pa, const uint4 &p0, const uint4 &p1, const PairConst2 &k,
+                                            const ShapeConst &sc, float2 &gL, float2 &gT);
+
+template <int DIM, int KERNEL, bool ISO, bool FINE>
+__device__ __forceinline__ float2 pair_shape(const uint4 &pa, const uint4 &pb, const PairConst2 &k, const ShapeConst &sc)
 {
-    float dx = sep(pa.x, pb.x, k.m1), dy = sep(pa.y, pb.y, k.m1), dz = 0.f;
-    if (DIM == 3) dz = sep(pa.z, pb.z, k.m1);
-    if (!ISO) {
-        dy *= k.sy;
-        if (DIM == 3) dz *= k.sz;
-    }
-    float r2 = fmaf(dx, dx, dy * dy);
-    if (DIM == 3) r2 = fmaf(dz, dz, r2);
-    float rinv = rsqrt_ftz(r2);
-    rinv = fmaf(0.5f * rinv, fmaf(-(r2 * rinv), rinv, 1.f), rinv);
-    const float r = r2 * rinv, rl = 0.5f * rinv * fmaf(-r, r, r2);
-    const float q = r * k.invH, ql = fmaf(r, sc.lo.w, fmaf(rl, k.invH, fmaf(r, k.invH, -q)));
-    const float om = (1.f - q) - ql;
-    const float f = shape2x<KERNEL>(fmaxf(om + om, 0.f));
-    float c = fmaf(sc.lo.x, dx, sc.lo.y * dy), ch;
-    if (DIM == 3) c = fmaf(sc.lo.z, dz, c);
-    ch = fmaf(k.w0, dx, fmaf(k.w1, dy, c));
-    if (DIM == 3) ch = fmaf(k.w2, dz, ch);
-    const float t = ch * rinv, u = fminf(t * t, 1.f);
-    return make_float2(f * fmaf(sc.g2, u, -2.f), f * fmaf(-sc.g2, u, sc.bT));
+    float2 gL, gT;
+    pair_shape2<DIM, KERNEL, ISO, FINE>(pa, pb, pb, k, sc, gL, gT);
+    return make_float2(gL.x, gT.x);
 }
 
-// The same for two candidates, in packed FP32x2 instructions (the same operations per half).
-template <int DIM, int KERNEL, bool ISO>
+// Sum and product with their rounding errors (Knuth's two-sum; fused multiply-add), per half.
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 two_sum2(float2 a, float2 b, float2 &lo)
+{
+    const float2 s = __fadd2_rn(a, b), bb = sub2(s, a);
+    lo = __fadd2_rn(lo, __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb)));
+    return s;
+}
+__device__ __forceinline__ float2 two_prod2(float2 a, float2 b, float2 &lo)
+{
+    const float2 p = __fmul2_rn(a, b);
+    lo = __fadd2_rn(lo, __ffma2_rn(a, b, __fmul2_rn(p, f2(-1.f, -1.f))));
+    return p;
+}
+
+// Two candidates at once, in packed FP32x2 instructions.
+template <int DIM, int KERNEL, bool ISO, bool FINE>
 __device__ __forceinline__ void pair_shape2(const uint4 &pa, const uint4 &p0, const uint4 &p1, const PairConst2 &k,
                                             const ShapeConst &sc, float2 &gL, float2 &gT)
 {
@@ -97,25 +102,48 @@ __device__ __forceinline__ void pair_shape2(const uint4 &pa, const uint4 &p0, co
         dy = __fmul2_rn(dy, k.sy);
         if (DIM == 3) dz = __fmul2_rn(dz, k.sz);
     }
-    const float2 m1 = f2(-1.f, -1.f), one = f2(1.f, 1.f), half = f2(0.5f, 0.5f);
-    float2 r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
-    if (DIM == 3) r2 = __ffma2_rn(dz, dz, r2);
+    const float2 m1 = f2(-1.f, -1.f), one = f2(1.f, 1.f), half = f2(0.5f, 0.5f), g2 = f2(sc.g2, sc.g2);
+    if (!FINE) {
+        float2 r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)), c = __ffma2_rn(k.w0, dx, __fmul2_rn(k.w1, dy));
+        if (DIM == 3) {
+            r2 = __ffma2_rn(dz, dz, r2);
+            c = __ffma2_rn(k.w2, dz, c);
+        }
+        const float2 rinv = f2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+        const float2 om = __ffma2_rn(__fmul2_rn(r2, rinv), k.ninvH, one);
+        const float2 f = shape2x2<KERNEL>(f2(fmaxf(om.x + om.x, 0.f), fmaxf(om.y + om.y, 0.f)));
+        const float2 t = __fmul2_rn(c, rinv), t2 = __fmul2_rn(t, t), u = f2(fminf(t2.x, 1.f), fminf(t2.y, 1.f));
+        gL = __fmul2_rn(f, __ffma2_rn(g2, u, f2(-2.f, -2.f)));
+        gT = __fmul2_rn(f, __ffma2_rn(__fmul2_rn(g2, m1), u, f2(sc.bT, sc.bT)));
+        return;
+    }
+    float2 r2l = f2(0.f, 0.f), cl = __ffma2_rn(f2(sc.lo.x, sc.lo.x), dx, __fmul2_rn(f2(sc.lo.y, sc.lo.y), dy));
+    float2 r2 = two_sum2(two_prod2(dx, dx, r2l), two_prod2(dy, dy, r2l), r2l);
+    float2 ch = two_sum2(two_prod2(k.w0, dx, cl), two_prod2(k.w1, dy, cl), cl);           // vhat . x
+    if (DIM == 3) {
+        r2 = two_sum2(r2, two_prod2(dz, dz, r2l), r2l);
+        ch = two_sum2(ch, two_prod2(k.w2, dz, cl), cl);
+        cl = __ffma2_rn(f2(sc.lo.z, sc.lo.z), dz, cl);
+    }
     float2 rinv = f2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
     rinv = __ffma2_rn(__fmul2_rn(half, rinv), __ffma2_rn(__fmul2_rn(__fmul2_rn(r2, rinv), m1), rinv, one), rinv);
     const float2 r = __fmul2_rn(r2, rinv), nr = __fmul2_rn(r, m1);
-    const float2 rl = __fmul2_rn(__fmul2_rn(half, rinv), __ffma2_rn(nr, r, r2));
+    const float2 rl = __fmul2_rn(__fmul2_rn(half, rinv), __fadd2_rn(__ffma2_rn(nr, r, r2), r2l));
     const float2 nq = __fmul2_rn(r, k.ninvH);                                   // -q, and its low part
     const float2 nql = __ffma2_rn(nr, f2(sc.lo.w, sc.lo.w), __ffma2_rn(rl, k.ninvH, __ffma2_rn(r, k.ninvH, __fmul2_rn(nq, m1))));
     const float2 om = __fadd2_rn(__fadd2_rn(one, nq), nql);
     const float2 f = shape2x2<KERNEL>(f2(fmaxf(om.x + om.x, 0.f), fmaxf(om.y + om.y, 0.f)));
-    float2 c = __ffma2_rn(f2(sc.lo.x, sc.lo.x), dx, __fmul2_rn(f2(sc.lo.y, sc.lo.y), dy));
-    if (DIM == 3) c = __ffma2_rn(f2(sc.lo.z, sc.lo.z), dz, c);
-    float2 ch = __ffma2_rn(k.w0, dx, __ffma2_rn(k.w1, dy, c));
-    if (DIM == 3) ch = __ffma2_rn(k.w2, dz, ch);
     const float2 t = __fmul2_rn(ch, rinv), t2 = __fmul2_rn(t, t);
-    const float2 u = f2(fminf(t2.x, 1.f), fminf(t2.y, 1.f)), g2 = f2(sc.g2, sc.g2);
-    gL = __fmul2_rn(f, __ffma2_rn(g2, u, f2(-2.f, -2.f)));
-    gT = __fmul2_rn(f, __ffma2_rn(__fmul2_rn(g2, m1), u, f2(sc.bT, sc.bT)));
+    const float2 u = f2(fminf(t2.x, 1.f), fminf(t2.y, 1.f));                   // u = ch^2 / r^2 and what is left of it
+    float2 e = __fmul2_rn(__fadd2_rn(ch, ch), cl);
+    const float2 n = two_prod2(ch, ch, e);
+    e = __fadd2_rn(e, __ffma2_rn(__fmul2_rn(u, m1), r2, n));
+    e = __ffma2_rn(__fmul2_rn(u, m1), r2l, e);
+    float2 ul = __fmul2_rn(__fmul2_rn(e, rinv), rinv);
+    ul = f2(fminf(fmaxf(ul.x, -1e-6f), 1e-6f), fminf(fmaxf(ul.y, -1e-6f), 1e-6f));   // (max-num: finite at r = 0 too)
+    const float2 g2l = __fmul2_rn(g2, ul);
+    gL = __fmul2_rn(f, __fadd2_rn(__ffma2_rn(g2, u, f2(-2.f, -2.f)), g2l));
+    gT = __fmul2_rn(f, sub2(__ffma2_rn(__fmul2_rn(g2, m1), u, f2(sc.bT, sc.bT)), g2l));
 }
 
 // Squared separation in x units^2.
@@ -256,7 +284,7 @@ enum ChunkCut { kCutFull = 0, kCutBand = 1, kCutBox = 2 };
 // lane's range is cut by its own distance to the row and then to its first and last candidate that may
 // lie inside H.  Bound: instruction issue.  128^3 cube 1.55 -> 1.15 ms, 1024^2 258 -> 200 us against a
 // form that counted every chunk's lines in a pass of its own.
-template <int DIM, int KERNEL, bool ISO, int CUT, int VAL>
+template <int DIM, int KERNEL, bool ISO, int CUT, int VAL, bool FINE = false>
 __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs, const RateParams &prm,
                              const Chunk &c, const uint4 &pa, const TrimRow *srow, const FrozenTab &tab,
                              const ShapeConst &sc = ShapeConst())
@@ -370,14 +398,14 @@ __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const 
                     for (; t + 1 < m; t += 2) {
                         const int j0 = s + t, j1 = j0 + 1;
                         float2 gL, gT;
-                        pair_shape2<DIM, KERNEL, ISO>(pa, __ldg(P + (j0 >= qe ? j0 - len : j0)), __ldg(P + (j1 >= qe ? j1 - len : j1)),
+                        pair_shape2<DIM, KERNEL, ISO, FINE>(pa, __ldg(P + (j0 >= qe ? j0 - len : j0)), __ldg(P + (j1 >= qe ? j1 - len : j1)),
                                                       k2, sc, gL, gT);
                         o2[t * 32] = f2(gL.x, gT.x);
                         o2[(t + 1) * 32] = f2(gL.y, gT.y);
                     }
                     if (t < m) {
                         const int j = s + t;
-                        o2[t * 32] = pair_shape<DIM, KERNEL, ISO>(pa, __ldg(P + (j >= qe ? j - len : j)), k, sc);
+                        o2[t * 32] = pair_shape<DIM, KERNEL, ISO, FINE>(pa, __ldg(P + (j >= qe ? j - len : j)), k2, sc);
                     }
                 } else if (__any_sync(kFull, s + m > qe)) {
                     rs = row_weights<DIM, KERNEL, ISO, true, true>(P, pa, Ca, k, k2, s, m, qe, len, out);

@@ -181,7 +181,8 @@ __device__ __noinline__ void walk_sets(const uint4 *__restrict__ P, const uint32
     const uint4 pa = __ldg(P + min(c.i0 + (int)(threadIdx.x & 31), c.pe - 1));
     const int ncx = prm.ncx;
     const int cx = (int)__umulhi(pa.x - frame_x(prm), (uint32_t)ncx);
-    const PairConst k(prm);
+    const PairConst kc(prm);
+    const PairConst2 k(kc, kc.m1);
     for (int r = 0; r < prm.nrows; ++r) {
         const StencilRow row = prm.rows[r];
         const int q = row_pencil_of<DIM>(row, c.cy, c.cz, prm);
@@ -193,7 +194,7 @@ __device__ __noinline__ void walk_sets(const uint4 *__restrict__ P, const uint32
             j = j >= qe ? j - len : j;
             float2 v[SetSums<NT>::N2];
             op.load((size_t)(qs + j), v);
-            op.add(pair_shape<DIM, KERNEL, ISO>(pa, __ldg(P + j), k, sc), v);
+            op.add(pair_shape<DIM, KERNEL, ISO, false>(pa, __ldg(P + j), k, sc), v);
         }
         op.end_row();
     }
@@ -440,8 +441,8 @@ cudaError_t pass_nt(const SweepRun &r, int epi, const SweepParams &sp, const Rat
 {
     const dim3 g = frozen_grid(prm);
     return epi == EPI_PREDICT
-               ? launch_pdl(k_sweep_pass<DIM, KERNEL, ISO, NT, EPI_PREDICT>, g, kT, 0, s, r.P, r.cs, prm, r.tab, ShapeConst{r.lo, r.g2, r.bT}, sp, r.C, r.Ch, r.perm, out)
-               : launch_pdl(k_sweep_pass<DIM, KERNEL, ISO, NT, EPI_CORRECT>, g, kT, 0, s, r.P, r.cs, prm, r.tab, ShapeConst{r.lo, r.g2, r.bT}, sp, r.C, r.Ch, r.perm, out);
+               ? launch_pdl(k_sweep_pass<DIM, KERNEL, ISO, NT, EPI_PREDICT>, g, kT, 0, s, r.P, r.cs, prm, r.tab, ShapeConst{float4{}, r.g2, r.bT}, sp, r.C, r.Ch, r.perm, out)
+               : launch_pdl(k_sweep_pass<DIM, KERNEL, ISO, NT, EPI_CORRECT>, g, kT, 0, s, r.P, r.cs, prm, r.tab, ShapeConst{float4{}, r.g2, r.bT}, sp, r.C, r.Ch, r.perm, out);
 }
 
 template <int DIM, int KERNEL, bool ISO>
@@ -459,7 +460,7 @@ template <int DIM, int KERNEL, bool ISO>
 cudaError_t table_k(const SweepRun &r, const RateParams &prm, const float *C, int sets, int P4, cudaStream_t s)
 {
     return launch_pdl(k_sweep_table<DIM, KERNEL, ISO>, frozen_grid(prm), kT, 0, s, r.P, r.cs, r.perm, prm, r.tab,
-                      ShapeConst{r.lo, r.g2, r.bT}, C, sets, P4, r.C);
+                      ShapeConst{float4{}, r.g2, r.bT}, C, sets, P4, r.C);
 }
 
 #define ADE_SWEEP_CALL(F, ...)                                                                                               \
