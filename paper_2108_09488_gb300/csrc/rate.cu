@@ -300,9 +300,9 @@ __global__ __launch_bounds__(kRateThreads) void k_rate_batch(const uint4 *__rest
     constexpr int kWords = (int)(sizeof(RateParams) / sizeof(int));
     static_assert(sizeof(RateParams) % sizeof(int) == 0, "RateParams is copied word by word");
     const int lane = threadIdx.x & 31;
+    __shared__ uint3 sorg[kRateThreads / 32];
     RateParams &mine = sp[threadIdx.x >> 5];
     int cur = -1;
-    uint3 org = make_uint3(0u, 0u, 0u);
     unsigned cnt = 0u;
     for (;;) {
         int item = 0;
@@ -316,9 +316,11 @@ __global__ __launch_bounds__(kRateThreads) void k_rate_batch(const uint4 *__rest
             for (int w = lane; w < kWords; w += 32) dst[w] = __ldg(src + w);
             cur = t.plume;
             __syncwarp();
-            org = cell_origin(mine);
+            if (lane == 0) sorg[threadIdx.x >> 5] = cell_origin(mine);   // (registers would cost 3 % of the batch)
+            __syncwarp();
         }
         const RateParams &prm = mine;
+        const uint3 &org = sorg[threadIdx.x >> 5];
         EpiOut o = out;
         if (EPI == EPI_CORRECT) o.xq = out.xq + (size_t)prm.goff * (DIM - 1);
         if (PAIRED && !COUNT) {

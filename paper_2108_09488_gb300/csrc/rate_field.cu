@@ -10,9 +10,9 @@
 // with W'(r)/r = kc f(q) as in rate.cu.  Particles drift with their own velocities, so relative
 // positions change during a step: the cell list is built for the radius H + dt vmax (the skin
 // covers the relative drift up to the half step, |v_a - v_b| dt/2 <= dt vmax) while the support
-// test uses H.  One thread per cell-sorted particle walks the stencil rows of its build-time
-// cell as in the direct kernel; the row sums of both terms are added with Neumaier compensation
-// in a fixed order, so results are deterministic.
+// test uses H.  Each cell-sorted particle's candidates are those of the stencil rows of its
+// build-time cell, cut to the chord its own position leaves; the sums of both terms over a row (2D) or
+// a list (3D) are added with Neumaier compensation in a fixed order, so results are deterministic.
 // Records of v and D are formed once per field in the caller's order (v is constant in time) and
 // permuted into the cell-sorted order after every cell build (k_field_permute), so the pair
 // loop's loads stay contiguous: candidates of a row are consecutive sorted indices.

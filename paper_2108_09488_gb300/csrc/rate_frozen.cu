@@ -77,7 +77,10 @@ __global__ __launch_bounds__(kT) void k_frozen_build(const uint4 *__restrict__ P
     });
 }
 
-// One evaluation from the table.
+// One evaluation from the table.  Bound: HBM where the table exceeds L2 (4 bytes per pair and the idle
+// tails of rows), latency below.  Per evaluation, walk / table: 128^3 cube, 250 neighbours, 700 / 412 us
+// (2.6 GB, 6.2 TB/s of the 6.7 a copy reaches); 1024^2, 120 neighbours 124 / 101; 512^2, 60 about 30 / 18.5;
+// 256^2, 28 7.5 / 5.3.  Twelve CTAs per SM: the loads in flight are what the stream lives on.
 template <int DIM, int KERNEL, bool ISO, int EPI>
 __global__ __launch_bounds__(kT, 12) void k_frozen_rate(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
                                                     const RateParams prm, const FrozenTab tab, const FrozenState st)

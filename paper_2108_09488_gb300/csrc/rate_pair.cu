@@ -16,9 +16,9 @@ namespace {
 // Paired kernel: thread t evaluates sorted particles 2t and 2t + 1; a pair that cannot share a
 // candidate stream (can_pair) takes the one-target walk for each particle.  The branch-free
 // full-row walk is held to 10 resident CTAs per SM (<= 48 registers), which measured faster on the
-// 1024^2 ladder; the trimmed and branched walks are left to the compiler.
+// 1024^2 ladder, and the 2D trimmed one to 9 (<= 56); the others are left to the compiler.
 template <int DIM, int KERNEL, int EPI, bool ISO, bool TRIM, bool BF>
-__global__ __launch_bounds__(kRateThreads, (BF && !TRIM) ? 10 : 0) void k_rate_pair(const uint4 *__restrict__ Pe,
+__global__ __launch_bounds__(kRateThreads, BF ? (!TRIM ? 10 : DIM == 2 ? 9 : 0) : 0) void k_rate_pair(const uint4 *__restrict__ Pe,
                                                             const uint4 *__restrict__ Pc,
                                                             const uint32_t *__restrict__ cs,
                                                             const uint32_t *__restrict__ perm,

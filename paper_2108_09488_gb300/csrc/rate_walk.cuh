@@ -26,9 +26,10 @@ __device__ __forceinline__ uint3 cell_origin(const P &prm)
 {
     uint3 o = make_uint3(prm.back[0], prm.back[1], prm.back[2]);
     if (prm.frame) {
-        o.x += __ldg(prm.frame + 4);
-        o.y += __ldg(prm.frame + 5);
-        o.z += __ldg(prm.frame + 6);
+        const uint4 f = __ldg(reinterpret_cast<const uint4 *>(prm.frame + 4));
+        o.x += f.x;
+        o.y += f.y;
+        o.z += f.z;
     }
     return o;
 }
