@@ -87,7 +87,8 @@ typedef struct ade_params {
     double dt_coef;    /* coefficient of the rule; <= 0 selects 0.1 (Eq. 10) */
     int cell_subdiv;   /* cells per support radius along each axis, 1..6; 0 = automatic */
     unsigned flags;    /* 0 (library's choice: without ade_autotune the branch-free walk over trimmed rows
-                          in 3D and from 100 expected neighbours on, over full rows otherwise; kept pair
+                          on 3D grids of about one particle per cell and from 100 expected
+                          neighbours on in 2D, over full rows otherwise; kept pair
                           weights in calls of several steps), ADE_FLAG_DIRECT, ADE_FLAG_TILED, ADE_FLAG_BRANCHED,
                           or ADE_FLAG_TRIMMED alone or with DIRECT or BRANCHED */
     double vmax;       /* 0: uniform velocity v.  > 0: velocity-field mode -- each particle carries

@@ -191,8 +191,16 @@ double grid_cost(const Grid &g, int n)
     return cand + 4.0 * g.nrows;
 }
 
+// 3D grids whose pencils hold about one line of particles, where the pencil boxes of the trimmed walk are tight.
+bool about_one_per_cell(const Grid &g, int n) { return (double)n >= 0.999 * g.ncells && (double)n <= 1.5 * g.ncells; }
+
 int choose_grid(const ade_params &p, double H, int n, Grid *g)
 {
+    bool finest = p.dim == 3 && p.vmax > 0.0;
+    for (int k = 1; p.dim == 3 && k <= ade::kMaxSubdiv; ++k) {
+        Grid t;
+        finest = finest || (make_grid(p, H, k, &t) && about_one_per_cell(t, n));
+    }
     if (p.cell_subdiv > 0) {
         if (p.cell_subdiv > ade::kMaxSubdiv || !make_grid(p, H, p.cell_subdiv, g))
             return fail(ADE_ERR_ARG, "cell_subdiv=%d does not fit the box (need >= 2k+1 cells per axis, <= 2^24 cells)",
@@ -204,11 +212,13 @@ int choose_grid(const ade_params &p, double H, int n, Grid *g)
     for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
         Grid t;
         if (!make_grid(p, H, k, &t)) continue;
-        // 3D: the finest grid of at least one particle per cell on average (else the coarsest).  Finer
+        // 3D velocity fields, and where it holds at most 1.5: the finest grid of at least one particle per cell on average (else the coarsest).  Finer
         // ones leave rows of few candidates and pencils of few particles (us per step at this rule's
         // choice and one finer: 45^3 jittered, velocity field 504 / 536, weights kept 121 / 205; 64^3 at one
-        // per cell, field 1882 / 2304, weights kept 165 / 179), coarser ones longer ranges.
-        if (p.dim == 3) {
+        // per cell, field 1882 / 2304, weights kept 165 / 179), coarser ones longer ranges.  Other sets keep
+        // the cost model and the full rows (49^3 jittered, 2 per cell, one
+        // rate: 237 us, trimmed at this rule's grid 271; 57^3 C4, 1.1 per cell 294 / 244).
+        if (finest) {
             if (found && (double)n < 0.999 * t.ncells) break;
             *g = t;
             found = true;
@@ -826,11 +836,12 @@ int plume_constants(const ade_params *p, int n, const Derived &d, double *D, dou
     rp.m1 = -1;
     rp.variant = d.tiles.variant == 1 ? 1 : ((p->flags & ADE_FLAG_BRANCHED) ? 2 : 0);
     if (rp.variant != 1 && (p->flags & ADE_FLAG_TRIMMED)) rp.variant = rp.variant == 2 ? 4 : 3;  // trimmed rows
-    // The library's choice without autotuning: trimmed rows in 3D, and in 2D from about 100 neighbours on
-    // (us per step, full / trimmed: 128^3 4424 / 2298, 57^3 jittered 505 / 439, 2D 160^2 with 2,700
+    // The library's choice without autotuning: trimmed rows on 3D grids of about one particle per
+    // cell and in 2D from 100 neighbours on (us per step, full / trimmed: 57^3 jittered C4 505 / 439, 2D 160^2 with 2,700
     // neighbours 828 / 693, 1024^2 with 120 385 / 375; 300^2 jittered with 45 68 / 82).  The paired walks
     // are left to the autotuner: on an irregular set they lose (57^3 980).
-    if (p->flags == 0u && !(p->vmax > 0.0) && *iso && (p->dim == 3 || expected_neighbours(*p, d.H, n) >= 100.0))
+    if (p->flags == 0u && !(p->vmax > 0.0) && *iso &&
+        (p->dim == 3 ? about_one_per_cell(d.g, n) : expected_neighbours(*p, d.H, n) >= 100.0))
         rp.variant = 3;
     if (p->flags & ADE_FLAG_PAIRED)                                                           // paired walks
         rp.variant = (p->flags & ADE_FLAG_BRANCHED) ? ((p->flags & ADE_FLAG_TRIMMED) ? 8 : 7)
