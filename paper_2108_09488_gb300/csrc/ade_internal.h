@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "../../include/ade_sph.h"
+#include "pool.h"
 
 struct ade_ctx;
 

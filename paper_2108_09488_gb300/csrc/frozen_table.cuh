@@ -10,14 +10,13 @@
 // kept twice per pencil, back to back (particle j of pencil [ps, pe) at ps + j and again at pe + j),
 // so that a range that runs over the periodic x seam stays contiguous.  A chunk that finds no room in
 // the table is marked and evaluated from the positions instead (the same sums), so a table that is
-// too small costs time, never a result.
+// too small costs time, never a result (claim_lines in pool.h never hands out a line twice).
 //
 // A value is one word (the weight for one tensor: VAL 1) or two (g_L and g_T, from which every
 // uniform tensor's weight follows: VAL 2, lane l's pair in words 2l, 2l + 1 of two lines).
 #pragma once
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr unsigned kNoRoom = 0xffffffffu;
 
 // Where one warp's chunk lies: particles [i0, min(i0 + 32, pe)) of pencil p (cy, cz).
 struct Chunk {
@@ -382,7 +381,7 @@ __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const 
                 const int m = (int)__reduce_max_sync(kFull, (unsigned)cnt);
                 if (m == 0) continue;
                 // idle tail iterations of a shorter lane stay inside the doubled pencil (m <= len)
-                used += 1u + (unsigned)(m * VAL);
+                used = add_lines(used, 1u + (unsigned)(m * VAL));
                 const bool keep = used <= room;
                 if (keep) {
                     if (lane == 0) hdr[R] = __int_as_float(m);
@@ -421,11 +420,16 @@ __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const 
         if (used <= room || attempt == 1) break;
         // outgrown: once more into the pool
         unsigned at = 0u;
-        if (lane == 0) at = atomicAdd(tab.cursor, used);
+        if (lane == 0)
+            at = claim_lines(*(volatile unsigned *)tab.cursor, tab.cap, used,
+                             [&](unsigned seen, unsigned next) { return atomicCAS(tab.cursor, seen, next); });
         at = __shfl_sync(kFull, at, 0);
+        if (at == kNoRoom) {
+            room = 0u;
+            break;
+        }
         base = tab.pool + at;
-        room = at <= tab.cap && tab.cap - at >= used ? used : 0u;
-        if (room == 0u) break;
+        room = used;
     }
     if (lane == 0) tab.slots[c.slot] = make_uint4(used <= room ? base : kNoRoom, R, used, hs);
     if (VAL == 1 && used > room) return walk_chunk<DIM, KERNEL, ISO>(P, cs, prm, c, nullptr);
