@@ -162,14 +162,22 @@ struct SweepOut {
 
 // Weight table of the evaluations over one cell list (rate_frozen.cu), in lines of 32 words: a region of
 // RateParams::fz_stride lines per chunk from RateParams::fz_base on, and from line `pool` on `cap` lines
-// that an atomic cursor hands out to chunks that outgrow theirs; slots[chunk] = {first line of the
-// chunk's stream, rows, lines, header lines}.
+// that an atomic cursor hands out to chunks that outgrow theirs; slots: two words of 16 bytes per chunk
+// number (put_chunk in frozen_table.cuh).
 constexpr int kFrozenThreads = 128;
+// Numbers given to the chunks of n particles in np pencils (find_chunk in frozen_table.cuh), and from how many
+// on they are counted (launch_chunk_numbers).  Without the count one number per pencil may belong to no chunk,
+// and the warps that get them idle in their block: on a chip that is full (a wave: 152 SMs of 48 warps) they
+// cost what their share of the warps is (per step: 128^3, four chunks and a gap per pencil, 989 us against
+// 955; 57^3 190 against 160), on less they cost nothing and the launch would (2 us a call).
+__host__ __device__ inline int chunk_numbers(int n, int np) { return (n >> 5) + np; }
+constexpr int kCountChunksFrom = 152 * 48;
 struct FrozenTab {
     float *words;
     uint4 *slots;
     unsigned *cursor;
     unsigned pool, cap;
+    uint32_t *dense;       // chunks before each pencil (launch_chunk_numbers; NULL: numbers with gaps)
 };
 // Concentrations (and Eq. 14's flux) of such a run in sorted order: C at level l, Ch at l + 1/2, each
 // pencil's twice back to back ([2n] words).
@@ -180,10 +188,9 @@ struct FrozenState {
     float tau_inv;
 };
 
-// Batched plumes: chunks y, y + ny, ... of one pencil of one plume; p0: pencils of the plumes before it.
+// Batched plumes: chunk number `chunk` of one plume; its slot is the item's index.
 struct FrozenItem {
-    int plume, pencil, p0;
-    unsigned short y, ny;
+    int plume, chunk;
 };
 
 // Steps of one sweep call: sorted positions, cell table, weight table, concentrations (planes of
@@ -313,12 +320,14 @@ cudaError_t launch_rate_field(int dim, int kernel, int epi, const uint4 *Pe, con
                               const uint32_t *perm, const FieldWork &fw, const RateParams &prm,
                               const FieldParams &fp, const EpiOut &out, cudaStream_t s);
 
-// Launch grid of the table's kernels (kFrozenThreads threads a block).
-dim3 frozen_grid(const RateParams &prm);
-// Lines and slots of a table with `val` words per pair (lines bounded by the table's size limit), and blocks
-// of frozen_grid, enough for every grid the context may switch to; and the table's division among the
-// chunks of the grid in use (fz_base, fz_stride, pool, cap).
-void frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots, int *blocks);
+// Blocks of the table's kernels (kFrozenThreads threads): a warp per chunk number.
+unsigned frozen_blocks(const RateParams &prm);
+// dense[p] = chunks of the pencils before p, p = 0..np (nothing where dense is NULL).
+cudaError_t launch_chunk_numbers(const uint32_t *cs, const RateParams &prm, uint32_t *dense, cudaStream_t s);
+// Lines and slots of a table with `val` words per pair (lines bounded by the table's size limit), enough for
+// every grid the context may switch to; and the table's division among the chunks of the grid in use
+// (fz_base, fz_stride, pool, cap).
+void frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots);
 void frozen_divide(const ade_ctx *c, int val, size_t lines, RateParams *rp, FrozenTab *tab);
 // Evaluations over one cell list with stored weights (rate_frozen.cu): the table, one predictor or
 // corrector (prm.dt), and the final state in the caller's order (prm.inc: the drift of all steps).

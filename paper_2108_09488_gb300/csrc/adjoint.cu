@@ -105,11 +105,12 @@ __device__ __noinline__ void walk_sums(const uint4 *__restrict__ P, const uint32
     const uint4 pa = __ldg(P + min(c.i0 + (int)(threadIdx.x & 31), c.pe - 1));
     const int ncx = prm.ncx;
     const int cx = (int)__umulhi(pa.x - frame_x(prm), (uint32_t)ncx);
+    const int cy = c.p % prm.ncy, cz = c.p / prm.ncy;
     const PairConst kc(prm);
     const PairConst2 k(kc, kc.m1);
     for (int r = 0; r < prm.nrows; ++r) {
         const StencilRow row = prm.rows[r];
-        const int q = row_pencil_of<DIM>(row, c.cy, c.cz, prm);
+        const int q = row_pencil_of<DIM>(row, cy, cz, prm);
         const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
         int s, cnt;
         cyclic_range(cs, q * ncx, cx - (int)row.w, cx + row.w + 1, ncx, qs, qe, s, cnt);
@@ -132,12 +133,15 @@ __global__ __launch_bounds__(kT) void k_adj_table(const uint4 *__restrict__ P, c
     pdl_wait();
     __shared__ TrimRow srow[ISO ? kMaxRows : 1];
     if (ISO) stage_trim_rows(srow, prm);
-    for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), gridDim.y * (kT / 32), [&](const Chunk &c) {
-        const int i = c.i0 + (threadIdx.x & 31);
-        const uint4 pa = __ldg(P + min(i, c.pe - 1));
-        build_chunk<DIM, KERNEL, ISO, ISO ? kCutBox : kCutFull, 2, true>(P, cs, prm, c, pa, srow, tab, sc);
-        if (i < c.pe) C0[c.ps + i] = C0[c.pe + i] = __uint_as_float(pa.w);
-    });
+    Chunk c;
+    const int t = warp_number();
+    const bool has = find_chunk(cs, prm, tab.dense, t, c);
+    if (t < chunk_numbers(prm.n, prm.ncy * prm.ncz)) put_chunk(tab, c, has);
+    if (!has) return;
+    const int i = c.i0 + (threadIdx.x & 31);
+    const uint4 pa = __ldg(P + min(i, c.pe - 1));
+    build_chunk<DIM, KERNEL, ISO, ISO ? kCutBox : kCutFull, 2, true>(P, cs, prm, c, pa, srow, tab, sc);
+    if (i < c.pe) C0[c.ps + i] = C0[c.pe + i] = __uint_as_float(pa.w);
 }
 
 // One pass over the table; fields doubled per pencil.
@@ -204,7 +208,9 @@ __global__ __launch_bounds__(kT) void k_adj_pass(const uint4 *__restrict__ P, co
     double dot[ND];
 #pragma unroll
     for (int q = 0; q < ND; ++q) dot[q] = 0.0;
-    for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), gridDim.y * (kT / 32), [&](const Chunk &c) {
+    Chunk c;
+    uint4 sl;
+    if (my_chunk(tab, prm, c, sl)) {
         const int i = c.i0 + (threadIdx.x & 31);
         const int at = c.ps + min(i, c.pe - 1);
         ShapeSums<NR> op;
@@ -215,48 +221,48 @@ __global__ __launch_bounds__(kT) void k_adj_pass(const uint4 *__restrict__ P, co
             op.x[NR - 1] = ps.x0;
             op.xa[NR - 1] = ps.x0[at];
         }
-        const uint4 sl = __ldg(tab.slots + c.slot);
         if (sl.x != kNoRoom) stream_rows<2>(sl, tab, op);
         else walk_sums<DIM, KERNEL, ISO, NR>(P, cs, prm, c, ps.sc, op);
-        if (i >= c.pe) return;
-        const int again = c.pe + i;
-        const float L1 = combine(ps, op.s0(0), op.s1(0));
-        const float p = MODE == HALF || MODE == BACK1 ? op.xa[0] : ps.base[at];
-        ps.out1[at] = ps.out1[again] = fmaf(ps.step, L1, p);
-        if (BACK) {
-            const float s0 = op.s0(NR - 1), s1 = op.s1(NR - 1);
-            dot[0] = fma((double)p, (double)s0, dot[0]);
-            dot[1] = fma((double)p, (double)s1, dot[1]);
-            if (MODE == BACK1) {
-                dot[2 % ND] = fma((double)L1, (double)s0, dot[2 % ND]);
-                dot[3 % ND] = fma((double)L1, (double)s1, dot[3 % ND]);
-                ps.out0[at] = ps.out0[again] = combine(ps, s0, s1);
+        if (i < c.pe) {
+            const int again = c.pe + i;
+            const float L1 = combine(ps, op.s0(0), op.s1(0));
+            const float p = MODE == HALF || MODE == BACK1 ? op.xa[0] : ps.base[at];
+            ps.out1[at] = ps.out1[again] = fmaf(ps.step, L1, p);
+            if (BACK) {
+                const float s0 = op.s0(NR - 1), s1 = op.s1(NR - 1);
+                dot[0] = fma((double)p, (double)s0, dot[0]);
+                dot[1] = fma((double)p, (double)s1, dot[1]);
+                if (MODE == BACK1) {
+                    dot[2 % ND] = fma((double)L1, (double)s0, dot[2 % ND]);
+                    dot[3 % ND] = fma((double)L1, (double)s1, dot[3 % ND]);
+                    ps.out0[at] = ps.out0[again] = combine(ps, s0, s1);
+                }
             }
         }
-    });
+    }
     if (BACK)
-        block_sums<ND>(dot, ps.partials + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kDots + (MODE == BACK2 ? 4 : 0));
+        block_sums<ND>(dot, ps.partials + (size_t)blockIdx.x * kDots + (MODE == BACK2 ? 4 : 0));
 }
 
 // lambda^N = C^N - C* (doubled per pencil) and its squares' block sums.
-template <int DIM>
-__global__ __launch_bounds__(kT) void k_adj_misfit(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
-                                                   const uint32_t *__restrict__ perm, const RateParams prm,
+__global__ __launch_bounds__(kT) void k_adj_misfit(const uint32_t *__restrict__ perm, const RateParams prm, const FrozenTab tab,
                                                    const float *__restrict__ CN, const float *__restrict__ target,
                                                    float *__restrict__ p, double *__restrict__ partials)
 {
     pdl_wait();
     double d[kDots] = {0.0};
-    for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), gridDim.y * (kT / 32), [&](const Chunk &c) {
-        const int i = c.i0 + (threadIdx.x & 31);
-        if (i >= c.pe) return;
+    Chunk c = {};
+    uint4 sl;
+    const bool has = my_chunk(tab, prm, c, sl);
+    const int i = c.i0 + (int)(threadIdx.x & 31);
+    if (has && i < c.pe) {
         const uint32_t a = __ldg(perm + i);
         const float t = a < (uint32_t)prm.n ? __ldg(target + a) : 0.f;
         const float v = fmaf(-1.f, t, CN[c.ps + i]);
         p[c.ps + i] = p[c.pe + i] = v;
-        d[0] = fma((double)v, (double)v, d[0]);
-    });
-    block_sums<kDots>(d, partials + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kDots);
+        d[0] = (double)v * (double)v;
+    }
+    block_sums<kDots>(d, partials + (size_t)blockIdx.x * kDots);
 }
 
 // out[step][q] = sum over the blocks' partials, one CTA per step, in a fixed order.
@@ -287,16 +293,17 @@ __global__ __launch_bounds__(kFoldT) void k_adj_fold(const double *__restrict__ 
 }
 
 // out[perm[i]] = the doubled field's value of sorted particle i.
-__global__ __launch_bounds__(kT) void k_adj_scatter(const uint32_t *__restrict__ cs, const uint32_t *__restrict__ perm,
-                                                    const RateParams prm, const float *__restrict__ x, float *__restrict__ out)
+__global__ __launch_bounds__(kT) void k_adj_scatter(const uint32_t *__restrict__ perm, const RateParams prm, const FrozenTab tab,
+                                                    const float *__restrict__ x, float *__restrict__ out)
 {
     pdl_wait();
-    for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), gridDim.y * (kT / 32), [&](const Chunk &c) {
-        const int i = c.i0 + (threadIdx.x & 31);
-        if (i >= c.pe) return;
-        const uint32_t a = __ldg(perm + i);
-        if (a < (uint32_t)prm.n) out[a] = x[c.ps + i];
-    });
+    Chunk c;
+    uint4 sl;
+    if (!my_chunk(tab, prm, c, sl)) return;
+    const int i = c.i0 + (threadIdx.x & 31);
+    if (i >= c.pe) return;
+    const uint32_t a = __ldg(perm + i);
+    if (a < (uint32_t)prm.n) out[a] = x[c.ps + i];
 }
 
 // Everything one call needs.
@@ -307,7 +314,7 @@ struct Adj {
     FrozenTab tab;
     float ca, cb, cal, cbl;   // L(theta) x = ca S_L + cb S_T (hi + lo)
     ShapeConst sc;
-    dim3 grid;
+    unsigned blocks;
 };
 
 template <int DIM, int KERNEL, bool ISO>
@@ -316,17 +323,17 @@ cudaError_t pass_t(const Adj &A, int mode, const AdjPass &ps)
     const uint4 *P = A.c->w.P0;
     const uint32_t *cs = A.c->w.cell_start;
     switch (mode) {
-    case HALF: return launch_pdl(k_adj_pass<DIM, KERNEL, ISO, HALF>, A.grid, kT, 0, A.s, P, cs, A.rp, A.tab, ps);
-    case FULL: return launch_pdl(k_adj_pass<DIM, KERNEL, ISO, FULL>, A.grid, kT, 0, A.s, P, cs, A.rp, A.tab, ps);
-    case BACK1: return launch_pdl(k_adj_pass<DIM, KERNEL, ISO, BACK1>, A.grid, kT, 0, A.s, P, cs, A.rp, A.tab, ps);
-    default: return launch_pdl(k_adj_pass<DIM, KERNEL, ISO, BACK2>, A.grid, kT, 0, A.s, P, cs, A.rp, A.tab, ps);
+    case HALF: return launch_pdl(k_adj_pass<DIM, KERNEL, ISO, HALF>, A.blocks, kT, 0, A.s, P, cs, A.rp, A.tab, ps);
+    case FULL: return launch_pdl(k_adj_pass<DIM, KERNEL, ISO, FULL>, A.blocks, kT, 0, A.s, P, cs, A.rp, A.tab, ps);
+    case BACK1: return launch_pdl(k_adj_pass<DIM, KERNEL, ISO, BACK1>, A.blocks, kT, 0, A.s, P, cs, A.rp, A.tab, ps);
+    default: return launch_pdl(k_adj_pass<DIM, KERNEL, ISO, BACK2>, A.blocks, kT, 0, A.s, P, cs, A.rp, A.tab, ps);
     }
 }
 
 template <int DIM, int KERNEL, bool ISO>
 cudaError_t table_t(const Adj &A, float *C0)
 {
-    return launch_pdl(k_adj_table<DIM, KERNEL, ISO>, A.grid, kT, 0, A.s, A.c->w.P0, A.c->w.cell_start, A.rp, A.tab, A.sc, C0);
+    return launch_pdl(k_adj_table<DIM, KERNEL, ISO>, A.blocks, kT, 0, A.s, A.c->w.P0, A.c->w.cell_start, A.rp, A.tab, A.sc, C0);
 }
 
 #define ADE_ADJ_CALL(F, ...)                                                                                          \
@@ -364,7 +371,7 @@ cudaError_t fwd_step(const Adj &A, const float *u, float *h, float *out, float d
 
 // Adjoint workspace: fields (doubled per pencil), the weight table, FP64 partials of one segment.
 struct AdjLayout {
-    size_t ckpt, seg, h, p, hp, a, dots, partials, words, slots, cursor, total;
+    size_t ckpt, seg, h, p, hp, a, dots, partials, words, slots, dense, cursor, total;
     size_t lines;
     int nck, blocks;
 };
@@ -380,7 +387,8 @@ AdjLayout adj_layout(const ade_ctx *c, int nsteps, int ck)
     };
     const size_t f2 = (size_t)c->n * 8;
     size_t slots = 0;
-    frozen_extent(c, 2, &L.lines, &slots, &L.blocks);
+    frozen_extent(c, 2, &L.lines, &slots);
+    L.blocks = (int)((slots + kT / 32 - 1) / (kT / 32));
     L.nck = (nsteps + ck - 1) / ck;
     L.ckpt = take(f2 * (L.nck + 1));
     L.seg = take(f2 * std::min(ck, nsteps));
@@ -391,7 +399,8 @@ AdjLayout adj_layout(const ade_ctx *c, int nsteps, int ck)
     L.dots = take(((size_t)nsteps + 1) * kDots * 8);
     L.partials = take((size_t)L.blocks * std::min(ck, nsteps) * kDots * 8);
     L.words = take(L.lines * 128);
-    L.slots = take(slots * 16);
+    L.slots = take(slots * 32);
+    L.dense = take(slots * 4);
     L.cursor = take(64);
     L.total = off;
     return L;
@@ -464,7 +473,7 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     A.cb = (float)(pf * sb);
     A.cal = (float)(pf * sa - (double)A.ca);
     A.cbl = (float)(pf * sb - (double)A.cb);
-    A.grid = frozen_grid(A.rp);
+    A.blocks = frozen_blocks(A.rp);
     char *base = static_cast<char *>(aws);
     auto field = [&](size_t o) { return reinterpret_cast<float *>(base + o); };
     const size_t n2 = 2 * (size_t)n;
@@ -474,17 +483,20 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     A.tab.words = field(L.words);
     A.tab.slots = reinterpret_cast<uint4 *>(base + L.slots);
     A.tab.cursor = reinterpret_cast<unsigned *>(base + L.cursor);
+    const bool count = chunk_numbers(n, A.rp.ncy * A.rp.ncz) > kCountChunksFrom;
+    A.tab.dense = count ? reinterpret_cast<uint32_t *>(base + L.dense) : nullptr;
     frozen_divide(c, 2, L.lines, &A.rp, &A.tab);
-    const int nb = (int)(A.grid.x * A.grid.y);
+    const int nb = (int)A.blocks;
     if (nb > L.blocks) return ade::report_error(ADE_ERR_CAPACITY, "adjoint partials exceed the workspace");
     const float dt = (float)c->dt;
     cudaStream_t s = A.s;
-    const uint32_t *cs = c->w.cell_start, *perm = c->w.perm;
+    const uint32_t *perm = c->w.perm;
 
     // frozen geometry: one cell list at the current positions (counts and tile totals cleared first)
     ADJ_CK(cudaMemsetAsync(A.tab.cursor, 0, sizeof(unsigned), s));
     ADJ_CK(ade::launch_build_cells(c->dim, c->xq, c->C, n, c->nc, c->ncells, c->w, s));
     c->cells_framed = false;
+    ADJ_CK(launch_chunk_numbers(c->w.cell_start, A.rp, A.tab.dense, s));
     ADJ_CK(table(A, ckpt));
     // forward: checkpoints every ckpt_every steps, the last segment's states straight into seg
     const int l0_last = (L.nck - 1) * ckpt_every;
@@ -501,10 +513,9 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     }
     // C^N sits in checkpoint slot nck (the last step always writes a slot)
     const float *CN = ckpt + (size_t)L.nck * n2;
-    if (C_final_dev) ADJ_CK(launch_pdl(k_adj_scatter, A.grid, kT, 0, s, cs, perm, A.rp, CN, C_final_dev));
+    if (C_final_dev) ADJ_CK(launch_pdl(k_adj_scatter, A.blocks, kT, 0, s, perm, A.rp, A.tab, CN, C_final_dev));
     // lambda^N = C^N - C*, J = 1/2 |lambda^N|^2
-    if (c->dim == 2) ADJ_CK(launch_pdl(k_adj_misfit<2>, A.grid, kT, 0, s, c->w.P0, cs, perm, A.rp, CN, C_target_dev, p, partials));
-    else ADJ_CK(launch_pdl(k_adj_misfit<3>, A.grid, kT, 0, s, c->w.P0, cs, perm, A.rp, CN, C_target_dev, p, partials));
+    ADJ_CK(launch_pdl(k_adj_misfit, A.blocks, kT, 0, s, perm, A.rp, A.tab, CN, C_target_dev, p, partials));
     ADJ_CK(launch_pdl(k_adj_fold, 1, kFoldT, 0, s, partials, nb, dots + (size_t)nsteps * kDots));
     // backward, segment by segment
     AdjPass ps;
@@ -540,7 +551,7 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
         }
         ADJ_CK(launch_pdl(k_adj_fold, (unsigned)(l1 - l0), kFoldT, 0, s, partials, nb, dots + (size_t)l0 * kDots));
     }
-    if (dJdC0_dev) ADJ_CK(launch_pdl(k_adj_scatter, A.grid, kT, 0, s, cs, perm, A.rp, (const float *)p, dJdC0_dev));
+    if (dJdC0_dev) ADJ_CK(launch_pdl(k_adj_scatter, A.blocks, kT, 0, s, perm, A.rp, A.tab, (const float *)p, dJdC0_dev));
     std::vector<double> hd(((size_t)nsteps + 1) * kDots);
     ADJ_CK(cudaMemcpyAsync(hd.data(), dots, hd.size() * 8, cudaMemcpyDeviceToHost, s));
     ADJ_CK(cudaStreamSynchronize(s));

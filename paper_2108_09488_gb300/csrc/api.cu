@@ -325,7 +325,7 @@ void choose_tiles(int dim, int n, const Grid &g, bool iso, unsigned flags, ade::
 
 struct Layout {
     size_t keys, rank, count, block_sums, perm_tmp, perm, cell_start, P0, P1, partials, wpart, stats,
-        cf_partials, status, pairs, pencil, tile_sums, frame, fz_words, fz_slots, fz_C, fz_cursor, fVc, fDAc, fDBc, fIncC, fV, fDA, fDB, fInc,
+        cf_partials, status, pairs, pencil, tile_sums, frame, fz_words, fz_slots, fz_dense, fz_C, fz_cursor, fVc, fDAc, fDBc, fIncC, fV, fDA, fDB, fInc,
         fbits, Q, Qh, total;
 };
 
@@ -363,7 +363,8 @@ Layout layout(int n, int ncells, int nb_partials, int nw_partials, int field_dim
     L.tile_sums = take(ade::tile_sums_bytes(ncells));
     L.frame = take(ade::kFrameWords * 4);
     L.fz_words = take(fz_lines * 128);
-    L.fz_slots = take(fz_slots * 16);
+    L.fz_slots = take(fz_slots * 32);
+    L.fz_dense = take(fz_slots * 4);
     L.fz_C = take(fz_slots > 0 ? (size_t)n * 16 : 0);
     L.fz_cursor = take(64);
     L.fVc = L.fDAc = L.fDBc = L.fIncC = L.fV = L.fDA = L.fDB = L.fInc = L.fbits = 0;
@@ -717,6 +718,8 @@ int enqueue_frozen(ade_ctx *c, int steps, cudaStream_t s)
     }
     ade::FrozenTab tab = c->frozen_tab;
     ade::frozen_divide(c, 1, c->frozen_lines, &rp, &tab);
+    if (ade::chunk_numbers(c->n, rp.ncy * rp.ncz) <= ade::kCountChunksFrom) tab.dense = nullptr;
+    ADE_CK(ade::launch_chunk_numbers(c->w.cell_start, rp, tab.dense, s));
     rp.dt = (float)(0.5 * c->dt);
     ADE_CK(ade::launch_frozen_build(c->dim, c->p.kernel, c->iso, c->w.P0, c->w.cell_start, c->w.perm, rp, tab, st, s));
     for (int k = 0; k < steps; ++k) {
@@ -865,10 +868,9 @@ T *at(void *base, size_t off)
 
 }  // namespace
 
-void ade::frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots, int *blocks)
+void ade::frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots)
 {
     *lines = *slots = 0;
-    *blocks = 1;
     const bool fixed = c->p.cell_subdiv > 0 || c->p.flags != 0u;   // no autotuning: the grid in use
     // (the same before and after autotuning: callers size a workspace with it; a grid that needs more has
     // chunks evaluated from the positions)
@@ -888,13 +890,6 @@ void ade::frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots,
         if ((fixed && k != c->subdiv) || !make_grid(c->p, c->Hgrid, k, &g)) continue;
         *lines = std::max(*lines, std::min(room, frozen_lines(c->p, c->H, c->n, g, val)));
         *slots = std::max(*slots, frozen_slots(c->n, g));
-        ade::RateParams rp;
-        memset(&rp, 0, sizeof(rp));
-        rp.n = c->n;
-        rp.ncy = g.nc[1];
-        rp.ncz = g.nc[2];
-        const dim3 d = ade::frozen_grid(rp);
-        *blocks = std::max(*blocks, (int)(d.x * d.y));
     }
     *lines = std::min(*lines, (size_t)(kFrozenMaxBytes / 128.0));
 }
@@ -1000,6 +995,7 @@ int ade_init_particles(ade_ctx **out, const ade_params *p, int n, uint32_t *xq_d
     c->frozen = d.fz_lines > 0;
     c->frozen_tab.words = at<float>(workspace_dev, d.L.fz_words);
     c->frozen_tab.slots = at<uint4>(workspace_dev, d.L.fz_slots);
+    c->frozen_tab.dense = at<uint32_t>(workspace_dev, d.L.fz_dense);
     c->frozen_C = at<float>(workspace_dev, d.L.fz_C);
     c->frozen_tab.cursor = at<unsigned>(workspace_dev, d.L.fz_cursor);
     c->frozen_lines = d.fz_lines;
@@ -1610,7 +1606,7 @@ struct BatchLayout {
 
 // Size of a batch's weight table over every subdivision its plumes may be given (0: none).
 struct BatchFrozen {
-    size_t lines = 0, pencils = 0, items = 0;
+    size_t lines = 0, items = 0;
     std::vector<size_t> plume;          // lines of each plume
 };
 
@@ -1619,7 +1615,7 @@ BatchFrozen batch_frozen_size(int P, const ade_params *p, const int *n)
     BatchFrozen f;
     for (int i = 0; i < P; ++i) {
         const double H = p[i].kernel == ADE_WENDLAND_C2 ? 2.0 * p[i].h : p[i].h;
-        size_t lines = 0, pencils = 0, items = 0, least = 0;
+        size_t lines = 0, items = 0, least = 0;
         for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
             Grid g;
             if (!make_grid(p[i], H, k, &g)) continue;
@@ -1631,12 +1627,10 @@ BatchFrozen batch_frozen_size(int P, const ade_params *p, const int *n)
             if (!make_grid(p[i], H, k, &g)) continue;
             const size_t np = (size_t)(g.ncells / g.nc[0]), l = frozen_lines(p[i], H, n[i], g);
             if (l <= least + least / 5) lines = std::max(lines, l);   // (see frozen_room)
-            pencils = std::max(pencils, np);
-            items = std::max(items, np + (size_t)n[i] / 32);
+            items = std::max(items, (size_t)ade::chunk_numbers(n[i], (int)np));
         }
         f.lines += lines;
         f.plume.push_back(lines);
-        f.pencils += pencils;
         f.items += items;
     }
     if (128.0 * (double)f.lines > kFrozenMaxBytes) f = BatchFrozen();
@@ -1653,7 +1647,7 @@ BatchLayout batch_layout(int P, int N, int NC_max, int max_tiles, const BatchFro
         return o;
     };
     L.fz_words = take(fz.lines * 128);
-    L.fz_slots = take(fz.lines > 0 ? ((size_t)N / 32 + fz.pencils + 2) * 16 : 0);
+    L.fz_slots = take(fz.items * 32);
     L.fz_C = take(fz.lines > 0 ? (size_t)N * 16 : 0);
     L.fz_cursor = take(64);
     L.fz_items = take(fz.items * sizeof(ade::FrozenItem));
@@ -1735,7 +1729,6 @@ int batch_plan(ade_batch *b)
 {
     b->NC = 0;
     b->items.clear();
-    int p0 = 0;
     unsigned fz_line = 0u;
     b->frozen_fits = true;
     std::vector<std::pair<double, ade::BatchTile>> items;
@@ -1778,15 +1771,8 @@ int batch_plan(ade_batch *b)
         }
         b->pred[i] = pr;
         b->corr[i] = co;
-        // chunks of the weight table: enough items per pencil for its mean population
-        if (b->frozen) {
-            const int np = d.g.ncells / d.g.nc[0];
-            const int ny = std::max(1, std::min(65535, b->n[i] / np / 32));
-            for (int q = 0; q < np; ++q)
-                for (int y = 0; y < ny; ++y)
-                    b->items.push_back(ade::FrozenItem{i, q, p0, (unsigned short)y, (unsigned short)ny});
-            p0 += np;
-        }
+        if (b->frozen)   // chunks of the weight table
+            for (int t = 0; t < ade::chunk_numbers(b->n[i], d.g.ncells / d.g.nc[0]); ++t) b->items.push_back(ade::FrozenItem{i, t});
         // work items and their estimated cost: candidates per particle x particles
         const double ppc = (double)b->n[i] / d.g.ncells;
         double cand = 0.0;
@@ -2375,7 +2361,7 @@ namespace {
 
 struct SweepLayout {
     Derived d;
-    size_t Cs0, Cs1, pstats, words, slots, cursor, lines, total;
+    size_t Cs0, Cs1, pstats, words, slots, dense, cursor, lines, total;
 };
 
 // Common parameters and workspace of a sweep.  theta may be NULL (workspace size only: the layout
@@ -2436,7 +2422,8 @@ int sweep_layout(const ade_params *p, int n, int P, const double *theta, ade_par
     L->pstats = take((size_t)3 * P * 8);
     L->lines = n > 0 ? std::min(frozen_lines(pp, L->d.H, n, L->d.g, 2), (size_t)(kFrozenMaxBytes / 128.0)) : 0;
     L->words = take(L->lines * 128);
-    L->slots = take(frozen_slots(n, L->d.g) * 16);
+    L->slots = take(frozen_slots(n, L->d.g) * 32);
+    L->dense = take(frozen_slots(n, L->d.g) * 4);
     L->cursor = take(64);
     L->total = off;
     if (pp_out) *pp_out = pp;
@@ -2649,6 +2636,7 @@ int ade_sweep_init(ade_sweep **out, const ade_params *p, int n, int ntheta, cons
     sw->run.Ch = sw->Cs1;
     sw->run.tab.words = at<float>(workspace_dev, L.words);
     sw->run.tab.slots = at<uint4>(workspace_dev, L.slots);
+    if (ade::chunk_numbers(n, L.d.g.nc[1] * L.d.g.nc[2]) > ade::kCountChunksFrom) sw->run.tab.dense = at<uint32_t>(workspace_dev, L.dense);
     sw->run.tab.cursor = at<unsigned>(workspace_dev, L.cursor);
     sw->rp.fz_stride = n > 0 ? frozen_stride(pp, L.d.H, n, L.d.g, 2, L.lines) : 0u;
     sw->run.tab.pool = (unsigned)(frozen_slots(n, L.d.g) * sw->rp.fz_stride);

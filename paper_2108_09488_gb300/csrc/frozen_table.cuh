@@ -18,11 +18,84 @@
 
 constexpr unsigned kFull = 0xffffffffu;
 
-// Where one warp's chunk lies: particles [i0, min(i0 + 32, pe)) of pencil p (cy, cz).
+// Where one warp's chunk lies: particles [i0, min(i0 + 32, pe)) of pencil p (cy, cz), which holds [ps, pe).
 struct Chunk {
-    int cy, cz, i0, ps, pe;
+    int cy, cz, i0, ps, pe, p;
     int local, slot;       // the chunk's number within its plume, and in the slot table
 };
+
+// Chunk number t of a plume.  Pencil p's first chunk has the number dense[p] (counted), or where that is NULL
+// (first particle >> 5) + p: strictly increasing, with at most one number per pencil that no chunk has.
+// So a launch takes one warp per number whatever the set: a pencil's share of the warps is its share of the particles
+// (launched by pencil, with the mean pencil's number of warps each, a set that fills 5 % of the box ran 4 to 9
+// times slower, and more particles than 65,535 blocks of one pencil could not be launched).
+// The warp finds the pencil by its lanes looking at 32 pencils around the place an even set has it in, one
+// latency on a lattice, and otherwise by a search that divides the pencils in 32 each time.
+// False where no chunk has the number.
+__device__ __forceinline__ bool find_chunk(const uint32_t *__restrict__ cs, const RateParams &prm, const uint32_t *__restrict__ dense, int t,
+                                           Chunk &c)
+{
+    const int lane = threadIdx.x & 31, np = prm.ncy * prm.ncz, ncx = prm.ncx;
+    const int total = dense ? (int)__ldg(dense + np) : chunk_numbers(prm.n, np);
+    if (t >= total) return false;
+    auto first = [&](int q, int &s) {      // the number of pencil q's first chunk; s: its first particle
+        s = (int)__ldg(cs + (size_t)q * ncx);
+        return dense ? (int)__ldg(dense + q) : ((s - prm.goff) >> 5) + q;
+    };
+    const int lo = max(0, min((int)((float)t * ((float)np / (float)total)) - 15, np - 31));
+    int s;
+    int k = __popc(__ballot_sync(kFull, first(min(lo + lane, np), s) <= t && lo + lane < np));
+    if (k > 0 && k < 32) {
+        c.p = lo + k - 1;
+        c.ps = __shfl_sync(kFull, s, k - 1);
+        c.pe = __shfl_sync(kFull, s, k);
+    } else {
+        int a = k > 0 ? lo + 31 : 0, b = k > 0 ? np : lo;   // pencil a begins at or before t, pencil b after it
+        while (b - a > 1) {
+            const int step = (b - a + 31) >> 5, q = min(a + step * lane, b);
+            k = __popc(__ballot_sync(kFull, q < b && first(q, s) <= t));
+            b = min(a + step * k, b);
+            a += step * (k - 1);
+        }
+        c.p = a;
+        c.ps = (int)__ldg(cs + (size_t)a * ncx);
+        c.pe = (int)__ldg(cs + (size_t)a * ncx + ncx);
+    }
+    c.i0 = c.ps + 32 * (t - (dense ? (int)__ldg(dense + c.p) : ((c.ps - prm.goff) >> 5) + c.p));
+    c.cy = c.p % prm.ncy;
+    c.cz = c.p / prm.ncy;
+    c.local = c.slot = t;
+    return c.i0 < c.pe;
+}
+
+// The slot table: per number {first line, rows, lines, header lines} and {first particle, pencil's first,
+// pencil's end, pencil}.  The kernel that fills the table writes both, later passes read them.
+__device__ __forceinline__ void put_chunk(const FrozenTab &tab, const Chunk &c, bool has)
+{
+    if ((threadIdx.x & 31) == 0)
+        tab.slots[2 * (size_t)c.slot + 1] = has ? make_uint4((unsigned)c.i0, (unsigned)c.ps, (unsigned)c.pe, (unsigned)c.p)
+                                                : make_uint4(0u, 0u, 0u, 0u);
+}
+
+__device__ __forceinline__ bool get_chunk(const FrozenTab &tab, const RateParams &prm, int slot, Chunk &c, uint4 &sl)
+{
+    const uint4 w = __ldg(tab.slots + 2 * (size_t)slot + 1);
+    sl = __ldg(tab.slots + 2 * (size_t)slot);
+    c.i0 = (int)w.x;
+    c.ps = (int)w.y;
+    c.pe = (int)w.z;
+    c.p = (int)w.w;
+    c.slot = slot;
+    return c.i0 < c.pe;
+}
+
+// This warp's number in a launch of frozen_blocks blocks, and the same for a chunk already in the table.
+__device__ __forceinline__ int warp_number() { return blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); }
+__device__ __forceinline__ bool my_chunk(const FrozenTab &tab, const RateParams &prm, Chunk &c, uint4 &sl)
+{
+    const int t = warp_number();
+    return t < chunk_numbers(prm.n, prm.ncy * prm.ncz) && get_chunk(tab, prm, t, c, sl);
+}
 
 // Origin of the build's cell grid along x (the records hold the positions of the build: no drift).
 __device__ __forceinline__ uint32_t frame_x(const RateParams &prm) { return prm.frame ? __ldg(prm.frame + 4) : 0u; }
@@ -251,11 +324,12 @@ __device__ __noinline__ float walk_chunk(const uint4 *__restrict__ P, const uint
     const float Ca = C ? C[c.ps + i] : __uint_as_float(pa.w);
     const int ncx = prm.ncx;
     const int cx = (int)__umulhi(pa.x - frame_x(prm), (uint32_t)ncx);
+    const int cy = c.p % prm.ncy, cz = c.p / prm.ncy;
     const PairConst k(prm);
     float acc = 0.f, comp = 0.f;
     for (int r = 0; r < prm.nrows; ++r) {
         const StencilRow row = prm.rows[r];
-        const int q = row_pencil_of<DIM>(row, c.cy, c.cz, prm);
+        const int q = row_pencil_of<DIM>(row, cy, cz, prm);
         const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
         int s, cnt;
         cyclic_range(cs, q * ncx, cx - (int)row.w, cx + row.w + 1, ncx, qs, qe, s, cnt);
@@ -431,7 +505,7 @@ __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const 
         base = tab.pool + at;
         room = used;
     }
-    if (lane == 0) tab.slots[c.slot] = make_uint4(used <= room ? base : kNoRoom, R, used, hs);
+    if (lane == 0) tab.slots[2 * (size_t)c.slot] = make_uint4(used <= room ? base : kNoRoom, R, used, hs);
     if (VAL == 1 && used > room) return walk_chunk<DIM, KERNEL, ISO>(P, cs, prm, c, nullptr);
     return acc + comp;
 }
@@ -531,21 +605,4 @@ __device__ __forceinline__ float stream_chunk(const uint4 sl, const FrozenTab &t
     WeightedSum op{C, Ca, 0.f, 0.f, 0.f};
     stream_rows<1>(sl, tab, op);
     return op.acc + op.comp;
-}
-
-// The warp's chunks: warp v of pencil p takes chunks v, v + nv, ...
-template <class F>
-__device__ __forceinline__ void for_chunks(const uint32_t *__restrict__ cs, const RateParams &prm, int p, int p0, int v, int nv,
-                                           F f)
-{
-    Chunk c;
-    c.cy = p % prm.ncy;
-    c.cz = p / prm.ncy;
-    c.ps = (int)__ldg(cs + p * prm.ncx);
-    c.pe = (int)__ldg(cs + p * prm.ncx + prm.ncx);
-    for (c.i0 = c.ps + 32 * v; c.i0 < c.pe; c.i0 += 32 * nv) {
-        c.local = ((c.i0 - prm.goff) >> 5) + p;   // increases strictly from chunk to chunk
-        c.slot = (c.i0 >> 5) + p0 + p;
-        f(c);
-    }
 }

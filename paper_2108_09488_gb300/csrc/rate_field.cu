@@ -368,7 +368,7 @@ __global__ __launch_bounds__(kT) void k_rate_field2(const uint4 *__restrict__ Pe
     warp_finish<EPI, false, kT>(acc, out);
 }
 
-// 3D: a warp takes chunks of up to 32 consecutive particles of one pencil (for_chunks), so its lanes share the
+// 3D: a warp takes up to 32 consecutive particles of one pencil (find_chunk), so its lanes share the
 // stencil rows; each lane's range of a row is cut by the distance its own cell position leaves to the
 // row's cell band, for the grid's radius H + dt vmax (positions of the build: the drift since cannot
 // bring a pair within H that was beyond it).  The candidates are only tested first, and those in support
@@ -399,11 +399,10 @@ __global__ __launch_bounds__(kT) void k_rate_field3(const uint4 *__restrict__ Pe
     unsigned *list = lists[wid] + lane;
     TrimGeom g(prm);
     g.Hm2 = prm.Hg2 * (1.f + 1.f / 2048.f);
-    const int v = SPLIT > 1 ? blockIdx.y : blockIdx.y * (kT / 32) + wid;
-    const int nv = SPLIT > 1 ? gridDim.y : gridDim.y * (kT / 32);
-    for_chunks(cs, prm, blockIdx.x, 0, v, nv, [&](const Chunk &c) {
+    Chunk c;
+    if (find_chunk(cs, prm, nullptr, SPLIT > 1 ? (int)blockIdx.x : warp_number(), c)) {   // (SPLIT: the same for the whole block)
         const int i = c.i0 + lane;
-        const bool valid = i < c.pe;
+        bool valid = i < c.pe;
         const int ii = valid ? i : c.pe - 1;
         const uint4 pa = __ldg(Pe + ii);
         // fixed-point drift of this particle; the cell of the cell build is the evaluation position
@@ -467,11 +466,11 @@ __global__ __launch_bounds__(kT) void k_rate_field3(const uint4 *__restrict__ Pe
                     cc += o.w;
                 }
             __syncthreads();
-            if (wid != 0) return;
+            if (wid != 0) valid = false;
         }
-        if (!valid) return;
         const float rate = fmaf(prm.pf, sd + cd, fp.pconv * t.Ca * (sc + cc));
-        if (EPI == EPI_RATE) {
+        if (!valid) {
+        } else if (EPI == EPI_RATE) {
             if (out.rate) {
                 const uint32_t a = __ldg(perm + i);
                 if (a < (uint32_t)prm.n) out.rate[a] = rate;
@@ -505,18 +504,15 @@ __global__ __launch_bounds__(kT) void k_rate_field3(const uint4 *__restrict__ Pe
             acc.mn = fminf(acc.mn, Cn);
             acc.mx = fmaxf(acc.mx, Cn);
         }
-    });
-    if (EPI == EPI_CORRECT) {   // one partial per warp that took chunks (SPLIT: the block's first)
+    }
+    if (EPI == EPI_CORRECT) {   // one partial per warp (SPLIT: the block's first)
         const float4 r = warp_partial(acc);
-        if (lane == 0 && (SPLIT == 1 || wid == 0)) {
-            const size_t blk = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
-            out.wpart[SPLIT == 1 ? blk * (kT / 32) + wid : blk] = r;
-        }
+        if (lane == 0 && (SPLIT == 1 || wid == 0)) out.wpart[SPLIT == 1 ? warp_number() : (int)blockIdx.x] = r;
     }
 }
 
 template <int KERNEL, int SPLIT>
-cudaError_t launch_field3(int epi, dim3 grid, const uint4 *Pe, const uint32_t *cs, const uint32_t *perm,
+cudaError_t launch_field3(int epi, unsigned grid, const uint4 *Pe, const uint32_t *cs, const uint32_t *perm,
                           const FieldWork &fw, const RateParams &prm, const FieldParams &fp, const EpiOut &out,
                           cudaStream_t s)
 {
@@ -548,20 +544,15 @@ cudaError_t launch_field2(int epi, const uint4 *Pe, const uint32_t *cs, const ui
 // Chunks of a set that fills the chip less than about twice (152 SMs of 24 warps) are shared by the four
 // warps of a block.
 bool field_split(const RateParams &prm) { return prm.n / 32 < 2 * 152 * 24; }
-unsigned field_split_y(const RateParams &prm)   // a block per chunk of the mean pencil
-{
-    return (unsigned)std::max(1, (prm.n / (prm.ncy * prm.ncz) + 31) / 32);
-}
+int field_chunks(const RateParams &prm) { return chunk_numbers(prm.n, prm.ncy * prm.ncz); }
 
 template <int KERNEL>
 cudaError_t launch_field_k(int dim, int epi, const uint4 *Pe, const uint32_t *cs, const uint32_t *perm, const FieldWork &fw,
                     const RateParams &prm, const FieldParams &fp, const EpiOut &out, cudaStream_t s)
 {
     if (dim == 2) return launch_field2<KERNEL>(epi, Pe, cs, perm, fw, prm, fp, out, s);
-    dim3 g = frozen_grid(prm);
-    if (!field_split(prm)) return launch_field3<KERNEL, 1>(epi, g, Pe, cs, perm, fw, prm, fp, out, s);
-    g.y = field_split_y(prm);
-    return launch_field3<KERNEL, 4>(epi, g, Pe, cs, perm, fw, prm, fp, out, s);
+    if (!field_split(prm)) return launch_field3<KERNEL, 1>(epi, frozen_blocks(prm), Pe, cs, perm, fw, prm, fp, out, s);
+    return launch_field3<KERNEL, 4>(epi, (unsigned)field_chunks(prm), Pe, cs, perm, fw, prm, fp, out, s);
 }
 
 }  // namespace
@@ -569,8 +560,7 @@ cudaError_t launch_field_k(int dim, int epi, const uint4 *Pe, const uint32_t *cs
 int field_partials(int dim, const RateParams &prm)
 {
     if (dim == 2) return (prm.n + kT - 1) / kT * (kT / 32);
-    const dim3 g = frozen_grid(prm);
-    return field_split(prm) ? (int)(g.x * field_split_y(prm)) : (int)(g.x * g.y) * (kT / 32);
+    return field_split(prm) ? field_chunks(prm) : (int)frozen_blocks(prm) * (kT / 32);
 }
 
 cudaError_t launch_field_records(int dim, const float *v_dev, int n, const FieldParams &fp, const FieldWork &fw,

@@ -59,47 +59,52 @@ __global__ __launch_bounds__(kT) void k_frozen_build(const uint4 *__restrict__ P
     pdl_wait();
     __shared__ TrimRow srow[ISO ? kMaxRows : 1];
     if (ISO) stage_trim_rows(srow, prm);
-    const int nv = gridDim.y * (kT / 32);
-    for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), nv, [&](const Chunk &c) {
-        const int i = c.i0 + (threadIdx.x & 31);
-        const uint4 pa = __ldg(P + min(i, c.pe - 1));
-        const float sum = build_chunk<DIM, KERNEL, ISO, ISO ? kCutBox : kCutFull, 1>(P, cs, prm, c, pa, srow, tab);
-        if (i >= c.pe) return;
-        const float Cl = __uint_as_float(pa.w);
-        st.C[c.ps + i] = st.C[c.pe + i] = Cl;
-        float ql = 0.f;
-        if (st.Qs) {
-            const uint32_t a = __ldg(perm + i);
-            ql = a < (uint32_t)prm.n ? st.Q[a] : 0.f;
-            st.Qs[i] = ql;
-        }
-        frozen_epilogue<EPI_PREDICT>(prm, st, c, i, prm.upf * shape_unscale<KERNEL>() * sum, Cl, ql);
-    });
+    Chunk c;
+    const int t = warp_number();
+    const bool has = find_chunk(cs, prm, tab.dense, t, c);
+    if (t < chunk_numbers(prm.n, prm.ncy * prm.ncz)) put_chunk(tab, c, has);
+    if (!has) return;
+    const int i = c.i0 + (threadIdx.x & 31);
+    const uint4 pa = __ldg(P + min(i, c.pe - 1));
+    const float sum = build_chunk<DIM, KERNEL, ISO, ISO ? kCutBox : kCutFull, 1>(P, cs, prm, c, pa, srow, tab);
+    if (i >= c.pe) return;
+    const float Cl = __uint_as_float(pa.w);
+    st.C[c.ps + i] = st.C[c.pe + i] = Cl;
+    float ql = 0.f;
+    if (st.Qs) {
+        const uint32_t a = __ldg(perm + i);
+        ql = a < (uint32_t)prm.n ? st.Q[a] : 0.f;
+        st.Qs[i] = ql;
+    }
+    frozen_epilogue<EPI_PREDICT>(prm, st, c, i, prm.upf * shape_unscale<KERNEL>() * sum, Cl, ql);
 }
 
 // One evaluation from the table.  Bound: HBM where the table exceeds L2 (4 bytes per pair and the idle
 // tails of rows), latency below.  Per evaluation, walk / table: 128^3 cube, 250 neighbours, 700 / 412 us
 // (2.6 GB, 6.2 TB/s of the 6.7 a copy reaches); 1024^2, 120 neighbours 124 / 101; 512^2, 60 about 30 / 18.5;
-// 256^2, 28 7.5 / 5.3.  Twelve CTAs per SM: the loads in flight are what the stream lives on.
-template <int DIM, int KERNEL, bool ISO, int EPI>
-__global__ __launch_bounds__(kT, 12) void k_frozen_rate(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
+// 256^2, 28 7.5 / 5.3.  The loads in flight are what the stream lives on: CTAS per SM, 12 (40 registers) on
+// large sets and 16 (32, of which three words spill) up to kWideFrom chunk numbers, where a last wave that is
+// nearly empty weighs more (per step, 12 / 16: 512^2 41.8 / 36.3 us, 64^3 175 / 163, 72^3 272 / 253; 100^3
+// 595 / 601, 128^3 955 / 961).
+constexpr int kWideFrom = 4 * 152 * 48;
+template <int DIM, int KERNEL, bool ISO, int EPI, int CTAS>
+__global__ __launch_bounds__(kT, CTAS) void k_frozen_rate(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
                                                     const RateParams prm, const FrozenTab tab, const FrozenState st)
 {
     pdl_wait();
-    const int nv = gridDim.y * (kT / 32);
-    for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), nv, [&](const Chunk &c) {
-        const float *Ce = EPI == EPI_PREDICT ? st.C : st.Ch;
-        const int i = c.i0 + (threadIdx.x & 31);
-        const uint4 sl = __ldg(tab.slots + c.slot);
-        const float sum = sl.x != kNoRoom ? stream_chunk(sl, tab, Ce, Ce[c.ps + min(i, c.pe - 1)])
-                                          : walk_chunk<DIM, KERNEL, ISO>(P, cs, prm, c, Ce);
-        if (i >= c.pe) return;
-        frozen_epilogue<EPI>(prm, st, c, i, prm.upf * shape_unscale<KERNEL>() * sum, st.C[c.ps + i], st.Qs ? st.Qs[i] : 0.f);
-    });
+    Chunk c;
+    uint4 sl;
+    if (!my_chunk(tab, prm, c, sl)) return;
+    const float *Ce = EPI == EPI_PREDICT ? st.C : st.Ch;
+    const int i = c.i0 + (threadIdx.x & 31);
+    const float sum = sl.x != kNoRoom ? stream_chunk(sl, tab, Ce, Ce[c.ps + min(i, c.pe - 1)])
+                                      : walk_chunk<DIM, KERNEL, ISO>(P, cs, prm, c, Ce);
+    if (i >= c.pe) return;
+    frozen_epilogue<EPI>(prm, st, c, i, prm.upf * shape_unscale<KERNEL>() * sum, st.C[c.ps + i], st.Qs ? st.Qs[i] : 0.f);
 }
 
-// Batched plumes: one work item per warp, chunks y, y + ny, ... of one pencil of one plume (the cell
-// table and the sorted arrays are the batch's; no pencil boxes).
+// Batched plumes: one chunk of one plume per warp (the cell table and the sorted arrays are the batch's; no
+// pencil boxes).
 template <int DIM, int KERNEL>
 __global__ __launch_bounds__(kT) void k_frozen_build_batch(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
                                                            const RateParams *__restrict__ descs,
@@ -111,15 +116,18 @@ __global__ __launch_bounds__(kT) void k_frozen_build_batch(const uint4 *__restri
     if (w >= nitems) return;
     const FrozenItem it = items[w];
     const RateParams &prm = descs[it.plume];
-    for_chunks(cs + prm.coff, prm, it.pencil, it.p0, it.y, it.ny, [&](const Chunk &c) {
-        const int i = c.i0 + (threadIdx.x & 31);
-        const uint4 pa = __ldg(P + min(i, c.pe - 1));
-        const float sum = build_chunk<DIM, KERNEL, true, kCutBand, 1>(P, cs + prm.coff, prm, c, pa, nullptr, tab);
-        if (i >= c.pe) return;
-        const float Cl = __uint_as_float(pa.w);
-        st.C[c.ps + i] = st.C[c.pe + i] = Cl;
-        frozen_epilogue<EPI_PREDICT>(prm, st, c, i, prm.upf * shape_unscale<KERNEL>() * sum, Cl, 0.f);
-    });
+    Chunk c;
+    const bool has = find_chunk(cs + prm.coff, prm, nullptr, it.chunk, c);
+    c.slot = w;
+    put_chunk(tab, c, has);
+    if (!has) return;
+    const int i = c.i0 + (threadIdx.x & 31);
+    const uint4 pa = __ldg(P + min(i, c.pe - 1));
+    const float sum = build_chunk<DIM, KERNEL, true, kCutBand, 1>(P, cs + prm.coff, prm, c, pa, nullptr, tab);
+    if (i >= c.pe) return;
+    const float Cl = __uint_as_float(pa.w);
+    st.C[c.ps + i] = st.C[c.pe + i] = Cl;
+    frozen_epilogue<EPI_PREDICT>(prm, st, c, i, prm.upf * shape_unscale<KERNEL>() * sum, Cl, 0.f);
 }
 
 template <int DIM, int KERNEL, int EPI>
@@ -131,17 +139,56 @@ __global__ __launch_bounds__(kT, 12) void k_frozen_rate_batch(const uint4 *__res
     pdl_wait();
     const int w = blockIdx.x * (kT / 32) + (threadIdx.x >> 5);
     if (w >= nitems) return;
-    const FrozenItem it = items[w];
-    const RateParams &prm = descs[it.plume];
-    for_chunks(cs + prm.coff, prm, it.pencil, it.p0, it.y, it.ny, [&](const Chunk &c) {
-        const float *Ce = EPI == EPI_PREDICT ? st.C : st.Ch;
-        const int i = c.i0 + (threadIdx.x & 31);
-        const uint4 sl = __ldg(tab.slots + c.slot);
-        const float sum = sl.x != kNoRoom ? stream_chunk(sl, tab, Ce, Ce[c.ps + min(i, c.pe - 1)])
-                                          : walk_chunk<DIM, KERNEL, true>(P, cs + prm.coff, prm, c, Ce);
-        if (i >= c.pe) return;
-        frozen_epilogue<EPI>(prm, st, c, i, prm.upf * shape_unscale<KERNEL>() * sum, st.C[c.ps + i], 0.f);
-    });
+    const RateParams &prm = descs[items[w].plume];
+    Chunk c;
+    uint4 sl;
+    if (!get_chunk(tab, prm, w, c, sl)) return;
+    const float *Ce = EPI == EPI_PREDICT ? st.C : st.Ch;
+    const int i = c.i0 + (threadIdx.x & 31);
+    const float sum = sl.x != kNoRoom ? stream_chunk(sl, tab, Ce, Ce[c.ps + min(i, c.pe - 1)])
+                                      : walk_chunk<DIM, KERNEL, true>(P, cs + prm.coff, prm, c, Ce);
+    if (i >= c.pe) return;
+    frozen_epilogue<EPI>(prm, st, c, i, prm.upf * shape_unscale<KERNEL>() * sum, st.C[c.ps + i], 0.f);
+}
+
+constexpr int kCountT = 1024, kCountItems = 16;
+
+// Chunks before each pencil: one block, kCountItems pencils per thread at a time (their loads in flight
+// together: 16,384 pencils in one go).
+__global__ __launch_bounds__(kCountT) void k_chunk_numbers(const uint32_t *__restrict__ cs, int np, int ncx,
+                                                           uint32_t *__restrict__ dense)
+{
+    pdl_wait();
+    __shared__ uint32_t warp_sum[kCountT / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t carry = 0u;
+    for (int base = 0; base < np; base += kCountT * kCountItems) {
+        const int q0 = base + (int)threadIdx.x * kCountItems;
+        uint32_t at[kCountItems + 1], sum = 0u;
+#pragma unroll
+        for (int k = 0; k <= kCountItems; ++k) at[k] = __ldg(cs + (size_t)min(q0 + k, np) * ncx);
+#pragma unroll
+        for (int k = 0; k < kCountItems; ++k) sum += (at[k + 1] - at[k] + 31u) >> 5;
+        uint32_t incl = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(kFull, incl, o);
+            incl += lane >= o ? v : 0u;
+        }
+        if (lane == 31) warp_sum[wid] = incl;
+        __syncthreads();
+        uint32_t run = carry + incl - sum;
+        for (int w = 0; w < kCountT / 32; ++w) {
+            run += w < wid ? warp_sum[w] : 0u;
+            carry += warp_sum[w];
+        }
+#pragma unroll
+        for (int k = 0; k < kCountItems; ++k) {
+            if (q0 + k < np) dense[q0 + k] = run;
+            run += (at[k + 1] - at[k] + 31u) >> 5;
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) dense[np] = carry;
 }
 
 // The state after `steps` steps of every plume, in the caller's order (descs: the correctors').
@@ -214,31 +261,30 @@ template <int DIM, int KERNEL, bool ISO>
 cudaError_t build_t(const uint4 *P, const uint32_t *cs, const uint32_t *perm, const RateParams &prm,
                     const FrozenTab &tab, const FrozenState &st, cudaStream_t s)
 {
-    return launch_pdl(k_frozen_build<DIM, KERNEL, ISO>, frozen_grid(prm), kT, 0, s, P, cs, perm, prm, tab, st);
+    return launch_pdl(k_frozen_build<DIM, KERNEL, ISO>, frozen_blocks(prm), kT, 0, s, P, cs, perm, prm, tab, st);
 }
 
 template <int DIM, int KERNEL, bool ISO>
 cudaError_t rate_t(int epi, const uint4 *P, const uint32_t *cs, const RateParams &prm, const FrozenTab &tab,
                    const FrozenState &st, cudaStream_t s)
 {
-    return epi == EPI_PREDICT
-               ? launch_pdl(k_frozen_rate<DIM, KERNEL, ISO, EPI_PREDICT>, frozen_grid(prm), kT, 0, s, P, cs, prm, tab, st)
-               : launch_pdl(k_frozen_rate<DIM, KERNEL, ISO, EPI_CORRECT>, frozen_grid(prm), kT, 0, s, P, cs, prm, tab, st);
+    auto go = [&](auto kernel) { return launch_pdl(kernel, frozen_blocks(prm), kT, 0, s, P, cs, prm, tab, st); };
+    if (chunk_numbers(prm.n, prm.ncy * prm.ncz) > kWideFrom)
+        return epi == EPI_PREDICT ? go(k_frozen_rate<DIM, KERNEL, ISO, EPI_PREDICT, 12>) : go(k_frozen_rate<DIM, KERNEL, ISO, EPI_CORRECT, 12>);
+    return epi == EPI_PREDICT ? go(k_frozen_rate<DIM, KERNEL, ISO, EPI_PREDICT, 16>) : go(k_frozen_rate<DIM, KERNEL, ISO, EPI_CORRECT, 16>);
 }
 
 }  // namespace
 
-// Grid: one block column per pencil, enough blocks along y for the mean pencil's chunks (a fuller
-// pencil's warps take several).  A grid of less than about four waves gets twice that, so that on a
-// small set one full pencil (two lattice lines where the others hold one) does not make a tail:
-// 256^2 at 3 cells per H 11.6 -> 8.3 us per evaluation.
-dim3 frozen_grid(const RateParams &prm)
+unsigned frozen_blocks(const RateParams &prm)
 {
-    const int np = prm.ncy * prm.ncz;
-    const int mean = (prm.n + np - 1) / np;
-    int y = (mean + kT - 1) / kT;
-    if ((long long)np * y < 8192) y *= 2;
-    return dim3((unsigned)np, (unsigned)(y > 0 ? y : 1), 1);
+    return (unsigned)((chunk_numbers(prm.n, prm.ncy * prm.ncz) + kT / 32 - 1) / (kT / 32));
+}
+
+cudaError_t launch_chunk_numbers(const uint32_t *cs, const RateParams &prm, uint32_t *dense, cudaStream_t s)
+{
+    if (!dense) return cudaSuccess;
+    return launch_pdl(k_chunk_numbers, 1u, kCountT, 0, s, cs, prm.ncy * prm.ncz, prm.ncx, dense);
 }
 
 cudaError_t launch_frozen_build(int dim, int kernel, bool iso, const uint4 *P, const uint32_t *cs, const uint32_t *perm,

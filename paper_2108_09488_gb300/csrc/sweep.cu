@@ -75,13 +75,6 @@ __device__ __forceinline__ void store_group(float *p, size_t plane, size_t j, co
 // The group's first plane, at its first set's word.
 __device__ __forceinline__ size_t group_base(int g0, size_t plane) { return (size_t)(g0 >> 2) * plane * 4 + (size_t)(g0 & 3); }
 
-// The warp's chunks of the block's pencil.
-template <class F>
-__device__ __forceinline__ void block_chunks(const uint32_t *__restrict__ cs, const RateParams &prm, F f)
-{
-    for_chunks(cs, prm, blockIdx.x, 0, blockIdx.y * (kT / 32) + (threadIdx.x >> 5), gridDim.y * (kT / 32), f);
-}
-
 // Sorted concentrations of one particle, C[p n + perm[i]], at words j0 and j1.
 __device__ __forceinline__ void gather_sets(const uint32_t *__restrict__ perm, const float *__restrict__ C, size_t n, int P,
                                             int P4, int i, size_t plane, size_t j0, size_t j1, float *__restrict__ Cs)
@@ -116,12 +109,15 @@ __global__ __launch_bounds__(kT) void k_sweep_table(const uint4 *__restrict__ P,
     pdl_wait();
     __shared__ TrimRow srow[ISO ? kMaxRows : 1];
     if (ISO) stage_trim_rows(srow, prm);
-    block_chunks(cs, prm, [&](const Chunk &c) {
-        const int i = c.i0 + (threadIdx.x & 31);
-        if (i < c.pe) gather_sets(perm, C, (size_t)prm.n, sets, P4, i, 2 * (size_t)prm.n, (size_t)(c.ps + i), (size_t)(c.pe + i), Cs);
-        const uint4 pa = __ldg(P + min(i, c.pe - 1));
-        build_chunk<DIM, KERNEL, ISO, ISO ? kCutBox : kCutFull, 2>(P, cs, prm, c, pa, srow, tab, sc);
-    });
+    Chunk c;
+    const int t = warp_number();
+    const bool has = find_chunk(cs, prm, tab.dense, t, c);
+    if (t < chunk_numbers(prm.n, prm.ncy * prm.ncz)) put_chunk(tab, c, has);
+    if (!has) return;
+    const int i = c.i0 + (threadIdx.x & 31);
+    if (i < c.pe) gather_sets(perm, C, (size_t)prm.n, sets, P4, i, 2 * (size_t)prm.n, (size_t)(c.ps + i), (size_t)(c.pe + i), Cs);
+    const uint4 pa = __ldg(P + min(i, c.pe - 1));
+    build_chunk<DIM, KERNEL, ISO, ISO ? kCutBox : kCutFull, 2>(P, cs, prm, c, pa, srow, tab, sc);
 }
 
 // sum_b (d_L g_L + d_T g_T)(C_a - C_b) of NT sets, two sets to a packed FP32x2 instruction.
@@ -181,11 +177,12 @@ __device__ __noinline__ void walk_sets(const uint4 *__restrict__ P, const uint32
     const uint4 pa = __ldg(P + min(c.i0 + (int)(threadIdx.x & 31), c.pe - 1));
     const int ncx = prm.ncx;
     const int cx = (int)__umulhi(pa.x - frame_x(prm), (uint32_t)ncx);
+    const int cy = c.p % prm.ncy, cz = c.p / prm.ncy;
     const PairConst kc(prm);
     const PairConst2 k(kc, kc.m1);
     for (int r = 0; r < prm.nrows; ++r) {
         const StencilRow row = prm.rows[r];
-        const int q = row_pencil_of<DIM>(row, c.cy, c.cz, prm);
+        const int q = row_pencil_of<DIM>(row, cy, cz, prm);
         const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
         int s, cnt;
         cyclic_range(cs, q * ncx, cx - (int)row.w, cx + row.w + 1, ncx, qs, qe, s, cnt);
@@ -214,57 +211,57 @@ __global__ __launch_bounds__(kT, 5) void k_sweep_pass(const uint4 *__restrict__ 
 {
     pdl_wait();
     const bool last = EPI == EPI_CORRECT && out.C;
-    if (last && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *tab.cursor = 0u;   // the next table starts empty
+    if (last && blockIdx.x == 0 && threadIdx.x == 0) *tab.cursor = 0u;   // the next table starts empty
     const int g0 = sp.g0;
-    block_chunks(cs, prm, [&](const Chunk &c) {
-        const int i = c.i0 + (threadIdx.x & 31);
-        const size_t plane = 2 * (size_t)prm.n, at = (size_t)(c.ps + min(i, c.pe - 1)), gb = group_base(g0, plane);
-        SetSums<NT> op;
-        op.C = (EPI == EPI_PREDICT ? C : Ch) + gb;
-        op.plane = plane;
-        op.load(at, op.Ca);
+    Chunk c;
+    uint4 sl;
+    if (!my_chunk(tab, prm, c, sl)) return;
+    const int i = c.i0 + (threadIdx.x & 31);
+    const size_t plane = 2 * (size_t)prm.n, at = (size_t)(c.ps + min(i, c.pe - 1)), gb = group_base(g0, plane);
+    SetSums<NT> op;
+    op.C = (EPI == EPI_PREDICT ? C : Ch) + gb;
+    op.plane = plane;
+    op.load(at, op.Ca);
 #pragma unroll
-        for (int k = 0; k < SetSums<NT>::N2; ++k) {
-            op.dL[k] = f2(sp.dL[2 * k], sp.dL[2 * k + 1]);
-            op.dT[k] = f2(sp.dT[2 * k], sp.dT[2 * k + 1]);
-            op.rs[k] = op.acc[k] = op.comp[k] = f2(0.f, 0.f);
-        }
-        const uint4 sl = __ldg(tab.slots + c.slot);
-        if (sl.x != kNoRoom) stream_rows<2>(sl, tab, op);
-        else walk_sets<DIM, KERNEL, ISO, NT>(P, cs, prm, c, sc, op);
-        if (i >= c.pe) return;
-        const float pf = prm.pf * shape_unscale<KERNEL>();
-        float Cl[NT], o[NT];
-        if (EPI == EPI_CORRECT) load_group<NT>(C + gb, plane, at, Cl);
+    for (int k = 0; k < SetSums<NT>::N2; ++k) {
+        op.dL[k] = f2(sp.dL[2 * k], sp.dL[2 * k + 1]);
+        op.dT[k] = f2(sp.dT[2 * k], sp.dT[2 * k + 1]);
+        op.rs[k] = op.acc[k] = op.comp[k] = f2(0.f, 0.f);
+    }
+    if (sl.x != kNoRoom) stream_rows<2>(sl, tab, op);
+    else walk_sets<DIM, KERNEL, ISO, NT>(P, cs, prm, c, sc, op);
+    if (i >= c.pe) return;
+    const float pf = prm.pf * shape_unscale<KERNEL>();
+    float Cl[NT], o[NT];
+    if (EPI == EPI_CORRECT) load_group<NT>(C + gb, plane, at, Cl);
+#pragma unroll
+    for (int k = 0; k < NT; ++k) {
+        const float2 a2 = op.acc[k / 2], c2 = op.comp[k / 2], ca = op.Ca[k / 2];
+        const float rate = pf * (k & 1 ? a2.y + c2.y : a2.x + c2.x);
+        o[k] = fmaf(prm.dt, rate, EPI == EPI_CORRECT ? Cl[k] : (k & 1 ? ca.y : ca.x));
+    }
+    if (last) {
+        const uint32_t a = __ldg(perm + i);
+        const size_t n = (size_t)prm.n;
+        if (a >= (uint32_t)n) return;
+        bool bad = false;
 #pragma unroll
         for (int k = 0; k < NT; ++k) {
-            const float2 a2 = op.acc[k / 2], c2 = op.comp[k / 2], ca = op.Ca[k / 2];
-            const float rate = pf * (k & 1 ? a2.y + c2.y : a2.x + c2.x);
-            o[k] = fmaf(prm.dt, rate, EPI == EPI_CORRECT ? Cl[k] : (k & 1 ? ca.y : ca.x));
+            out.C[(size_t)(g0 + k) * n + a] = o[k];
+            bad |= !isfinite(o[k]);
         }
-        if (last) {
-            const uint32_t a = __ldg(perm + i);
-            const size_t n = (size_t)prm.n;
-            if (a >= (uint32_t)n) return;
-            bool bad = false;
-#pragma unroll
-            for (int k = 0; k < NT; ++k) {
-                out.C[(size_t)(g0 + k) * n + a] = o[k];
-                bad |= !isfinite(o[k]);
-            }
-            if (bad) atomicOr(out.status, 1);
-            if (g0 == 0) {
-                const uint4 q = __ldg(P + i);
-                out.xq[a] = q.x + prm.inc[0];
-                out.xq[n + a] = q.y + prm.inc[1];
-                if (DIM == 3) out.xq[2 * n + a] = q.z + prm.inc[2];
-            }
-            return;
+        if (bad) atomicOr(out.status, 1);
+        if (g0 == 0) {
+            const uint4 q = __ldg(P + i);
+            out.xq[a] = q.x + prm.inc[0];
+            out.xq[n + a] = q.y + prm.inc[1];
+            if (DIM == 3) out.xq[2 * n + a] = q.z + prm.inc[2];
         }
-        float *to = (EPI == EPI_PREDICT ? Ch : C) + gb;
-        store_group<NT>(to, plane, at, o);
-        store_group<NT>(to, plane, (size_t)(c.pe + i), o);
-    });
+        return;
+    }
+    float *to = (EPI == EPI_PREDICT ? Ch : C) + gb;
+    store_group<NT>(to, plane, at, o);
+    store_group<NT>(to, plane, (size_t)(c.pe + i), o);
 }
 
 // One evaluation with the geometry computed on the fly: the rate or pair count, or a predictor (Ce -> out.Cout)
@@ -439,7 +436,7 @@ void launch_sweep_k(int epi, bool count, int blocks, const uint4 *Pe, const floa
 template <int DIM, int KERNEL, bool ISO, int NT>
 cudaError_t pass_nt(const SweepRun &r, int epi, const SweepParams &sp, const RateParams &prm, const SweepOut &out, cudaStream_t s)
 {
-    const dim3 g = frozen_grid(prm);
+    const unsigned g = frozen_blocks(prm);
     return epi == EPI_PREDICT
                ? launch_pdl(k_sweep_pass<DIM, KERNEL, ISO, NT, EPI_PREDICT>, g, kT, 0, s, r.P, r.cs, prm, r.tab, ShapeConst{float4{}, r.g2, r.bT}, sp, r.C, r.Ch, r.perm, out)
                : launch_pdl(k_sweep_pass<DIM, KERNEL, ISO, NT, EPI_CORRECT>, g, kT, 0, s, r.P, r.cs, prm, r.tab, ShapeConst{float4{}, r.g2, r.bT}, sp, r.C, r.Ch, r.perm, out);
@@ -459,7 +456,7 @@ cudaError_t pass_k(const SweepRun &r, int epi, const SweepParams &sp, const Rate
 template <int DIM, int KERNEL, bool ISO>
 cudaError_t table_k(const SweepRun &r, const RateParams &prm, const float *C, int sets, int P4, cudaStream_t s)
 {
-    return launch_pdl(k_sweep_table<DIM, KERNEL, ISO>, frozen_grid(prm), kT, 0, s, r.P, r.cs, r.perm, prm, r.tab,
+    return launch_pdl(k_sweep_table<DIM, KERNEL, ISO>, frozen_blocks(prm), kT, 0, s, r.P, r.cs, r.perm, prm, r.tab,
                       ShapeConst{float4{}, r.g2, r.bT}, C, sets, P4, r.C);
 }
 
@@ -482,6 +479,8 @@ cudaError_t launch_sweep_gather(const uint32_t *perm, const float *C, int n, int
 cudaError_t launch_sweep_table(int dim, int kernel, bool iso, const SweepRun &r, const RateParams &prm, const float *C,
                                int sets, int P4, cudaStream_t s)
 {
+    const cudaError_t e = launch_chunk_numbers(r.cs, prm, r.tab.dense, s);
+    if (e != cudaSuccess) return e;
     return ADE_SWEEP_CALL(table_k, r, prm, C, sets, P4, s);
 }
 
