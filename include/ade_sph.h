@@ -165,10 +165,9 @@ int ade_count_pairs(ade_ctx *ctx, long long *pairs_host, void *stream);
 /* nsteps predictor-corrector steps (Eq. 8-9), each: cell build, rate at level l with the fused
  * predictor, rate at level l+1/2 with the fused corrector (which writes one partial of sum C,
  * min C and max C per warp), and the fold of those partials into the step's FP64 statistics.
- * In a uniform flow the separations do not change: a call of several steps on a context with
- * flags = 0 builds the cell list and the pair weights once and evaluates every step from them
- * (the workspace holds them unless they would exceed 16 GB); results are the same bits as one step
- * at a time, and as any split of the steps into calls. */
+ * In a uniform flow the separations do not change: with a weights buffer (ade_set_weights) a call of
+ * several steps builds the cell list and the pair weights once and evaluates every step from them;
+ * results are the same bits as one step at a time, and as any split of the steps into calls. */
 int ade_step(ade_ctx *ctx, int nsteps, void *stream);
 
 /* As ade_step, replaying captured CUDA graphs: one graph of 32 steps per whole multiple of 32
@@ -178,6 +177,25 @@ int ade_step(ade_ctx *ctx, int nsteps, void *stream);
  * waits for the stream and fills in the last step's statistics (those of the state it wrote; with
  * nsteps = 0, those of the current state as ade_get_stats); with NULL it only enqueues. */
 int ade_run(ade_ctx *ctx, int nsteps, ade_stats *stats_host, void *stream);
+
+/* Weights buffer: where calls of two and more steps keep the pair weights (4 bytes per pair and the idle
+ * ends of rows: about 2.6 GB for 128^3 particles with 250 neighbours on a lattice, up to three times the
+ * pairs' bytes on an irregular set).  It is scratch: every call fills it from the positions and leaves
+ * nothing in it for the next.  Without one, calls step as one step at a time does.
+ * ade_weights_bytes: the bytes that hold every weight on the grid in use.  counted nonzero: builds the cell
+ * list of the current positions and counts, so the size is what the set needs, however uneven it is; waits for
+ * the stream; ADE_ERR_STATE while the stream is captured.  counted 0: an estimate for an even set, host only, for
+ * a first call that should not wait (up to four times what a lattice needs; a set with dense spots keeps
+ * fewer of its weights in it).  0 where weights are not kept: flags other than 0, a velocity field, more than
+ * 500 expected neighbours with more than 80,000 particles (the walks are as fast there), more than 16 GB
+ * counted or 4 GB estimated.
+ * ade_set_weights: gives the context a buffer (device, 256-byte aligned, valid until the context is destroyed
+ * or another or NULL is set; no work in flight may use the old one).  A smaller buffer than asked for
+ * holds what fits, and the other particles' weights are evaluated at every step (ADE_ERR_CAPACITY below the
+ * part that is not weights).  Needs an ade_weights_bytes since the last change of grid
+ * (ADE_ERR_STATE otherwise); ade_autotune takes the buffer away, so ask and set again after it. */
+int ade_weights_bytes(ade_ctx *ctx, int counted, size_t *bytes, void *stream);
+int ade_set_weights(ade_ctx *ctx, void *weights_dev, size_t bytes);
 
 /* One step (as ade_step) bracketed by CUDA events on `stream`; waits for it and returns the device
  * time of each phase in phase_ms_host[4] = {cell build, predictor rate, corrector rate, fold of
@@ -268,8 +286,12 @@ int ade_checkpoint_load(ade_ctx *ctx, const void *host_buf, size_t bytes, void *
  * list built at the current positions, and keeps C every ckpt_every steps; segments are recomputed
  * on the way back.  Pair arithmetic is FP32; J and the dot products are FP64. */
 
-/* Device workspace of ade_adjoint for nsteps steps with checkpoints every ckpt_every steps. */
+/* Device workspace of ade_adjoint for nsteps steps with checkpoints every ckpt_every steps.  A larger one
+ * keeps pair weights for the length of the call in what is beyond: ade_adjoint_weights_bytes (counted or
+ * estimated, as ade_weights_bytes) reports how much of it serves, at most 16 GB;
+ * where it is less, the weights that do not fit are evaluated in every pass.  */
 int ade_adjoint_workspace_bytes(const ade_ctx *ctx, int nsteps, int ckpt_every, size_t *bytes);
+int ade_adjoint_weights_bytes(ade_ctx *ctx, int counted, size_t *bytes, void *stream);
 
 /* C_target_dev [n] (caller order): the target field C*.  Outputs: dJdC0_dev [n] (caller order, may
  * be NULL), dJdtheta_host[3] = dJ/d(alpha_L, alpha_T, D_m) (may be NULL), J_host (may be NULL),
@@ -306,6 +328,11 @@ int ade_batch_step(ade_batch *b, int nsteps, void *stream);
 /* As ade_batch_step, replaying captured CUDA graphs (of up to 32 steps where several steps share the
  * pair weights, as in ade_step); only enqueues. */
 int ade_batch_run(ade_batch *b, int nsteps, void *stream);
+
+/* Weights buffer of a batch, as ade_weights_bytes and ade_set_weights (set uploads the plumes'
+ * shares on `stream` and waits, unless they are the estimate's; ade_batch_autotune and ade_batch_set_config take it away). */
+int ade_batch_weights_bytes(ade_batch *b, int counted, size_t *bytes, void *stream);
+int ade_batch_set_weights(ade_batch *b, void *weights_dev, size_t bytes, void *stream);
 
 /* FP64 per-plume mass, min and max (stats_host[nplumes]); waits for the stream. */
 int ade_batch_stats(ade_batch *b, ade_stats *stats_host, void *stream);
@@ -369,6 +396,10 @@ int ade_sweep_count_pairs(ade_sweep *sw, long long *pairs_host, void *stream);
 /* nsteps predictor-corrector steps (Eq. 8-9) of every set; ade_sweep_run replays a captured graph. */
 int ade_sweep_step(ade_sweep *sw, int nsteps, void *stream);
 int ade_sweep_run(ade_sweep *sw, int nsteps, void *stream);
+/* Weights buffer of a sweep, as ade_weights_bytes and ade_set_weights: 8 bytes per pair and twice the
+ * concentrations, used by calls of four evaluations (2 x nsteps x groups of sets) and more. */
+int ade_sweep_weights_bytes(ade_sweep *sw, int counted, size_t *bytes, void *stream);
+int ade_sweep_set_weights(ade_sweep *sw, void *weights_dev, size_t bytes);
 /* One step bracketed by events; waits; phase_ms_host[4] = {cell build, predictors, correctors, 0}. */
 int ade_sweep_step_timed(ade_sweep *sw, double *phase_ms_host, void *stream);
 int ade_sweep_launches_per_step(const ade_sweep *sw, int *launches);

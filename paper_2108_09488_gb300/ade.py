@@ -47,7 +47,9 @@ EXPORTS = ("ade_workspace_bytes", "ade_init_particles", "ade_get_info", "ade_bui
            "ade_sweep_workspace_bytes", "ade_sweep_init", "ade_sweep_get_info", "ade_sweep_rate",
            "ade_sweep_count_pairs", "ade_sweep_step", "ade_sweep_run", "ade_sweep_step_timed",
            "ade_sweep_launches_per_step", "ade_sweep_stats", "ade_sweep_destroy", "ade_set_flux",
-           "ade_get_flux", "ade_checkpoint_bytes", "ade_checkpoint_save", "ade_checkpoint_load")
+           "ade_get_flux", "ade_checkpoint_bytes", "ade_checkpoint_save", "ade_checkpoint_load",
+           "ade_weights_bytes", "ade_set_weights", "ade_batch_weights_bytes", "ade_batch_set_weights",
+           "ade_sweep_weights_bytes", "ade_sweep_set_weights", "ade_adjoint_weights_bytes")
 NOALLOC_MAX_PARTICLES = 1 << 20
 NOALLOC_MAX_CELLS = 1 << 20
 
@@ -151,6 +153,13 @@ def load():
         "ade_adjoint_workspace_bytes": (I, [P, I, I, ctypes.POINTER(SZ)]),
         "ade_adjoint": (I, [P, P, I, I, P, SZ, P, ctypes.POINTER(ctypes.c_double),
                             ctypes.POINTER(ctypes.c_double), P, V]),
+        "ade_weights_bytes": (I, [P, I, ctypes.POINTER(SZ), V]),
+        "ade_set_weights": (I, [P, P, SZ]),
+        "ade_batch_weights_bytes": (I, [P, I, ctypes.POINTER(SZ), V]),
+        "ade_batch_set_weights": (I, [P, P, SZ, V]),
+        "ade_sweep_weights_bytes": (I, [P, I, ctypes.POINTER(SZ), V]),
+        "ade_sweep_set_weights": (I, [P, P, SZ]),
+        "ade_adjoint_weights_bytes": (I, [P, I, ctypes.POINTER(SZ), V]),
         "ade_batch_destroy": (None, [P]),
         "ade_destroy": (None, [P]),
         "ade_last_error": (ctypes.c_char_p, []),
@@ -307,7 +316,44 @@ def destroy(ctx):
 
 
 # ---- device-memory owner ----------------------------------------------------------------------
-class Simulation:
+class _KeptWeights:
+    """Weights buffer of a context's multi-step calls (ade_weights_bytes, ade_set_weights): allocated when the first
+    such call is made, not where only single steps and rates are.  The first call takes the estimated size, which
+    costs no wait; from the second on the buffer has the size counted for the set.  Where the device has no room
+    the context steps without; in a stream capture the question is put off to the next call."""
+
+    _weights = None          # the buffer
+    _weights_asked = 0       # 1: estimated, 2: counted, since the last change of grid
+
+    def _forget_weights(self):
+        self._weights, self._weights_asked = None, 0
+
+    def _weights_bytes(self, kind, counted):
+        n = ctypes.c_size_t(0)
+        _check(getattr(load(), f"ade_{kind}weights_bytes")(self.ctx, counted, ctypes.byref(n), self.stream))
+        return n.value
+
+    def _keep_weights(self, kind):
+        t = self.torch
+        if self._weights_asked == 2 or t.cuda.is_current_stream_capturing():
+            return
+        nbytes = self._weights_bytes(kind, 0) if self._weights_asked == 0 else 0
+        self._weights_asked = 1 if nbytes else 2
+        if not nbytes:
+            nbytes = self._weights_bytes(kind, 1)     # (waits: the last call has left the old buffer)
+        self._weights = None
+        if nbytes:
+            try:
+                self._weights = t.empty(nbytes + 256, dtype=t.uint8, device=self.C.device)
+            except t.cuda.OutOfMemoryError:
+                pass
+        if self._weights is None:
+            self._set_weights(None, 0)
+        else:
+            self._set_weights((self._weights.data_ptr() + 255) // 256 * 256, nbytes)
+
+
+class Simulation(_KeptWeights):
     """Particle state + workspace on the current CUDA device, bound to one library context.
 
     ``xq`` (int32 [dim][n], the uint32 fixed-point words) and ``C`` (float32 [n]) are torch CUDA
@@ -328,6 +374,7 @@ class Simulation:
         self.ws_bytes = nbytes
         self.ctx = init_particles(p, self.n, self.xq.data_ptr(), self.C.data_ptr(), self.ws_ptr, nbytes)
         self.info = get_info(self.ctx)
+        self._adjoint_weights, self._adjoint_asked = 0, 0     # bytes of pair weights an adjoint call keeps
 
     @property
     def stream(self):
@@ -354,10 +401,17 @@ class Simulation:
         return count_pairs(self.ctx, self.stream)
 
     def step(self, nsteps=1):
+        if nsteps > 1:
+            self._keep_weights("")
         step(self.ctx, nsteps, self.stream)
 
     def run(self, nsteps, stats=True):
+        if nsteps > 1:
+            self._keep_weights("")
         return run(self.ctx, nsteps, self.stream, stats)
+
+    def _set_weights(self, ptr, nbytes):
+        _check(load().ade_set_weights(self.ctx, ptr, nbytes))
 
     def step_timed(self):
         return step_timed(self.ctx, self.stream)
@@ -373,6 +427,8 @@ class Simulation:
         and two evaluations per configuration (ade_autotune); returns that time in ms."""
         ms = ctypes.c_double(0.0)
         _check(load().ade_autotune(self.ctx, ctypes.byref(ms), self.stream))
+        self._forget_weights()
+        self._adjoint_asked = 0
         self.info = get_info(self.ctx)
         return ms.value
 
@@ -423,13 +479,23 @@ class Simulation:
         tgt = t.as_tensor(C_target, dtype=t.float32, device=self.C.device).contiguous()
         nbytes = ctypes.c_size_t(0)
         _check(load().ade_adjoint_workspace_bytes(self.ctx, nsteps, ckpt_every, ctypes.byref(nbytes)))
-        aws = t.empty(nbytes.value + 256, dtype=t.uint8, device=self.C.device)
+        if self._adjoint_asked < 2:     # as _keep_weights
+            self._adjoint_weights = self._weights_bytes("adjoint_", 0) if self._adjoint_asked == 0 else 0
+            self._adjoint_asked = 1 if self._adjoint_weights else 2
+            if not self._adjoint_weights:
+                self._adjoint_weights = self._weights_bytes("adjoint_", 1)
+        size = nbytes.value + self._adjoint_weights
+        try:
+            aws = t.empty(size + 256, dtype=t.uint8, device=self.C.device)
+        except t.cuda.OutOfMemoryError:     # without the pair weights
+            size = nbytes.value
+            aws = t.empty(size + 256, dtype=t.uint8, device=self.C.device)
         aws_ptr = (aws.data_ptr() + 255) // 256 * 256
         dC0 = t.empty(max(self.n, 1), dtype=t.float32, device=self.C.device) if want_dC0 else None
         fin = t.empty(max(self.n, 1), dtype=t.float32, device=self.C.device) if want_final else None
         g = (ctypes.c_double * 3)()
         J = ctypes.c_double(0.0)
-        _check(load().ade_adjoint(self.ctx, tgt.data_ptr(), nsteps, ckpt_every, aws_ptr, nbytes.value,
+        _check(load().ade_adjoint(self.ctx, tgt.data_ptr(), nsteps, ckpt_every, aws_ptr, size,
                                   dC0.data_ptr() if dC0 is not None else None, g, ctypes.byref(J),
                                   fin.data_ptr() if fin is not None else None, self.stream))
         return (J.value, np.array(list(g)), dC0[: self.n] if dC0 is not None else None,
@@ -468,7 +534,7 @@ def batch_workspace_bytes(plist, ns):
     return out.value
 
 
-class Batch:
+class Batch(_KeptWeights):
     """Many plumes stepped together through the ade_batch_* entry points.
 
     ``xq_list[p]`` (uint32 [dim][n_p]) and ``C_list[p]`` (float32 [n_p]) are copied into one
@@ -500,10 +566,17 @@ class Batch:
         return ctypes.c_void_p(self.torch.cuda.current_stream().cuda_stream)
 
     def step(self, nsteps=1):
+        if nsteps > 1:
+            self._keep_weights("batch_")
         _check(load().ade_batch_step(self.ctx, nsteps, self.stream))
 
     def run(self, nsteps):
+        if nsteps > 1:
+            self._keep_weights("batch_")
         _check(load().ade_batch_run(self.ctx, nsteps, self.stream))
+
+    def _set_weights(self, ptr, nbytes):
+        _check(load().ade_batch_set_weights(self.ctx, ptr, nbytes, self.stream))
 
     def stats(self):
         st = (Stats * self.P)()
@@ -525,6 +598,7 @@ class Batch:
     def autotune(self):
         ms = ctypes.c_double(0.0)
         _check(load().ade_batch_autotune(self.ctx, ctypes.byref(ms), self.stream))
+        self._forget_weights()
         return ms.value
 
     def config(self):
@@ -539,6 +613,7 @@ class Batch:
         another batch's config() after its autotune."""
         _check(load().ade_batch_set_config(self.ctx, int(cfg[0]), int(cfg[1]), int(cfg[2]), int(cfg[3]),
                                            self.stream))
+        self._forget_weights()
 
     def launches_per_step(self):
         v = ctypes.c_int(0)
@@ -576,7 +651,7 @@ def sweep_workspace_bytes(p, n, ntheta):
     return out.value
 
 
-class Sweep:
+class Sweep(_KeptWeights):
     """P dispersivity sets theta[k] = (alpha_L, alpha_T, D_m) on one particle set through the
     ade_sweep_* entry points.  ``C`` is a float32 [P][n] torch CUDA tensor (set k's field in row k),
     ``xq`` the shared int32 [dim][n] positions; both are updated in place."""
@@ -618,10 +693,19 @@ class Sweep:
         return v.value
 
     def step(self, nsteps=1):
+        self._weights_for(nsteps)
         _check(load().ade_sweep_step(self.ctx, nsteps, self.stream))
 
     def run(self, nsteps):
+        self._weights_for(nsteps)
         _check(load().ade_sweep_run(self.ctx, nsteps, self.stream))
+
+    def _weights_for(self, nsteps):
+        if 2 * nsteps * self.info.tile[0] >= 4:     # evaluations of the call
+            self._keep_weights("sweep_")
+
+    def _set_weights(self, ptr, nbytes):
+        _check(load().ade_sweep_set_weights(self.ctx, ptr, nbytes))
 
     def step_timed(self):
         out = (ctypes.c_double * 4)()

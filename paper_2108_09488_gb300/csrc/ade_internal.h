@@ -105,7 +105,8 @@ struct RateParams {
     int cap;         // staged-particle capacity of a tile
     double u[3];     // FP64 length of one fixed-point unit per axis (L_i / 2^32)
     double H2d;      // FP64 support radius squared (pair counting decides support in FP64)
-    unsigned fz_base, fz_stride;   // weight table: first line and lines per chunk (FrozenTab)
+    unsigned fz_base, fz_stride, fz_regions;   // weight table: first line, lines of a chunk's region (0: no
+                     // table) and chunks that have one (FrozenTab)
     int goff;        // batched plumes: first particle (caller and sorted order) of this plume
     int coff;        // batched plumes: first cell of this plume in the global cell table
     int m1;               // -1: the multiplier of the walks' separations (see sep in rate_common.cuh)
@@ -161,7 +162,7 @@ struct SweepOut {
 };
 
 // Weight table of the evaluations over one cell list (rate_frozen.cu), in lines of 32 words: a region of
-// RateParams::fz_stride lines per chunk from RateParams::fz_base on, and from line `pool` on `cap` lines
+// RateParams::fz_stride lines for each of the first fz_regions chunks from RateParams::fz_base on, and from line `pool` on `cap` lines
 // that an atomic cursor hands out to chunks that outgrow theirs; slots: two words of 16 bytes per chunk
 // number (put_chunk in frozen_table.cuh).
 constexpr int kFrozenThreads = 128;
@@ -175,9 +176,20 @@ constexpr int kCountChunksFrom = 152 * 48;
 struct FrozenTab {
     float *words;
     uint4 *slots;
-    unsigned *cursor;
+    unsigned long long *cursor;
     unsigned pool, cap;
     uint32_t *dense;       // chunks before each pencil (launch_chunk_numbers; NULL: numbers with gaps)
+};
+// Lines that a set's chunks need, counted by size: two bins per octave.
+struct ChunkBin {
+    unsigned count, most;
+    unsigned long long sum;
+};
+constexpr int kChunkBins = 64;
+// How a table is divided: `lines` hold every chunk, `regions` of them `stride` lines each and the others in the pool.
+struct TablePlan {
+    unsigned stride, regions;
+    size_t lines;
 };
 // Concentrations (and Eq. 14's flux) of such a run in sorted order: C at level l, Ch at l + 1/2, each
 // pencil's twice back to back ([2n] words).
@@ -324,11 +336,23 @@ cudaError_t launch_rate_field(int dim, int kernel, int epi, const uint4 *Pe, con
 unsigned frozen_blocks(const RateParams &prm);
 // dense[p] = chunks of the pencils before p, p = 0..np (nothing where dense is NULL).
 cudaError_t launch_chunk_numbers(const uint32_t *cs, const RateParams &prm, uint32_t *dense, cudaStream_t s);
-// Lines and slots of a table with `val` words per pair (lines bounded by the table's size limit), enough for
-// every grid the context may switch to; and the table's division among the chunks of the grid in use
-// (fz_base, fz_stride, pool, cap).
-void frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots);
-void frozen_divide(const ade_ctx *c, int val, size_t lines, RateParams *rp, FrozenTab *tab);
+// Slots of a table, enough for every grid the context may switch to.
+size_t table_slots(const ade_ctx *c);
+// The plan of a table with `val` words per pair (`lines` 0: above the limit; then `stride` is that of the whole table
+// all the same): counted for the current positions (waits for the stream; the limit is kTableMaxBytes), or the
+// estimate for an even set (host only; kEstimateMaxBytes).
+int plan_context_table(ade_ctx *c, int val, bool counted, TablePlan *plan, cudaStream_t s);
+constexpr double kTableMaxBytes = 16e9, kEstimateMaxBytes = 4e9;
+// Division of `lines` lines (fz_base, fz_stride, fz_regions, pool, cap).
+void divide_table(const TablePlan &plan, size_t lines, RateParams *rp, FrozenTab *tab);
+// Cell build of the current positions in the steps' moving frame.
+int framed_cells(ade_ctx *c, cudaStream_t s);
+// Adds the lines that every chunk needs to bins[kChunkBins]; batch: items [first, last), bins of the plumes from
+// that of the first item on.
+cudaError_t launch_chunk_need(int dim, bool iso, const uint4 *P, const uint32_t *cs, const RateParams &prm, int val,
+                              ChunkBin *bins, cudaStream_t s);
+cudaError_t launch_chunk_need_batch(int dim, const uint4 *P, const uint32_t *cs, const RateParams *descs, const FrozenItem *items,
+                                    int first, int last, ChunkBin *bins, cudaStream_t s);
 // Evaluations over one cell list with stored weights (rate_frozen.cu): the table, one predictor or
 // corrector (prm.dt), and the final state in the caller's order (prm.inc: the drift of all steps).
 cudaError_t launch_frozen_build(int dim, int kernel, bool iso, const uint4 *P, const uint32_t *cs, const uint32_t *perm,
@@ -401,12 +425,15 @@ struct ade_ctx {
     cudaEvent_t ev[5];    // per-phase timing events (created on first timed step)
     bool ev_ready;
     bool frame_set;       // w.frame holds the frame of the current step
-    bool cells_framed;    // the last build was a step's (in the moving frame)
-    bool frozen;          // steps of one call may keep the pair weights (frozen_tab)
+    bool cells_framed;    // the last build was in the moving frame, of the positions cells_add before the current
+    uint32_t cells_add[3];
+    // weight table of multi-step calls (ade_set_weights), in the caller's buffer
+    bool frozen;          // there is one for the grid in use
+    bool cursor_clean;    // its pool's counter has been cleared
     ade::FrozenTab frozen_tab;
     size_t frozen_lines;  // lines of the table
-    bool frozen_fits;     // the table has room for the grid in use
     float *frozen_C;      // [2][2n] concentrations of such a call (FrozenState)
+    ade::TablePlan plan, adj_plan;   // as last asked for (stride 0: not since the last change of grid)
     // velocity-field mode (p.vmax > 0)
     bool field;
     bool field_set;       // a valid field has been copied in

@@ -371,8 +371,7 @@ cudaError_t fwd_step(const Adj &A, const float *u, float *h, float *out, float d
 
 // Adjoint workspace: fields (doubled per pencil), the weight table, FP64 partials of one segment.
 struct AdjLayout {
-    size_t ckpt, seg, h, p, hp, a, dots, partials, words, slots, dense, cursor, total;
-    size_t lines;
+    size_t ckpt, seg, h, p, hp, a, dots, partials, slots, dense, cursor, total;
     int nck, blocks;
 };
 
@@ -386,8 +385,7 @@ AdjLayout adj_layout(const ade_ctx *c, int nsteps, int ck)
         return o;
     };
     const size_t f2 = (size_t)c->n * 8;
-    size_t slots = 0;
-    frozen_extent(c, 2, &L.lines, &slots);
+    const size_t slots = table_slots(c);
     L.blocks = (int)((slots + kT / 32 - 1) / (kT / 32));
     L.nck = (nsteps + ck - 1) / ck;
     L.ckpt = take(f2 * (L.nck + 1));
@@ -398,7 +396,6 @@ AdjLayout adj_layout(const ade_ctx *c, int nsteps, int ck)
     L.a = take(f2);
     L.dots = take(((size_t)nsteps + 1) * kDots * 8);
     L.partials = take((size_t)L.blocks * std::min(ck, nsteps) * kDots * 8);
-    L.words = take(L.lines * 128);
     L.slots = take(slots * 32);
     L.dense = take(slots * 4);
     L.cursor = take(64);
@@ -429,6 +426,18 @@ extern "C" int ade_adjoint_workspace_bytes(const ade_ctx *c, int nsteps, int ckp
     return ADE_OK;
 }
 
+extern "C" int ade_adjoint_weights_bytes(ade_ctx *c, int counted, size_t *bytes, void *stream)
+{
+    if (!c || !bytes) return ade::report_error(ADE_ERR_ARG, "NULL argument");
+    *bytes = 0;
+    if (c->field || c->n == 0) return ADE_OK;
+    const int rc = plan_context_table(c, 2, counted != 0, &c->adj_plan, (cudaStream_t)stream);
+    if (rc || c->adj_plan.stride == 0u || (!counted && c->adj_plan.lines == 0)) return rc;
+    // above the limit: as many chunks as fit
+    *bytes = c->adj_plan.lines > 0 ? c->adj_plan.lines * 128 : (size_t)kTableMaxBytes / 256 * 256;
+    return ADE_OK;
+}
+
 extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, int ckpt_every, void *aws,
                            size_t aws_bytes, float *dJdC0_dev, double *dJdtheta_host, double *J_host,
                            float *C_final_dev, void *stream)
@@ -456,7 +465,8 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     A.c = c;
     A.s = (cudaStream_t)stream;
     A.rp = c->rp;
-    A.rp.frame = nullptr;
+    A.rp.frame = c->w.frame;
+    for (int i = 0; i < 3; ++i) A.rp.back[i] = 0u;
     A.rp.ub = 0.f;
     float lo[3];
     for (int i = 0; i < 3; ++i) {
@@ -480,22 +490,22 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     float *ckpt = field(L.ckpt), *seg = field(L.seg), *h = field(L.h), *p = field(L.p), *hp = field(L.hp), *a = field(L.a);
     double *dots = reinterpret_cast<double *>(base + L.dots);
     double *partials = reinterpret_cast<double *>(base + L.partials);
-    A.tab.words = field(L.words);
+    A.tab.words = field(L.total);   // what the caller gave beyond the fields
     A.tab.slots = reinterpret_cast<uint4 *>(base + L.slots);
-    A.tab.cursor = reinterpret_cast<unsigned *>(base + L.cursor);
+    A.tab.cursor = reinterpret_cast<unsigned long long *>(base + L.cursor);
     const bool count = chunk_numbers(n, A.rp.ncy * A.rp.ncz) > kCountChunksFrom;
     A.tab.dense = count ? reinterpret_cast<uint32_t *>(base + L.dense) : nullptr;
-    frozen_divide(c, 2, L.lines, &A.rp, &A.tab);
+    divide_table(c->adj_plan, std::min((aws_bytes - L.total) / 128, (size_t)kTableMaxBytes / 128), &A.rp, &A.tab);
     const int nb = (int)A.blocks;
     if (nb > L.blocks) return ade::report_error(ADE_ERR_CAPACITY, "adjoint partials exceed the workspace");
     const float dt = (float)c->dt;
     cudaStream_t s = A.s;
     const uint32_t *perm = c->w.perm;
 
-    // frozen geometry: one cell list at the current positions (counts and tile totals cleared first)
-    ADJ_CK(cudaMemsetAsync(A.tab.cursor, 0, sizeof(unsigned), s));
-    ADJ_CK(ade::launch_build_cells(c->dim, c->xq, c->C, n, c->nc, c->ncells, c->w, s));
-    c->cells_framed = false;
+    // frozen geometry: one cell list at the current positions
+    ADJ_CK(cudaMemsetAsync(A.tab.cursor, 0, sizeof(*A.tab.cursor), s));
+    const int rc = framed_cells(c, s);
+    if (rc) return rc;
     ADJ_CK(launch_chunk_numbers(c->w.cell_start, A.rp, A.tab.dense, s));
     ADJ_CK(table(A, ckpt));
     // forward: checkpoints every ckpt_every steps, the last segment's states straight into seg

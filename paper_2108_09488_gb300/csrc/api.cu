@@ -325,7 +325,7 @@ void choose_tiles(int dim, int n, const Grid &g, bool iso, unsigned flags, ade::
 
 struct Layout {
     size_t keys, rank, count, block_sums, perm_tmp, perm, cell_start, P0, P1, partials, wpart, stats,
-        cf_partials, status, pairs, pencil, tile_sums, frame, fz_words, fz_slots, fz_dense, fz_C, fz_cursor, fVc, fDAc, fDBc, fIncC, fV, fDA, fDB, fInc,
+        cf_partials, status, pairs, pencil, tile_sums, frame, fVc, fDAc, fDBc, fIncC, fV, fDA, fDB, fInc,
         fbits, Q, Qh, total;
 };
 
@@ -335,7 +335,7 @@ constexpr size_t kStatusAt = 64, kStatsBytes = 128;
 // nw_partials: per-warp corrector partials of the widest rate launch.  npencils: pencil boxes of
 // the trimmed walks (0: none).
 Layout layout(int n, int ncells, int nb_partials, int nw_partials, int field_dim = 0, bool catt = false,
-              int npencils = 0, size_t fz_lines = 0, size_t fz_slots = 0)
+              int npencils = 0)
 {
     Layout L;
     size_t off = 0;
@@ -362,11 +362,6 @@ Layout layout(int n, int ncells, int nb_partials, int nw_partials, int field_dim
     L.pencil = npencils > 0 ? take((size_t)npencils * 16) : 0;
     L.tile_sums = take(ade::tile_sums_bytes(ncells));
     L.frame = take(ade::kFrameWords * 4);
-    L.fz_words = take(fz_lines * 128);
-    L.fz_slots = take(fz_slots * 32);
-    L.fz_dense = take(fz_slots * 4);
-    L.fz_C = take(fz_slots > 0 ? (size_t)n * 16 : 0);
-    L.fz_cursor = take(64);
     L.fVc = L.fDAc = L.fDBc = L.fIncC = L.fV = L.fDA = L.fDB = L.fInc = L.fbits = 0;
     if (field_dim) {
         const size_t rec = (size_t)n * 16, rec3 = field_dim == 3 ? (size_t)n * 16 : 16;
@@ -400,8 +395,6 @@ struct Derived {
     int nw_partials;
     int ncells_cap;
     int pencils_cap;     // pencils (ncy * ncz) of the largest grid the context may use
-    size_t fz_lines;     // weight table of multi-step calls: lines (0: none) and chunk slots
-    size_t fz_slots;
     ade::RateParams tiles;
     Layout L;
 };
@@ -414,11 +407,48 @@ double expected_neighbours(const ade_params &p, double H, int n)
     return nb;
 }
 
-// Weight table of multi-step calls (rate_frozen.cu) for grid g.  chunk_lines: lines one chunk may need.  A
-// row is as long as its longest lane's range: the particles of the row's pencil within the chord that
-// the smallest transverse distance between the two pencils leaves, plus what the cells at its ends hold
-// outside of it and the spread of 32 lanes' counts on an irregular set.
-unsigned chunk_lines(const ade_params &p, double H, int n, const Grid &g, int val)
+// ---- weight table of multi-step calls (rate_frozen.cu), in a buffer of the caller's ----
+
+size_t table_slots(int n, const Grid &g) { return (size_t)ade::chunk_numbers(n, g.ncells / g.nc[0]) + 1; }
+
+// Whether the chunks of a grid are counted (see kCountChunksFrom).
+bool counts_chunks(int n, int pencils) { return ade::chunk_numbers(n, pencils) > ade::kCountChunksFrom; }
+
+// A division for chunks that need what the bins say: regions of one size for all, large enough for the chunks
+// up to some bin, and the others in the pool.  The cheapest in memory would have many chunks filled twice, so
+// the largest regions within half more of that: an even set gets regions of its longest chunk (512^2
+// jittered, 27 neighbours, per step of eight: 46 us at the cheapest, 35 so), a set with a few dense spots
+// short ones and a pool.
+ade::TablePlan plan_table(const ade::ChunkBin *bins, size_t numbers, bool counted)
+{
+    ade::TablePlan plan = {};
+    size_t chunks = 0;
+    for (int b = 0; b < ade::kChunkBins; ++b) chunks += bins[b].count;
+    const size_t regions = counted ? chunks : numbers;
+    size_t least = 0;
+    for (int pass = 0; pass < 2; ++pass) {       // the least, then the largest regions near it
+        size_t above = 0;
+        for (int b = ade::kChunkBins - 1; b >= 0 && plan.stride == 0u; --b) {
+            if (bins[b].count == 0) continue;
+            const size_t lines = regions * bins[b].most + above + 64;
+            if (pass == 0) {
+                least = least ? std::min(least, lines) : lines;
+            } else if (lines <= least + least / 2) {
+                plan.stride = bins[b].most;
+                plan.lines = lines;
+            }
+            above += (size_t)bins[b].sum;
+        }
+    }
+    plan.regions = chunks > 0 ? (unsigned)regions : 0u;
+    return plan;
+}
+
+// The same without looking at the set: what an even one, lattice or jittered, needs.  A row is as long as its
+// longest lane's range: the particles of the row's pencil within the chord that the smallest transverse
+// distance between the two pencils leaves, plus what the cells at its ends hold outside of it and the spread of
+// 32 lanes' counts; an eighth more for chunks that outgrow their regions.  (Up to four times what a lattice needs.)
+ade::TablePlan estimate_table(const ade_params &p, double H, int n, const Grid &g, int val)
 {
     const double per = (double)n / g.ncells;                  // particles per cell
     const double sx = p.box[0] / g.nc[0], sy = p.box[1] / g.nc[1], sz = p.dim == 3 ? p.box[2] / g.nc[2] : 0.0;
@@ -428,41 +458,46 @@ unsigned chunk_lines(const ade_params &p, double H, int n, const Grid &g, int va
         const double mu = 2.0 * sqrt(fmax(H * H - ey * ey - ez * ez, 0.0)) / sx * per;
         lines += val * (mu + 1.2 * sqrt(mu) + 0.8 * per + 0.5) + 1.0;   // whole cells at the ends; the first indices
     }
-    return (unsigned)fmin(ceil(lines), 1e9);
+    ade::TablePlan plan;
+    plan.stride = (unsigned)fmin(ceil(lines), 1e9);
+    plan.regions = n > 0 ? (unsigned)ade::chunk_numbers(n, g.ncells / g.nc[0]) : 0u;
+    plan.lines = (size_t)plan.regions * plan.stride;
+    plan.lines += plan.lines / 8 + 64;
+    return plan;
 }
 
-size_t frozen_slots(int n, const Grid &g) { return (size_t)n / 32 + (size_t)(g.ncells / g.nc[0]) + 2; }
-
-// A region per chunk, and an eighth more for chunks that outgrow theirs.
-size_t frozen_lines(const ade_params &p, double H, int n, const Grid &g, int val = 1)
+// A set's buffer: counter, slots, chunk counts, concentrations (`fields` words per particle) and lines.
+struct TableLayout {
+    size_t cursor, slots, dense, C, words;
+};
+TableLayout table_layout(size_t slots, size_t C_bytes)
 {
-    const size_t l = frozen_slots(n, g) * chunk_lines(p, H, n, g, val);
-    return l + l / 8 + 64;
+    TableLayout L;
+    L.cursor = 0;
+    L.slots = 256;
+    L.dense = L.slots + align256(slots * 32);
+    L.C = L.dense + align256(slots * 4);
+    L.words = L.C + align256(C_bytes);
+    return L;
 }
 
-// Lines of a chunk's region when `lines` are at hand.
-unsigned frozen_stride(const ade_params &p, double H, int n, const Grid &g, int val, size_t lines)
+// The lines a buffer holds behind `words`, and why it cannot serve.
+int table_lines(const void *buf, size_t bytes, size_t words, unsigned stride, size_t *lines)
 {
-    return (unsigned)std::min<size_t>(chunk_lines(p, H, n, g, val), lines / frozen_slots(n, g));
+    if (((uintptr_t)buf & 255u) != 0u) return fail(ADE_ERR_ARG, "weights buffer must be 256-byte aligned");
+    if (stride == 0u) return fail(ADE_ERR_STATE, "ask for the size of the weights buffer first (since the last change of grid)");
+    if (bytes < words) return fail(ADE_ERR_CAPACITY, "weights buffer too small: %zu < %zu bytes", bytes, words);
+    *lines = std::min((bytes - words) / 128, (size_t)(ade::kTableMaxBytes / 128.0));
+    return ADE_OK;
 }
 
-// Lines a table may take on the grids the autotuner may switch to: a fifth more than the smallest, and what
-// the grid in use needs.  (Coarse grids hold several lattice lines per pencil and need much more; a
-// context tuned to one evaluates every step anew.)
-size_t frozen_room(const ade_params &p, double Hgrid, double H, int n, const Grid &in_use, bool fixed, int val)
+// A query runs kernels and waits: not inside a stream capture.
+int not_capturing(cudaStream_t s)
 {
-    size_t least = frozen_lines(p, H, n, in_use, val);
-    const size_t own = least;
-    for (int k = 1; !fixed && k <= ade::kMaxSubdiv; ++k) {
-        Grid g;
-        if (make_grid(p, Hgrid, k, &g)) least = std::min(least, frozen_lines(p, H, n, g, val));
-    }
-    return std::max(own, least + least / 5);
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    ADE_CK(cudaStreamIsCapturing(s, &st));
+    return st == cudaStreamCaptureStatusNone ? ADE_OK : fail(ADE_ERR_STATE, "the size of the weights buffer cannot be asked for during a capture");
 }
-
-// Above this the table is left out and every evaluation computes its weights (a few per cent of the
-// device's memory; a plume of 10^6 particles with 31,000 neighbours would need 125 GB).
-constexpr double kFrozenMaxBytes = 16e9;
 
 int derive(const ade_params *p, int n, Derived *d)
 {
@@ -522,31 +557,10 @@ int derive(const ade_params *p, int n, Derived *d)
         }
     }
     d->ncells_cap = ncells_cap;
-    d->fz_lines = d->fz_slots = 0;
-    // Wide kernels on sets that fill the chip stay with the walks: a table of 12 GB streams no faster than
-    // they evaluate (405^2 irregular, 9,400 neighbours: 2.2 ms either way; 248^2, 4,900, whose 1,900 warps do
-    // not fill it: 0.58 against 0.93 ms).
-    const bool wide = expected_neighbours(*p, d->H, n) > 500.0 && n > 80000;
-    if (p->flags == 0u && !(p->vmax > 0.0) && n > 0 && !wide) {
-        // the library's choice of walk: multi-step calls keep the weights, on any grid it may pick
-        size_t lines = 0, slots = 0;
-        const size_t room = frozen_room(*p, d->Hgrid, d->H, n, d->g, p->cell_subdiv > 0, 1);
-        for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
-            Grid g;
-            if ((p->cell_subdiv > 0 && k != p->cell_subdiv) || !make_grid(*p, d->Hgrid, k, &g)) continue;
-            if (frozen_lines(*p, d->H, n, g) > room) continue;
-            lines = std::max(lines, frozen_lines(*p, d->H, n, g));
-            slots = std::max(slots, frozen_slots(n, g));
-        }
-        if (128.0 * (double)lines <= kFrozenMaxBytes) {
-            d->fz_lines = lines;
-            d->fz_slots = slots;
-        }
-    }
     // pencil boxes serve the trimmed walks of the uniform-velocity kernels
     d->pencils_cap = p->vmax > 0.0 ? 0 : pencils_cap;
     d->L = layout(n, ncells_cap, d->nb_partials, d->nw_partials, p->vmax > 0.0 ? p->dim : 0, p->tau > 0.0,
-                  d->pencils_cap, d->fz_lines, d->fz_slots);
+                  d->pencils_cap);
     return ADE_OK;
 }
 
@@ -590,8 +604,11 @@ int clean_counts(ade_ctx *c, cudaStream_t s)
         ADE_CK(cudaMemsetAsync(c->w.count, 0, (size_t)c->ncells_cap * sizeof(uint32_t), s));
         // the one-pass scan's flags and {ticket, epoch}: from then on each scan leaves them valid
         ADE_CK(cudaMemsetAsync(c->w.tile_sums, 0, ade::tile_sums_bytes(c->ncells_cap), s));
-        if (c->frozen) ADE_CK(cudaMemsetAsync(c->frozen_tab.cursor, 0, sizeof(unsigned), s));
         c->count_clean = true;
+    }
+    if (c->frozen && !c->cursor_clean) {   // (the kernel that ends a call leaves the pool's counter at 0)
+        ADE_CK(cudaMemsetAsync(c->frozen_tab.cursor, 0, sizeof(*c->frozen_tab.cursor), s));
+        c->cursor_clean = true;
     }
     return ADE_OK;
 }
@@ -611,8 +628,8 @@ int set_frame_once(ade_ctx *c, cudaStream_t s)
 
 // Enqueue one cell build; in velocity-field mode followed by the permutation of the v and D
 // records into the sorted order.  steps > 0: the build of that many steps of a uniform flow, in the
-// moving frame; 0: on the absolute grid.
-int enqueue_cells(ade_ctx *c, cudaStream_t s, int steps = 0)
+// moving frame; 0: on the absolute grid, or in the moving frame where it stands (framed).
+int enqueue_cells(ade_ctx *c, cudaStream_t s, int steps = 0, bool framed = false)
 {
     int rc = need_field(c);
     if (rc) return rc;
@@ -621,10 +638,13 @@ int enqueue_cells(ade_ctx *c, cudaStream_t s, int steps = 0)
     rc = clean_counts(c, s);
     if (rc) return rc;
     ade::CellFrame frame;
-    c->cells_framed = steps > 0 && !c->field;
+    c->cells_framed = (steps > 0 || framed) && !c->field;
     if (c->cells_framed) {
         frame.words = c->w.frame;
-        for (int i = 0; i < 3; ++i) frame.adv[i] = (uint32_t)steps * c->inc[i];
+        for (int i = 0; i < 3; ++i) {
+            frame.adv[i] = (uint32_t)steps * c->inc[i];
+            c->cells_add[i] = steps > 0 ? c->inc[i] : 0u;
+        }
     }
     cudaError_t e = ade::launch_build_cells(c->dim, c->xq, c->C, c->n, c->nc, c->ncells, c->w, s, true, frame);
     if (e != cudaSuccess) {
@@ -717,8 +737,8 @@ int enqueue_frozen(ade_ctx *c, int steps, cudaStream_t s)
         rp.inc[i] = (uint32_t)steps * c->inc[i];
     }
     ade::FrozenTab tab = c->frozen_tab;
-    ade::frozen_divide(c, 1, c->frozen_lines, &rp, &tab);
-    if (ade::chunk_numbers(c->n, rp.ncy * rp.ncz) <= ade::kCountChunksFrom) tab.dense = nullptr;
+    ade::divide_table(c->plan, c->frozen_lines, &rp, &tab);
+    if (!counts_chunks(c->n, rp.ncy * rp.ncz)) tab.dense = nullptr;
     ADE_CK(ade::launch_chunk_numbers(c->w.cell_start, rp, tab.dense, s));
     rp.dt = (float)(0.5 * c->dt);
     ADE_CK(ade::launch_frozen_build(c->dim, c->p.kernel, c->iso, c->w.P0, c->w.cell_start, c->w.perm, rp, tab, st, s));
@@ -739,7 +759,7 @@ int enqueue_frozen(ade_ctx *c, int steps, cudaStream_t s)
 // from the second step on (two steps, us per step: 128^3 1241 against 1465, 1024^2 276 against 285,
 // 512^2 59 against 72, 256^2 23 against 38).  A single step stays with the walks (the cube's would
 // take 1.5 ms).
-bool use_frozen(const ade_ctx *c, int steps) { return c->frozen && c->frozen_fits && steps >= 2; }
+bool use_frozen(const ade_ctx *c, int steps) { return c->frozen && steps >= 2; }
 
 // Enqueue one predictor-corrector step (Eq. 8-9) and the fold of its diagnostics.
 int enqueue_step(ade_ctx *c, cudaStream_t s)
@@ -868,40 +888,59 @@ T *at(void *base, size_t off)
 
 }  // namespace
 
-void ade::frozen_extent(const ade_ctx *c, int val, size_t *lines, size_t *slots)
+size_t ade::table_slots(const ade_ctx *c)
 {
-    *lines = *slots = 0;
     const bool fixed = c->p.cell_subdiv > 0 || c->p.flags != 0u;   // no autotuning: the grid in use
-    // (the same before and after autotuning: callers size a workspace with it; a grid that needs more has
-    // chunks evaluated from the positions)
-    Grid first;
-    size_t room = 0;
-    for (int k = 1; k <= ade::kMaxSubdiv && room == 0; ++k)
-        if ((!fixed || k == c->subdiv) && make_grid(c->p, c->Hgrid, k, &first)) {
-            Grid best = first;
-            for (int q = k; !fixed && q <= ade::kMaxSubdiv; ++q) {
-                Grid g;
-                if (make_grid(c->p, c->Hgrid, q, &g) && frozen_lines(c->p, c->H, c->n, g, val) < frozen_lines(c->p, c->H, c->n, best, val)) best = g;
-            }
-            room = frozen_room(c->p, c->Hgrid, c->H, c->n, best, fixed, val);
-        }
+    size_t slots = 0;
     for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
         Grid g;
-        if ((fixed && k != c->subdiv) || !make_grid(c->p, c->Hgrid, k, &g)) continue;
-        *lines = std::max(*lines, std::min(room, frozen_lines(c->p, c->H, c->n, g, val)));
-        *slots = std::max(*slots, frozen_slots(c->n, g));
+        if ((!fixed || k == c->subdiv) && make_grid(c->p, c->Hgrid, k, &g)) slots = std::max(slots, ::table_slots(c->n, g));
     }
-    *lines = std::min(*lines, (size_t)(kFrozenMaxBytes / 128.0));
+    return slots;
 }
 
-void ade::frozen_divide(const ade_ctx *c, int val, size_t lines, RateParams *rp, FrozenTab *tab)
+void ade::divide_table(const TablePlan &plan, size_t lines, RateParams *rp, FrozenTab *tab)
 {
-    Grid g;
-    if (!make_grid(c->p, c->Hgrid, c->subdiv, &g)) return;   // (the grid in use fits)
     rp->fz_base = 0u;
-    rp->fz_stride = frozen_stride(c->p, c->H, c->n, g, val, lines);
-    tab->pool = (unsigned)(frozen_slots(c->n, g) * rp->fz_stride);
+    rp->fz_stride = lines > 0 ? plan.stride : 0u;
+    rp->fz_regions = plan.stride > 0u ? (unsigned)std::min<size_t>(plan.regions, lines / plan.stride) : 0u;
+    tab->pool = rp->fz_regions * plan.stride;
     tab->cap = (unsigned)(lines - tab->pool);
+}
+
+int ade::framed_cells(ade_ctx *c, cudaStream_t s)
+{
+    const int rc = set_frame_once(c, s);
+    return rc ? rc : enqueue_cells(c, s, 0, true);
+}
+
+int ade::plan_context_table(ade_ctx *c, int val, bool counted, TablePlan *plan, cudaStream_t s)
+{
+    *plan = TablePlan{};
+    const size_t bytes = kChunkBins * sizeof(ChunkBin);
+    if (!counted || (size_t)c->n * 16 < bytes) {   // (the bins lie in the half-step state, free between steps)
+        Grid g;
+        if (!make_grid(c->p, c->Hgrid, c->subdiv, &g)) return ADE_OK;   // (the grid in use fits)
+        *plan = estimate_table(c->p, c->H, c->n, g, val);
+        if (128.0 * (double)plan->lines > kEstimateMaxBytes) plan->lines = 0;
+        return ADE_OK;
+    }
+    int rc = not_capturing(s);
+    if (rc == ADE_OK) rc = framed_cells(c, s);
+    if (rc) return rc;
+    ChunkBin bins[kChunkBins];
+    ChunkBin *dev = reinterpret_cast<ChunkBin *>(c->w.P1);
+    RateParams rp = c->rp;
+    rp.frame = c->w.frame;
+    for (int i = 0; i < 3; ++i) rp.back[i] = 0u;
+    ADE_CK(cudaMemsetAsync(dev, 0, bytes, s));
+    ADE_CK(launch_chunk_need(c->dim, c->iso, c->w.P0, c->w.cell_start, rp, val, dev, s));
+    ADE_CK(cudaMemcpyAsync(bins, dev, bytes, cudaMemcpyDeviceToHost, s));
+    ADE_CK(cudaStreamSynchronize(s));
+    const int np = rp.ncy * rp.ncz;
+    *plan = plan_table(bins, (size_t)chunk_numbers(c->n, np), counts_chunks(c->n, np));
+    if (128.0 * (double)plan->lines > kTableMaxBytes) plan->lines = 0;
+    return ADE_OK;
 }
 
 // Eq. 3 gives D = d_T I + (d_L - d_T) vhat vhat^T with d_T = alpha_T |v| + D_m, d_L = alpha_L |v| + D_m;
@@ -992,15 +1031,6 @@ int ade_init_particles(ade_ctx **out, const ade_params *p, int n, uint32_t *xq_d
     c->w.pencil = d.pencils_cap > 0 ? at<uint4>(workspace_dev, d.L.pencil) : nullptr;
     c->w.tile_sums = at<uint32_t>(workspace_dev, d.L.tile_sums);
     c->w.frame = at<uint32_t>(workspace_dev, d.L.frame);
-    c->frozen = d.fz_lines > 0;
-    c->frozen_tab.words = at<float>(workspace_dev, d.L.fz_words);
-    c->frozen_tab.slots = at<uint4>(workspace_dev, d.L.fz_slots);
-    c->frozen_tab.dense = at<uint32_t>(workspace_dev, d.L.fz_dense);
-    c->frozen_C = at<float>(workspace_dev, d.L.fz_C);
-    c->frozen_tab.cursor = at<unsigned>(workspace_dev, d.L.fz_cursor);
-    c->frozen_lines = d.fz_lines;
-    c->frozen_fits = true;
-
     rc = plume_constants(p, n, d, c->D, &c->dt, c->inc, c->inc_half, &c->rp, &c->iso);
     if (rc) {
         delete c;
@@ -1101,7 +1131,8 @@ int apply_config(ade_ctx *c, int k, int variant)
     for (int i = 0; i < 3; ++i) c->nc[i] = g.nc[i];
     c->ncells = g.ncells;
     c->subdiv = g.subdiv;
-    c->frozen_fits = frozen_lines(c->p, c->H, c->n, g) <= c->frozen_lines;
+    c->frozen = false;   // (a weight table is for one grid)
+    c->plan = c->adj_plan = ade::TablePlan{};
     ade::RateParams &rp = c->rp;
     rp.ncx = g.nc[0];
     rp.ncy = g.nc[1];
@@ -1124,6 +1155,43 @@ int apply_config(ade_ctx *c, int k, int variant)
 }  // namespace
 
 extern "C" {
+
+int ade_weights_bytes(ade_ctx *c, int counted, size_t *bytes, void *stream)
+{
+    if (!c || !bytes) return fail(ADE_ERR_ARG, "NULL argument");
+    *bytes = 0;
+    // Wide kernels on sets that fill the chip stay with the walks: a table of 12 GB streams no faster than
+    // they evaluate (405^2 irregular, 9,400 neighbours: 2.2 ms either way; 248^2, 4,900, whose 1,900 warps do
+    // not fill it: 0.58 against 0.93 ms).
+    const bool wide = expected_neighbours(c->p, c->H, c->n) > 500.0 && c->n > 80000;
+    if (c->p.flags != 0u || c->field || c->n == 0 || wide) return ADE_OK;
+    const int rc = ade::plan_context_table(c, 1, counted != 0, &c->plan, (cudaStream_t)stream);
+    if (rc || c->plan.lines == 0) return rc;
+    const size_t slots = (size_t)ade::chunk_numbers(c->n, c->nc[1] * c->nc[2]) + 1;
+    *bytes = table_layout(slots, (size_t)c->n * 16).words + c->plan.lines * 128;
+    return ADE_OK;
+}
+
+int ade_set_weights(ade_ctx *c, void *weights_dev, size_t bytes)
+{
+    if (!c) return fail(ADE_ERR_ARG, "ctx is NULL");
+    if (weights_dev) {
+        const TableLayout L = table_layout((size_t)ade::chunk_numbers(c->n, c->nc[1] * c->nc[2]) + 1, (size_t)c->n * 16);
+        size_t lines = 0;
+        const int rc = table_lines(weights_dev, bytes, L.words, c->plan.stride, &lines);
+        if (rc) return rc;
+        c->frozen_lines = lines;
+        c->frozen_tab.words = at<float>(weights_dev, L.words);
+        c->frozen_tab.slots = at<uint4>(weights_dev, L.slots);
+        c->frozen_tab.dense = at<uint32_t>(weights_dev, L.dense);
+        c->frozen_tab.cursor = at<unsigned long long>(weights_dev, L.cursor);
+        c->frozen_C = at<float>(weights_dev, L.C);
+        c->cursor_clean = false;
+    }
+    c->frozen = weights_dev && c->frozen_lines > 0;
+    drop_graphs(c);
+    return ADE_OK;
+}
 
 int ade_autotune(ade_ctx *c, double *best_ms_host, void *stream)
 {
@@ -1314,12 +1382,12 @@ int ade_get_cells(ade_ctx *c, uint32_t *perm_dev, uint32_t *cell_start_dev, void
     if (!c) return fail(ADE_ERR_ARG, "ctx is NULL");
     cudaStream_t s = (cudaStream_t)stream;
     if (c->cells_framed && c->n > 0) {
-        // a step built its list in the moving frame: the absolute grid's list of the last step's
-        // positions (the current ones minus one drift)
+        // the list was built in the moving frame: the absolute grid's list of the same positions (the
+        // current ones, minus one drift after steps)
         int rc = clean_counts(c, s);
         if (rc) return rc;
         ade::CellFrame frame;
-        for (int i = 0; i < 3; ++i) frame.add[i] = c->inc[i];
+        for (int i = 0; i < 3; ++i) frame.add[i] = c->cells_add[i];
         ADE_CK(ade::launch_build_cells(c->dim, c->xq, c->C, c->n, c->nc, c->ncells, c->w, s, true, frame));
         c->cells_framed = false;
     }
@@ -1430,7 +1498,10 @@ int ade_run(ade_ctx *c, int nsteps, ade_stats *st, void *stream)
     if (rc0) return rc0;
     for (int k = 0; k < nmulti; ++k) ADE_CK(cudaGraphLaunch(c->graph_exec[ade::kGraphSteps], s));
     for (int k = 0; k < rest; k += per) ADE_CK(cudaGraphLaunch(c->graph_exec[per], s));
-    c->cells_framed = (nsteps > 0 && !c->field) || c->cells_framed;
+    if (nsteps > 0 && !c->field) {
+        c->cells_framed = true;
+        for (int i = 0; i < 3; ++i) c->cells_add[i] = c->inc[i];
+    }
     c->step += nsteps;
     c->t += nsteps * c->dt;
     if (!st) return ADE_OK;
@@ -1589,55 +1660,40 @@ struct ade_batch {
     cudaGraphExec_t graph_exec[ade::kGraphSteps + 1] = {};
     cudaStream_t cap_stream = nullptr;
     // weight table of multi-step calls (rate_frozen.cu)
-    bool frozen = false, frozen_fits = false;   // frozen_fits: room for the grids in use
+    bool frozen = false;               // there is one for the grids in use (ade_batch_set_weights)
     ade::FrozenTab frozen_tab = {};
     ade::FrozenItem *d_items = nullptr;
     float *frozen_C = nullptr;
     std::vector<ade::FrozenItem> items;
-    std::vector<size_t> frozen_plume;   // table lines of each plume
+    std::vector<ade::TablePlan> plans;  // per plume: for an even set, or as last counted
+    size_t plan_lines = 0;              // their lines
+    size_t divided = 0;                 // lines the uploaded constants divide (0: those of other plans)
 };
 
 namespace {
 
 struct BatchLayout {
-    size_t fz_words, fz_slots, fz_C, fz_cursor, fz_items, frames, keys, rank, count, block_sums, tile_sums, perm_tmp, perm, cell_start, P0, P1, pred, corr, tiles,
+    size_t fz_items, frames, keys, rank, count, block_sums, tile_sums, perm_tmp, perm, cell_start, P0, P1, pred, corr, tiles,
         queue, plume_of, offsets, stats, status, pairs, total;
 };
 
-// Size of a batch's weight table over every subdivision its plumes may be given (0: none).
-struct BatchFrozen {
-    size_t lines = 0, items = 0;
-    std::vector<size_t> plume;          // lines of each plume
-};
-
-BatchFrozen batch_frozen_size(int P, const ade_params *p, const int *n)
+// Chunks of the weight table over every subdivision the plumes may be given.
+size_t batch_max_items(int P, const ade_params *p, const int *n)
 {
-    BatchFrozen f;
+    size_t items = 0;
     for (int i = 0; i < P; ++i) {
         const double H = p[i].kernel == ADE_WENDLAND_C2 ? 2.0 * p[i].h : p[i].h;
-        size_t lines = 0, items = 0, least = 0;
+        size_t most = 0;
         for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
             Grid g;
-            if (!make_grid(p[i], H, k, &g)) continue;
-            const size_t l = frozen_lines(p[i], H, n[i], g);
-            least = least ? std::min(least, l) : l;
+            if (make_grid(p[i], H, k, &g)) most = std::max(most, (size_t)ade::chunk_numbers(n[i], g.ncells / g.nc[0]));
         }
-        for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
-            Grid g;
-            if (!make_grid(p[i], H, k, &g)) continue;
-            const size_t np = (size_t)(g.ncells / g.nc[0]), l = frozen_lines(p[i], H, n[i], g);
-            if (l <= least + least / 5) lines = std::max(lines, l);   // (see frozen_room)
-            items = std::max(items, (size_t)ade::chunk_numbers(n[i], (int)np));
-        }
-        f.lines += lines;
-        f.plume.push_back(lines);
-        f.items += items;
+        items += most;
     }
-    if (128.0 * (double)f.lines > kFrozenMaxBytes) f = BatchFrozen();
-    return f;
+    return items;
 }
 
-BatchLayout batch_layout(int P, int N, int NC_max, int max_tiles, const BatchFrozen &fz)
+BatchLayout batch_layout(int P, int N, int NC_max, int max_tiles, size_t items)
 {
     BatchLayout L;
     size_t off = 0;
@@ -1646,11 +1702,7 @@ BatchLayout batch_layout(int P, int N, int NC_max, int max_tiles, const BatchFro
         off += align256(bytes > 0 ? bytes : 1);
         return o;
     };
-    L.fz_words = take(fz.lines * 128);
-    L.fz_slots = take(fz.items * 32);
-    L.fz_C = take(fz.lines > 0 ? (size_t)N * 16 : 0);
-    L.fz_cursor = take(64);
-    L.fz_items = take(fz.items * sizeof(ade::FrozenItem));
+    L.fz_items = take(items * sizeof(ade::FrozenItem));
     L.frames = take((size_t)P * ade::kFrameWords * 4);
     L.keys = take((size_t)N * 4);
     L.rank = take((size_t)N * 4);
@@ -1725,12 +1777,32 @@ int batch_max_tiles(int P, const int *n)
 
 // Plan the batch for the current subdivision mode and tile size: per-plume constants, global
 // cell offsets and the work list, ordered by decreasing estimated cost (candidates per item).
+// Divides `lines` lines among the plumes' regions, one plume behind the other; what is left is the pool.
+void batch_divide(ade_batch *b, size_t lines)
+{
+    size_t line = 0;
+    for (int i = 0; i < b->P; ++i) {
+        ade::RateParams &rp = b->pred[i];
+        rp.fz_stride = std::max(1u, b->plans[i].stride);
+        rp.fz_regions = (unsigned)std::min<size_t>(b->plans[i].regions, (lines - line) / rp.fz_stride);
+        rp.fz_base = (unsigned)line;
+        line += (size_t)rp.fz_regions * rp.fz_stride;
+        b->corr[i].fz_stride = rp.fz_stride;
+        b->corr[i].fz_regions = rp.fz_regions;
+        b->corr[i].fz_base = rp.fz_base;
+    }
+    b->frozen_tab.pool = (unsigned)line;
+    b->frozen_tab.cap = (unsigned)(lines - line);
+    b->divided = lines;
+}
+
 int batch_plan(ade_batch *b)
 {
     b->NC = 0;
+    b->frozen = false;   // (a weight table is for one set of grids)
+    b->plans.clear();
+    b->plan_lines = 0;
     b->items.clear();
-    unsigned fz_line = 0u;
-    b->frozen_fits = true;
     std::vector<std::pair<double, ade::BatchTile>> items;
     for (int i = 0; i < b->P; ++i) {
         ade_params pp = b->params[i];
@@ -1751,12 +1823,9 @@ int batch_plan(ade_batch *b)
         rp.goff = b->offsets[i];
         rp.coff = b->NC;
         rp.frame = b->w.frame + (size_t)i * ade::kFrameWords;
-        if (b->frozen) {   // the plume's chunks' regions, one plume behind the other; what is left is the pool
-            b->frozen_fits = b->frozen_fits && frozen_lines(pp, d.H, b->n[i], d.g) <= b->frozen_plume[i];
-            rp.fz_base = fz_line;
-            rp.fz_stride = frozen_stride(pp, d.H, b->n[i], d.g, 1, b->frozen_plume[i]);
-            fz_line += (unsigned)(frozen_slots(b->n[i], d.g) * rp.fz_stride);
-        }
+        b->plans.push_back(estimate_table(pp, d.H, b->n[i], d.g, 1));
+        b->plan_lines += b->plans[i].lines;
+        for (int t = 0; t < ade::chunk_numbers(b->n[i], d.g.ncells / d.g.nc[0]); ++t) b->items.push_back(ade::FrozenItem{i, t});
         b->ncells[i] = d.g.ncells;
         b->subdiv_choice[i] = d.g.subdiv;
         b->NC += d.g.ncells;
@@ -1771,8 +1840,6 @@ int batch_plan(ade_batch *b)
         }
         b->pred[i] = pr;
         b->corr[i] = co;
-        if (b->frozen)   // chunks of the weight table
-            for (int t = 0; t < ade::chunk_numbers(b->n[i], d.g.ncells / d.g.nc[0]); ++t) b->items.push_back(ade::FrozenItem{i, t});
         // work items and their estimated cost: candidates per particle x particles
         const double ppc = (double)b->n[i] / d.g.ncells;
         double cand = 0.0;
@@ -1787,10 +1854,7 @@ int batch_plan(ade_batch *b)
         }
     }
     if (b->NC > b->NC_max) return fail(ADE_ERR_CAPACITY, "batch cell table exceeds the workspace");
-    size_t fz_total = 0;
-    for (size_t l : b->frozen_plume) fz_total += l;
-    b->frozen_tab.pool = fz_line;
-    b->frozen_tab.cap = (unsigned)(fz_total - fz_line);
+    batch_divide(b, b->plan_lines);
     std::stable_sort(items.begin(), items.end(),
                      [](const std::pair<double, ade::BatchTile> &x, const std::pair<double, ade::BatchTile> &y) {
                          return x.first > y.first;
@@ -1883,8 +1947,16 @@ int batch_enqueue_frozen(ade_batch *b, int steps, cudaStream_t s)
     return ADE_OK;
 }
 
+// Where the parts of a batch's weights buffer lie (behind the counter); returns where the lines begin.
+size_t batch_table(const ade_batch *b, size_t *slots, size_t *C)
+{
+    *slots = 256;
+    *C = *slots + align256(b->items.size() * 32);
+    return *C + align256((size_t)b->N * 16);
+}
+
 // Whether `steps` steps of one call keep the pair weights.
-bool batch_use_frozen(const ade_batch *b, int steps) { return b->frozen && b->frozen_fits && b->N > 0 && steps >= 2; }
+bool batch_use_frozen(const ade_batch *b, int steps) { return b->frozen && steps >= 2; }
 
 int batch_enqueue_steps(ade_batch *b, int steps, cudaStream_t s)
 {
@@ -1941,7 +2013,7 @@ int ade_batch_workspace_bytes(int nplumes, const ade_params *p, const int *n, si
     if (rc) return rc;
     long long N = 0;
     for (int i = 0; i < nplumes; ++i) N += n[i];
-    *bytes = batch_layout(nplumes, (int)N, (int)ncm, batch_max_tiles(nplumes, n), batch_frozen_size(nplumes, p, n)).total;
+    *bytes = batch_layout(nplumes, (int)N, (int)ncm, batch_max_tiles(nplumes, n), batch_max_items(nplumes, p, n)).total;
     return ADE_OK;
 }
 
@@ -1973,8 +2045,7 @@ int ade_batch_init(ade_batch **out, int nplumes, const ade_params *p, const int 
     b->corr.resize(nplumes);
     b->dt.assign(nplumes, 0.0);
     b->D.assign(9 * (size_t)nplumes, 0.0);
-    const BatchFrozen fz = batch_frozen_size(nplumes, p, n);
-    const BatchLayout L = batch_layout(nplumes, b->N, b->NC_max, b->max_tiles, fz);
+    const BatchLayout L = batch_layout(nplumes, b->N, b->NC_max, b->max_tiles, batch_max_items(nplumes, p, n));
     if (b->N > 0 && (!xq_dev || !C_dev)) {
         delete b;
         return fail(ADE_ERR_ARG, "xq_dev and C_dev must be non-NULL");
@@ -2001,12 +2072,6 @@ int ade_batch_init(ade_batch **out, int nplumes, const ade_params *p, const int 
     b->w.cell_start = at<uint32_t>(workspace_dev, L.cell_start);
     b->w.tile_sums = at<uint32_t>(workspace_dev, L.tile_sums);   // cleared with the counts every build
     b->w.frame = at<uint32_t>(workspace_dev, L.frames);
-    b->frozen = fz.lines > 0;
-    b->frozen_tab.words = at<float>(workspace_dev, L.fz_words);
-    b->frozen_tab.slots = at<uint4>(workspace_dev, L.fz_slots);
-    b->frozen_tab.cursor = at<unsigned>(workspace_dev, L.fz_cursor);
-    b->frozen_plume = fz.plume;
-    b->frozen_C = at<float>(workspace_dev, L.fz_C);
     b->d_items = at<ade::FrozenItem>(workspace_dev, L.fz_items);
     b->w.P0 = at<uint4>(workspace_dev, L.P0);
     b->w.P1 = at<uint4>(workspace_dev, L.P1);
@@ -2038,7 +2103,6 @@ int ade_batch_init(ade_batch **out, int nplumes, const ade_params *p, const int 
         std::fill(pid.begin() + b->offsets[i], pid.begin() + b->offsets[i + 1], (uint16_t)i);
     e = cudaSuccess;
     if (b->N > 0) e = cudaMemcpyAsync(b->plume_of, pid.data(), pid.size() * 2, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->frozen_tab.cursor, 0, sizeof(unsigned), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->w.frame, 0, (size_t)nplumes * ade::kFrameWords * 4, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->d_offsets, b->offsets.data(), b->offsets.size() * 4, cudaMemcpyHostToDevice, s);
@@ -2053,6 +2117,69 @@ int ade_batch_init(ade_batch **out, int nplumes, const ade_params *p, const int 
     }
     *out = b;
     return ADE_OK;
+}
+
+int ade_batch_weights_bytes(ade_batch *b, int counted, size_t *bytes, void *stream)
+{
+    if (!b || !bytes) return fail(ADE_ERR_ARG, "NULL argument");
+    *bytes = 0;
+    cudaStream_t s = (cudaStream_t)stream;
+    // the plumes' bins lie in the half-step state, free between steps: as many plumes at a time as fit
+    const size_t one = ade::kChunkBins * sizeof(ade::ChunkBin), at_once = std::min((size_t)b->N * 16 / one, (size_t)b->P);
+    if (counted && at_once > 0) {
+        int rc = not_capturing(s);
+        if (rc == ADE_OK) rc = batch_cells(b, s);
+        if (rc) return rc;
+        ade::ChunkBin *dev = reinterpret_cast<ade::ChunkBin *>(b->w.P1);
+        std::vector<ade::ChunkBin> bins(at_once * ade::kChunkBins);
+        std::vector<ade::TablePlan> plans(b->P);
+        size_t lines = 0;
+        int item = 0;
+        for (int p0 = 0; p0 < b->P; p0 += (int)at_once) {
+            const int m = std::min(b->P - p0, (int)at_once);
+            int last = item;
+            for (int i = 0; i < m; ++i) last += ade::chunk_numbers(b->pred[p0 + i].n, b->pred[p0 + i].ncy * b->pred[p0 + i].ncz);
+            ADE_CK(cudaMemsetAsync(dev, 0, m * one, s));
+            ADE_CK(ade::launch_chunk_need_batch(b->dim, b->w.P0, b->w.cell_start, b->d_pred, b->d_items, item, last, dev, s));
+            ADE_CK(cudaMemcpyAsync(bins.data(), dev, m * one, cudaMemcpyDeviceToHost, s));
+            ADE_CK(cudaStreamSynchronize(s));
+            item = last;
+            for (int i = 0; i < m; ++i) {
+                const ade::RateParams &rp = b->pred[p0 + i];
+                plans[p0 + i] = plan_table(bins.data() + (size_t)i * ade::kChunkBins, (size_t)ade::chunk_numbers(rp.n, rp.ncy * rp.ncz), false);
+                lines += plans[p0 + i].lines;
+            }
+        }
+        b->plans = plans;
+        b->plan_lines = lines;
+        b->divided = 0;
+    }
+    if (b->N == 0 || 128.0 * (double)b->plan_lines > (counted ? ade::kTableMaxBytes : ade::kEstimateMaxBytes)) return ADE_OK;
+    size_t slots, C;
+    *bytes = batch_table(b, &slots, &C) + b->plan_lines * 128;
+    return ADE_OK;
+}
+
+int ade_batch_set_weights(ade_batch *b, void *weights_dev, size_t bytes, void *stream)
+{
+    if (!b) return fail(ADE_ERR_ARG, "batch is NULL");
+    size_t slots, C, lines = 0;
+    if (weights_dev) {
+        const size_t words = batch_table(b, &slots, &C);
+        const int rc = table_lines(weights_dev, bytes, words, 1u, &lines);
+        if (rc) return rc;
+        lines = std::min(lines, b->plan_lines);
+        b->frozen_tab.cursor = at<unsigned long long>(weights_dev, 0);
+        b->frozen_tab.slots = at<uint4>(weights_dev, slots);
+        b->frozen_C = at<float>(weights_dev, C);
+        b->frozen_tab.words = at<float>(weights_dev, words);
+        ADE_CK(cudaMemsetAsync(b->frozen_tab.cursor, 0, sizeof(*b->frozen_tab.cursor), (cudaStream_t)stream));
+    }
+    b->frozen = weights_dev && lines > 0 && b->N > 0;
+    batch_drop_graphs(b);
+    if (!b->frozen || lines == b->divided) return ADE_OK;
+    batch_divide(b, lines);
+    return batch_upload(b, (cudaStream_t)stream);
 }
 
 int ade_batch_step(ade_batch *b, int nsteps, void *stream)
@@ -2348,6 +2475,8 @@ struct ade_sweep {
     long long step = 0, pairs = 0;
     uint32_t inc[3], inc_half[3];
     bool status_cleared = false, count_clean = false, iso = false;
+    bool table = false, cursor_clean = false;   // a weight table (ade_sweep_set_weights) and its counter
+    ade::TablePlan plan = {}, estimate = {};    // as last asked for; for an even set
     ade::SweepRun run = {};
     // captured runs of 1..kGraphSteps steps, each on the first call that needs it
     cudaGraph_t graph[ade::kGraphSteps + 1] = {};
@@ -2361,7 +2490,7 @@ namespace {
 
 struct SweepLayout {
     Derived d;
-    size_t Cs0, Cs1, pstats, words, slots, dense, cursor, lines, total;
+    size_t Cs0, Cs1, pstats, total;
 };
 
 // Common parameters and workspace of a sweep.  theta may be NULL (workspace size only: the layout
@@ -2417,14 +2546,9 @@ int sweep_layout(const ade_params *p, int n, int P, const double *theta, ade_par
         off += align256(bytes > 0 ? bytes : 1);
         return o;
     };
-    L->Cs0 = take((size_t)n * P4 * 8);   // each pencil twice
-    L->Cs1 = take((size_t)n * P4 * 8);
+    L->Cs0 = take((size_t)n * P4 * 4);
+    L->Cs1 = take((size_t)n * P4 * 4);
     L->pstats = take((size_t)3 * P * 8);
-    L->lines = n > 0 ? std::min(frozen_lines(pp, L->d.H, n, L->d.g, 2), (size_t)(kFrozenMaxBytes / 128.0)) : 0;
-    L->words = take(L->lines * 128);
-    L->slots = take(frozen_slots(n, L->d.g) * 32);
-    L->dense = take(frozen_slots(n, L->d.g) * 4);
-    L->cursor = take(64);
     L->total = off;
     if (pp_out) *pp_out = pp;
     return ADE_OK;
@@ -2437,9 +2561,12 @@ int sweep_clear_once(ade_sweep *sw, cudaStream_t s)
     if (!sw->count_clean) {
         ADE_CK(cudaMemsetAsync(sw->w.count, 0, (size_t)sw->ncells * sizeof(uint32_t), s));
         ADE_CK(cudaMemsetAsync(sw->w.tile_sums, 0, ade::tile_sums_bytes(sw->ncells), s));
-        ADE_CK(cudaMemsetAsync(sw->run.tab.cursor, 0, sizeof(unsigned), s));
         ADE_CK(cudaMemsetAsync(sw->w.frame, 0, ade::kFrameWords * 4, s));
         sw->count_clean = true;
+    }
+    if (sw->table && !sw->cursor_clean) {
+        ADE_CK(cudaMemsetAsync(sw->run.tab.cursor, 0, sizeof(*sw->run.tab.cursor), s));
+        sw->cursor_clean = true;
     }
     return ADE_OK;
 }
@@ -2489,7 +2616,7 @@ int sweep_begin(ade_sweep *sw, int steps, cudaStream_t s)
 
 // Whether a call of `steps` steps fills the table: it costs about three evaluations' gain (512^2, 8 sets:
 // 71 us against 95 - 72 per evaluation), so from four evaluations on.
-bool sweep_use_table(const ade_sweep *sw, int steps) { return 2 * steps * (int)sw->groups.size() >= 4; }
+bool sweep_use_table(const ade_sweep *sw, int steps) { return sw->table && 2 * steps * (int)sw->groups.size() >= 4; }
 
 // The predictors or correctors of every group with the geometry on the fly (one step).
 int sweep_evals_fly(ade_sweep *sw, int epi, cudaStream_t s)
@@ -2521,11 +2648,15 @@ int sweep_begin_fly(ade_sweep *sw, cudaStream_t s)
 // `steps` steps of one call.
 int sweep_steps(ade_sweep *sw, int steps, cudaStream_t s)
 {
-    if (!sweep_use_table(sw, steps)) {   // (one step of one group)
-        int rc = sweep_begin_fly(sw, s);
-        if (rc || sw->n == 0) return rc;
-        rc = sweep_evals_fly(sw, ade::EPI_PREDICT, s);
-        return rc ? rc : sweep_evals_fly(sw, ade::EPI_CORRECT, s);
+    if (!sweep_use_table(sw, steps)) {
+        int rc = ADE_OK;
+        for (int k = 0; rc == ADE_OK && k < steps; ++k) {
+            rc = sweep_begin_fly(sw, s);
+            if (rc || sw->n == 0) continue;
+            rc = sweep_evals_fly(sw, ade::EPI_PREDICT, s);
+            if (rc == ADE_OK) rc = sweep_evals_fly(sw, ade::EPI_CORRECT, s);
+        }
+        return rc;
     }
     int rc = sweep_begin(sw, steps, s);
     for (int k = 0; rc == ADE_OK && sw->n > 0 && k < steps; ++k) {
@@ -2545,6 +2676,16 @@ int sweep_eval_fly(ade_sweep *sw, bool count, const ade::SweepOut &out, cudaStre
         if (count) break;   // the geometry is the same for every group
     }
     return ADE_OK;
+}
+
+void sweep_drop_graphs(ade_sweep *sw)
+{
+    for (int k = 0; k <= ade::kGraphSteps; ++k) {
+        if (sw->graph_exec[k]) cudaGraphExecDestroy(sw->graph_exec[k]);
+        if (sw->graph[k]) cudaGraphDestroy(sw->graph[k]);
+        sw->graph_exec[k] = nullptr;
+        sw->graph[k] = nullptr;
+    }
 }
 
 int sweep_clear_status_once(ade_sweep *sw, cudaStream_t s)
@@ -2629,18 +2770,10 @@ int ade_sweep_init(ade_sweep **out, const ade_params *p, int n, int ntheta, cons
     sw->w.pencil = at<uint4>(workspace_dev, W.pencil);
     sw->rp.frame = sw->w.frame;
     sw->rp.pencil = sw->w.pencil;
+    sw->estimate = estimate_table(pp, L.d.H, n, L.d.g, 2);
     sw->run.P = sw->w.P0;
     sw->run.cs = sw->w.cell_start;
     sw->run.perm = sw->w.perm;
-    sw->run.C = sw->Cs0;
-    sw->run.Ch = sw->Cs1;
-    sw->run.tab.words = at<float>(workspace_dev, L.words);
-    sw->run.tab.slots = at<uint4>(workspace_dev, L.slots);
-    if (ade::chunk_numbers(n, L.d.g.nc[1] * L.d.g.nc[2]) > ade::kCountChunksFrom) sw->run.tab.dense = at<uint32_t>(workspace_dev, L.dense);
-    sw->run.tab.cursor = at<unsigned>(workspace_dev, L.cursor);
-    sw->rp.fz_stride = n > 0 ? frozen_stride(pp, L.d.H, n, L.d.g, 2, L.lines) : 0u;
-    sw->run.tab.pool = (unsigned)(frozen_slots(n, L.d.g) * sw->rp.fz_stride);
-    sw->run.tab.cap = (unsigned)L.lines - sw->run.tab.pool;
     sw->theta.assign(theta_host, theta_host + 3 * ntheta);
     // Dcal = a u + b per set (uniform v, K = 2D)
     const int dm = pp.dim;
@@ -2688,6 +2821,54 @@ int ade_sweep_get_info(const ade_sweep *sw, ade_info *info)
     info->stencil_rows = sw->rp.nrows;
     info->sort_passes = 1;
     info->tile[0] = (int)sw->groups.size();   // launches per evaluation
+    return ADE_OK;
+}
+
+int ade_sweep_weights_bytes(ade_sweep *sw, int counted, size_t *bytes, void *stream)
+{
+    if (!sw || !bytes) return fail(ADE_ERR_ARG, "NULL argument");
+    *bytes = 0;
+    cudaStream_t s = (cudaStream_t)stream;
+    const int np = sw->nc[1] * sw->nc[2];
+    ade::TablePlan plan = sw->estimate;
+    ade::ChunkBin bins[ade::kChunkBins];
+    if (counted && (size_t)sw->n * 16 >= sizeof(bins)) {
+        int rc = not_capturing(s);
+        if (rc == ADE_OK) rc = sweep_cells(sw, 0, s);
+        if (rc) return rc;
+        ade::ChunkBin *dev = reinterpret_cast<ade::ChunkBin *>(sw->w.P1);
+        ADE_CK(cudaMemsetAsync(dev, 0, sizeof(bins), s));
+        ADE_CK(ade::launch_chunk_need(sw->dim, sw->iso, sw->w.P0, sw->w.cell_start, sw->rp, 2, dev, s));
+        ADE_CK(cudaMemcpyAsync(bins, dev, sizeof(bins), cudaMemcpyDeviceToHost, s));
+        ADE_CK(cudaStreamSynchronize(s));
+        plan = plan_table(bins, (size_t)ade::chunk_numbers(sw->n, np), counts_chunks(sw->n, np));
+    }
+    if (sw->n == 0 || 128.0 * (double)plan.lines > (counted ? ade::kTableMaxBytes : ade::kEstimateMaxBytes)) return ADE_OK;
+    sw->plan = plan;
+    *bytes = table_layout((size_t)ade::chunk_numbers(sw->n, np) + 1, (size_t)sw->n * sw->P4 * 16).words + plan.lines * 128;
+    return ADE_OK;
+}
+
+int ade_sweep_set_weights(ade_sweep *sw, void *weights_dev, size_t bytes)
+{
+    if (!sw) return fail(ADE_ERR_ARG, "sweep is NULL");
+    size_t lines = 0;
+    if (weights_dev) {
+        const int np = sw->nc[1] * sw->nc[2];
+        const TableLayout L = table_layout((size_t)ade::chunk_numbers(sw->n, np) + 1, (size_t)sw->n * sw->P4 * 16);
+        const int rc = table_lines(weights_dev, bytes, L.words, sw->plan.stride, &lines);
+        if (rc) return rc;
+        sw->run.tab.words = at<float>(weights_dev, L.words);
+        sw->run.tab.slots = at<uint4>(weights_dev, L.slots);
+        sw->run.tab.cursor = at<unsigned long long>(weights_dev, L.cursor);
+        sw->run.tab.dense = counts_chunks(sw->n, np) ? at<uint32_t>(weights_dev, L.dense) : nullptr;
+        sw->run.C = at<float>(weights_dev, L.C);
+        sw->run.Ch = sw->run.C + 2 * (size_t)sw->n * sw->P4;
+        ade::divide_table(sw->plan, lines, &sw->rp, &sw->run.tab);
+        sw->cursor_clean = false;
+    }
+    sw->table = weights_dev && lines > 0;
+    sweep_drop_graphs(sw);
     return ADE_OK;
 }
 
@@ -2853,10 +3034,7 @@ int ade_sweep_stats(ade_sweep *sw, ade_stats *st, void *stream)
 void ade_sweep_destroy(ade_sweep *sw)
 {
     if (!sw) return;
-    for (int k = 0; k <= ade::kGraphSteps; ++k) {
-        if (sw->graph_exec[k]) cudaGraphExecDestroy(sw->graph_exec[k]);
-        if (sw->graph[k]) cudaGraphDestroy(sw->graph[k]);
-    }
+    sweep_drop_graphs(sw);
     if (sw->cap_stream) cudaStreamDestroy(sw->cap_stream);
     if (sw->ev_ready)
         for (int k = 0; k < 4; ++k) cudaEventDestroy(sw->ev[k]);

@@ -350,17 +350,13 @@ __device__ __noinline__ float walk_chunk(const uint4 *__restrict__ P, const uint
 // transverse boxes (kCutBox), as in the trimmed walks.
 enum ChunkCut { kCutFull = 0, kCutBand = 1, kCutBox = 2 };
 
-// Weights (VAL 1) or g_L, g_T (VAL 2) of one chunk into the table; VAL 1 returns the row sums of the
-// first evaluation (the concentrations of the records).  One pass over the rows: the chunk's lines go
-// to a region of fixed size (prm.fz_stride lines, the host's estimate for the grid) and only a chunk that
-// outgrows it is done again into room taken from the pool behind.  Rows are tested once per warp, each
-// lane's range is cut by its own distance to the row and then to its first and last candidate that may
-// lie inside H.  Bound: instruction issue.  128^3 cube 1.55 -> 1.15 ms, 1024^2 258 -> 200 us against a
-// form that counted every chunk's lines in a pass of its own.
-template <int DIM, int KERNEL, bool ISO, int CUT, int VAL, bool FINE = false>
-__device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs, const RateParams &prm,
-                             const Chunk &c, const uint4 &pa, const TrimRow *srow, const FrozenTab &tab,
-                             const ShapeConst &sc = ShapeConst())
+// Calls f(q's first and end particle, first candidate s, longest lane's count m, row word) for each row of
+// chunk c that holds a candidate within H of some lane: the lanes' contiguous ranges of the row's pencil,
+// cut as CUT says.  Rows are tested once per warp, each lane's range is cut by its own distance to the row
+// and then to its first and last candidate that may lie inside H.
+template <int DIM, bool ISO, int CUT, class F>
+__device__ __forceinline__ void chunk_rows(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs, const RateParams &prm,
+                                           const Chunk &c, const uint4 &pa, const TrimRow *srow, F f)
 {
     const int lane = threadIdx.x & 31;
     const int ncx = prm.ncx, nrows = prm.nrows;
@@ -371,132 +367,152 @@ __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const 
     const TrimGeom g(prm);
     const float wpc = 4294967296.f / (float)ncx;     // x words per cell
     const PairConst k(prm);
-    const PairConst2 k2(k, k.m1);
     const float far2 = prm.H2 * (1.f + 1.f / 4096.f);   // beyond this the weight is exactly 0
-    const float Ca = __uint_as_float(pa.w);
     if (CUT != kCutFull) {
         me = trim_self<DIM>(pa, c.cy, c.cz, prm);
         ylo = yhi = me.fy;
         zlo = zhi = me.fz;
         warp_interval<DIM>(ylo, yhi, zlo, zhi);
     }
-    const unsigned hs = (unsigned)(nrows + 31) >> 5;    // header lines: a word per row
-    unsigned base = prm.fz_base + (unsigned)c.local * prm.fz_stride, room = prm.fz_stride;
+    for (int rb = 0; rb < nrows; rb += 32) {
+        float xe = 0.f;
+        int pidx = 0, wx = 0;
+        bool reach = rb + lane < nrows;
+        if (CUT == kCutBox) {
+            reach = warp_row_test<DIM>(rb, srow, nrows, me, c.cy, c.cz, prm, g, ylo, yhi, zlo, zhi, xe, pidx, wx);
+        } else if (reach) {
+            const StencilRow r = prm.rows[rb + lane];
+            pidx = row_pencil_of<DIM>(r, c.cy, c.cz, prm);
+            wx = (r.w & 0xff) | (r.dy == 0 && (DIM == 2 || r.dz == 0) ? 1 << 24 : 0);
+            if (CUT == kCutBand) {
+                const TrimRow tr{(float)r.dy, (float)r.dz, 0, 0};
+                const float e2 = row_gap2<DIM>(make_float4(0.f, 1.f, 0.f, DIM == 3 ? 1.f : 0.f), tr, ylo, yhi, yhi - ylo, zlo, zhi,
+                                               zhi - zlo, g);
+                const float t = fmaxf(g.Hm2 - e2, 0.f);
+                xe = fmaf(t * rsqrt_ftz(fmaxf(t, 1.f)), g.inv_wx, 1.f / 4096.f);
+                reach = e2 < g.Hm2;
+            }
+        }
+        for (unsigned mask = __ballot_sync(kFull, reach); mask != 0u; mask &= mask - 1u) {
+            const int b = __ffs(mask) - 1;
+            const int q = __shfl_sync(kFull, pidx, b), wb = __shfl_sync(kFull, wx, b), w = wb & 0xff;
+            int dlo = -w, dhi = w, xw = 0x7fffffff;          // xw: the lane's x half-extent in words
+            if (CUT == kCutBox) {
+                const TrimRow tr = srow[rb + b];
+                const float e2 = row_gap2<DIM>(load_box(prm, q), tr, me.fy, me.fy, 0.f, me.fz, me.fz, 0.f, g);
+                const float t = g.Hm2 - e2, xl = t > 0.f ? fmaf(t * rsqrt_ftz(t), g.inv_wx, 1.f / 4096.f) : 0.f;
+                dlo = max(__float2int_rd(me.fx - xl), -w);
+                dhi = min(__float2int_rd(me.fx + xl), w);
+                xw = t > 0.f ? __float2int_ru(fminf(xl * wpc, 2.0e9f)) : -1;
+            } else if (CUT == kCutBand) {
+                const float xeb = __shfl_sync(kFull, xe, b);
+                dlo = max(__float2int_rd(me.fx - xeb), -w);
+                dhi = min(__float2int_rd(me.fx + xeb), w);
+            }
+            const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
+            int s, cnt;
+            cyclic_range(cs, q * ncx, cx + dlo, cx + dhi + 1, ncx, qs, qe, s, cnt);
+            if (!valid || xw < 0) cnt = 0;
+            if (s >= qe) s = qs;                     // (the range's first cells are empty)
+            // Both ends' two outermost candidates are looked at together (one latency): farther than xw
+            // along x, or than H, their weight is exactly 0.
+            auto out_of = [&](int t) {
+                const int j = s + t, jj = j >= qe ? j - len : j;
+                if (CUT == kCutBox) {
+                    const int d = (int)(__ldg(&P[jj].x) - pa.x);
+                    return d < -xw || d > xw;
+                }
+                return !(sep2<DIM, ISO>(pa, __ldg(P + jj), k) < far2);
+            };
+            while (cnt > 0) {
+                const bool f0 = out_of(0), f1 = out_of(min(1, cnt - 1)), b0 = out_of(cnt - 1), b1 = out_of(max(cnt - 2, 0));
+                const int df = f0 ? (f1 ? 2 : 1) : 0, db = b0 ? (b1 ? 2 : 1) : 0, left = cnt - df - db;
+                if (left <= 0) {                     // the ends meet: what is left, if anything, lies between
+                    if (f0 && f1 && b0 && b1 && cnt <= 4) cnt = 0;
+                    break;
+                }
+                s += df;
+                if (s >= qe) s -= len;
+                cnt = left;
+                if (df < 2 && db < 2) break;
+            }
+            const int m = (int)__reduce_max_sync(kFull, (unsigned)cnt);
+            if (m > 0) f(qs, qe, s, m, wb);
+        }
+    }
+}
+
+// Lines that hold the rows' lengths, a word per row.
+__device__ __forceinline__ unsigned header_lines(const RateParams &prm) { return (unsigned)(prm.nrows + 31) >> 5; }
+
+// Weights (VAL 1) or g_L, g_T (VAL 2) of one chunk into the table; VAL 1 returns the row sums of the
+// first evaluation (the concentrations of the records).  One pass over the rows: the chunk's lines go
+// to its region (prm.fz_stride lines, what nearly every chunk needs: plan_table in api.cu) and only a chunk
+// that outgrows it is done again into room taken from the pool behind; fz_stride 0: no table.
+// Bound: instruction issue.  128^3 cube 1.55 -> 1.15 ms, 1024^2 258 -> 200 us against a
+// form that counted every chunk's lines in a pass of its own.
+template <int DIM, int KERNEL, bool ISO, int CUT, int VAL, bool FINE = false>
+__device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs, const RateParams &prm,
+                             const Chunk &c, const uint4 &pa, const TrimRow *srow, const FrozenTab &tab,
+                             const ShapeConst &sc = ShapeConst())
+{
+    const int lane = threadIdx.x & 31;
+    const PairConst k(prm);
+    const PairConst2 k2(k, k.m1);
+    const float Ca = __uint_as_float(pa.w);
+    const unsigned hs = header_lines(prm);
+    unsigned base = prm.fz_base + (unsigned)c.local * prm.fz_stride, room = (unsigned)c.local < prm.fz_regions ? prm.fz_stride : 0u;
     float acc = 0.f, comp = 0.f;
-    unsigned R = 0u, used = 0u;
-    for (int attempt = 0; attempt < 2; ++attempt) {
+    unsigned R = 0u, used = 0xffffffffu;
+    for (int attempt = 0; attempt < (prm.fz_stride > 0u ? 2 : 0); ++attempt) {
         acc = comp = 0.f;
         R = 0u;
         used = hs;
         float *hdr = tab.words + (size_t)base * 32;
         float *out = hdr + hs * 32 + lane;
-        for (int rb = 0; rb < nrows; rb += 32) {
-            float xe = 0.f;
-            int pidx = 0, wx = 0;
-            bool reach = rb + lane < nrows;
-            if (CUT == kCutBox) {
-                reach = warp_row_test<DIM>(rb, srow, nrows, me, c.cy, c.cz, prm, g, ylo, yhi, zlo, zhi, xe, pidx, wx);
-            } else if (reach) {
-                const StencilRow r = prm.rows[rb + lane];
-                pidx = row_pencil_of<DIM>(r, c.cy, c.cz, prm);
-                wx = (r.w & 0xff) | (r.dy == 0 && (DIM == 2 || r.dz == 0) ? 1 << 24 : 0);
-                if (CUT == kCutBand) {
-                    const TrimRow tr{(float)r.dy, (float)r.dz, 0, 0};
-                    const float e2 = row_gap2<DIM>(make_float4(0.f, 1.f, 0.f, DIM == 3 ? 1.f : 0.f), tr, ylo, yhi, yhi - ylo, zlo, zhi,
-                                                   zhi - zlo, g);
-                    const float t = fmaxf(g.Hm2 - e2, 0.f);
-                    xe = fmaf(t * rsqrt_ftz(fmaxf(t, 1.f)), g.inv_wx, 1.f / 4096.f);
-                    reach = e2 < g.Hm2;
-                }
+        chunk_rows<DIM, ISO, CUT>(P, cs, prm, c, pa, srow, [&](int qs, int qe, int s, int m, int wb) {
+            const int len = qe - qs;
+            // idle tail iterations of a shorter lane stay inside the doubled pencil (m <= len)
+            used = add_lines(used, 1u + (unsigned)(m * VAL));
+            const bool keep = used <= room;
+            if (keep) {
+                if (lane == 0) hdr[R] = __int_as_float(m);
+                out[0] = __int_as_float(s + qs);     // index into the doubled concentrations
             }
-            for (unsigned mask = __ballot_sync(kFull, reach); mask != 0u; mask &= mask - 1u) {
-                const int b = __ffs(mask) - 1;
-                const int q = __shfl_sync(kFull, pidx, b), wb = __shfl_sync(kFull, wx, b), w = wb & 0xff;
-                int dlo = -w, dhi = w, xw = 0x7fffffff;          // xw: the lane's x half-extent in words
-                if (CUT == kCutBox) {
-                    const TrimRow tr = srow[rb + b];
-                    const float e2 = row_gap2<DIM>(load_box(prm, q), tr, me.fy, me.fy, 0.f, me.fz, me.fz, 0.f, g);
-                    const float t = g.Hm2 - e2, xl = t > 0.f ? fmaf(t * rsqrt_ftz(t), g.inv_wx, 1.f / 4096.f) : 0.f;
-                    dlo = max(__float2int_rd(me.fx - xl), -w);
-                    dhi = min(__float2int_rd(me.fx + xl), w);
-                    xw = t > 0.f ? __float2int_ru(fminf(xl * wpc, 2.0e9f)) : -1;
-                } else if (CUT == kCutBand) {
-                    const float xeb = __shfl_sync(kFull, xe, b);
-                    dlo = max(__float2int_rd(me.fx - xeb), -w);
-                    dhi = min(__float2int_rd(me.fx + xeb), w);
+            ++R;
+            if (!keep) return;                       // to be done again
+            out += 32;
+            float rs = 0.f;
+            if (VAL == 2) {
+                float2 *o2 = reinterpret_cast<float2 *>(out + lane);
+                int t = 0;
+                for (; t + 1 < m; t += 2) {
+                    const int j0 = s + t, j1 = j0 + 1;
+                    float2 gL, gT;
+                    pair_shape2<DIM, KERNEL, ISO, FINE>(pa, __ldg(P + (j0 >= qe ? j0 - len : j0)), __ldg(P + (j1 >= qe ? j1 - len : j1)),
+                                                  k2, sc, gL, gT);
+                    o2[t * 32] = f2(gL.x, gT.x);
+                    o2[(t + 1) * 32] = f2(gL.y, gT.y);
                 }
-                const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
-                int s, cnt;
-                cyclic_range(cs, q * ncx, cx + dlo, cx + dhi + 1, ncx, qs, qe, s, cnt);
-                if (!valid || xw < 0) cnt = 0;
-                if (s >= qe) s = qs;                     // (the range's first cells are empty)
-                // Both ends' two outermost candidates are looked at together (one latency): farther than xw
-                // along x, or than H, their weight is exactly 0.
-                auto out_of = [&](int t) {
-                    const int j = s + t, jj = j >= qe ? j - len : j;
-                    if (CUT == kCutBox) {
-                        const int d = (int)(__ldg(&P[jj].x) - pa.x);
-                        return d < -xw || d > xw;
-                    }
-                    return !(sep2<DIM, ISO>(pa, __ldg(P + jj), k) < far2);
-                };
-                while (cnt > 0) {
-                    const bool f0 = out_of(0), f1 = out_of(min(1, cnt - 1)), b0 = out_of(cnt - 1), b1 = out_of(max(cnt - 2, 0));
-                    const int df = f0 ? (f1 ? 2 : 1) : 0, db = b0 ? (b1 ? 2 : 1) : 0, left = cnt - df - db;
-                    if (left <= 0) {                     // the ends meet: what is left, if anything, lies between
-                        if (f0 && f1 && b0 && b1 && cnt <= 4) cnt = 0;
-                        break;
-                    }
-                    s += df;
-                    if (s >= qe) s -= len;
-                    cnt = left;
-                    if (df < 2 && db < 2) break;
+                if (t < m) {
+                    const int j = s + t;
+                    o2[t * 32] = pair_shape<DIM, KERNEL, ISO, FINE>(pa, __ldg(P + (j >= qe ? j - len : j)), k2, sc);
                 }
-                const int m = (int)__reduce_max_sync(kFull, (unsigned)cnt);
-                if (m == 0) continue;
-                // idle tail iterations of a shorter lane stay inside the doubled pencil (m <= len)
-                used = add_lines(used, 1u + (unsigned)(m * VAL));
-                const bool keep = used <= room;
-                if (keep) {
-                    if (lane == 0) hdr[R] = __int_as_float(m);
-                    out[0] = __int_as_float(s + qs);     // index into the doubled concentrations
-                }
-                ++R;
-                if (!keep) continue;                     // to be done again
-                out += 32;
-                float rs = 0.f;
-                if (VAL == 2) {
-                    float2 *o2 = reinterpret_cast<float2 *>(out + lane);
-                    int t = 0;
-                    for (; t + 1 < m; t += 2) {
-                        const int j0 = s + t, j1 = j0 + 1;
-                        float2 gL, gT;
-                        pair_shape2<DIM, KERNEL, ISO, FINE>(pa, __ldg(P + (j0 >= qe ? j0 - len : j0)), __ldg(P + (j1 >= qe ? j1 - len : j1)),
-                                                      k2, sc, gL, gT);
-                        o2[t * 32] = f2(gL.x, gT.x);
-                        o2[(t + 1) * 32] = f2(gL.y, gT.y);
-                    }
-                    if (t < m) {
-                        const int j = s + t;
-                        o2[t * 32] = pair_shape<DIM, KERNEL, ISO, FINE>(pa, __ldg(P + (j >= qe ? j - len : j)), k2, sc);
-                    }
-                } else if (__any_sync(kFull, s + m > qe)) {
-                    rs = row_weights<DIM, KERNEL, ISO, true, true>(P, pa, Ca, k, k2, s, m, qe, len, out);
-                } else if ((wb >> 24) != 0) {
-                    rs = row_weights<DIM, KERNEL, ISO, true, false>(P, pa, Ca, k, k2, s, m, qe, len, out);
-                } else {
-                    rs = row_weights<DIM, KERNEL, ISO, false, false>(P, pa, Ca, k, k2, s, m, qe, len, out);
-                }
-                out += m * 32 * VAL;
-                neumaier_add(acc, comp, rs);
+            } else if (__any_sync(kFull, s + m > qe)) {
+                rs = row_weights<DIM, KERNEL, ISO, true, true>(P, pa, Ca, k, k2, s, m, qe, len, out);
+            } else if ((wb >> 24) != 0) {
+                rs = row_weights<DIM, KERNEL, ISO, true, false>(P, pa, Ca, k, k2, s, m, qe, len, out);
+            } else {
+                rs = row_weights<DIM, KERNEL, ISO, false, false>(P, pa, Ca, k, k2, s, m, qe, len, out);
             }
-        }
+            out += m * 32 * VAL;
+            neumaier_add(acc, comp, rs);
+        });
         if (used <= room || attempt == 1) break;
         // outgrown: once more into the pool
         unsigned at = 0u;
         if (lane == 0)
-            at = claim_lines(*(volatile unsigned *)tab.cursor, tab.cap, used,
-                             [&](unsigned seen, unsigned next) { return atomicCAS(tab.cursor, seen, next); });
+            at = claim_lines(atomicAdd(tab.cursor, (unsigned long long)used), tab.cap, used);
         at = __shfl_sync(kFull, at, 0);
         if (at == kNoRoom) {
             room = 0u;

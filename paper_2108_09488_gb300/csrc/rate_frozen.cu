@@ -151,6 +151,50 @@ __global__ __launch_bounds__(kT, 12) void k_frozen_rate_batch(const uint4 *__res
     frozen_epilogue<EPI>(prm, st, c, i, prm.upf * shape_unscale<KERNEL>() * sum, st.C[c.ps + i], 0.f);
 }
 
+// Lines one chunk needs (the rows and ranges of build_chunk) into two bins per octave.
+template <int DIM, bool ISO, int CUT>
+__device__ __forceinline__ void bin_chunk(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs, const RateParams &prm,
+                                          const Chunk &c, const TrimRow *srow, int val, ChunkBin *__restrict__ bins)
+{
+    const int lane = threadIdx.x & 31;
+    const uint4 pa = __ldg(P + min(c.i0 + lane, c.pe - 1));
+    unsigned used = header_lines(prm);
+    chunk_rows<DIM, ISO, CUT>(P, cs, prm, c, pa, srow,
+                              [&](int, int, int, int m, int) { used = add_lines(used, 1u + (unsigned)(m * val)); });
+    if (lane != 0) return;
+    const int top = 31 - __clz((int)used);
+    ChunkBin *b = bins + 2 * top + (top > 0 ? (used >> (top - 1)) & 1 : 0);
+    atomicAdd(&b->count, 1u);
+    atomicMax(&b->most, used);
+    atomicAdd(&b->sum, (unsigned long long)used);
+}
+
+template <int DIM, bool ISO>
+__global__ __launch_bounds__(kT) void k_chunk_need(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
+                                                   const RateParams prm, int val, ChunkBin *__restrict__ bins)
+{
+    pdl_wait();
+    __shared__ TrimRow srow[ISO ? kMaxRows : 1];
+    if (ISO) stage_trim_rows(srow, prm);
+    Chunk c;
+    if (find_chunk(cs, prm, nullptr, warp_number(), c)) bin_chunk<DIM, ISO, ISO ? kCutBox : kCutFull>(P, cs, prm, c, srow, val, bins);
+}
+
+template <int DIM>
+__global__ __launch_bounds__(kT) void k_chunk_need_batch(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
+                                                         const RateParams *__restrict__ descs, const FrozenItem *__restrict__ items,
+                                                         int first, int last, ChunkBin *__restrict__ bins)
+{
+    pdl_wait();
+    const int w = first + warp_number();
+    if (w >= last) return;
+    const FrozenItem it = items[w];
+    const RateParams &prm = descs[it.plume];
+    Chunk c;
+    if (find_chunk(cs + prm.coff, prm, nullptr, it.chunk, c))
+        bin_chunk<DIM, true, kCutBand>(P, cs + prm.coff, prm, c, nullptr, 1, bins + (size_t)(it.plume - items[first].plume) * kChunkBins);
+}
+
 constexpr int kCountT = 1024, kCountItems = 16;
 
 // Chunks before each pencil: one block, kCountItems pencils per thread at a time (their loads in flight
@@ -202,7 +246,7 @@ __global__ __launch_bounds__(kT) void k_frozen_finish_batch(const uint4 *__restr
     pdl_wait();
     pdl_trigger();
     const int i = blockIdx.x * kT + threadIdx.x;
-    if (i == 0) *tab.cursor = 0u;
+    if (i == 0) *tab.cursor = 0ull;
     if (i >= n) return;
     const uint32_t a = __ldg(perm + i);
     if (a >= (uint32_t)n) return;
@@ -232,7 +276,7 @@ __global__ __launch_bounds__(kT) void k_frozen_finish(const uint4 *__restrict__ 
     pdl_wait();
     pdl_trigger();
     const int i = blockIdx.x * kT + threadIdx.x;
-    if (i == 0) *tab.cursor = 0u;   // the next call's table starts empty
+    if (i == 0) *tab.cursor = 0ull;   // the next call's table starts empty
     Acc acc{0.f, 0.f, __int_as_float(0x7f800000), __int_as_float(0xff800000), 0u};
     if (i < prm.n) {
         const uint32_t a = __ldg(perm + i);
@@ -279,6 +323,23 @@ cudaError_t rate_t(int epi, const uint4 *P, const uint32_t *cs, const RateParams
 unsigned frozen_blocks(const RateParams &prm)
 {
     return (unsigned)((chunk_numbers(prm.n, prm.ncy * prm.ncz) + kT / 32 - 1) / (kT / 32));
+}
+
+cudaError_t launch_chunk_need(int dim, bool iso, const uint4 *P, const uint32_t *cs, const RateParams &prm, int val,
+                              ChunkBin *bins, cudaStream_t s)
+{
+    auto go = [&](auto kernel) { return launch_pdl(kernel, frozen_blocks(prm), kT, 0, s, P, cs, prm, val, bins); };
+    if (iso) return dim == 2 ? go(k_chunk_need<2, true>) : go(k_chunk_need<3, true>);
+    return dim == 2 ? go(k_chunk_need<2, false>) : go(k_chunk_need<3, false>);
+}
+
+cudaError_t launch_chunk_need_batch(int dim, const uint4 *P, const uint32_t *cs, const RateParams *descs, const FrozenItem *items,
+                                    int first, int last, ChunkBin *bins, cudaStream_t s)
+{
+    if (last <= first) return cudaSuccess;
+    const unsigned nb = (unsigned)((last - first + kT / 32 - 1) / (kT / 32));
+    return dim == 2 ? launch_pdl(k_chunk_need_batch<2>, nb, kT, 0, s, P, cs, descs, items, first, last, bins)
+                    : launch_pdl(k_chunk_need_batch<3>, nb, kT, 0, s, P, cs, descs, items, first, last, bins);
 }
 
 cudaError_t launch_chunk_numbers(const uint32_t *cs, const RateParams &prm, uint32_t *dense, cudaStream_t s)

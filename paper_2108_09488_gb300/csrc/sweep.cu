@@ -211,7 +211,7 @@ __global__ __launch_bounds__(kT, 5) void k_sweep_pass(const uint4 *__restrict__ 
 {
     pdl_wait();
     const bool last = EPI == EPI_CORRECT && out.C;
-    if (last && blockIdx.x == 0 && threadIdx.x == 0) *tab.cursor = 0u;   // the next table starts empty
+    if (last && blockIdx.x == 0 && threadIdx.x == 0) *tab.cursor = 0ull;   // the next table starts empty
     const int g0 = sp.g0;
     Chunk c;
     uint4 sl;

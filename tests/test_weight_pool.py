@@ -1,6 +1,6 @@
 """The counter of the weight table's pool of lines (csrc/pool.h), on the CPU: a sequence of claims
-whose demands pass 2^32 lines several times over never gets a line twice and never lines beyond the
-pool, whatever the interleaving of the compare-and-swaps."""
+whose demands pass 2^32 lines many times over never gets a line twice and never lines beyond the
+pool.  The same check finds out a 32-bit counter."""
 import os
 import shutil
 import subprocess
@@ -16,66 +16,41 @@ SRC = r"""
 #include <vector>
 #include "pool.h"
 
-// Claims of 1..most lines from a pool of `cap` until `demand` lines were asked for; every third
-// compare-and-swap first lets another claimant through.  plain_add: the counter that every demand is
-// added to, which the check has to find out.
-static int check(unsigned cap, unsigned most, unsigned long long demand, bool plain_add = false)
+// Claims of 1..most lines from a pool of `cap` until `demand` lines were asked for.
+template <class Counter>
+static int check(unsigned cap, unsigned most, unsigned long long demand)
 {
     std::mt19937 g(7);
     std::vector<std::uint8_t> owned(cap, 0);
-    unsigned cursor = 0;
-    unsigned long long asked = 0, granted = 0;
-    int turn = 0;
-    auto take = [&](unsigned at, unsigned used) {
-        if (at == ade::kNoRoom) return true;
-        if (at > cap || used > cap - at) return false;
+    Counter cursor = 0;
+    unsigned long long granted = 0;
+    for (unsigned long long asked = 0; asked < demand;) {
+        const unsigned used = 1u + g() % most;
+        const Counter before = cursor;
+        asked += used;
+        cursor += used;
+        const unsigned at = ade::claim_lines(before, cap, used);
+        if (at == ade::kNoRoom) continue;
+        if (at > cap || used > cap - at) return 1;
         for (unsigned k = 0; k < used; ++k) {
-            if (owned[at + k]) return false;
+            if (owned[at + k]) return 1;
             owned[at + k] = 1;
         }
         granted += used;
-        return true;
-    };
-    auto plain = [&](unsigned seen, unsigned next) {
-        const unsigned was = cursor;
-        if (was == seen) cursor = next;
-        return was;
-    };
-    while (asked < demand) {
-        const unsigned used = 1u + g() % most;
-        asked += used;
-        bool ok = true;
-        auto crossed = [&](unsigned seen, unsigned next) {
-            if (++turn % 3 == 0) {
-                const unsigned other = 1u + g() % most;
-                asked += other;
-                ok = ok && take(ade::claim_lines(cursor, cap, other, plain), other);
-            }
-            return plain(seen, next);
-        };
-        unsigned at;
-        if (plain_add) {
-            at = cursor;
-            cursor += used;
-            if (!(at <= cap && cap - at >= used)) at = ade::kNoRoom;
-            if (!take(at, used)) return 1;
-            continue;
-        }
-        at = ade::claim_lines(cursor, cap, used, crossed);
-        if (!ok || !take(at, used) || cursor > cap) return 1;
     }
     return granted > cap ? 2 : 0;
 }
 
 int main()
 {
+    using Counter = unsigned long long;
     int bad = 0;
-    bad |= check(0u, 5u, 1ull << 12);
-    bad |= check(1000u, 40u, 1ull << 20);
+    bad |= check<Counter>(0u, 5u, 1ull << 12);
+    bad |= check<Counter>(1000u, 40u, 1ull << 20);
     // demands that pass 2^32 many times, on a pool of 8 GB
-    bad |= check(1u << 26, 1u << 25, 60ull << 32);
-    bad |= check(1u << 26, 0x7fffffffu, 60ull << 32);
-    if (check(1u << 26, 1u << 25, 60ull << 32, true) == 0) bad |= 8;
+    bad |= check<Counter>(1u << 26, 1u << 25, 60ull << 32);
+    bad |= check<Counter>(1u << 26, 0x7fffffffu, 60ull << 32);
+    if (check<std::uint32_t>(1u << 26, 1u << 25, 60ull << 32) == 0) bad |= 8;
     // a chunk's own count does not wrap either
     unsigned used = 6u;
     for (int r = 0; r < 169; ++r) {
@@ -99,3 +74,8 @@ def test_claims_never_overlap_beyond_2_to_32_lines(tmp_path):
     inc = os.path.join(ROOT, "paper_2108_09488_gb300", "csrc")
     subprocess.run([cxx, "-std=c++17", "-O2", "-I", inc, str(src), "-o", str(exe)], check=True)
     assert subprocess.run([str(exe)], capture_output=True, text=True).stdout.strip() == "0"
+
+
+def test_the_tables_counter_has_64_bits():
+    src = open(os.path.join(ROOT, "paper_2108_09488_gb300", "csrc", "ade_internal.h")).read()
+    assert "unsigned long long *cursor;" in src
