@@ -393,7 +393,8 @@ int ade_sweep_get_info(const ade_sweep *sw, ade_info *info_host);
 int ade_sweep_rate(ade_sweep *sw, float *dCdt_dev, void *stream);
 /* Ordered in-support pairs of the shared geometry (each set evaluates them all); waits. */
 int ade_sweep_count_pairs(ade_sweep *sw, long long *pairs_host, void *stream);
-/* nsteps predictor-corrector steps (Eq. 8-9) of every set; ade_sweep_run replays a captured graph. */
+/* nsteps predictor-corrector steps (Eq. 8-9) of every set; ade_sweep_run replays captured graphs.  The results
+ * are the same bits however the steps are split into calls, with a weights buffer or without. */
 int ade_sweep_step(ade_sweep *sw, int nsteps, void *stream);
 int ade_sweep_run(ade_sweep *sw, int nsteps, void *stream);
 /* Weights buffer of a sweep, as ade_weights_bytes and ade_set_weights: 8 bytes per pair and twice the

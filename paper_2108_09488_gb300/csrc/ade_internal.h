@@ -144,8 +144,7 @@ constexpr int kSweepGroup = 8;
 constexpr int kSweepMax = 64;     // parameter sets per sweep
 struct SweepParams {
     float vh[3];                  // unit vector of the uniform velocity (x axis when v = 0)
-    float a[kSweepGroup];         // Dcal = a u + b per set of the group, u = (vhat . e)^2
-    float b[kSweepGroup];
+    float g2, bT;                 // 2 Gamma, 2 (Gamma - d) + 2
     int g0;                       // first set of the group
     int nt;                       // sets in the group: 1, 2, 4 or 8
     float dL[kSweepGroup];        // alpha_L |v| + D_m and alpha_T |v| + D_m per set (0 beyond nt)
@@ -212,7 +211,7 @@ struct SweepRun {
     const uint32_t *cs, *perm;
     FrozenTab tab;
     float *C, *Ch;
-    float g2, bT;                 // 2 Gamma, 2 (Gamma - d) + 2
+    float g2, bT;                 // as in SweepParams
 };
 
 // One work item of the batched rate kernel: `count` sorted particles of plume `plume` starting

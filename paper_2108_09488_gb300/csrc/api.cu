@@ -2786,8 +2786,8 @@ int ade_sweep_init(ade_sweep **out, const ade_params *p, int n, int ntheta, cons
     for (int i = 0; i < 3; ++i) base.vh[i] = vabs > 0.0 ? (float)(i < dm ? pp.v[i] / vabs : 0.0) : (i == 0 ? 1.f : 0.f);
     for (int i = 0; i < 3; ++i) sw->rp.uw[i] = base.vh[i];   // the table's weights take u = (vhat . e)^2
     sw->rp.ub = 0.f;
-    sw->run.g2 = (float)(2.0 * gamma);
-    sw->run.bT = (float)(2.0 * (gamma - dm) + 2.0);
+    sw->run.g2 = base.g2 = (float)(2.0 * gamma);
+    sw->run.bT = base.bT = (float)(2.0 * (gamma - dm) + 2.0);
     for (int g0 = 0; g0 < ntheta;) {
         int nt = ade::kSweepGroup;
         while (nt > ntheta - g0) nt >>= 1;
@@ -2797,8 +2797,6 @@ int ade_sweep_init(ade_sweep **out, const ade_params *p, int n, int ntheta, cons
         for (int k = 0; k < nt; ++k) {
             const double aL = theta_host[3 * (g0 + k)], aT = theta_host[3 * (g0 + k) + 1],
                          Dm = theta_host[3 * (g0 + k) + 2];
-            g.a[k] = (float)(2.0 * gamma * (aL - aT) * vabs);
-            g.b[k] = (float)(2.0 * (gamma - dm) * (aT * vabs + Dm) - 2.0 * (aL - aT) * vabs);
             g.dL[k] = (float)(aL * vabs + Dm);
             g.dT[k] = (float)(aT * vabs + Dm);
         }

@@ -2,21 +2,19 @@
 // (alpha_L, alpha_T, D_m)_p that share the particles, the uniform velocity and the time step, each
 // with its own concentration field (a parameter sweep or the forward runs of an inversion).
 //
-// With a uniform v, K = 2D (Eq. 5 with equal tensors) and e = x_ab / r, the pair factor of Eq. 5 is
-//     Dcal = Gamma e^T K e - tr K = a_p u + b_p,    u = (vhat . e)^2,
-//     a_p = 2 Gamma (aL - aT) |v|,
-//     b_p = 2 (Gamma - d) (aT |v| + Dm) - 2 (aL - aT) |v|,
-// (substitute D of Eq. 3), so a pair's geometry -- separation, kernel shape f and u -- is computed
-// once and each parameter set costs one fused multiply-add for Dcal, a multiply by f, the
-// concentration difference and the accumulation.  The cell list, the positions and the drift are
+// With a uniform v, K = 2D (Eq. 5 with equal tensors) and e = x_ab / r, a pair's weight for the tensor of Eq. 3
+// is d_L,p g_L + d_T,p g_T with d_L = alpha_L |v| + D_m, d_T = alpha_T |v| + D_m and, f the kernel shape,
+//     g_L = f (2 Gamma u - 2),  g_T = f (-2 Gamma u + 2 (Gamma - d) + 2),  u = (vhat . e)^2,
+// so a pair's geometry -- separation, f and u -- is computed once and each parameter set costs a
+// multiplication and a fused multiply-add for its weight, the concentration difference and the accumulation.  The cell list, the positions and the drift are
 // shared; only the concentrations are per set.  Parameter sets are evaluated in groups of up to 8
 // per launch (registers); the sorted concentrations lie in planes of four sets, 16 bytes per particle, so
 // that a group's values are one or two 16-byte loads per candidate.
 // Summation as in rate.cu: FP32 row sums, Neumaier across rows, fixed order.
 //
-// Calls of four evaluations and more keep the geometry in a table (frozen_table.cuh: g_L and g_T per pair,
-// from which set k's weight is d_L,k g_L + d_T,k g_T) and stream it once per group and evaluation
-// (k_sweep_pass); shorter ones (k_rate_sweep) compute it on the fly.  Bound of a pass with 8 sets: the
+// Calls of four evaluations and more keep g_L and g_T of every pair in a table (frozen_table.cuh) and stream it
+// once per group and evaluation (k_sweep_pass); shorter ones (k_rate_sweep) compute them on the fly, with the
+// same operations in the same order, so that a run's bits do not depend on how it is split into calls.  Bound of a pass with 8 sets: the
 // latency of L1 and L2 at 27 % occupancy (32 bytes of concentrations a candidate, 96 registers).
 // 512^2, 60 neighbours, 8 sets, per evaluation: 95 us on the fly, 71 us from the table.
 #include "ade_internal.h"
@@ -291,8 +289,8 @@ __global__ __launch_bounds__(kT) void k_rate_sweep(const uint4 *__restrict__ Pe,
     const int cx = (int)__umulhi(pa.x - org.x, (uint32_t)ncx);
     const int cy = (int)__umulhi(pa.y - org.y, (uint32_t)ncy);
     const int cz = DIM == 3 ? (int)__umulhi(pa.z - org.z, (uint32_t)ncz) : 0;
-    const float H2 = prm.H2, invH = prm.invH, sy = prm.sy, sz = prm.sz;
-    const float vx = sp.vh[0], vy = sp.vh[1], vz = sp.vh[2];
+    const float far2 = prm.H2 * (1.f + 1.f / 4096.f), invH = prm.invH, sy = prm.sy, sz = prm.sz;   // far2: as chunk_rows
+    const float vx = sp.vh[0], vy = sp.vh[1], vz = sp.vh[2], g2 = sp.g2, bT = sp.bT;
     float acc[NT], comp[NT];
 #pragma unroll
     for (int k = 0; k < NT; ++k) acc[k] = comp[k] = 0.f;
@@ -348,17 +346,21 @@ __global__ __launch_bounds__(kT) void k_rate_sweep(const uint4 *__restrict__ Pe,
                 const float dz = DIM == 3 ? (float)iz * sz : 0.f;
                 float r2 = fmaf(dx, dx, dy * dy);
                 if (DIM == 3) r2 = fmaf(dz, dz, r2);
-                if (r2 < H2 && r2 > 0.f) {
-                    const float rinv = rsqrtf(r2);
-                    const float f = shape<KERNEL>(fmaf(-(r2 * rinv), invH, 1.f));
+                if (r2 < far2 && r2 > 0.f) {
+                    // the operations of pair_shape and SetSums::add, so that a step has the same bits here and
+                    // from the table; a candidate between H and far2 has f = 0
+                    const float rinv = rsqrt_ftz(r2);
+                    const float om = fmaf(-(r2 * rinv), invH, 1.f);
+                    const float f = shape2x<KERNEL>(fmaxf(om + om, 0.f));
                     float c = fmaf(vx, dx, vy * dy);
                     if (DIM == 3) c = fmaf(vz, dz, c);
-                    const float cr = c * rinv;
-                    const float u = cr * cr;
+                    const float t = c * rinv;
+                    const float u = fminf(t * t, 1.f);
+                    const float gL = f * fmaf(g2, u, -2.f), gT = f * fmaf(-g2, u, bT);
                     float Cb[NT];
                     load_group<NT>(Cg, (size_t)prm.n, (size_t)j, Cb);
 #pragma unroll
-                    for (int k = 0; k < NT; ++k) rs[k] = fmaf(f * fmaf(sp.a[k], u, sp.b[k]), Ca[k] - Cb[k], rs[k]);
+                    for (int k = 0; k < NT; ++k) rs[k] = fmaf(fmaf(sp.dL[k], gL, sp.dT[k] * gT), Ca[k] - Cb[k], rs[k]);
                 }
             }
 #pragma unroll
@@ -372,7 +374,7 @@ __global__ __launch_bounds__(kT) void k_rate_sweep(const uint4 *__restrict__ Pe,
     if (!valid) return;
     float rate[NT];
 #pragma unroll
-    for (int k = 0; k < NT; ++k) rate[k] = prm.pf * (acc[k] + comp[k]);
+    for (int k = 0; k < NT; ++k) rate[k] = (prm.pf * shape_unscale<KERNEL>()) * (acc[k] + comp[k]);
     const size_t n = (size_t)prm.n;
     if (EPI == EPI_PREDICT) {
         float o[NT];
