@@ -186,7 +186,8 @@ int ade_run(ade_ctx *ctx, int nsteps, ade_stats *stats_host, void *stream);
  * list of the current positions and counts, so the size is what the set needs, however uneven it is; waits for
  * the stream; ADE_ERR_STATE while the stream is captured.  counted 0: an estimate for an even set, host only, for
  * a first call that should not wait (up to four times what a lattice needs; a set with dense spots keeps
- * fewer of its weights in it).  0 where weights are not kept: flags other than 0, a velocity field, more than
+ * fewer of its weights in it).  0 where weights are not kept: flags other than 0, a velocity field, an
+ * autotuned walk that is tiled or branched, more than
  * 500 expected neighbours with more than 80,000 particles (the walks are as fast there), more than 16 GB
  * counted or 4 GB estimated.
  * ade_set_weights: gives the context a buffer (device, 256-byte aligned, valid until the context is destroyed

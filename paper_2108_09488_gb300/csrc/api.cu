@@ -1164,7 +1164,13 @@ int ade_weights_bytes(ade_ctx *c, int counted, size_t *bytes, void *stream)
     // they evaluate (405^2 irregular, 9,400 neighbours: 2.2 ms either way; 248^2, 4,900, whose 1,900 warps do
     // not fill it: 0.58 against 0.93 ms).
     const bool wide = expected_neighbours(c->p, c->H, c->n) > 500.0 && c->n > 80000;
-    if (c->p.flags != 0u || c->field || c->n == 0 || wide) return ADE_OK;
+    // The table's sums are those of the branch-free walks (variants 0, 3, 5, 6), bit for bit: a context tuned to
+    // another keeps to that, so that its bits do not depend on how steps are split into calls (and it was the
+    // faster one: 160^2 with 2,700 neighbours, tiles 347 us per step, table 613).
+    const int v = c->rp.variant;
+    const bool branch_free = v == 0 || v == 3 || v == 5 || v == 6;
+    c->plan = ade::TablePlan{};
+    if (c->p.flags != 0u || c->field || c->n == 0 || wide || !branch_free) return ADE_OK;
     const int rc = ade::plan_context_table(c, 1, counted != 0, &c->plan, (cudaStream_t)stream);
     if (rc || c->plan.lines == 0) return rc;
     const size_t slots = (size_t)ade::chunk_numbers(c->n, c->nc[1] * c->nc[2]) + 1;
