@@ -171,9 +171,9 @@ int ade_count_pairs(ade_ctx *ctx, long long *pairs_host, void *stream);
 int ade_step(ade_ctx *ctx, int nsteps, void *stream);
 
 /* As ade_step, replaying captured CUDA graphs: one graph of 32 steps per whole multiple of 32
- * (no launch gap between those steps) and one of the remaining steps (a graph of one step, where the
- * pair weights are not kept), each captured on the first call that needs it, outside any capture of
- * the caller's.  With stats_host non-NULL it
+ * (no launch gap between those steps), and for the rest one of one step, or where the pair weights are
+ * kept one of all its steps once two calls in a row have the same remainder (launched as ade_step does
+ * until then).  They are captured when first needed, outside any capture of the caller's.  With stats_host non-NULL it
  * waits for the stream and fills in the last step's statistics (those of the state it wrote; with
  * nsteps = 0, those of the current state as ade_get_stats); with NULL it only enqueues. */
 int ade_run(ade_ctx *ctx, int nsteps, ade_stats *stats_host, void *stream);

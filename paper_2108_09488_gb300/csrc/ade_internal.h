@@ -388,6 +388,15 @@ int rate_launch_warps(int dim, const RateParams &prm, bool iso);
 size_t tiled_smem_bytes(int dim, const RateParams &prm);
 int closed_form_blocks(int n);
 
+// Captured steps of a context's run calls, three at most: kGraphSteps steps, one step, and the remainder
+// that the last calls had in common (run_graphs in api.cu).
+struct StepGraphs {
+    cudaGraph_t graph[3];
+    cudaGraphExec_t exec[3];
+    int rest;                // steps of the last remainder
+    cudaStream_t stream;     // captured on
+};
+
 }  // namespace ade
 
 struct ade_ctx {
@@ -416,10 +425,7 @@ struct ade_ctx {
     double t;
     long long step;
     long long pairs;
-    // captured runs of 1..kGraphSteps steps (ade_run), each on the first call that needs it
-    cudaGraph_t graph[ade::kGraphSteps + 1];
-    cudaGraphExec_t graph_exec[ade::kGraphSteps + 1];
-    cudaStream_t cap_stream;
+    ade::StepGraphs graphs;   // of ade_run
     bool status_cleared;
     cudaEvent_t ev[5];    // per-phase timing events (created on first timed step)
     bool ev_ready;

@@ -491,6 +491,73 @@ int table_lines(const void *buf, size_t bytes, size_t words, unsigned stride, si
     return ADE_OK;
 }
 
+// Forget the captured steps (the configuration they were captured with has changed).
+void drop_graph(ade::StepGraphs &g, int slot)
+{
+    if (g.exec[slot]) cudaGraphExecDestroy(g.exec[slot]);
+    if (g.graph[slot]) cudaGraphDestroy(g.graph[slot]);
+    g.exec[slot] = nullptr;
+    g.graph[slot] = nullptr;
+}
+
+void drop_graphs(ade::StepGraphs &g)
+{
+    for (int k = 0; k < 3; ++k) drop_graph(g, k);
+    g.rest = 0;
+}
+
+void destroy_graphs(ade::StepGraphs &g)
+{
+    drop_graphs(g);
+    if (g.stream) cudaStreamDestroy(g.stream);
+    g.stream = nullptr;
+}
+
+// Launches the graph of `steps` steps in `slot` n times, capturing what enqueue(steps, stream) enqueues first.
+template <class Enqueue>
+int launch_graph(ade::StepGraphs &G, int slot, int steps, int n, cudaStream_t s, Enqueue enqueue)
+{
+    if (!G.exec[slot]) {
+        if (!G.stream) ADE_CK(cudaStreamCreateWithFlags(&G.stream, cudaStreamNonBlocking));
+        ADE_CK(cudaStreamBeginCapture(G.stream, cudaStreamCaptureModeThreadLocal));
+        const int rc = enqueue(steps, G.stream);
+        cudaGraph_t g = nullptr;
+        const cudaError_t e = cudaStreamEndCapture(G.stream, &g);
+        if (rc) {
+            if (g) cudaGraphDestroy(g);
+            return rc;
+        }
+        ADE_CK(e);
+        const cudaError_t ei = cudaGraphInstantiate(&G.exec[slot], g, 0);
+        if (ei != cudaSuccess) {
+            cudaGraphDestroy(g);
+            G.exec[slot] = nullptr;
+            return fail(ADE_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(ei));
+        }
+        G.graph[slot] = g;
+    }
+    for (int k = 0; k < n; ++k) ADE_CK(cudaGraphLaunch(G.exec[slot], s));
+    return ADE_OK;
+}
+
+// nsteps steps of a run call: whole multiples of kGraphSteps (multi) replay one graph of that many (no launch
+// gap between them).  The rest replays a graph of one step, or where the steps of a call share the pair weights
+// (shared) has a graph of its own once two calls in a row have the same remainder; until then it
+// is launched as it is, which the GPU does not wait for (a capture costs more than the launches), and
+// a context holds three graphs however its calls vary.
+template <class Enqueue>
+int run_graphs(ade::StepGraphs &G, int nsteps, bool multi, bool shared, cudaStream_t s, Enqueue enqueue)
+{
+    const int big = multi ? nsteps / ade::kGraphSteps : 0, rest = nsteps - big * ade::kGraphSteps;
+    int rc = big > 0 ? launch_graph(G, 0, ade::kGraphSteps, big, s, enqueue) : ADE_OK;
+    if (rc || rest == 0) return rc;
+    if (!shared) return launch_graph(G, 1, 1, rest, s, enqueue);
+    if (G.rest == rest) return launch_graph(G, 2, rest, 1, s, enqueue);
+    drop_graph(G, 2);
+    G.rest = rest;
+    return enqueue(rest, s);
+}
+
 // A query runs kernels and waits: not inside a stream capture.
 int not_capturing(cudaStream_t s)
 {
@@ -1068,17 +1135,6 @@ int ade_init_particles(ade_ctx **out, const ade_params *p, int n, uint32_t *xq_d
 
 namespace {
 
-// Forget the captured step graphs (the configuration they were captured with has changed).
-void drop_graphs(ade_ctx *c)
-{
-    for (int k = 0; k <= ade::kGraphSteps; ++k) {
-        if (c->graph_exec[k]) cudaGraphExecDestroy(c->graph_exec[k]);
-        if (c->graph[k]) cudaGraphDestroy(c->graph[k]);
-        c->graph_exec[k] = nullptr;
-        c->graph[k] = nullptr;
-    }
-}
-
 // Enqueue `steps` steps of one call.
 int enqueue_steps(ade_ctx *c, int steps, cudaStream_t s)
 {
@@ -1086,30 +1142,6 @@ int enqueue_steps(ade_ctx *c, int steps, cudaStream_t s)
     int rc = ADE_OK;
     for (int k = 0; k < steps && rc == ADE_OK; ++k) rc = enqueue_step(c, s);
     return rc;
-}
-
-// Capture `steps` consecutive steps into one graph (once).
-int capture_steps(ade_ctx *c, int steps)
-{
-    if (c->graph_exec[steps]) return ADE_OK;
-    if (!c->cap_stream) ADE_CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
-    ADE_CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-    const int rc = enqueue_steps(c, steps, c->cap_stream);
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
-    if (rc) {
-        if (g) cudaGraphDestroy(g);
-        return rc;
-    }
-    ADE_CK(e);
-    cudaError_t ei = cudaGraphInstantiate(&c->graph_exec[steps], g, 0);
-    if (ei != cudaSuccess) {
-        cudaGraphDestroy(g);
-        c->graph_exec[steps] = nullptr;
-        return fail(ADE_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(ei));
-    }
-    c->graph[steps] = g;
-    return ADE_OK;
 }
 
 // Switch a context to cell subdivision k and kernel variant (tiled or direct); the workspace
@@ -1148,7 +1180,7 @@ int apply_config(ade_ctx *c, int k, int variant)
     rp.nty = t.nty;
     rp.ntz = t.ntz;
     rp.cap = t.cap;
-    drop_graphs(c);
+    drop_graphs(c->graphs);
     return ADE_OK;
 }
 
@@ -1195,7 +1227,7 @@ int ade_set_weights(ade_ctx *c, void *weights_dev, size_t bytes)
         c->cursor_clean = false;
     }
     c->frozen = weights_dev && c->frozen_lines > 0;
-    drop_graphs(c);
+    drop_graphs(c->graphs);
     return ADE_OK;
 }
 
@@ -1350,7 +1382,7 @@ int ade_set_dispersivity(ade_ctx *c, double alpha_L, double alpha_T, double D_m)
         c->fp.Dm = D_m;
         c->field_dirty = true;   // tensors re-formed on the caller's stream before the next use
     }
-    drop_graphs(c);
+    drop_graphs(c->graphs);
     return ADE_OK;
 }
 
@@ -1494,16 +1526,9 @@ int ade_run(ade_ctx *c, int nsteps, ade_stats *st, void *stream)
     if (rc0) return rc0;
     rc0 = refresh_field(c, s);
     if (rc0) return rc0;
-    // whole multiples of kGraphSteps replay one graph of kGraphSteps steps (no launch gap between
-    // them), the rest one graph of the remaining steps where they keep the pair weights, else a graph
-    // of one step
-    const int nmulti = nsteps / ade::kGraphSteps, rest = nsteps % ade::kGraphSteps;
-    const int per = use_frozen(c, rest) ? rest : 1;
-    rc0 = nmulti > 0 ? capture_steps(c, ade::kGraphSteps) : ADE_OK;
-    if (rc0 == ADE_OK && rest > 0) rc0 = capture_steps(c, per);
+    rc0 = run_graphs(c->graphs, nsteps, true, use_frozen(c, nsteps % ade::kGraphSteps), s,
+                     [c](int steps, cudaStream_t st) { return enqueue_steps(c, steps, st); });
     if (rc0) return rc0;
-    for (int k = 0; k < nmulti; ++k) ADE_CK(cudaGraphLaunch(c->graph_exec[ade::kGraphSteps], s));
-    for (int k = 0; k < rest; k += per) ADE_CK(cudaGraphLaunch(c->graph_exec[per], s));
     if (nsteps > 0 && !c->field) {
         c->cells_framed = true;
         for (int i = 0; i < 3; ++i) c->cells_add[i] = c->inc[i];
@@ -1620,8 +1645,7 @@ int ade_closed_form_error(ade_ctx *c, const double *x0, double w, double C0, int
 void ade_destroy(ade_ctx *c)
 {
     if (!c) return;
-    drop_graphs(c);
-    if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
+    destroy_graphs(c->graphs);
     if (c->ev_ready)
         for (int k = 0; k < 5; ++k) cudaEventDestroy(c->ev[k]);
     delete c;
@@ -1661,10 +1685,7 @@ struct ade_batch {
     int max_tiles = 0;
     long long step = 0;
     bool status_cleared = false;
-    // captured runs of 1..kGraphSteps steps, each on the first call that needs it
-    cudaGraph_t graph[ade::kGraphSteps + 1] = {};
-    cudaGraphExec_t graph_exec[ade::kGraphSteps + 1] = {};
-    cudaStream_t cap_stream = nullptr;
+    ade::StepGraphs graphs = {};
     // weight table of multi-step calls (rate_frozen.cu)
     bool frozen = false;               // there is one for the grids in use (ade_batch_set_weights)
     ade::FrozenTab frozen_tab = {};
@@ -1871,16 +1892,6 @@ int batch_plan(ade_batch *b)
     return ADE_OK;
 }
 
-void batch_drop_graphs(ade_batch *b)
-{
-    for (int k = 0; k <= ade::kGraphSteps; ++k) {
-        if (b->graph_exec[k]) cudaGraphExecDestroy(b->graph_exec[k]);
-        if (b->graph[k]) cudaGraphDestroy(b->graph[k]);
-        b->graph_exec[k] = nullptr;
-        b->graph[k] = nullptr;
-    }
-}
-
 int batch_upload(ade_batch *b, cudaStream_t s)
 {
     ADE_CK(cudaMemcpyAsync(b->d_pred, b->pred.data(), b->P * sizeof(ade::RateParams), cudaMemcpyHostToDevice, s));
@@ -1892,7 +1903,7 @@ int batch_upload(ade_batch *b, cudaStream_t s)
         ADE_CK(cudaMemcpyAsync(b->d_items, b->items.data(), b->items.size() * sizeof(ade::FrozenItem),
                                cudaMemcpyHostToDevice, s));
     ADE_CK(cudaStreamSynchronize(s));   // the host vectors may change before the next call
-    batch_drop_graphs(b);
+    drop_graphs(b->graphs);
     return ADE_OK;
 }
 
@@ -1970,30 +1981,6 @@ int batch_enqueue_steps(ade_batch *b, int steps, cudaStream_t s)
     int rc = ADE_OK;
     for (int k = 0; k < steps && rc == ADE_OK; ++k) rc = batch_enqueue_step(b, s);
     return rc;
-}
-
-// Capture `steps` steps into one graph (once).
-int batch_capture(ade_batch *b, int steps)
-{
-    if (b->graph_exec[steps]) return ADE_OK;
-    if (!b->cap_stream) ADE_CK(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking));
-    ADE_CK(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
-    const int rc = batch_enqueue_steps(b, steps, b->cap_stream);
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamEndCapture(b->cap_stream, &g);
-    if (rc) {
-        if (g) cudaGraphDestroy(g);
-        return rc;
-    }
-    ADE_CK(e);
-    cudaError_t ei = cudaGraphInstantiate(&b->graph_exec[steps], g, 0);
-    if (ei != cudaSuccess) {
-        cudaGraphDestroy(g);
-        b->graph_exec[steps] = nullptr;
-        return fail(ADE_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(ei));
-    }
-    b->graph[steps] = g;
-    return ADE_OK;
 }
 
 int batch_clear_status_once(ade_batch *b, cudaStream_t s)
@@ -2182,7 +2169,7 @@ int ade_batch_set_weights(ade_batch *b, void *weights_dev, size_t bytes, void *s
         ADE_CK(cudaMemsetAsync(b->frozen_tab.cursor, 0, sizeof(*b->frozen_tab.cursor), (cudaStream_t)stream));
     }
     b->frozen = weights_dev && lines > 0 && b->N > 0;
-    batch_drop_graphs(b);
+    drop_graphs(b->graphs);
     if (!b->frozen || lines == b->divided) return ADE_OK;
     batch_divide(b, lines);
     return batch_upload(b, (cudaStream_t)stream);
@@ -2207,15 +2194,9 @@ int ade_batch_run(ade_batch *b, int nsteps, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     int rc = batch_clear_status_once(b, s);
     if (rc) return rc;
-    // graphs of kGraphSteps steps and one of the rest where they keep the pair weights, else of one step
-    const int big = batch_use_frozen(b, nsteps) ? ade::kGraphSteps : 1;
-    for (int left = nsteps; left > 0;) {
-        const int k = std::min(left, big);
-        rc = batch_capture(b, k);
-        if (rc) return rc;
-        ADE_CK(cudaGraphLaunch(b->graph_exec[k], s));
-        left -= k;
-    }
+    rc = run_graphs(b->graphs, nsteps, batch_use_frozen(b, nsteps), batch_use_frozen(b, nsteps % ade::kGraphSteps), s,
+                    [b](int steps, cudaStream_t st) { return batch_enqueue_steps(b, steps, st); });
+    if (rc) return rc;
     b->step += nsteps;
     return ADE_OK;
 }
@@ -2453,8 +2434,7 @@ int ade_batch_launches_per_step(const ade_batch *b, int *launches)
 void ade_batch_destroy(ade_batch *b)
 {
     if (!b) return;
-    batch_drop_graphs(b);
-    if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
+    destroy_graphs(b->graphs);
     delete b;
 }
 
@@ -2484,10 +2464,7 @@ struct ade_sweep {
     bool table = false, cursor_clean = false;   // a weight table (ade_sweep_set_weights) and its counter
     ade::TablePlan plan = {}, estimate = {};    // as last asked for; for an even set
     ade::SweepRun run = {};
-    // captured runs of 1..kGraphSteps steps, each on the first call that needs it
-    cudaGraph_t graph[ade::kGraphSteps + 1] = {};
-    cudaGraphExec_t graph_exec[ade::kGraphSteps + 1] = {};
-    cudaStream_t cap_stream = nullptr;
+    ade::StepGraphs graphs = {};
     cudaEvent_t ev[4];
     bool ev_ready = false;
 };
@@ -2684,16 +2661,6 @@ int sweep_eval_fly(ade_sweep *sw, bool count, const ade::SweepOut &out, cudaStre
     return ADE_OK;
 }
 
-void sweep_drop_graphs(ade_sweep *sw)
-{
-    for (int k = 0; k <= ade::kGraphSteps; ++k) {
-        if (sw->graph_exec[k]) cudaGraphExecDestroy(sw->graph_exec[k]);
-        if (sw->graph[k]) cudaGraphDestroy(sw->graph[k]);
-        sw->graph_exec[k] = nullptr;
-        sw->graph[k] = nullptr;
-    }
-}
-
 int sweep_clear_status_once(ade_sweep *sw, cudaStream_t s)
 {
     if (!sw->status_cleared) {
@@ -2872,7 +2839,7 @@ int ade_sweep_set_weights(ade_sweep *sw, void *weights_dev, size_t bytes)
         sw->cursor_clean = false;
     }
     sw->table = weights_dev && lines > 0;
-    sweep_drop_graphs(sw);
+    drop_graphs(sw->graphs);
     return ADE_OK;
 }
 
@@ -2934,30 +2901,10 @@ int ade_sweep_run(ade_sweep *sw, int nsteps, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     int rc = sweep_clear_status_once(sw, s);
     if (rc) return rc;
-    for (int left = nsteps; left > 0;) {   // graphs of kGraphSteps steps and one of the rest
-        const int k = std::min(left, ade::kGraphSteps);
-        if (!sw->graph_exec[k]) {
-            if (!sw->cap_stream) ADE_CK(cudaStreamCreateWithFlags(&sw->cap_stream, cudaStreamNonBlocking));
-            ADE_CK(cudaStreamBeginCapture(sw->cap_stream, cudaStreamCaptureModeThreadLocal));
-            rc = sweep_steps(sw, k, sw->cap_stream);
-            cudaGraph_t g = nullptr;
-            cudaError_t e = cudaStreamEndCapture(sw->cap_stream, &g);
-            if (rc) {
-                if (g) cudaGraphDestroy(g);
-                return rc;
-            }
-            ADE_CK(e);
-            cudaError_t ei = cudaGraphInstantiate(&sw->graph_exec[k], g, 0);
-            if (ei != cudaSuccess) {
-                cudaGraphDestroy(g);
-                sw->graph_exec[k] = nullptr;
-                return fail(ADE_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(ei));
-            }
-            sw->graph[k] = g;
-        }
-        ADE_CK(cudaGraphLaunch(sw->graph_exec[k], s));
-        left -= k;
-    }
+    const int rest = nsteps % ade::kGraphSteps;
+    rc = run_graphs(sw->graphs, nsteps, sw->table, rest > 0 && sweep_use_table(sw, rest), s,
+                    [sw](int steps, cudaStream_t st) { return sweep_steps(sw, steps, st); });
+    if (rc) return rc;
     sw->step += nsteps;
     sw->t += nsteps * sw->dt;
     return ADE_OK;
@@ -3038,8 +2985,7 @@ int ade_sweep_stats(ade_sweep *sw, ade_stats *st, void *stream)
 void ade_sweep_destroy(ade_sweep *sw)
 {
     if (!sw) return;
-    sweep_drop_graphs(sw);
-    if (sw->cap_stream) cudaStreamDestroy(sw->cap_stream);
+    destroy_graphs(sw->graphs);
     if (sw->ev_ready)
         for (int k = 0; k < 4; ++k) cudaEventDestroy(sw->ev[k]);
     delete sw;
