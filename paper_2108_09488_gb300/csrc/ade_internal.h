@@ -287,6 +287,9 @@ int cell_build_launches(int n, int ncells, bool onepass);
 cudaError_t launch_build_cells(int dim, const uint32_t *xq, const float *C, int n, const int *nc,
                                int ncells, const Work &w, cudaStream_t s, bool count_zero = false,
                                const CellFrame &frame = CellFrame());
+// Positions of the last build (its sorted records), in the caller's order and moved by add, into xq [dim][n].
+cudaError_t launch_build_positions(const uint4 *P, const uint32_t *perm, int n, int dim, const uint32_t *add, uint32_t *xq,
+                                   cudaStream_t s);
 // Writes a CellFrame's words: the next build's origin, and the last build's.
 cudaError_t launch_set_frame(uint32_t *words, const uint32_t *origin, cudaStream_t s);
 // Batched plumes: keys are coff_p + local key; plume_of[i] gives the plume of caller particle i.
@@ -430,8 +433,8 @@ struct ade_ctx {
     cudaEvent_t ev[5];    // per-phase timing events (created on first timed step)
     bool ev_ready;
     bool frame_set;       // w.frame holds the frame of the current step
-    bool cells_framed;    // the last build was in the moving frame, of the positions cells_add before the current
-    uint32_t cells_add[3];
+    bool cells_framed;    // the last build was in the moving frame; the last step that used it started from its
+    uint32_t cells_add[3];   // positions moved by cells_add
     // weight table of multi-step calls (ade_set_weights), in the caller's buffer
     bool frozen;          // there is one for the grid in use
     bool cursor_clean;    // its pool's counter has been cleared

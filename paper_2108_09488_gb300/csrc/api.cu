@@ -710,7 +710,7 @@ int enqueue_cells(ade_ctx *c, cudaStream_t s, int steps = 0, bool framed = false
         frame.words = c->w.frame;
         for (int i = 0; i < 3; ++i) {
             frame.adv[i] = (uint32_t)steps * c->inc[i];
-            c->cells_add[i] = steps > 0 ? c->inc[i] : 0u;
+            c->cells_add[i] = steps > 1 ? (uint32_t)(steps - 1) * c->inc[i] : 0u;
         }
     }
     cudaError_t e = ade::launch_build_cells(c->dim, c->xq, c->C, c->n, c->nc, c->ncells, c->w, s, true, frame);
@@ -1420,13 +1420,14 @@ int ade_get_cells(ade_ctx *c, uint32_t *perm_dev, uint32_t *cell_start_dev, void
     if (!c) return fail(ADE_ERR_ARG, "ctx is NULL");
     cudaStream_t s = (cudaStream_t)stream;
     if (c->cells_framed && c->n > 0) {
-        // the list was built in the moving frame: the absolute grid's list of the same positions (the
-        // current ones, minus one drift after steps)
+        // the list was built in the moving frame: the absolute grid's list of the positions the last step
+        // started from, which the build's records give (the caller's may have changed since); they lie in the
+        // half-step state, free between steps
         int rc = clean_counts(c, s);
         if (rc) return rc;
-        ade::CellFrame frame;
-        for (int i = 0; i < 3; ++i) frame.add[i] = c->cells_add[i];
-        ADE_CK(ade::launch_build_cells(c->dim, c->xq, c->C, c->n, c->nc, c->ncells, c->w, s, true, frame));
+        uint32_t *xq = reinterpret_cast<uint32_t *>(c->w.P1);
+        ADE_CK(ade::launch_build_positions(c->w.P0, c->w.perm, c->n, c->dim, c->cells_add, xq, s));
+        ADE_CK(ade::launch_build_cells(c->dim, xq, c->C, c->n, c->nc, c->ncells, c->w, s, true));
         c->cells_framed = false;
     }
     if (perm_dev && c->n > 0)
@@ -1529,9 +1530,10 @@ int ade_run(ade_ctx *c, int nsteps, ade_stats *st, void *stream)
     rc0 = run_graphs(c->graphs, nsteps, true, use_frozen(c, nsteps % ade::kGraphSteps), s,
                      [c](int steps, cudaStream_t st) { return enqueue_steps(c, steps, st); });
     if (rc0) return rc0;
-    if (nsteps > 0 && !c->field) {
+    if (nsteps > 0 && !c->field) {   // (a replayed graph's last build, as enqueue_cells notes it)
+        const int rest = nsteps % ade::kGraphSteps, last = rest > 0 ? rest : ade::kGraphSteps;
         c->cells_framed = true;
-        for (int i = 0; i < 3; ++i) c->cells_add[i] = c->inc[i];
+        for (int i = 0; i < 3; ++i) c->cells_add[i] = use_frozen(c, last) ? (uint32_t)(last - 1) * c->inc[i] : 0u;
     }
     c->step += nsteps;
     c->t += nsteps * c->dt;

@@ -699,6 +699,20 @@ __global__ void k_set_frame(uint32_t *words, uint32_t x, uint32_t y, uint32_t z)
     if (threadIdx.x < kFrameWords) words[threadIdx.x] = t == 0 ? x : (t == 1 ? y : (t == 2 ? z : 0u));
 }
 
+// Caller-order positions of a build from its sorted records, moved by add.
+__global__ __launch_bounds__(kThreads) void k_build_positions(const uint4 *__restrict__ P, const uint32_t *__restrict__ perm, int n,
+                                                              int dim, uint3 add, uint32_t *__restrict__ xq)
+{
+    const int i = blockIdx.x * kThreads + threadIdx.x;
+    if (i >= n) return;
+    const uint32_t a = perm[i];
+    if (a >= (uint32_t)n) return;
+    const uint4 p = P[i];
+    xq[a] = p.x + add.x;
+    xq[(size_t)n + a] = p.y + add.y;
+    if (dim == 3) xq[2 * (size_t)n + a] = p.z + add.z;
+}
+
 struct BatchRec {
     const uint32_t *xq;
     const float *C;
@@ -745,6 +759,13 @@ __global__ __launch_bounds__(kThreads) void k_order_batch(const uint32_t *__rest
 cudaError_t launch_set_frame(uint32_t *words, const uint32_t *origin, cudaStream_t s)
 {
     k_set_frame<<<1, 32, 0, s>>>(words, origin[0], origin[1], origin[2]);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_build_positions(const uint4 *P, const uint32_t *perm, int n, int dim, const uint32_t *add, uint32_t *xq,
+                                   cudaStream_t s)
+{
+    if (n > 0) k_build_positions<<<(n + kThreads - 1) / kThreads, kThreads, 0, s>>>(P, perm, n, dim, make_uint3(add[0], add[1], add[2]), xq);
     return cudaGetLastError();
 }
 
