@@ -178,6 +178,7 @@ struct FrozenTab {
     unsigned long long *cursor;
     unsigned pool, cap;
     uint32_t *dense;       // chunks before each pencil (launch_chunk_numbers; NULL: numbers with gaps)
+    float *low;            // plane of low parts, half as many lines (the adjoint's table)
 };
 // Lines that a set's chunks need, counted by size: two bins per octave.
 struct ChunkBin {
@@ -420,6 +421,7 @@ struct ade_ctx {
     ade::Work w;
     double H;
     double dt;
+    double pf;            // RateParams::pf in FP64
     double D[9];
     ade::RateParams rp;   // rate constants (dt/inc set per use)
     uint32_t inc[3];

@@ -26,9 +26,14 @@
 // they are computed once (frozen_table.cuh) and an evaluation streams them; the state and the adjoint
 // state of a backward step share one pass, and the dot products are taken in that pass from S_L and S_T,
 // so a backward step is two launches and a forward step two.
-// Bound: L2 / HBM, 8 bytes a pair.  512^2 lattice, 20 neighbours, 40 steps: 13.5 -> 4.3 ms (the dot
+// Bound: L2 / HBM, 8 bytes a pair (10 on average with the low parts that the backward passes read).  512^2 lattice,
+// 20 neighbours, 40 steps: 13.3 -> 4.05 ms (the dot
 // products' kernel alone took 97 us a step: nine threads folded 1024 FP64 partials one by one).
-// Pair arithmetic is FP32 with compensated row sums (as in rate.cu); dot products and J are FP64.
+// Precision: the states are FP32 (C, half steps, L u), everything else that all pairs or steps share is kept to FP64
+// or nearly (weights to 32 bits with their low parts, the geometry behind them, the time step, prefactor and
+// coefficients), and the sums behind the dot products take every rounding along: dJ/dtheta is within 1e-9 (one
+// case 8e-9) of an FP64 computation with the states rounded alike, and the states' roundings move it by up to 1.4e-7
+// (6 plumes of 85^2 to 512^2 against FP64: 5e-10..5e-8; with weights and sums in FP32 4e-9..2e-7).
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -52,77 +57,96 @@ constexpr int kT = kFrozenThreads;
 constexpr double kTwo32 = 4294967296.0;
 constexpr int kDots = 6;   // per backward step: p.S_L u, p.S_T u, b.S_L u, b.S_T u (b = L p), p.S_L a, p.S_T a (a = L u)
 
-// S_L (0) and S_T (1) of NR fields.
-template <int NR>
+// S_L (x) and S_T (y) of NR fields, rows summed in FP32 and added up with Neumaier's compensation.  LOW (the dot
+// products of the backward passes): the last field's sums take the weights' low parts and the rounding of every
+// product and addition, for on a lattice the weights' and the row sums' roundings bias all particles alike
+// (dJ/dtheta by up to 2e-7).  The states do not need that: they are rounded to FP32 themselves.
+template <int NR, bool LOW>
 struct ShapeSums {
     const float *x[NR];
-    float xa[NR], r0[NR], r1[NR], a0[NR], c0[NR], a1[NR], c1[NR];
+    const float *words, *low;
+    float xa[NR];
+    float2 r[NR], a[NR], c[NR];
     __device__ __forceinline__ void zero()
     {
 #pragma unroll
-        for (int q = 0; q < NR; ++q) r0[q] = r1[q] = a0[q] = c0[q] = a1[q] = c1[q] = 0.f;
+        for (int q = 0; q < NR; ++q) r[q] = a[q] = c[q] = f2(0.f, 0.f);
     }
-    __device__ __forceinline__ void add(int q, float2 w, float xb)
+    __device__ __forceinline__ void add(int q, float2 w, float2 lo, float xb)
     {
-        const float d = xa[q] - xb;
-        r0[q] = fmaf(w.x, d, r0[q]);
-        r1[q] = fmaf(w.y, d, r1[q]);
+        const float2 d = both(xa[q] - xb);
+        if (LOW && q == NR - 1) {
+            c[q] = __ffma2_rn(lo, d, c[q]);
+            r[q] = two_sum2(r[q], two_prod2(w, d, c[q]), c[q]);
+        } else {
+            r[q] = __ffma2_rn(w, d, r[q]);
+        }
+    }
+    __device__ __forceinline__ void prefetch(const float *base, int first, int n) const
+    {
+        if (LOW) prefetch_l2(low + (((size_t)(base - words) >> 5) + first) / 2 * 32, (unsigned)(n / 2) * 128u + 128u);
     }
     template <int M>
     __device__ __forceinline__ void lines(const float *w, int s)
     {
         float2 wv[M];
-        float xv[NR][M];
+        float lv[M], xv[NR][M];
+        const int lane = threadIdx.x & 31;
+        const float *lw = low + (((size_t)(w - words) - 2 * lane) >> 6) * 32 + lane;
 #pragma unroll
         for (int u = 0; u < M; ++u) {
             wv[u] = __ldg(reinterpret_cast<const float2 *>(w) + u * 32);
+            lv[u] = LOW ? ld_weight(lw + u * 32) : 0.f;
 #pragma unroll
             for (int q = 0; q < NR; ++q) xv[q][u] = x[q][s + u];
         }
 #pragma unroll
-        for (int u = 0; u < M; ++u)
+        for (int u = 0; u < M; ++u) {
+            const float2 lo = unpack_low(lv[u]);
 #pragma unroll
-            for (int q = 0; q < NR; ++q) add(q, wv[u], xv[q][u]);
+            for (int q = 0; q < NR; ++q) add(q, wv[u], lo, xv[q][u]);
+        }
     }
     __device__ __forceinline__ void end_row()
     {
 #pragma unroll
         for (int q = 0; q < NR; ++q) {
-            neumaier_add(a0[q], c0[q], r0[q]);
-            neumaier_add(a1[q], c1[q], r1[q]);
-            r0[q] = r1[q] = 0.f;
+            neumaier_add2(a[q], c[q], r[q]);
+            r[q] = f2(0.f, 0.f);
         }
     }
-    __device__ __forceinline__ float s0(int q) const { return a0[q] + c0[q]; }
-    __device__ __forceinline__ float s1(int q) const { return a1[q] + c1[q]; }
+    __device__ __forceinline__ float s0(int q) const { return a[q].x + c[q].x; }
+    __device__ __forceinline__ float s1(int q) const { return a[q].y + c[q].y; }
+    __device__ __forceinline__ double d0(int q) const { return (double)a[q].x + (double)c[q].x; }
+    __device__ __forceinline__ double d1(int q) const { return (double)a[q].y + (double)c[q].y; }
 };
 
-// The same sums over the positions, for a chunk without room in the table.
-template <int DIM, int KERNEL, bool ISO, int NR>
-__device__ __noinline__ void walk_sums(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs, const RateParams &prm,
-                                       const Chunk &c, const ShapeConst sc, ShapeSums<NR> &op)
+// The same sums over the positions, for a chunk without room in the table: the rows and ranges of the table's
+// chunks (cut by the cell bands), two candidates at a time.
+template <int DIM, int KERNEL, bool ISO, int NR, bool LOW>
+__device__ __noinline__ void walk_sums(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs, const RateParams &prm, Chunk c,
+                                       const ShapeConst sc, ShapeSums<NR, LOW> &op)
 {
     const uint4 pa = __ldg(P + min(c.i0 + (int)(threadIdx.x & 31), c.pe - 1));
-    const int ncx = prm.ncx;
-    const int cx = (int)__umulhi(pa.x - frame_x(prm), (uint32_t)ncx);
-    const int cy = c.p % prm.ncy, cz = c.p / prm.ncy;
+    c.cy = c.p % prm.ncy;
+    c.cz = c.p / prm.ncy;
     const PairConst kc(prm);
     const PairConst2 k(kc, kc.m1);
-    for (int r = 0; r < prm.nrows; ++r) {
-        const StencilRow row = prm.rows[r];
-        const int q = row_pencil_of<DIM>(row, cy, cz, prm);
-        const int qs = (int)__ldg(cs + q * ncx), qe = (int)__ldg(cs + q * ncx + ncx), len = qe - qs;
-        int s, cnt;
-        cyclic_range(cs, q * ncx, cx - (int)row.w, cx + row.w + 1, ncx, qs, qe, s, cnt);
-        for (int t = 0; t < cnt; ++t) {
-            int j = s + t;
-            j = j >= qe ? j - len : j;
-            const float2 w = pair_shape<DIM, KERNEL, ISO, true>(pa, __ldg(P + j), k, sc);
+    chunk_rows<DIM, ISO, ISO ? kCutBand : kCutFull>(P, cs, prm, c, pa, nullptr, [&](int qs, int qe, int s, int m, int) {
+        const int len = qe - qs;
+        for (int t = 0; t < m; t += 2) {
+            const int j0 = s + t, j1 = min(t + 1, m - 1) + s;
+            const int i0 = j0 >= qe ? j0 - len : j0, i1 = j1 >= qe ? j1 - len : j1;
+            Double2 gL, gT;
+            pair_fine2<DIM, KERNEL, ISO>(pa, __ldg(P + i0), __ldg(P + i1), k, sc, gL, gT);
 #pragma unroll
-            for (int f = 0; f < NR; ++f) op.add(f, w, op.x[f][qs + j]);
+            for (int f = 0; f < NR; ++f) {
+                op.add(f, f2(gL.h.x, gT.h.x), f2(gL.l.x, gT.l.x), op.x[f][qs + i0]);
+                if (t + 1 < m) op.add(f, f2(gL.h.y, gT.h.y), f2(gL.l.y, gT.l.y), op.x[f][qs + i1]);
+            }
         }
         op.end_row();
-    }
+    });
 }
 
 // The table (prm.uw = vhat, prm.ub = 0) and the initial concentrations, doubled per pencil.
@@ -213,8 +237,10 @@ __global__ __launch_bounds__(kT) void k_adj_pass(const uint4 *__restrict__ P, co
     if (my_chunk(tab, prm, c, sl)) {
         const int i = c.i0 + (threadIdx.x & 31);
         const int at = c.ps + min(i, c.pe - 1);
-        ShapeSums<NR> op;
+        ShapeSums<NR, BACK> op;
         op.zero();
+        op.words = tab.words;
+        op.low = tab.low;
         op.x[0] = ps.x1;
         op.xa[0] = ps.x1[at];
         if (BACK) {
@@ -222,20 +248,20 @@ __global__ __launch_bounds__(kT) void k_adj_pass(const uint4 *__restrict__ P, co
             op.xa[NR - 1] = ps.x0[at];
         }
         if (sl.x != kNoRoom) stream_rows<2>(sl, tab, op);
-        else walk_sums<DIM, KERNEL, ISO, NR>(P, cs, prm, c, ps.sc, op);
+        else walk_sums<DIM, KERNEL, ISO, NR, BACK>(P, cs, prm, c, ps.sc, op);
         if (i < c.pe) {
             const int again = c.pe + i;
             const float L1 = combine(ps, op.s0(0), op.s1(0));
             const float p = MODE == HALF || MODE == BACK1 ? op.xa[0] : ps.base[at];
             ps.out1[at] = ps.out1[again] = fmaf(ps.step, L1, p);
             if (BACK) {
-                const float s0 = op.s0(NR - 1), s1 = op.s1(NR - 1);
-                dot[0] = fma((double)p, (double)s0, dot[0]);
-                dot[1] = fma((double)p, (double)s1, dot[1]);
+                const double s0 = op.d0(NR - 1), s1 = op.d1(NR - 1);
+                dot[0] = (double)p * s0;
+                dot[1] = (double)p * s1;
                 if (MODE == BACK1) {
-                    dot[2 % ND] = fma((double)L1, (double)s0, dot[2 % ND]);
-                    dot[3 % ND] = fma((double)L1, (double)s1, dot[3 % ND]);
-                    ps.out0[at] = ps.out0[again] = combine(ps, s0, s1);
+                    dot[2 % ND] = (double)L1 * s0;
+                    dot[3 % ND] = (double)L1 * s1;
+                    ps.out0[at] = ps.out0[again] = combine(ps, op.s0(NR - 1), op.s1(NR - 1));
                 }
             }
         }
@@ -434,7 +460,7 @@ extern "C" int ade_adjoint_weights_bytes(ade_ctx *c, int counted, size_t *bytes,
     const int rc = plan_context_table(c, 2, counted != 0, &c->adj_plan, (cudaStream_t)stream);
     if (rc || c->adj_plan.stride == 0u || (!counted && c->adj_plan.lines == 0)) return rc;
     // above the limit: as many chunks as fit
-    *bytes = c->adj_plan.lines > 0 ? c->adj_plan.lines * 128 : (size_t)kTableMaxBytes / 256 * 256;
+    *bytes = c->adj_plan.lines > 0 ? c->adj_plan.lines * 192 + 256 : (size_t)kTableMaxBytes / 256 * 256;
     return ADE_OK;
 }
 
@@ -460,7 +486,7 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     for (int i = 0; i < c->dim; ++i) vabs += c->p.v[i] * c->p.v[i];
     vabs = sqrt(vabs);
     // the table's shapes are those of 2 (1 - q): 2^3 f (C2) or 2^5 f (C4), undone in the prefactor
-    const double pf = (double)c->rp.pf * (c->p.kernel == ADE_WENDLAND_C2 ? 0.125 : 0.03125);
+    const double pf = c->pf * (c->p.kernel == ADE_WENDLAND_C2 ? 0.125 : 0.03125);
     Adj A;
     A.c = c;
     A.s = (cudaStream_t)stream;
@@ -469,16 +495,24 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     for (int i = 0; i < 3; ++i) A.rp.back[i] = 0u;
     A.rp.ub = 0.f;
     float lo[3];
+    auto left = [](double v) { return (float)(v - (double)(float)v); };   // what FP32 leaves of v
     for (int i = 0; i < 3; ++i) {
         const double vh = vabs > 0.0 ? (i < c->dim ? c->p.v[i] / vabs : 0.0) : (i == 0 ? 1.0 : 0.0);
         A.rp.uw[i] = (float)vh;
-        lo[i] = (float)(vh - (double)A.rp.uw[i]);
+        lo[i] = left(vh);
     }
     // 1/H in x-axis words, and the part of it that FP32 leaves
-    A.sc.lo = make_float4(lo[0], lo[1], lo[2], (float)(c->p.box[0] / kTwo32 / c->H - (double)c->rp.invH));
+    A.sc.vl = make_float4(lo[0], lo[1], lo[2], (float)(c->p.box[0] / kTwo32 / c->H - (double)c->rp.invH));
     A.sc.g2 = (float)(2.0 * gamma);
     A.sc.bT = (float)(2.0 * (gamma - c->dim) + 2.0);
-    const double sa = c->p.alpha_L * vabs + c->p.D_m, sb = c->p.alpha_T * vabs + c->p.D_m;
+    A.sc.g2l = left(2.0 * gamma);
+    A.sc.bTl = left(2.0 * (gamma - c->dim) + 2.0);
+    A.sc.syl = (float)(c->p.box[1] / c->p.box[0] - (double)c->rp.sy);
+    A.sc.szl = c->dim == 3 ? (float)(c->p.box[2] / c->p.box[0] - (double)c->rp.sz) : 0.f;
+    // the passes step by dt rounded to FP32; what that leaves is put into L's coefficients
+    const float dt = (float)c->dt;
+    const double fit = dt > 0.f ? c->dt / (double)dt : 1.0;
+    const double sa = fit * (c->p.alpha_L * vabs + c->p.D_m), sb = fit * (c->p.alpha_T * vabs + c->p.D_m);
     A.ca = (float)(pf * sa);
     A.cb = (float)(pf * sb);
     A.cal = (float)(pf * sa - (double)A.ca);
@@ -495,10 +529,11 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     A.tab.cursor = reinterpret_cast<unsigned long long *>(base + L.cursor);
     const bool count = chunk_numbers(n, A.rp.ncy * A.rp.ncz) > kCountChunksFrom;
     A.tab.dense = count ? reinterpret_cast<uint32_t *>(base + L.dense) : nullptr;
-    divide_table(c->adj_plan, std::min((aws_bytes - L.total) / 128, (size_t)kTableMaxBytes / 128), &A.rp, &A.tab);
+    const size_t kept = std::min(aws_bytes - L.total, (size_t)kTableMaxBytes), lines = kept > 256 ? (kept - 256) / 192 : 0;
+    A.tab.low = A.tab.words + lines * 32;      // (a line more than half of the table's: 256 bytes)
+    divide_table(c->adj_plan, lines, &A.rp, &A.tab);
     const int nb = (int)A.blocks;
     if (nb > L.blocks) return ade::report_error(ADE_ERR_CAPACITY, "adjoint partials exceed the workspace");
-    const float dt = (float)c->dt;
     cudaStream_t s = A.s;
     const uint32_t *perm = c->w.perm;
 
@@ -567,12 +602,12 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     ADJ_CK(cudaStreamSynchronize(s));
     if (J_host) *J_host = 0.5 * hd[(size_t)nsteps * kDots];
     if (dJdtheta_host) {
-        // sum_l dt p.(L_k u) + dt^2/2 (p.(L_k a) + b.(L_k u)) of S_L and S_T
-        const double dtd = (double)dt;
+        // sum_l dt p.(L_k u) + dt^2/2 (p.(L_k a) + b.(L_k u)) of S_L and S_T; a and b hold the factor `fit`
+        const double dtd = c->dt, dt2 = c->dt * (double)dt;
         double g[2] = {0.0, 0.0};
         for (int l = 0; l < nsteps; ++l) {
             const double *d = hd.data() + (size_t)l * kDots;
-            for (int q = 0; q < 2; ++q) g[q] += dtd * d[q] + 0.5 * dtd * dtd * (d[4 + q] + d[2 + q]);
+            for (int q = 0; q < 2; ++q) g[q] += dtd * d[q] + 0.5 * dt2 * (d[4 + q] + d[2 + q]);
         }
         dJdtheta_host[0] = pf * vabs * g[0];
         dJdtheta_host[1] = pf * vabs * g[1];

@@ -1103,6 +1103,7 @@ int ade_init_particles(ade_ctx **out, const ade_params *p, int n, uint32_t *xq_d
         delete c;
         return rc;
     }
+    c->pf = 0.5 * (p->mass / p->rho) * kernel_kc(p->kernel, p->dim, d.H);
     c->rp.pencil = c->w.pencil;
     c->Hgrid = d.Hgrid;
     c->skin = d.skin;

@@ -13,7 +13,8 @@
 // too small costs time, never a result (claim_lines in pool.h never hands out a line twice).
 //
 // A value is one word (the weight for one tensor: VAL 1) or two (g_L and g_T, from which every
-// uniform tensor's weight follows: VAL 2, lane l's pair in words 2l, 2l + 1 of two lines).
+// uniform tensor's weight follows: VAL 2, lane l's pair in words 2l, 2l + 1 of two lines); with low parts
+// (FINE), those of the pair that begins in line k of the table lie in line k / 2 of a plane of their own.
 #pragma once
 
 constexpr unsigned kFull = 0xffffffffu;
@@ -123,30 +124,51 @@ __device__ __forceinline__ float pair_weight(const uint4 &pa, const uint4 &pb, c
 // The pair's weights for D = vhat vhat^T and D = I - vhat vhat^T (Eq. 3-5 with K = 2D),
 //   g_L = f (2 Gamma u - 2),  g_T = f (-2 Gamma u + 2 (Gamma - d) + 2),  u = (vhat . e)^2,
 // from which every uniform tensor's weight is (alpha_L |v| + D_m) g_L + (alpha_T |v| + D_m) g_T (sums of
-// f and f u would cancel in that).  Both 0 outside the support and at zero separation.  FINE (the adjoint):
-// 1/r takes a Newton step, and r, 1/H, vhat (sc.lo: low parts {vhat, 1/H}) and u are taken to twice FP32.
-// On a lattice the same few separations recur, so their rounding biases every pair alike, and dJ/dtheta adds
-// the pairs of all steps: 1e-8..2e-7 of its components with FINE, 4e-9..3e-7 with the low parts of vhat, r and
-// 1/H alone (six plumes of 85^2 to 512^2).  The sweep's concentrations do not feel it (2e-8..1.1e-7 both ways,
-// and without the table), and a call of four steps with 8 sets on 512^2 takes 603 us instead of 654.
+// f and f u would cancel in that).  Both 0 outside the support and at zero separation.  Low parts (what FP32
+// leaves) of the constants: vl {vhat, 1/H}, g2l, bTl, syl, szl (pair_fine2 only).
 struct ShapeConst {
-    float4 lo;
+    float4 vl;
     float g2, bT;          // 2 Gamma, 2 (Gamma - d) + 2
+    float g2l, bTl, syl, szl;
 };
 
-template <int DIM, int KERNEL, bool ISO, bool FINE>
+// The sweep's: two candidates at once, in packed FP32x2 instructions.
+template <int DIM, int KERNEL, bool ISO>
 __device__ __forceinline__ void pair_shape2(const uint4 &pa, const uint4 &p0, const uint4 &p1, const PairConst2 &k,
-                                            const ShapeConst &sc, float2 &gL, float2 &gT);
+                                            const ShapeConst &sc, float2 &gL, float2 &gT)
+{
+    const float2 dx = f2(sep(pa.x, p0.x, k.m1), sep(pa.x, p1.x, k.m1));
+    float2 dy = f2(sep(pa.y, p0.y, k.m1), sep(pa.y, p1.y, k.m1));
+    float2 dz = f2(0.f, 0.f);
+    if (DIM == 3) dz = f2(sep(pa.z, p0.z, k.m1), sep(pa.z, p1.z, k.m1));
+    if (!ISO) {
+        dy = __fmul2_rn(dy, k.sy);
+        if (DIM == 3) dz = __fmul2_rn(dz, k.sz);
+    }
+    const float2 m1 = f2(-1.f, -1.f), one = f2(1.f, 1.f), g2 = f2(sc.g2, sc.g2);
+    float2 r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)), c = __ffma2_rn(k.w0, dx, __fmul2_rn(k.w1, dy));
+    if (DIM == 3) {
+        r2 = __ffma2_rn(dz, dz, r2);
+        c = __ffma2_rn(k.w2, dz, c);
+    }
+    const float2 rinv = f2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+    const float2 om = __ffma2_rn(__fmul2_rn(r2, rinv), k.ninvH, one);
+    const float2 f = shape2x2<KERNEL>(f2(fmaxf(om.x + om.x, 0.f), fmaxf(om.y + om.y, 0.f)));
+    const float2 t = __fmul2_rn(c, rinv), t2 = __fmul2_rn(t, t), u = f2(fminf(t2.x, 1.f), fminf(t2.y, 1.f));
+    gL = __fmul2_rn(f, __ffma2_rn(g2, u, f2(-2.f, -2.f)));
+    gT = __fmul2_rn(f, __ffma2_rn(__fmul2_rn(g2, m1), u, f2(sc.bT, sc.bT)));
+}
 
-template <int DIM, int KERNEL, bool ISO, bool FINE>
+template <int DIM, int KERNEL, bool ISO>
 __device__ __forceinline__ float2 pair_shape(const uint4 &pa, const uint4 &pb, const PairConst2 &k, const ShapeConst &sc)
 {
     float2 gL, gT;
-    pair_shape2<DIM, KERNEL, ISO, FINE>(pa, pb, pb, k, sc, gL, gT);
+    pair_shape2<DIM, KERNEL, ISO>(pa, pb, pb, k, sc, gL, gT);
     return make_float2(gL.x, gT.x);
 }
 
-// Sum and product with their rounding errors (Knuth's two-sum; fused multiply-add), per half.
+// Numbers of twice FP32's precision as unevaluated sums h + l, two at a time: sum and product with their
+// rounding errors (Knuth's two-sum; fused multiply-add), added to what l holds already.
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.f, -1.f), a); }
 __device__ __forceinline__ float2 two_sum2(float2 a, float2 b, float2 &lo)
 {
@@ -160,62 +182,104 @@ __device__ __forceinline__ float2 two_prod2(float2 a, float2 b, float2 &lo)
     lo = __fadd2_rn(lo, __ffma2_rn(a, b, __fmul2_rn(p, f2(-1.f, -1.f))));
     return p;
 }
-
-// Two candidates at once, in packed FP32x2 instructions.
-template <int DIM, int KERNEL, bool ISO, bool FINE>
-__device__ __forceinline__ void pair_shape2(const uint4 &pa, const uint4 &p0, const uint4 &p1, const PairConst2 &k,
-                                            const ShapeConst &sc, float2 &gL, float2 &gT)
+struct Double2 {
+    float2 h, l;
+};
+__device__ __forceinline__ Double2 mul22(const Double2 &a, const Double2 &b)
 {
-    float2 dx = f2(sep(pa.x, p0.x, k.m1), sep(pa.x, p1.x, k.m1));
-    float2 dy = f2(sep(pa.y, p0.y, k.m1), sep(pa.y, p1.y, k.m1));
-    float2 dz = f2(0.f, 0.f);
-    if (DIM == 3) dz = f2(sep(pa.z, p0.z, k.m1), sep(pa.z, p1.z, k.m1));
+    Double2 r;
+    r.l = __ffma2_rn(a.h, b.l, __fmul2_rn(a.l, b.h));
+    r.h = two_prod2(a.h, b.h, r.l);
+    return r;
+}
+__device__ __forceinline__ Double2 settle(const Double2 &a)     // |l| at most half a unit of h's last place
+{
+    const float2 h = __fadd2_rn(a.h, a.l);
+    return Double2{h, sub2(a.l, sub2(h, a.h))};
+}
+__device__ __forceinline__ float2 both(float x) { return f2(x, x); }
+// Separation of two candidates along one axis (h + l is the integer difference exactly).
+__device__ __forceinline__ Double2 sep22(uint32_t a, uint32_t b0, uint32_t b1)
+{
+    const int d0 = (int)(a - b0), d1 = (int)(a - b1);
+    const float h0 = (float)d0, h1 = (float)d1;
+    return Double2{f2(h0, h1), f2((float)(d0 - __float2int_rn(h0)), (float)(d1 - __float2int_rn(h1)))};
+}
+
+// g_L and g_T of two candidates to twice FP32 (the adjoint).  On a lattice the same few separations recur, so a
+// weight's rounding biases every pair alike, and dJ/dtheta adds the pairs of all steps: with weights rounded
+// to FP32 it was off by up to 2e-7 of its value.
+template <int DIM, int KERNEL, bool ISO>
+__device__ __forceinline__ void pair_fine2(const uint4 &pa, const uint4 &p0, const uint4 &p1, const PairConst2 &k,
+                                           const ShapeConst &sc, Double2 &gL, Double2 &gT)
+{
+    const float2 m1 = both(-1.f), half = both(0.5f), none = both(0.f);
+    const Double2 x = sep22(pa.x, p0.x, p1.x);
+    Double2 y = sep22(pa.y, p0.y, p1.y), z = Double2{none, none};
+    if (DIM == 3) z = sep22(pa.z, p0.z, p1.z);
     if (!ISO) {
-        dy = __fmul2_rn(dy, k.sy);
-        if (DIM == 3) dz = __fmul2_rn(dz, k.sz);
+        y = mul22(y, Double2{k.sy, both(sc.syl)});
+        if (DIM == 3) z = mul22(z, Double2{k.sz, both(sc.szl)});
     }
-    const float2 m1 = f2(-1.f, -1.f), one = f2(1.f, 1.f), half = f2(0.5f, 0.5f), g2 = f2(sc.g2, sc.g2);
-    if (!FINE) {
-        float2 r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)), c = __ffma2_rn(k.w0, dx, __fmul2_rn(k.w1, dy));
-        if (DIM == 3) {
-            r2 = __ffma2_rn(dz, dz, r2);
-            c = __ffma2_rn(k.w2, dz, c);
-        }
-        const float2 rinv = f2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-        const float2 om = __ffma2_rn(__fmul2_rn(r2, rinv), k.ninvH, one);
-        const float2 f = shape2x2<KERNEL>(f2(fmaxf(om.x + om.x, 0.f), fmaxf(om.y + om.y, 0.f)));
-        const float2 t = __fmul2_rn(c, rinv), t2 = __fmul2_rn(t, t), u = f2(fminf(t2.x, 1.f), fminf(t2.y, 1.f));
-        gL = __fmul2_rn(f, __ffma2_rn(g2, u, f2(-2.f, -2.f)));
-        gT = __fmul2_rn(f, __ffma2_rn(__fmul2_rn(g2, m1), u, f2(sc.bT, sc.bT)));
-        return;
-    }
-    float2 r2l = f2(0.f, 0.f), cl = __ffma2_rn(f2(sc.lo.x, sc.lo.x), dx, __fmul2_rn(f2(sc.lo.y, sc.lo.y), dy));
-    float2 r2 = two_sum2(two_prod2(dx, dx, r2l), two_prod2(dy, dy, r2l), r2l);
-    float2 ch = two_sum2(two_prod2(k.w0, dx, cl), two_prod2(k.w1, dy, cl), cl);           // vhat . x
+    // r^2 and vhat . x
+    float2 r2l = __fmul2_rn(__fadd2_rn(x.h, x.h), x.l), cl = __ffma2_rn(both(sc.vl.x), x.h, __fmul2_rn(k.w0, x.l));
+    r2l = __ffma2_rn(__fadd2_rn(y.h, y.h), y.l, r2l);
+    cl = __ffma2_rn(both(sc.vl.y), y.h, __ffma2_rn(k.w1, y.l, cl));
+    float2 r2 = two_prod2(x.h, x.h, r2l), ch = two_prod2(k.w0, x.h, cl);
+    r2 = two_sum2(r2, two_prod2(y.h, y.h, r2l), r2l);
+    ch = two_sum2(ch, two_prod2(k.w1, y.h, cl), cl);
     if (DIM == 3) {
-        r2 = two_sum2(r2, two_prod2(dz, dz, r2l), r2l);
-        ch = two_sum2(ch, two_prod2(k.w2, dz, cl), cl);
-        cl = __ffma2_rn(f2(sc.lo.z, sc.lo.z), dz, cl);
+        r2l = __ffma2_rn(__fadd2_rn(z.h, z.h), z.l, r2l);
+        cl = __ffma2_rn(both(sc.vl.z), z.h, __ffma2_rn(k.w2, z.l, cl));
+        r2 = two_sum2(r2, two_prod2(z.h, z.h, r2l), r2l);
+        ch = two_sum2(ch, two_prod2(k.w2, z.h, cl), cl);
     }
+    // 1/r with a Newton step, r and -q = -r/H, 1 - q
     float2 rinv = f2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-    rinv = __ffma2_rn(__fmul2_rn(half, rinv), __ffma2_rn(__fmul2_rn(__fmul2_rn(r2, rinv), m1), rinv, one), rinv);
+    rinv = __ffma2_rn(__fmul2_rn(half, rinv), __ffma2_rn(__fmul2_rn(__fmul2_rn(r2, rinv), m1), rinv, both(1.f)), rinv);
     const float2 r = __fmul2_rn(r2, rinv), nr = __fmul2_rn(r, m1);
     const float2 rl = __fmul2_rn(__fmul2_rn(half, rinv), __fadd2_rn(__ffma2_rn(nr, r, r2), r2l));
-    const float2 nq = __fmul2_rn(r, k.ninvH);                                   // -q, and its low part
-    const float2 nql = __ffma2_rn(nr, f2(sc.lo.w, sc.lo.w), __ffma2_rn(rl, k.ninvH, __ffma2_rn(r, k.ninvH, __fmul2_rn(nq, m1))));
-    const float2 om = __fadd2_rn(__fadd2_rn(one, nq), nql);
-    const float2 f = shape2x2<KERNEL>(f2(fmaxf(om.x + om.x, 0.f), fmaxf(om.y + om.y, 0.f)));
+    const float2 nq = __fmul2_rn(r, k.ninvH);
+    Double2 om;
+    om.l = __ffma2_rn(nr, both(sc.vl.w), __ffma2_rn(rl, k.ninvH, __ffma2_rn(r, k.ninvH, __fmul2_rn(nq, m1))));
+    om.h = two_sum2(both(1.f), nq, om.l);
+    om = settle(om);
+    // twice 1 - q, 0 outside the support (and at r = 0, where it is not a number)
+    const bool in0 = om.h.x > 0.f, in1 = om.h.y > 0.f;
+    const Double2 w{f2(in0 ? om.h.x + om.h.x : 0.f, in1 ? om.h.y + om.h.y : 0.f), f2(in0 ? om.l.x + om.l.x : 0.f, in1 ? om.l.y + om.l.y : 0.f)};
+    Double2 f = mul22(w, w);
+    if (KERNEL == ADE_WENDLAND_C2) {
+        f = mul22(f, w);
+    } else {
+        Double2 q{none, __fmul2_rn(both(-2.5f), w.l)};                          // 6 - 5 (1 - q)
+        q.h = two_sum2(both(6.f), two_prod2(both(-2.5f), w.h, q.l), q.l);
+        f = mul22(mul22(mul22(f, f), w), q);
+    }
+    // u = (vhat . x)^2 / r^2 and what is left of it
     const float2 t = __fmul2_rn(ch, rinv), t2 = __fmul2_rn(t, t);
-    const float2 u = f2(fminf(t2.x, 1.f), fminf(t2.y, 1.f));                   // u = ch^2 / r^2 and what is left of it
+    const float2 u = f2(fminf(t2.x, 1.f), fminf(t2.y, 1.f)), nu = __fmul2_rn(u, m1);
     float2 e = __fmul2_rn(__fadd2_rn(ch, ch), cl);
     const float2 n = two_prod2(ch, ch, e);
-    e = __fadd2_rn(e, __ffma2_rn(__fmul2_rn(u, m1), r2, n));
-    e = __ffma2_rn(__fmul2_rn(u, m1), r2l, e);
+    e = __fadd2_rn(e, __ffma2_rn(nu, r2, n));       // (exact: n and u r^2 agree to a few units)
+    e = __ffma2_rn(nu, r2l, e);
     float2 ul = __fmul2_rn(__fmul2_rn(e, rinv), rinv);
     ul = f2(fminf(fmaxf(ul.x, -1e-6f), 1e-6f), fminf(fmaxf(ul.y, -1e-6f), 1e-6f));   // (max-num: finite at r = 0 too)
-    const float2 g2l = __fmul2_rn(g2, ul);
-    gL = __fmul2_rn(f, __fadd2_rn(__ffma2_rn(g2, u, f2(-2.f, -2.f)), g2l));
-    gT = __fmul2_rn(f, sub2(__ffma2_rn(__fmul2_rn(g2, m1), u, f2(sc.bT, sc.bT)), g2l));
+    const float2 g2ul = __ffma2_rn(both(sc.g2), ul, __fmul2_rn(both(sc.g2l), u));
+    Double2 A{none, g2ul}, B{none, __ffma2_rn(g2ul, m1, both(sc.bTl))};
+    A.h = two_sum2(two_prod2(both(sc.g2), u, A.l), both(-2.f), A.l);
+    B.h = two_sum2(two_prod2(both(sc.g2), nu, B.l), both(sc.bT), B.l);
+    gL = settle(mul22(f, A));
+    gT = settle(mul22(f, B));
+}
+
+// Two low parts in one word, 16 bits each: FP32 hi and a low part cut to 8 bits are 32 bits of a weight.
+__device__ __forceinline__ float pack_low(float lL, float lT)
+{
+    return __uint_as_float((__float_as_uint(lT) & 0xffff0000u) | (__float_as_uint(lL) >> 16));
+}
+__device__ __forceinline__ float2 unpack_low(float w)
+{
+    return f2(__uint_as_float(__float_as_uint(w) << 16), __uint_as_float(__float_as_uint(w) & 0xffff0000u));
 }
 
 // Squared separation in x units^2.
@@ -445,7 +509,7 @@ __device__ __forceinline__ void chunk_rows(const uint4 *__restrict__ P, const ui
 // Lines that hold the rows' lengths, a word per row.
 __device__ __forceinline__ unsigned header_lines(const RateParams &prm) { return (unsigned)(prm.nrows + 31) >> 5; }
 
-// Weights (VAL 1) or g_L, g_T (VAL 2) of one chunk into the table; VAL 1 returns the row sums of the
+// Weights (VAL 1) or g_L, g_T (VAL 2; FINE: and their low parts) of one chunk into the table; VAL 1 returns the row sums of the
 // first evaluation (the concentrations of the records).  One pass over the rows: the chunk's lines go
 // to its region (prm.fz_stride lines, what nearly every chunk needs: plan_table in api.cu) and only a chunk
 // that outgrows it is done again into room taken from the pool behind; fz_stride 0: no table.
@@ -483,20 +547,36 @@ __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const 
             if (!keep) return;                       // to be done again
             out += 32;
             float rs = 0.f;
-            if (VAL == 2) {
+            if (FINE) {
+                const size_t line = (size_t)(out - lane - tab.words) >> 5;
+                for (int t = 0; t < m; t += 2) {
+                    const int j0 = s + t, j1 = min(t + 1, m - 1) + s;
+                    Double2 gL, gT;
+                    pair_fine2<DIM, KERNEL, ISO>(pa, __ldg(P + (j0 >= qe ? j0 - len : j0)), __ldg(P + (j1 >= qe ? j1 - len : j1)), k2, sc,
+                                                 gL, gT);
+                    float2 *o = reinterpret_cast<float2 *>(out + lane) + t * 32;
+                    float *low = tab.low + ((line >> 1) + t) * 32 + lane;
+                    o[0] = f2(gL.h.x, gT.h.x);
+                    low[0] = pack_low(gL.l.x, gT.l.x);
+                    if (t + 1 < m) {
+                        o[32] = f2(gL.h.y, gT.h.y);
+                        low[32] = pack_low(gL.l.y, gT.l.y);
+                    }
+                }
+            } else if (VAL == 2) {
                 float2 *o2 = reinterpret_cast<float2 *>(out + lane);
                 int t = 0;
                 for (; t + 1 < m; t += 2) {
                     const int j0 = s + t, j1 = j0 + 1;
                     float2 gL, gT;
-                    pair_shape2<DIM, KERNEL, ISO, FINE>(pa, __ldg(P + (j0 >= qe ? j0 - len : j0)), __ldg(P + (j1 >= qe ? j1 - len : j1)),
+                    pair_shape2<DIM, KERNEL, ISO>(pa, __ldg(P + (j0 >= qe ? j0 - len : j0)), __ldg(P + (j1 >= qe ? j1 - len : j1)),
                                                   k2, sc, gL, gT);
                     o2[t * 32] = f2(gL.x, gT.x);
                     o2[(t + 1) * 32] = f2(gL.y, gT.y);
                 }
                 if (t < m) {
                     const int j = s + t;
-                    o2[t * 32] = pair_shape<DIM, KERNEL, ISO, FINE>(pa, __ldg(P + (j >= qe ? j - len : j)), k2, sc);
+                    o2[t * 32] = pair_shape<DIM, KERNEL, ISO>(pa, __ldg(P + (j >= qe ? j - len : j)), k2, sc);
                 }
             } else if (__any_sync(kFull, s + m > qe)) {
                 rs = row_weights<DIM, KERNEL, ISO, true, true>(P, pa, Ca, k, k2, s, m, qe, len, out);
@@ -558,7 +638,10 @@ __device__ __forceinline__ void stream_rows(const uint4 sl, const FrozenTab &tab
     const float *w = base + lane;
     const int total = (int)sl.z;
     int ahead = min(total, kAhead);
-    if (lane == 0) prefetch_l2(base, (unsigned)ahead * 128u);
+    if (lane == 0) {
+        prefetch_l2(base, (unsigned)ahead * 128u);
+        op.prefetch(base, 0, ahead);
+    }
     const float *hdr = w;
     w += (size_t)sl.w * 32;
     int hm = 0;
@@ -573,7 +656,10 @@ __device__ __forceinline__ void stream_rows(const uint4 sl, const FrozenTab &tab
         const int pos = (int)((w - base) >> 5);
         if (ahead < total && pos + kAhead > ahead + kPiece) {
             const int n = min(total - ahead, pos + kAhead - ahead);
-            if (lane == 0) prefetch_l2(base + (size_t)ahead * 32, (unsigned)n * 128u);
+            if (lane == 0) {
+                prefetch_l2(base + (size_t)ahead * 32, (unsigned)n * 128u);
+                op.prefetch(base, ahead, n);
+            }
             ahead += n;
         }
         int k = m;
@@ -596,6 +682,7 @@ __device__ __forceinline__ void stream_rows(const uint4 sl, const FrozenTab &tab
 struct WeightedSum {
     const float *C;
     float Ca, rs, acc, comp;
+    __device__ __forceinline__ void prefetch(const float *, int, int) const {}
     template <int M>
     __device__ __forceinline__ void lines(const float *w, int s)
     {

@@ -125,6 +125,7 @@ struct SetSums {
     const float *C;            // doubled, from the group's first set
     size_t plane;
     float2 Ca[N2], rs[N2], acc[N2], comp[N2], dL[N2], dT[N2];
+    __device__ __forceinline__ void prefetch(const float *, int, int) const {}
     __device__ __forceinline__ void add(float2 g, const float2 (&Cb)[N2])
     {
         const float2 gl = f2(g.x, g.x), gt = f2(g.y, g.y), m1 = f2(-1.f, -1.f);
@@ -189,7 +190,7 @@ __device__ __noinline__ void walk_sets(const uint4 *__restrict__ P, const uint32
             j = j >= qe ? j - len : j;
             float2 v[SetSums<NT>::N2];
             op.load((size_t)(qs + j), v);
-            op.add(pair_shape<DIM, KERNEL, ISO, false>(pa, __ldg(P + j), k, sc), v);
+            op.add(pair_shape<DIM, KERNEL, ISO>(pa, __ldg(P + j), k, sc), v);
         }
         op.end_row();
     }
@@ -440,8 +441,8 @@ cudaError_t pass_nt(const SweepRun &r, int epi, const SweepParams &sp, const Rat
 {
     const unsigned g = frozen_blocks(prm);
     return epi == EPI_PREDICT
-               ? launch_pdl(k_sweep_pass<DIM, KERNEL, ISO, NT, EPI_PREDICT>, g, kT, 0, s, r.P, r.cs, prm, r.tab, ShapeConst{float4{}, r.g2, r.bT}, sp, r.C, r.Ch, r.perm, out)
-               : launch_pdl(k_sweep_pass<DIM, KERNEL, ISO, NT, EPI_CORRECT>, g, kT, 0, s, r.P, r.cs, prm, r.tab, ShapeConst{float4{}, r.g2, r.bT}, sp, r.C, r.Ch, r.perm, out);
+               ? launch_pdl(k_sweep_pass<DIM, KERNEL, ISO, NT, EPI_PREDICT>, g, kT, 0, s, r.P, r.cs, prm, r.tab, ShapeConst{float4{}, r.g2, r.bT, 0.f, 0.f, 0.f, 0.f}, sp, r.C, r.Ch, r.perm, out)
+               : launch_pdl(k_sweep_pass<DIM, KERNEL, ISO, NT, EPI_CORRECT>, g, kT, 0, s, r.P, r.cs, prm, r.tab, ShapeConst{float4{}, r.g2, r.bT, 0.f, 0.f, 0.f, 0.f}, sp, r.C, r.Ch, r.perm, out);
 }
 
 template <int DIM, int KERNEL, bool ISO>
@@ -459,7 +460,7 @@ template <int DIM, int KERNEL, bool ISO>
 cudaError_t table_k(const SweepRun &r, const RateParams &prm, const float *C, int sets, int P4, cudaStream_t s)
 {
     return launch_pdl(k_sweep_table<DIM, KERNEL, ISO>, frozen_blocks(prm), kT, 0, s, r.P, r.cs, r.perm, prm, r.tab,
-                      ShapeConst{float4{}, r.g2, r.bT}, C, sets, P4, r.C);
+                      ShapeConst{float4{}, r.g2, r.bT, 0.f, 0.f, 0.f, 0.f}, C, sets, P4, r.C);
 }
 
 #define ADE_SWEEP_CALL(F, ...)                                                                                               \
