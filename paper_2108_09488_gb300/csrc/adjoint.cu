@@ -149,10 +149,10 @@ __device__ __noinline__ void walk_sums(const uint4 *__restrict__ P, const uint32
     });
 }
 
-// The table (prm.uw = vhat, prm.ub = 0) and the initial concentrations, doubled per pencil.
+// The table (prm.uw = vhat, prm.ub = 0) and the initial concentrations, doubled per pencil and as kept.
 template <int DIM, int KERNEL, bool ISO>
 __global__ __launch_bounds__(kT) void k_adj_table(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
-                                                  const RateParams prm, const FrozenTab tab, const ShapeConst sc, float *__restrict__ C0)
+                                                  const RateParams prm, const FrozenTab tab, const ShapeConst sc, float *__restrict__ C0, float *__restrict__ kept)
 {
     pdl_wait();
     __shared__ TrimRow srow[ISO ? kMaxRows : 1];
@@ -165,10 +165,10 @@ __global__ __launch_bounds__(kT) void k_adj_table(const uint4 *__restrict__ P, c
     const int i = c.i0 + (threadIdx.x & 31);
     const uint4 pa = __ldg(P + min(i, c.pe - 1));
     build_chunk<DIM, KERNEL, ISO, ISO ? kCutBox : kCutFull, 2, true>(P, cs, prm, c, pa, srow, tab, sc);
-    if (i < c.pe) C0[c.ps + i] = C0[c.pe + i] = __uint_as_float(pa.w);
+    if (i < c.pe) C0[c.ps + i] = C0[c.pe + i] = kept[i] = __uint_as_float(pa.w);
 }
 
-// One pass over the table; fields doubled per pencil.
+// One pass over the table; fields doubled per pencil (states that are kept for later, once per particle).
 //   HALF, FULL  out1 = base + step L x1 (HALF: base = x1)
 //   BACK1       out0 = a = L x0 (x0 = u), out1 = x1 + step L x1 (x1 = p); dots of p and b = L p with S_L u, S_T u
 //   BACK2       out1 = base + step L x1 (x1 = hp, base = p; out1 may be base); dots of p with S_L a, S_T a (x0 = a)
@@ -178,6 +178,9 @@ struct AdjPass {
     float *out0, *out1;
     float ca, cb, cal, cbl;   // L x = ca S_L + cb S_T (hi + lo), pf folded in
     float step;
+    float *kept;           // FULL: out1 once per particle as well (NULL: not)
+    const float *next;     // BACK2: the kept state that the next step reads, doubled into next2 (NULL: none)
+    float *next2;
     ShapeConst sc;
     double *partials;      // [blocks][kDots] of the step (BACK1: the first four, BACK2: the last two)
 };
@@ -253,7 +256,10 @@ __global__ __launch_bounds__(kT) void k_adj_pass(const uint4 *__restrict__ P, co
             const int again = c.pe + i;
             const float L1 = combine(ps, op.s0(0), op.s1(0));
             const float p = MODE == HALF || MODE == BACK1 ? op.xa[0] : ps.base[at];
-            ps.out1[at] = ps.out1[again] = fmaf(ps.step, L1, p);
+            const float o = fmaf(ps.step, L1, p);
+            ps.out1[at] = ps.out1[again] = o;
+            if (MODE == FULL && ps.kept) ps.kept[i] = o;
+            if (MODE == BACK2 && ps.next) ps.next2[at] = ps.next2[again] = ps.next[i];
             if (BACK) {
                 const double s0 = op.d0(NR - 1), s1 = op.d1(NR - 1);
                 dot[0] = (double)p * s0;
@@ -270,7 +276,7 @@ __global__ __launch_bounds__(kT) void k_adj_pass(const uint4 *__restrict__ P, co
         block_sums<ND>(dot, ps.partials + (size_t)blockIdx.x * kDots + (MODE == BACK2 ? 4 : 0));
 }
 
-// lambda^N = C^N - C* (doubled per pencil) and its squares' block sums.
+// lambda^N = C^N - C* (doubled per pencil; C^N as kept) and its squares' block sums.
 __global__ __launch_bounds__(kT) void k_adj_misfit(const uint32_t *__restrict__ perm, const RateParams prm, const FrozenTab tab,
                                                    const float *__restrict__ CN, const float *__restrict__ target,
                                                    float *__restrict__ p, double *__restrict__ partials)
@@ -284,7 +290,7 @@ __global__ __launch_bounds__(kT) void k_adj_misfit(const uint32_t *__restrict__ 
     if (has && i < c.pe) {
         const uint32_t a = __ldg(perm + i);
         const float t = a < (uint32_t)prm.n ? __ldg(target + a) : 0.f;
-        const float v = fmaf(-1.f, t, CN[c.ps + i]);
+        const float v = fmaf(-1.f, t, CN[i]);
         p[c.ps + i] = p[c.pe + i] = v;
         d[0] = (double)v * (double)v;
     }
@@ -318,9 +324,9 @@ __global__ __launch_bounds__(kFoldT) void k_adj_fold(const double *__restrict__ 
     }
 }
 
-// out[perm[i]] = the doubled field's value of sorted particle i.
+// out[perm[i]] = the value of sorted particle i, of a doubled field or a kept one.
 __global__ __launch_bounds__(kT) void k_adj_scatter(const uint32_t *__restrict__ perm, const RateParams prm, const FrozenTab tab,
-                                                    const float *__restrict__ x, float *__restrict__ out)
+                                                    const float *__restrict__ x, bool doubled, float *__restrict__ out)
 {
     pdl_wait();
     Chunk c;
@@ -329,7 +335,19 @@ __global__ __launch_bounds__(kT) void k_adj_scatter(const uint32_t *__restrict__
     const int i = c.i0 + (threadIdx.x & 31);
     if (i >= c.pe) return;
     const uint32_t a = __ldg(perm + i);
-    if (a < (uint32_t)prm.n) out[a] = x[c.ps + i];
+    if (a < (uint32_t)prm.n) out[a] = x[doubled ? c.ps + i : i];
+}
+
+// A kept state doubled per pencil.
+__global__ __launch_bounds__(kT) void k_adj_double(const RateParams prm, const FrozenTab tab, const float *__restrict__ x,
+                                                   float *__restrict__ out)
+{
+    pdl_wait();
+    Chunk c;
+    uint4 sl;
+    if (!my_chunk(tab, prm, c, sl)) return;
+    const int i = c.i0 + (threadIdx.x & 31);
+    if (i < c.pe) out[c.ps + i] = out[c.pe + i] = x[i];
 }
 
 // Everything one call needs.
@@ -357,9 +375,9 @@ cudaError_t pass_t(const Adj &A, int mode, const AdjPass &ps)
 }
 
 template <int DIM, int KERNEL, bool ISO>
-cudaError_t table_t(const Adj &A, float *C0)
+cudaError_t table_t(const Adj &A, float *C0, float *kept)
 {
-    return launch_pdl(k_adj_table<DIM, KERNEL, ISO>, A.blocks, kT, 0, A.s, A.c->w.P0, A.c->w.cell_start, A.rp, A.tab, A.sc, C0);
+    return launch_pdl(k_adj_table<DIM, KERNEL, ISO>, A.blocks, kT, 0, A.s, A.c->w.P0, A.c->w.cell_start, A.rp, A.tab, A.sc, C0, kept);
 }
 
 #define ADE_ADJ_CALL(F, ...)                                                                                          \
@@ -371,10 +389,10 @@ cudaError_t table_t(const Adj &A, float *C0)
                           : (A.c->iso ? F<3, ADE_WENDLAND_C4, true>(__VA_ARGS__) : F<3, ADE_WENDLAND_C4, false>(__VA_ARGS__))))
 
 cudaError_t pass(const Adj &A, int mode, const AdjPass &ps) { return ADE_ADJ_CALL(pass_t, A, mode, ps); }
-cudaError_t table(const Adj &A, float *C0) { return ADE_ADJ_CALL(table_t, A, C0); }
+cudaError_t table(const Adj &A, float *C0, float *kept) { return ADE_ADJ_CALL(table_t, A, C0, kept); }
 
-// One forward step C_out = S C_in: h = u + dt/2 L u, C_out = u + dt L h.
-cudaError_t fwd_step(const Adj &A, const float *u, float *h, float *out, float dt)
+// One forward step C_out = S C_in: h = u + dt/2 L u, C_out = u + dt L h (kept: once per particle as well).
+cudaError_t fwd_step(const Adj &A, const float *u, float *h, float *out, float *kept, float dt)
 {
     AdjPass ps;
     memset(&ps, 0, sizeof(ps));
@@ -391,13 +409,15 @@ cudaError_t fwd_step(const Adj &A, const float *u, float *h, float *out, float d
     ps.x1 = h;
     ps.base = u;
     ps.out1 = out;
+    ps.kept = kept;
     ps.step = dt;
     return pass(A, FULL, ps);
 }
 
-// Adjoint workspace: fields (doubled per pencil), the weight table, FP64 partials of one segment.
+// Adjoint workspace: states kept once per particle (checkpoints, one segment), working fields doubled per pencil, FP64
+// partials of one segment; the weight table lies behind.
 struct AdjLayout {
-    size_t ckpt, seg, h, p, hp, a, dots, partials, slots, dense, cursor, total;
+    size_t ckpt, seg, u0, u1, h, p, hp, a, dots, partials, slots, dense, cursor, total;
     int nck, blocks;
 };
 
@@ -410,12 +430,14 @@ AdjLayout adj_layout(const ade_ctx *c, int nsteps, int ck)
         off += ((bytes > 0 ? bytes : 1) + 255) & ~(size_t)255;
         return o;
     };
-    const size_t f2 = (size_t)c->n * 8;
+    const size_t f1 = (size_t)c->n * 4, f2 = 2 * f1;
     const size_t slots = table_slots(c);
     L.blocks = (int)((slots + kT / 32 - 1) / (kT / 32));
     L.nck = (nsteps + ck - 1) / ck;
-    L.ckpt = take(f2 * (L.nck + 1));
-    L.seg = take(f2 * std::min(ck, nsteps));
+    L.ckpt = take(f1 * (L.nck + 1));
+    L.seg = take(f1 * std::min(ck, nsteps));
+    L.u0 = take(f2);
+    L.u1 = take(f2);
     L.h = take(f2);
     L.p = take(f2);
     L.hp = take(f2);
@@ -520,7 +542,7 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     A.blocks = frozen_blocks(A.rp);
     char *base = static_cast<char *>(aws);
     auto field = [&](size_t o) { return reinterpret_cast<float *>(base + o); };
-    const size_t n2 = 2 * (size_t)n;
+    const size_t n1 = (size_t)n;
     float *ckpt = field(L.ckpt), *seg = field(L.seg), *h = field(L.h), *p = field(L.p), *hp = field(L.hp), *a = field(L.a);
     double *dots = reinterpret_cast<double *>(base + L.dots);
     double *partials = reinterpret_cast<double *>(base + L.partials);
@@ -542,23 +564,22 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     const int rc = framed_cells(c, s);
     if (rc) return rc;
     ADJ_CK(launch_chunk_numbers(c->w.cell_start, A.rp, A.tab.dense, s));
-    ADJ_CK(table(A, ckpt));
+    float *U[2] = {field(L.u0), field(L.u1)};   // the running state: U[cur]
+    int cur = 0;
+    ADJ_CK(table(A, U[0], ckpt));
     // forward: checkpoints every ckpt_every steps, the last segment's states straight into seg
     const int l0_last = (L.nck - 1) * ckpt_every;
-    float *tmp[2] = {hp, a};   // free until the backward pass
-    const float *u = ckpt;
-    for (int l = 0; l < nsteps; ++l) {
-        float *out;
-        if (l + 1 == nsteps) out = ckpt + (size_t)L.nck * n2;
-        else if (l + 1 > l0_last) out = seg + (size_t)(l + 1 - l0_last) * n2;
-        else if ((l + 1) % ckpt_every == 0) out = ckpt + (size_t)((l + 1) / ckpt_every) * n2;
-        else out = tmp[l & 1];
-        ADJ_CK(fwd_step(A, u, h, out, dt));
-        u = out;
+    for (int l = 0; l < nsteps; ++l, cur ^= 1) {
+        float *keep = nullptr;
+        if (l + 1 == nsteps) keep = ckpt + (size_t)L.nck * n1;
+        else if (l + 1 > l0_last) keep = seg + (size_t)(l + 1 - l0_last) * n1;
+        else if ((l + 1) % ckpt_every == 0) keep = ckpt + (size_t)((l + 1) / ckpt_every) * n1;
+        ADJ_CK(fwd_step(A, U[cur], h, U[cur ^ 1], keep, dt));
     }
+    cur ^= 1;   // the state before the last step
     // C^N sits in checkpoint slot nck (the last step always writes a slot)
-    const float *CN = ckpt + (size_t)L.nck * n2;
-    if (C_final_dev) ADJ_CK(launch_pdl(k_adj_scatter, A.blocks, kT, 0, s, perm, A.rp, A.tab, CN, C_final_dev));
+    const float *CN = ckpt + (size_t)L.nck * n1;
+    if (C_final_dev) ADJ_CK(launch_pdl(k_adj_scatter, A.blocks, kT, 0, s, perm, A.rp, A.tab, CN, false, C_final_dev));
     // lambda^N = C^N - C*, J = 1/2 |lambda^N|^2
     ADJ_CK(launch_pdl(k_adj_misfit, A.blocks, kT, 0, s, perm, A.rp, A.tab, CN, C_target_dev, p, partials));
     ADJ_CK(launch_pdl(k_adj_fold, 1, kFoldT, 0, s, partials, nb, dots + (size_t)nsteps * kDots));
@@ -573,13 +594,15 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     for (int sgi = L.nck - 1; sgi >= 0; --sgi) {
         const int l0 = sgi * ckpt_every;
         const int l1 = l0 + ckpt_every < nsteps ? l0 + ckpt_every : nsteps;
-        auto state = [&](int l) { return l == l0 ? ckpt + (size_t)sgi * n2 : seg + (size_t)(l - l0) * n2; };
-        if (sgi < L.nck - 1)
-            for (int l = l0; l + 1 < l1; ++l) ADJ_CK(fwd_step(A, state(l), h, state(l + 1), dt));
-        for (int l = l1 - 1; l >= l0; --l) {
+        auto state = [&](int l) { return l == l0 ? ckpt + (size_t)sgi * n1 : seg + (size_t)(l - l0) * n1; };
+        if (sgi < L.nck - 1) {
+            ADJ_CK(launch_pdl(k_adj_double, A.blocks, kT, 0, s, A.rp, A.tab, (const float *)state(l0), U[cur]));
+            for (int l = l0; l + 1 < l1; ++l, cur ^= 1) ADJ_CK(fwd_step(A, U[cur], h, U[cur ^ 1], state(l + 1), dt));
+        }
+        for (int l = l1 - 1; l >= l0; --l, cur ^= 1) {
             // a = L u, b = L p, hp = p + dt/2 b, then lambda^l = p + dt L hp (into p)
             ps.partials = partials + (size_t)(l - l0) * nb * kDots;
-            ps.x0 = state(l);
+            ps.x0 = U[cur];
             ps.x1 = p;
             ps.base = nullptr;
             ps.out0 = a;
@@ -592,11 +615,13 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
             ps.out0 = nullptr;
             ps.out1 = p;
             ps.step = dt;
+            ps.next = l > l0 ? state(l - 1) : nullptr;
+            ps.next2 = U[cur ^ 1];
             ADJ_CK(pass(A, BACK2, ps));
         }
         ADJ_CK(launch_pdl(k_adj_fold, (unsigned)(l1 - l0), kFoldT, 0, s, partials, nb, dots + (size_t)l0 * kDots));
     }
-    if (dJdC0_dev) ADJ_CK(launch_pdl(k_adj_scatter, A.blocks, kT, 0, s, perm, A.rp, A.tab, (const float *)p, dJdC0_dev));
+    if (dJdC0_dev) ADJ_CK(launch_pdl(k_adj_scatter, A.blocks, kT, 0, s, perm, A.rp, A.tab, (const float *)p, true, dJdC0_dev));
     std::vector<double> hd(((size_t)nsteps + 1) * kDots);
     ADJ_CK(cudaMemcpyAsync(hd.data(), dots, hd.size() * 8, cudaMemcpyDeviceToHost, s));
     ADJ_CK(cudaStreamSynchronize(s));
