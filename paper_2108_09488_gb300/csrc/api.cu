@@ -212,12 +212,12 @@ int choose_grid(const ade_params &p, double H, int n, Grid *g)
     for (int k = 1; k <= ade::kMaxSubdiv; ++k) {
         Grid t;
         if (!make_grid(p, H, k, &t)) continue;
-        // 3D velocity fields, and where it holds at most 1.5: the finest grid of at least one particle per cell on average (else the coarsest).  Finer
-        // ones leave rows of few candidates and pencils of few particles (us per step at this rule's
-        // choice and one finer: 45^3 jittered, velocity field 504 / 536, weights kept 121 / 205; 64^3 at one
-        // per cell, field 1882 / 2304, weights kept 165 / 179), coarser ones longer ranges.  Other sets keep
-        // the cost model and the full rows (49^3 jittered, 2 per cell, one
-        // rate: 237 us, trimmed at this rule's grid 271; 57^3 C4, 1.1 per cell 294 / 244).
+        // Sets with `finest` (3D velocity fields, and 3D sets for which some grid has 1.0 to 1.5 particles per cell)
+        // take the finest grid of at least one particle per cell on average, or the coarsest where none has.
+        // Finer ones leave rows of few candidates and pencils of few particles (us per step at this rule's
+        // choice and one finer: 45^3 jittered, velocity field 504 / 536; 64^3 at one per cell, field 1882 / 2304),
+        // coarser ones longer ranges.  Other sets keep the cost model and the full rows (49^3 jittered, 2 per
+        // cell, one rate: 237 us, trimmed at this rule's grid 271; 57^3 C4 jittered, 1.1 per cell 294 / 244).
         if (finest) {
             if (found && (double)n < 0.999 * t.ncells) break;
             *g = t;
@@ -823,9 +823,9 @@ int enqueue_frozen(ade_ctx *c, int steps, cudaStream_t s)
 
 // Whether `steps` steps of one call keep the pair weights: filling the table takes 1.5 to 1.9 evaluations of
 // the tuned walk and gives the first predictor, a later evaluation from it takes 0.4 to 0.8, so it pays
-// from the second step on (two steps, us per step: 128^3 1241 against 1465, 1024^2 276 against 285,
-// 512^2 59 against 72, 256^2 23 against 38).  A single step stays with the walks (the cube's would
-// take 1.5 ms).
+// from the second step on (two steps, us per step: 128^3 1319 against 1470, 1024^2 279 against 284,
+// 512^2 57 against 80, 256^2 25 against 38).  A single step stays with the walks (the cube's would
+// take 1.8 ms).
 bool use_frozen(const ade_ctx *c, int steps) { return c->frozen && steps >= 2; }
 
 // Enqueue one predictor-corrector step (Eq. 8-9) and the fold of its diagnostics.
@@ -2600,8 +2600,8 @@ int sweep_begin(ade_sweep *sw, int steps, cudaStream_t s)
     return ADE_OK;
 }
 
-// Whether a call of `steps` steps fills the table: it costs about three evaluations' gain (512^2, 8 sets:
-// 71 us against 95 - 72 per evaluation), so from four evaluations on.
+// Whether a call of `steps` steps fills the table: it costs about two evaluations' gain (512^2, 8 sets:
+// 49 us against 90 - 66 per evaluation) and its memory, so from four evaluations on.
 bool sweep_use_table(const ade_sweep *sw, int steps) { return sw->table && 2 * steps * (int)sw->groups.size() >= 4; }
 
 // The predictors or correctors of every group with the geometry on the fly (one step).

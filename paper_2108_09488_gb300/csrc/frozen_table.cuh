@@ -513,8 +513,8 @@ __device__ __forceinline__ unsigned header_lines(const RateParams &prm) { return
 // first evaluation (the concentrations of the records).  One pass over the rows: the chunk's lines go
 // to its region (prm.fz_stride lines, what nearly every chunk needs: plan_table in api.cu) and only a chunk
 // that outgrows it is done again into room taken from the pool behind; fz_stride 0: no table.
-// Bound: instruction issue.  128^3 cube 1.55 -> 1.15 ms, 1024^2 258 -> 200 us against a
-// form that counted every chunk's lines in a pass of its own.
+// Bound: instruction issue.  128^3 cube 1.27 ms with the first predictor (ncu), 1024^2 204 us; a form that counted
+// every chunk's lines in a pass of its own took 0.4 ms and 55 us more.
 template <int DIM, int KERNEL, bool ISO, int CUT, int VAL, bool FINE = false>
 __device__ __forceinline__ float build_chunk(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs, const RateParams &prm,
                              const Chunk &c, const uint4 &pa, const TrimRow *srow, const FrozenTab &tab,
@@ -624,7 +624,7 @@ __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes)
 // load of the M in flight at once; op.end_row() closes a row.  Lane 0 keeps the stream kAhead lines
 // ahead in L2 with bulk prefetches; the next row's first indices are loaded before the current
 // row's lines.  Bound: memory.  Per evaluation of the 128^3 cube: a loop of four predicated lines 723 us
-// (latency), the switch on the row's length 559, with the prefetches and the early index line 412.  A ring
+// (latency), the switch on the row's length 559, with the prefetches and the early index line 418.  A ring
 // in shared memory filled by asynchronous copies was slower on the cube and at 1024^2 (fewer warps) and
 // 6 % faster at 512^2 only.
 constexpr int kAhead = 32, kPiece = 16;   // lines

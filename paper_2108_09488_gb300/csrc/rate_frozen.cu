@@ -3,7 +3,7 @@
 // In a uniform flow every particle drifts by the same fixed-point word, so the separations -- and
 // with them every weight w_ab of dC_a/dt = sum_b w_ab (C_a - C_b) -- do not change during a run:
 // only C does.  A call that evaluates Eq. 4 more than a few times therefore computes the weights
-// once (k_frozen_build, the pair arithmetic of the walks) into a table in the workspace and each
+// once (k_frozen_build, the pair arithmetic of the walks) into a table in the weights buffer and each
 // evaluation streams them (k_frozen_rate): 4 bytes, two loads and two FP32 operations per pair
 // instead of about 39 instructions.  The table belongs to one call: it is rebuilt from the
 // positions by every call that uses it.
@@ -80,9 +80,9 @@ __global__ __launch_bounds__(kT) void k_frozen_build(const uint4 *__restrict__ P
 }
 
 // One evaluation from the table.  Bound: HBM where the table exceeds L2 (4 bytes per pair and the idle
-// tails of rows), latency below.  Per evaluation, walk / table: 128^3 cube, 250 neighbours, 700 / 412 us
-// (2.6 GB, 6.2 TB/s of the 6.7 a copy reaches); 1024^2, 120 neighbours 124 / 101; 512^2, 60 about 30 / 18.5;
-// 256^2, 28 7.5 / 5.3.  The loads in flight are what the stream lives on: CTAS per SM, 12 (40 registers) on
+// tails of rows), latency below.  Per evaluation, tuned walk / table (ncu, cold caches): 128^3 cube, 250
+// neighbours, 700 / 418 us (2.6 GB, 6.2 TB/s of the 6.7 a copy reaches); 1024^2, 120 neighbours 124 / 98; 512^2,
+// 60 about 35 / 22; 256^2, 28 16 / 10.  The loads in flight are what the stream lives on: CTAS per SM, 12 (40 registers) on
 // large sets and 16 (32, of which three words spill) up to kWideFrom chunk numbers, where a last wave that is
 // nearly empty weighs more (per step, 12 / 16: 512^2 41.8 / 36.3 us, 64^3 175 / 163, 72^3 272 / 253; 100^3
 // 595 / 601, 128^3 955 / 961).

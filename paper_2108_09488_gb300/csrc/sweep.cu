@@ -16,7 +16,7 @@
 // once per group and evaluation (k_sweep_pass); shorter ones (k_rate_sweep) compute them on the fly, with the
 // same operations in the same order, so that a run's bits do not depend on how it is split into calls.  Bound of a pass with 8 sets: the
 // latency of L1 and L2 at 27 % occupancy (32 bytes of concentrations a candidate, 96 registers).
-// 512^2, 60 neighbours, 8 sets, per evaluation: 95 us on the fly, 71 us from the table.
+// 512^2, 60 neighbours, 8 sets, per evaluation: 90 us on the fly, 66 us from the table.
 #include "ade_internal.h"
 
 namespace ade {
@@ -199,9 +199,9 @@ __device__ __noinline__ void walk_sets(const uint4 *__restrict__ P, const uint32
 // One evaluation of one group from the table: predictor (C -> Ch) or corrector (C updated), Eq. 8-9.
 // out.C set (a call's last corrector): the state goes to the caller's order instead, with the positions
 // advanced by prm.inc (the drift of all steps; the first group writes them).
-// Eight sets' sums take up to 96 registers, five CTAs per SM; held to 80 they spill (97 against 75 us a
-// pass at 512^2), and two warps of four sets each on a chunk were slower (94 us: twice the weights'
-// traffic), as were rings of the stream in shared memory (81 us: fewer warps).
+// Eight sets' sums take up to 96 registers, five CTAs per SM; held to 80 they spill, which was a third slower
+// at 512^2, and so were two warps of four sets each on a chunk (twice the weights' traffic) and, a little,
+// rings of the stream in shared memory (fewer warps).
 template <int DIM, int KERNEL, bool ISO, int NT, int EPI>
 __global__ __launch_bounds__(kT, 5) void k_sweep_pass(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
                                                    const RateParams prm, const FrozenTab tab, const ShapeConst sc,
