@@ -100,17 +100,17 @@ KERNEL_FILES = {
     "sweep": ("sweep.cu", "rate_common.cuh", "ade_internal.h"),
 }
 # (workload, walk) -> (DRAM bytes read + written per launch, mean of one predictor and one corrector
-# from an ncu --set full capture, the profile that records it, kernel family, digest of its files)
+# from an ncu capture, the profile that records it, kernel family, digest of its files)
 TRAFFIC_PER_LAUNCH = {
-    ("cube-128-h2", "direct-branch-free-trimmed-paired"): (53.62e6, "profiles/k_rate_cube128.md", "pair", "dd0f33488e40561a"),
+    ("cube-128-h2", "direct-branch-free-trimmed-paired"): (53.30e6, "profiles/k_rate_cube128.md", "pair", "d7325ed398b05adc"),
     ("ladder-1024-n120-r10", "direct-branch-free-trimmed-paired"): (25.13e6, "profiles/k_rate_ladder1024.md", "pair",
-                                                              "dd0f33488e40561a"),
-    ("batched-64", None): (42.19e6, "profiles/k_rate_batch_batched64.md", "batch", "f85a9b4952214a0c"),
+                                                              "d7325ed398b05adc"),
+    ("batched-64", None): (42.04e6, "profiles/k_rate_batch_batched64.md", "batch", "d19ebfc622af6ea9"),
     ("paper-1m-n31k-c4", "direct-branch-free-trimmed-paired"): (16.09e6, "profiles/k_rate_paper1m.md", "pair",
-                                                          "dd0f33488e40561a"),
-    ("field-1024-n120-r10", "velocity-field-direct"): (82.34e6, "profiles/k_rate_field_field1024.md", "field",
-                                                       "33d53e1a706f6232"),
-    ("sweep-512-8", None): (18.25e6, "profiles/k_rate_sweep_sweep512.md", "sweep", "3fed28905bd475a7"),
+                                                          "d7325ed398b05adc"),
+    ("field-1024-n120-r10", "velocity-field-direct"): (80.04e6, "profiles/k_rate_field_field1024.md", "field",
+                                                       "4d4cb01321416fcc"),
+    ("sweep-512-8", None): (18.25e6, "profiles/k_rate_sweep_sweep512.md", "sweep", "35dd25d097d4e40f"),
 }
 
 
