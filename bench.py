@@ -57,7 +57,7 @@ FIELD_VMAX = {"field-1024-n120-r10": 0.2}
 # dispersivity sweep: alpha_T = 1e-3, alpha_L / alpha_T = 1 .. 100, D_m = 1e-6, on the 512^2 rung
 SWEEP_RATIOS = (1, 2, 5, 10, 20, 30, 50, 100)
 # minimum FP32-pipe instructions of the sweep kernel: 12 per pair for the shared geometry
-# (separation, r^2, r, 1 - q, f, u = (vhat . e)^2) and 4 per pair and set (a u + b, f s, C_a - C_b,
+# (separation, r^2, r, 1 - q, f, u = (vhat . e)^2) and 4 per pair and set (the set's weight, C_a - C_b,
 # accumulation)
 SWEEP_GEOM, SWEEP_PER_SET = 12, 4
 ADJ_THETA = (1e-2, 1e-3, 1e-6)

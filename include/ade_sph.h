@@ -191,7 +191,8 @@ int ade_run(ade_ctx *ctx, int nsteps, ade_stats *stats_host, void *stream);
  * 500 expected neighbours with more than 80,000 particles (the walks are as fast there), more than 16 GB
  * counted or 4 GB estimated.
  * ade_set_weights: gives the context a buffer (device, 256-byte aligned, valid until the context is destroyed
- * or another or NULL is set; no work in flight may use the old one).  A smaller buffer than asked for
+ * or another or NULL is set; no work in flight may use the old one, and a graph that
+ * the caller captured goes on using the one set at its capture).  A smaller buffer than asked for
  * holds what fits, and the other particles' weights are evaluated at every step (ADE_ERR_CAPACITY below the
  * part that is not weights).  Needs an ade_weights_bytes since the last change of grid
  * (ADE_ERR_STATE otherwise); ade_autotune takes the buffer away, so ask and set again after it. */

@@ -324,6 +324,7 @@ class _KeptWeights:
 
     _weights = None          # the buffer
     _weights_asked = 0       # 1: estimated, 2: counted, since the last change of grid
+    _weights_captured = ()   # buffers that captured calls use
 
     def _forget_weights(self):
         self._weights, self._weights_asked = None, 0
@@ -335,7 +336,11 @@ class _KeptWeights:
 
     def _keep_weights(self, kind):
         t = self.torch
-        if self._weights_asked == 2 or t.cuda.is_current_stream_capturing():
+        if t.cuda.is_current_stream_capturing():
+            if self._weights is not None:       # the caller's graph will use this buffer as long as the context lives
+                self._weights_captured = self._weights_captured + (self._weights,)
+            return
+        if self._weights_asked == 2:
             return
         nbytes = self._weights_bytes(kind, 0) if self._weights_asked == 0 else 0
         self._weights_asked = 1 if nbytes else 2

@@ -180,3 +180,28 @@ def test_capture_before_the_first_multi_step_call(lib):
     a.step(3)                # and outside it is asked for
     b.step(3)
     assert a._weights is not None and _bits(a.state()[1], b.state()[1])
+
+
+def test_a_captured_call_keeps_its_buffer(lib):
+    """The buffer that a captured call uses stays allocated when later calls get one of another size (or the grid is
+    tuned): the caller's graph can be replayed and writes nowhere else."""
+    import torch
+    xq, C, kw = CASES["2d-jitter"]()
+    a, b = (lib.Simulation(lib.params(**kw), xq, C) for _ in range(2))
+    a.step(3)                                   # the estimated buffer
+    first = a._weights.data_ptr()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        a.step(2)
+    a.step(3)                                   # the counted one
+    assert a._weights.data_ptr() != first
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    others = [torch.zeros(8 << 20, dtype=torch.uint8, device="cuda") for _ in range(16)]
+    g.replay()
+    b.step(3)
+    b.step(3)
+    b.step(2)
+    assert _bits(a.state()[1], b.state()[1])
+    assert not any(o.any() for o in others)
+    assert any(w.data_ptr() == first for w in a._weights_captured)
