@@ -549,7 +549,8 @@ extern "C" int ade_adjoint(ade_ctx *c, const float *C_target_dev, int nsteps, in
     A.tab.words = field(L.total);   // what the caller gave beyond the fields
     A.tab.slots = reinterpret_cast<uint4 *>(base + L.slots);
     A.tab.cursor = reinterpret_cast<unsigned long long *>(base + L.cursor);
-    const bool count = chunk_numbers(n, A.rp.ncy * A.rp.ncz) > kCountChunksFrom;
+    const int pencils = A.rp.ncy * A.rp.ncz, numbers = chunk_numbers(n, pencils);
+    const bool count = numbers > kCountChunksFrom || 4ll * pencils > numbers;   // (as counts_chunks in api.cu)
     A.tab.dense = count ? reinterpret_cast<uint32_t *>(base + L.dense) : nullptr;
     const size_t kept = std::min(aws_bytes - L.total, (size_t)kTableMaxBytes), lines = kept > 256 ? (kept - 256) / 192 : 0;
     A.tab.low = A.tab.words + lines * 32;      // (a line more than half of the table's: 256 bytes)

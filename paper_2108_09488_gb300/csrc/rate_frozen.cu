@@ -82,10 +82,10 @@ __global__ __launch_bounds__(kT) void k_frozen_build(const uint4 *__restrict__ P
 // One evaluation from the table.  Bound: HBM where the table exceeds L2 (4 bytes per pair and the idle
 // tails of rows), latency below.  Per evaluation, tuned walk / table (ncu, cold caches): 128^3 cube, 250
 // neighbours, 700 / 418 us (2.6 GB, 6.2 TB/s of the 6.7 a copy reaches); 1024^2, 120 neighbours 124 / 98; 512^2,
-// 60 about 35 / 22; 256^2, 28 16 / 10.  The loads in flight are what the stream lives on: CTAS per SM, 12 (40 registers) on
-// large sets and 16 (32, of which three words spill) up to kWideFrom chunk numbers, where a last wave that is
-// nearly empty weighs more (per step, 12 / 16: 512^2 41.8 / 36.3 us, 64^3 175 / 163, 72^3 272 / 253; 100^3
-// 595 / 601, 128^3 955 / 961).
+// 60 about 35 / 22; 256^2, 28 16 / 10.  The loads in flight are what the stream lives on: CTAS per SM, 12
+// (40 registers), but 16 (32, of which three words spill) between one wave and kWideFrom chunk numbers, where a
+// last wave that is nearly empty weighs more (per step, 12 / 16: 512^2 41.8 / 36.3 us, 64^3 175 / 163, 72^3 272 /
+// 253; outside of that 256^2 14.1 / 14.8, 45^3 67 / 69, 100^3 595 / 601, 128^3 955 / 961).
 constexpr int kWideFrom = 4 * 152 * 48;
 template <int DIM, int KERNEL, bool ISO, int EPI, int CTAS>
 __global__ __launch_bounds__(kT, CTAS) void k_frozen_rate(const uint4 *__restrict__ P, const uint32_t *__restrict__ cs,
@@ -312,8 +312,9 @@ template <int DIM, int KERNEL, bool ISO>
 cudaError_t rate_t(int epi, const uint4 *P, const uint32_t *cs, const RateParams &prm, const FrozenTab &tab,
                    const FrozenState &st, cudaStream_t s)
 {
+    const int numbers = chunk_numbers(prm.n, prm.ncy * prm.ncz);
     auto go = [&](auto kernel) { return launch_pdl(kernel, frozen_blocks(prm), kT, 0, s, P, cs, prm, tab, st); };
-    if (chunk_numbers(prm.n, prm.ncy * prm.ncz) > kWideFrom)
+    if (numbers <= kCountChunksFrom || numbers > kWideFrom)
         return epi == EPI_PREDICT ? go(k_frozen_rate<DIM, KERNEL, ISO, EPI_PREDICT, 12>) : go(k_frozen_rate<DIM, KERNEL, ISO, EPI_CORRECT, 12>);
     return epi == EPI_PREDICT ? go(k_frozen_rate<DIM, KERNEL, ISO, EPI_PREDICT, 16>) : go(k_frozen_rate<DIM, KERNEL, ISO, EPI_CORRECT, 16>);
 }

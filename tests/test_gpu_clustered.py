@@ -64,6 +64,19 @@ def test_kept_weights_give_the_walks_bits(lib, name, k):
     assert _bits(a.state()[0], b.state()[0]) and _bits(a.state()[1], b.state()[1])
 
 
+@pytest.mark.parametrize("side,h_dx", [(60, 11.0), (113, 9.0), (40, 6.0)])
+def test_long_chunks_on_few_warps(lib, side, h_dx):
+    """Sets of a few hundred chunks with hundreds of neighbours."""
+    p = inputs.Plume(2, side, h_dx, jitter=0.4, seed=3)
+    xq, C = p.initial_state()
+    a = lib.Simulation(lib.params_for(p), xq, C)
+    b = lib.Simulation(lib.params_for(p, cell_subdiv=a.info.cell_subdiv, flags=lib.FLAG_DIRECT), xq, C)
+    for n in (2, 3):
+        a.run(n)
+        b.run(n)
+        assert _bits(a.state()[0], b.state()[0]) and _bits(a.state()[1], b.state()[1])
+
+
 @pytest.mark.parametrize("name", sorted(SETS))
 def test_adjoint_matches_the_oracle(lib, orc, name):
     """J and dJ/d(alpha_L, alpha_T, D_m) at the bars of the adjoint's tests (1e-5, 1e-4)."""
