@@ -38,6 +38,7 @@ __device__ __forceinline__ bool find_chunk(const uint32_t *__restrict__ cs, cons
 {
     const int lane = threadIdx.x & 31, np = prm.ncy * prm.ncz, ncx = prm.ncx;
     const int total = dense ? (int)__ldg(dense + np) : chunk_numbers(prm.n, np);
+    c.local = c.slot = t;      // (also where there is no chunk: put_chunk marks the slot of every number)
     if (t >= total) return false;
     auto first = [&](int q, int &s) {      // the number of pencil q's first chunk; s: its first particle
         s = (int)__ldg(cs + (size_t)q * ncx);
@@ -65,7 +66,6 @@ __device__ __forceinline__ bool find_chunk(const uint32_t *__restrict__ cs, cons
     c.i0 = c.ps + 32 * (t - (dense ? (int)__ldg(dense + c.p) : ((c.ps - prm.goff) >> 5) + c.p));
     c.cy = c.p % prm.ncy;
     c.cz = c.p / prm.ncy;
-    c.local = c.slot = t;
     return c.i0 < c.pe;
 }
 

@@ -205,3 +205,29 @@ def test_a_captured_call_keeps_its_buffer(lib):
     assert _bits(a.state()[1], b.state()[1])
     assert not any(o.any() for o in others)
     assert any(w.data_ptr() == first for w in a._weights_captured)
+
+
+@pytest.mark.parametrize("dim,side,h_dx", [(3, 20, 1.5), (3, 13, 1.5), (2, 100, 1.2)])
+def test_every_slot_is_written(lib, dim, side, h_dx):
+    """Numbers that no chunk has (a count leaves them at the end, gaps lie in between) are marked as such in a
+    buffer that arrives with anything in it: {first particle, pencil's first, pencil's end, pencil}, all 0."""
+    import torch
+    xq, C, kw = _set(dim, side, h_dx, jitter=0.3)
+    a = lib.Simulation(lib.params(**kw), xq, C)
+    b = lib.Simulation(lib.params(cell_subdiv=a.info.cell_subdiv, flags=lib.FLAG_DIRECT, **kw), xq, C)
+    nbytes = _ask(lib, a)
+    _give(lib, a, nbytes, torch)
+    a._weights.fill_(0xff)
+    a.step(2)
+    b.step(2)
+    assert _bits(a.state()[1], b.state()[1])
+    nc, n = a.info.nc, len(C)
+    numbers = (n >> 5) + nc[1] * nc[2]
+    at = -a._weights.data_ptr() % 256 + 256      # the counter's line, then the slots
+    slots = a._weights[at:at + 32 * numbers].cpu().numpy().view(np.int32).reshape(numbers, 8)[:, 4:]
+    none = slots[slots[:, 0] >= slots[:, 2]]
+    assert len(none) > 0 and not none.any()
+    first, _, pe, pencil = slots[slots[:, 0] < slots[:, 2]].T
+    length = np.minimum(first + 32, pe) - first
+    assert np.array_equal(first, np.cumsum(length) - length) and length.sum() == n
+    assert (length > 0).all() and (np.diff(pencil) >= 0).all()
